@@ -70,6 +70,57 @@ __device__ __forceinline__ bool geo_identity(const Geo& g, int seq) { return geo
 __device__ __forceinline__ float ld_as_float(const float* p) { return *p; }
 __device__ __forceinline__ float ld_as_float(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 
+// Programmatic dependent launch.  Every kernel of the library is launched with the attribute that
+// lets it start while its predecessor on the stream still runs, and opens with pdl_wait(), which
+// returns once the predecessor has completed and its writes are visible: nothing but set-up that
+// touches no global memory comes before it.  pdl_launch() lets the successor's CTAs be scheduled as
+// soon as there is room for them; they then wait in their own pdl_wait().  What this hides is launch
+// latency (about 2 us from kernel to kernel becomes about 1), which short calls are made of.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Thread-block clusters: barrier over all threads of the cluster, and loads from another CTA's
+// shared memory (same variable, CTA `rank`).
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_map(const void* p, int rank)
+{
+    uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p)), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float ld_cluster_f32(const float* p, int rank)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_map(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ int ld_cluster_s32(const int* p, int rank)
+{
+    int v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_map(p, rank)) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ float warp_sum(float v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ double warp_sum(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ int warp_sum(int v)
+{
+    return __reduce_add_sync(0xffffffffu, v);
+}
+
 __device__ __forceinline__ float ex2_approx(float x)
 {
     float y;
@@ -128,6 +179,14 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p)
 {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
+
+// 16-byte asynchronous copy global -> shared (cp.async), grouped and waited for per thread.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {

@@ -33,14 +33,6 @@ struct DecodeArgs {
     float* lse;                                      // optional [n_prob][H]: natural log of the normaliser
 };
 
-// 16-byte asynchronous copy global -> shared (cp.async), grouped and waited for per thread.
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // A 16-byte piece of a row as packed fp32 pairs.
 template <typename T> struct DecVec;
 template <> struct DecVec<__nv_bfloat16> {

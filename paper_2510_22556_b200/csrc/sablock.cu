@@ -6,6 +6,8 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <atomic>
+
 #include "common.cuh"
 #include "stages.cuh"
 #include "score_simt.cuh"
@@ -61,7 +63,9 @@ struct Plan {
     bool use_fused;            // the persistent two-sweep kernel (Llama-shaped problems)
     int fu_cpp, fu_groups;     // its CTAs per problem group and number of groups
     int tpc1, tpc2;            // tiles per CTA of the tensor-core passes
+    SimtShape simt;            // shape of the SIMT passes
     int n_chunks;              // pass-1 partials per row
+    int units;                 // row blocks of pass 1 per problem
     int keep_words, long_cap, seg_tiles;
     // workspace offsets
     size_t o_status, o_ticket, o_long_count, o_tile_state, o_keep, o_arrive, o_done, o_top, control_bytes;
@@ -199,9 +203,37 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
         pl->tpc1 = (int)fmin(8.0, fmax(1.0, (double)(work1 / (sms * 4))));
         pl->tpc2 = (int)fmin(4.0, fmax(1.0, (double)(work2 / (sms * 4))));
         pl->n_chunks = (int)((tiles + pl->tpc1 - 1) / pl->tpc1);
+        pl->units = g.Hkv;
     } else {
+        // SIMT passes: as many heads per thread as the KV head has (up to four) and shared memory holds;
+        // pass 1 gets one wave of two CTAs per SM (what shared memory holds at D = 128) and at most
+        // kSimtMaxChunks partials per row.
+        SimtShape& sp = pl->simt;
+        sp.wp_log2 = 0;
+        while ((1 << sp.wp_log2) < p->window) ++sp.wp_log2;
+        sp.tok = kSimtTokLarge;
+        sp.tile = (kSimtThreads >> sp.wp_log2) * sp.tok;
+        sp.gb = g.G >= 3 ? 4 : g.G;
+        while (sp.gb > 1 && simt_smem_bytes(sp.gb, p->window, g.D, sp.tile) > kSimtSmemMax) sp.gb /= 2;
+        sp.batches = (g.G + sp.gb - 1) / sp.gb;
+        const long long units = (long long)g.Hkv * sp.batches;
+        if ((max_L + sp.tile - 1) / sp.tile * units * pl->n_prob < sm_count()) {
+            sp.tok = kSimtTokSmall;
+            sp.tile = (kSimtThreads >> sp.wp_log2) * sp.tok;
+        }
+        sp.smem = simt_smem_bytes(sp.gb, p->window, g.D, sp.tile);
+        const long long tl = (max_L + sp.tile - 1) / sp.tile;
+        long long tpc = (tl * units * pl->n_prob + sm_count() * 2 - 1) / (sm_count() * 2);
+        if (tpc < (tl + kSimtMaxChunks - 1) / kSimtMaxChunks) tpc = (tl + kSimtMaxChunks - 1) / kSimtMaxChunks;
+        sp.tpc = (int)(tpc < 1 ? 1 : tpc);
+        // pass 2 has one CTA per token tile; where that leaves SMs without four CTAs each, the KV heads
+        // of a tile are spread over a cluster
+        sp.split = 1;
+        while (sp.split * 2 <= kSimtMaxSplit && sp.split * 2 <= units && tl * pl->n_prob * sp.split * 2 <= sm_count() * 4LL)
+            sp.split *= 2;
         pl->tpc1 = pl->tpc2 = 1;
-        pl->n_chunks = (max_L + kSimtThreads - 1) / kSimtThreads;
+        pl->n_chunks = (int)((tl + sp.tpc - 1) / sp.tpc);
+        pl->units = (int)units;
     }
     pl->keep_words = (max_L + 31) / 32;
     pl->long_cap = max_L / kSegShort + 1;
@@ -214,7 +246,7 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     pl->o_long_count = take(sizeof(int) * pl->n_prob);
     pl->o_tile_state = take(sizeof(unsigned long long) * (size_t)n_seqs * pl->seg_tiles);
     pl->o_keep = take(sizeof(unsigned) * (size_t)pl->n_prob * pl->keep_words);
-    pl->o_arrive = take(sizeof(int) * (size_t)pl->n_prob * g.Hkv);
+    pl->o_arrive = take(sizeof(int) * (size_t)pl->n_prob * pl->units);
     pl->o_done = take(sizeof(int) * (size_t)pl->n_prob * g.Hkv);
     pl->o_top = take(sizeof(TopScratch) * (size_t)pl->n_prob);
     pl->control_bytes = o;
@@ -227,7 +259,7 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     pl->o_e = take(sizeof(float) * ntok);
     pl->o_sr = take(sizeof(float) * ntok);
     const size_t part_n = pl->use_tc ? (size_t)pl->n_prob * g.Hkv * pl->n_chunks * 128
-                                     : (size_t)pl->n_prob * g.H * g.window * pl->n_chunks;
+                                     : (size_t)pl->n_prob * pl->units * pl->n_chunks * pl->simt.gb * g.window;
     pl->o_part = take(sizeof(float2) * part_n);
     pl->o_lse = take(sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
     pl->o_neg_lse = take(sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
@@ -257,7 +289,47 @@ sablock_status_t check_launch()
     const cudaError_t err = cudaGetLastError();
     return err == cudaSuccess ? SABLOCK_OK : note_cuda_error(err, "kernel launch");
 }
-#define SAB_TRY(expr) do { sablock_status_t _s = (expr); if (_s != SABLOCK_OK) return _s; } while (0)
+
+// Launches a kernel with programmatic stream serialisation (see pdl_wait in common.cuh); `cluster` > 1
+// makes clusters of that many CTAs along x.
+template <typename... KArgs, typename... Args>
+sablock_status_t launch(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int cluster,
+                        Args&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+    ++t_launches;
+    if (err == cudaSuccess) return SABLOCK_OK;
+    cudaGetLastError();
+    return note_cuda_error(err, "kernel launch");
+}
+
+// Raises a kernel's limit of dynamic shared memory, once per device for as long as it suffices.
+template <auto Kern>
+sablock_status_t allow_smem(int bytes)
+{
+    static std::atomic<int> allowed[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return note_cuda_error(cudaGetLastError(), "current device");
+    if (bytes <= allowed[dev].load(std::memory_order_acquire)) return SABLOCK_OK;
+    const cudaError_t err = cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (err != cudaSuccess) {
+        cudaGetLastError();
+        return note_cuda_error(err, "shared memory of a kernel");
+    }
+    int seen = allowed[dev].load();
+    while (seen < bytes && !allowed[dev].compare_exchange_weak(seen, bytes)) { }
+    return SABLOCK_OK;
+}
+#define SAB_TRY(...) do { sablock_status_t _s = (__VA_ARGS__); if (_s != SABLOCK_OK) return _s; } while (0)
 
 // Diagnostic aid: with debug_sync set in the parameter block the pipeline waits for the stream
 // after every stage, so that a device fault is reported with the stage that raised it.
@@ -355,6 +427,24 @@ sablock_status_t launch_p2_tc(const Plan& pl, const CUtensorMap& tmQ, const CUte
     return check_launch();
 }
 
+template <typename T, int GB, int TOK>
+sablock_status_t launch_simt(const Plan& pl, const sablock_params_t* p, const SimtShape& sp, const void* q, const void* k,
+                             const Strides& ks, float c2, const ScoreBufs& sb, float* s, float* e, cudaStream_t stream)
+{
+    const Geo& g = pl.geo;
+    if (!p->row_lse) {
+        SAB_TRY(allow_smem<score_p1_simt<T, GB, TOK>>(sp.smem));
+        SAB_TRY(launch(score_p1_simt<T, GB, TOK>, dim3(pl.n_chunks, pl.units, pl.n_prob), kSimtThreads, sp.smem, stream, 1, g, sp,
+                       (const T*)q, (const T*)k, ks.tok, ks.head, ks.layer, c2, sb));
+    }
+    prof_mark(1, stream);
+    prof_mark(2, stream);
+    SAB_TRY(allow_smem<score_p2_simt<T, GB, TOK>>(sp.smem));
+    const int tiles = (pl.max_L + sp.tile - 1) / sp.tile;
+    return launch(score_p2_simt<T, GB, TOK>, dim3(tiles * sp.split, pl.n_prob), kSimtThreads, sp.smem, stream, sp.split, g, sp,
+                  (const T*)q, (const T*)k, ks.tok, ks.head, ks.layer, c2, p->eps, sb, s, e);
+}
+
 // Stage 2: window scores s (pre-pooling) and per-token entropy e.
 sablock_status_t run_score(const Plan& pl, const sablock_params_t* p, const void* q, const void* k, float* s,
                            float* e, void* ws, cudaStream_t stream)
@@ -365,6 +455,7 @@ sablock_status_t run_score(const Plan& pl, const sablock_params_t* p, const void
     ScoreBufs sb;
     sb.part = at<float2>(ws, pl.o_part);
     sb.lse2 = at<float>(ws, pl.o_lse);
+    sb.arrive = at<int>(ws, pl.o_arrive);
     sb.n_chunks = pl.n_chunks;
     int* status = at<int>(ws, pl.o_status);
     const Strides ks = k_strides(p, g.total_tokens);
@@ -467,46 +558,19 @@ sablock_status_t run_score(const Plan& pl, const sablock_params_t* p, const void
             default: return SABLOCK_ERR_UNSUPPORTED;
         }
     }
-    const int smem1 = (g.window * g.D + 2 * (kSimtThreads / 32) * g.window) * (int)sizeof(float);
-    const int smem2 = (kSimtWChunk * g.D + kSimtWChunk) * (int)sizeof(float);
-    dim3 grid1(pl.n_chunks, g.H, pl.n_prob);
-    dim3 grid2((pl.max_L + kSimtThreads - 1) / kSimtThreads, pl.n_prob);
-    dim3 gridm((g.H * g.window + 127) / 128, pl.n_prob);
-    if (p->dtype == SABLOCK_BF16) {
-        auto k1 = score_p1_simt<__nv_bfloat16>;
-        if (cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1) != cudaSuccess)
-            return SABLOCK_ERR_CUDA;
-        if (!have_lse) {
-            k1<<<grid1, kSimtThreads, smem1, stream>>>(g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, ks.tok, ks.head,
-                                                       ks.layer, c2, sb);
-            SAB_TRY(check_launch());
-        }
-        prof_mark(1, stream);
-        if (!have_lse) {
-            lse_merge_simt<<<gridm, 128, 0, stream>>>(g, sb);
-            SAB_TRY(check_launch());
-        }
-        prof_mark(2, stream);
-        score_p2_simt<__nv_bfloat16><<<grid2, kSimtThreads, smem2, stream>>>(
-            g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, ks.tok, ks.head, ks.layer, c2, p->eps, sb, s, e);
-    } else {
-        auto k1 = score_p1_simt<float>;
-        if (cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1) != cudaSuccess)
-            return SABLOCK_ERR_CUDA;
-        if (!have_lse) {
-            k1<<<grid1, kSimtThreads, smem1, stream>>>(g, (const float*)q, (const float*)k, ks.tok, ks.head, ks.layer, c2, sb);
-            SAB_TRY(check_launch());
-        }
-        prof_mark(1, stream);
-        if (!have_lse) {
-            lse_merge_simt<<<gridm, 128, 0, stream>>>(g, sb);
-            SAB_TRY(check_launch());
-        }
-        prof_mark(2, stream);
-        score_p2_simt<float><<<grid2, kSimtThreads, smem2, stream>>>(g, (const float*)q, (const float*)k, ks.tok,
-                                                                     ks.head, ks.layer, c2, p->eps, sb, s, e);
+    SimtShape sp = pl.simt;
+    sp.vec_q = (reinterpret_cast<uintptr_t>(q) & 15) == 0;              // D * element size is a multiple of 16
+    const int es = elem_size(p);
+    sp.vec_k = ((reinterpret_cast<uintptr_t>(k) | (uintptr_t)(ks.tok * es) | (uintptr_t)(ks.head * es) | (uintptr_t)(ks.layer * es)) & 15) == 0;
+    const bool bf = p->dtype == SABLOCK_BF16;
+#define SAB_SIMT(T, GB) (sp.tok == kSimtTokLarge ? launch_simt<T, GB, kSimtTokLarge>(pl, p, sp, q, k, ks, c2, sb, s, e, stream) \
+                                                 : launch_simt<T, GB, kSimtTokSmall>(pl, p, sp, q, k, ks, c2, sb, s, e, stream))
+    switch (sp.gb) {
+        case 4: return bf ? SAB_SIMT(__nv_bfloat16, 4) : SAB_SIMT(float, 4);
+        case 2: return bf ? SAB_SIMT(__nv_bfloat16, 2) : SAB_SIMT(float, 2);
+        default: return bf ? SAB_SIMT(__nv_bfloat16, 1) : SAB_SIMT(float, 1);
     }
-    return check_launch();
+#undef SAB_SIMT
 }
 
 // Stage 3 (with optional pooling first): s_raw -> s (pooled) -> s_refined.

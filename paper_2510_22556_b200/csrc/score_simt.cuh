@@ -3,23 +3,61 @@
 // row (h, w) over its causal keys (Eq. 2), pass 2 recomputes the logits, normalises, and
 // reduces over heads and window positions per token (Eqs. 3, 4 and the inner sum of Eq. 6).
 // Logits are kept in log2 units: x2 = (q . k) * log2(e) / sqrt(D).
+//
+// Both passes are the same register-tiled product.  A CTA of 256 threads holds a tile of key rows
+// and the window rows of GB query heads of one KV head in shared memory (fp32, rows padded by 16
+// bytes so that the eight lanes of a 16-byte shared-memory phase hit different banks).  A thread
+// owns one window position w and eight tokens and computes GB x 8 logits: the GB heads of a w are
+// summed inside the thread (Eq. 3), and per four elements of D the thread's 8 + GB shared-memory
+// loads feed 16 GB packed multiply-adds, so that with GB = 4 the FMA pipes and not the
+// shared-memory port are the busier unit.  Problems too small to give every SM a tile of that size
+// take two tokens per thread (four times the CTAs, a quarter of the serial work in each).  (One thread per token reading its key row straight from
+// global memory, the way this path used to work, took 225 + 1406 us for the two passes on a
+// 4096-token fp32 layer with 32 / 8 heads of 128; the tiled passes take 50 + 49 us, of which 2 x 17 us
+// are the multiply-adds at full rate and the rest loads that nothing overlaps and the merges.)
 #pragma once
 #include "common.cuh"
 
 namespace sab {
 
-constexpr int kSimtThreads = 128;
-constexpr int kSimtWChunk = 16;
+constexpr int kSimtThreads = 256;
+constexpr int kSimtTokLarge = 8, kSimtTokSmall = 2;     // tokens per thread
 constexpr int kSimtMaxW = 64;
 constexpr int kSimtMaxD = 256;
+constexpr int kSimtMaxSplit = 8;                        // CTAs of a cluster that share the KV heads of a token tile
+constexpr int kSimtMaxChunks = 64;                      // pass-1 partials per window row
+constexpr int kSimtSmemMax = 200 * 1024;
 
 // Partial row statistics of pass 1: (m, l) with m the running maximum (log2 units) and
 // l = sum exp2(x2 - m) over the keys seen.
 struct ScoreBufs {
-    float2* part;          // [n_prob][H*W][n_chunks]   (SIMT)  or [n_prob][Hkv][n_chunks][128] (tensor)
+    float2* part;          // [n_prob][Hkv * head batches][n_chunks][GB * W] (SIMT)  or [n_prob][Hkv][n_chunks][128] (tensor)
     float* lse2;           // [n_prob][H*W]
+    int* arrive;           // zeroed: CTAs that have left their partials, per row block of `part`
     int n_chunks;
 };
+
+// Shape of the SIMT passes for one parameter block.
+struct SimtShape {
+    int gb;                // query heads per thread (4, 2 or 1)
+    int batches;           // ceil(G / gb): units of one KV head
+    int wp_log2;           // window positions rounded up to a power of two: threads along w
+    int tok;               // tokens per thread (kSimtTokLarge or kSimtTokSmall)
+    int tile;              // tokens per tile
+    int smem;              // bytes of dynamic shared memory
+    int tpc;               // pass 1: tiles per CTA
+    int split;             // pass 2: CTAs (of one cluster) per tile
+    int vec_q, vec_k;      // rows start on 16-byte boundaries: loaded as 16-byte vectors
+};
+
+// Query rows, then the key tile; the end of each pass reuses the space for its merge.
+__host__ __device__ inline int simt_smem_bytes(int gb, int W, int D, int tile)
+{
+    const int keys = tile * (D + 4), red = kSimtThreads * gb * 2, sums = tile * (W + 1);
+    int n = gb * W * (D + 4) + (keys > red ? keys : red);
+    if (sums > n) n = sums;
+    return n * (int)sizeof(float);
+}
 
 // Single-sweep mode: the caller knows ln sum_j exp(logit_j) of every window row (the prefill's
 // attention kernel keeps it).  Converts it to the log2 units the score kernels work in, once as it
@@ -27,6 +65,8 @@ struct ScoreBufs {
 __global__ void lse_import_kernel(const float* __restrict__ row_lse, float* __restrict__ lse2,
                                   float* __restrict__ neg_lse2, size_t n)
 {
+    pdl_wait();
+    pdl_launch();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float v = row_lse[i] * 1.4426950408889634f;
@@ -34,156 +74,300 @@ __global__ void lse_import_kernel(const float* __restrict__ row_lse, float* __re
     neg_lse2[i] = -v;
 }
 
+// n_rows rows of D elements (row r at src + r * stride; rows >= n_valid read as row n_valid - 1) into
+// shared memory as fp32, row stride D + 4.  fp32 vectors go by cp.async (no registers, all in
+// flight at once): simt_load_wait() before the barrier.
 template <typename T>
-__global__ void __launch_bounds__(kSimtThreads)
-score_p1_simt(Geo g, const T* __restrict__ q, const T* __restrict__ k, long long ks_tok, long long ks_head,
+__device__ __forceinline__ void simt_load_rows(float* dst, const T* src, long long stride, int n_rows, int n_valid, int D,
+                                               bool vec)
+{
+    if (!vec) {
+        for (int i = threadIdx.x; i < n_rows * D; i += kSimtThreads) {
+            const int r = i / D, c = i - r * D;
+            dst[r * (D + 4) + c] = ld_as_float(src + (long long)min(r, n_valid - 1) * stride + c);
+        }
+        return;
+    }
+    constexpr int E = 16 / (int)sizeof(T);
+    const int vpr = D / E;
+    const int dr = kSimtThreads / vpr, dc = kSimtThreads - dr * vpr;      // what one step of kSimtThreads vectors adds
+    int r = threadIdx.x / vpr, c = threadIdx.x - r * vpr;
+    if constexpr (sizeof(T) == 4) {
+        while (r < n_rows) {
+            cp_async16(smem_u32(dst + r * (D + 4) + c * E), src + (long long)min(r, n_valid - 1) * stride + c * E);
+            r += dr;
+            c += dc;
+            if (c >= vpr) { c -= vpr; ++r; }
+        }
+    } else {
+        while (r < n_rows) {
+            uint4 u[4];
+            int rr[4], cc[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                rr[x] = r;
+                cc[x] = c;
+                u[x] = __ldg(reinterpret_cast<const uint4*>(src + (long long)min(r, n_valid - 1) * stride) + c);
+                r += dr;
+                c += dc;
+                if (c >= vpr) { c -= vpr; ++r; }
+            }
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                if (rr[x] >= n_rows) break;
+                float4* o = reinterpret_cast<float4*>(dst + rr[x] * (D + 4) + cc[x] * E);
+                o[0] = make_float4(__uint_as_float(u[x].x << 16), __uint_as_float(u[x].x & 0xffff0000u),
+                                   __uint_as_float(u[x].y << 16), __uint_as_float(u[x].y & 0xffff0000u));
+                o[1] = make_float4(__uint_as_float(u[x].z << 16), __uint_as_float(u[x].z & 0xffff0000u),
+                                   __uint_as_float(u[x].w << 16), __uint_as_float(u[x].w & 0xffff0000u));
+            }
+        }
+    }
+}
+__device__ __forceinline__ void simt_load_wait()
+{
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+}
+
+// Thread -> (window position, token group).  A warp covers at most 16 window positions: its query
+// loads then touch 16 rows (two shared-memory wavefronts per 16-byte load instead of four) and its
+// key loads two rows (still one wavefront).
+__device__ __forceinline__ void simt_place(int tid, int wp_log2, int& wi, int& tg)
+{
+    const int lo = min(wp_log2, 4), hi = wp_log2 - lo;          // bits of the window position inside and above the warp
+    wi = (tid & ((1 << lo) - 1)) | (((tid >> 5) & ((1 << hi) - 1)) << lo);
+    tg = ((tid & 31) >> lo) | ((tid >> (5 + hi)) << (5 - lo));
+}
+
+// x2[i][b] = c2 * (key row tg + TG i) . (window row of head b at position w)
+template <int GB, int kTok>
+__device__ __forceinline__ void simt_logits(const float* ks, const float* qs, int D, int TG, int tg, int w, int W, float c2,
+                                            float (&x)[kTok][GB])
+{
+    const int ld = D + 4;
+    uint64_t acc[kTok][GB];
+#pragma unroll
+    for (int i = 0; i < kTok; ++i)
+#pragma unroll
+        for (int b = 0; b < GB; ++b) acc[i][b] = pack2(0.f, 0.f);
+    const float* qw = qs + w * ld;
+    const float* kt = ks + tg * ld;
+#pragma unroll 1
+    for (int d = 0; d < D; d += 4) {
+        uint64_t q0[GB], q1[GB];
+#pragma unroll
+        for (int b = 0; b < GB; ++b) {
+            const float4 v = *reinterpret_cast<const float4*>(qw + b * W * ld + d);
+            q0[b] = pack2(v.x, v.y);
+            q1[b] = pack2(v.z, v.w);
+        }
+#pragma unroll
+        for (int i = 0; i < kTok; ++i) {
+            const float4 v = *reinterpret_cast<const float4*>(kt + i * TG * ld + d);
+            const uint64_t k0 = pack2(v.x, v.y), k1 = pack2(v.z, v.w);
+#pragma unroll
+            for (int b = 0; b < GB; ++b) acc[i][b] = fma2(q1[b], k1, fma2(q0[b], k0, acc[i][b]));
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kTok; ++i)
+#pragma unroll
+        for (int b = 0; b < GB; ++b) {
+            float lo, hi;
+            unpack2(acc[i][b], lo, hi);
+            x[i][b] = (lo + hi) * c2;
+        }
+}
+
+// Pass 1.  grid = (chunks, Hkv * batches, problems): row statistics of GB * W window rows over
+// `tpc` token tiles.  The CTA that is the last of a row block to leave its partials merges them, in
+// chunk order, into the rows' log-sum-exps: no launch of its own for the merge.
+template <typename T, int GB, int kTok>
+__global__ void __launch_bounds__(kSimtThreads, 2)
+score_p1_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict__ k, long long ks_tok, long long ks_head,
               long long ks_layer, float c2, ScoreBufs sb)
 {
+    pdl_wait();
+    pdl_launch();
     const int p = blockIdx.z, layer = p / g.n_seqs, seq = p % g.n_seqs;
     if (geo_identity(g, seq)) return;
     const int L = geo_L(g, seq), Tn = L - g.window, W = g.window, D = g.D;
-    const int chunk = blockIdx.x, h = blockIdx.y;
-    if (chunk * kSimtThreads >= L) return;
-    const int j = h / g.G;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    extern __shared__ float smem[];
-    float* qs = smem;                                   // [W][D]
-    float* wm = smem + W * D;                           // [4][W] warp maxima
-    float* wl = wm + (kSimtThreads / 32) * W;           // [4][W] warp sums
-    const T* qh = q + ((size_t)p * g.H + h) * W * D;
-    for (int i = tid; i < W * D; i += kSimtThreads) qs[i] = ld_as_float(qh + i);
-    __syncthreads();
-    const int i_key = chunk * kSimtThreads + tid;
-    const bool in_seq = i_key < L;
-    const T* kr = k + (size_t)layer * ks_layer + ((size_t)g.cu[seq] + (in_seq ? i_key : 0)) * ks_tok +
-                  (size_t)j * ks_head;
-    for (int w0 = 0; w0 < W; w0 += kSimtWChunk) {
-        float acc[kSimtWChunk];
+    const int chunk = blockIdx.x, unit = blockIdx.y, j = unit / sp.batches, b0 = (unit % sp.batches) * GB;
+    const int ntiles = (L + sp.tile - 1) / sp.tile;
+    const int nch = (ntiles + sp.tpc - 1) / sp.tpc;
+    if (chunk >= nch) return;
+    const int nh = min(GB, g.G - b0);                   // heads of this unit
+    extern __shared__ __align__(16) float smem[];
+    float* qs = smem;                                   // [GB * W][D + 4]
+    float* ks = smem + GB * W * (D + 4);                // [tile][D + 4]
+    const int WP = 1 << sp.wp_log2, TG = kSimtThreads >> sp.wp_log2;
+    const int tid = threadIdx.x;
+    int wi, tg;
+    simt_place(tid, sp.wp_log2, wi, tg);
+    const int w = min(wi, W - 1);
+    simt_load_rows(qs, q + ((size_t)p * g.H + j * g.G + b0) * W * D, (long long)D, GB * W, nh * W, D, sp.vec_q != 0);
+    float m[GB], l[GB];
 #pragma unroll
-        for (int u = 0; u < kSimtWChunk; ++u) acc[u] = 0.f;
-        for (int d = 0; d < D; ++d) {
-            const float kd = ld_as_float(kr + d);
+    for (int b = 0; b < GB; ++b) { m[b] = -INFINITY; l[b] = 0.f; }
+    const int t_end = min(ntiles, (chunk + 1) * sp.tpc);
+    for (int tl = chunk * sp.tpc; tl < t_end; ++tl) {
+        const int t0 = tl * sp.tile;
+        if (tl > chunk * sp.tpc) __syncthreads();
+        simt_load_rows(ks, k + (size_t)layer * ks_layer + (size_t)j * ks_head + ((size_t)g.cu[seq] + t0) * ks_tok, ks_tok,
+                       sp.tile, L - t0, D, sp.vec_k != 0);
+        simt_load_wait();
+        float x[kTok][GB];
+        simt_logits<GB, kTok>(ks, qs, D, TG, tg, w, W, c2, x);
+        const int lim = min(L - 1, Tn + w) - t0;        // causal (Eq. 2): tokens of the tile up to here are visible
 #pragma unroll
-            for (int u = 0; u < kSimtWChunk; ++u)
-                if (w0 + u < W) acc[u] = fmaf(qs[(w0 + u) * D + d], kd, acc[u]);
-        }
+        for (int b = 0; b < GB; ++b) {
+            float mx = m[b];
 #pragma unroll
-        for (int u = 0; u < kSimtWChunk; ++u) {
-            const int w = w0 + u;
-            if (w >= W) break;
-            const bool valid = in_seq && i_key <= Tn + w;        // causal (Eq. 2)
-            const float x2 = valid ? acc[u] * c2 : -INFINITY;
-            float m = x2;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            const float ms = (m == -INFINITY) ? 0.f : m;
-            float l = valid ? exp2f(x2 - ms) : 0.f;
-            l = warp_sum(l);
-            if (lane == 0) {
-                wm[warp * W + w] = m;
-                wl[warp * W + w] = l;
+            for (int i = 0; i < kTok; ++i) {
+                if (tg + TG * i > lim) x[i][b] = -INFINITY;
+                mx = fmaxf(mx, x[i][b]);
             }
+            const float ms = mx == -INFINITY ? 0.f : mx;
+            float s = 0.f;
+#pragma unroll
+            for (int i = 0; i < kTok; ++i) s += exp2f(x[i][b] - ms);
+            l[b] = l[b] * exp2f(m[b] - ms) + s;
+            m[b] = mx;
         }
     }
     __syncthreads();
-    if (tid < W) {
-        float m = -INFINITY;
-        for (int x = 0; x < kSimtThreads / 32; ++x) m = fmaxf(m, wm[x * W + tid]);
-        const float ms = (m == -INFINITY) ? 0.f : m;
-        float l = 0.f;
-        for (int x = 0; x < kSimtThreads / 32; ++x) l += wl[x * W + tid] * exp2f(wm[x * W + tid] - ms);
-        sb.part[((size_t)p * g.H * W + (size_t)h * W + tid) * sb.n_chunks + chunk] = make_float2(m, l);
+    // merge over the token groups, in order
+    float2* red = reinterpret_cast<float2*>(ks);        // [TG][GB][WP]: at most 512 entries, the key tile is larger
+#pragma unroll
+    for (int b = 0; b < GB; ++b) red[(tg * GB + b) * WP + wi] = make_float2(m[b], l[b]);
+    __syncthreads();
+    const int rows = GB * W;
+    const size_t blk = (size_t)p * gridDim.y + unit;
+    float2* dst = sb.part + (blk * sb.n_chunks + chunk) * rows;
+    for (int r = tid; r < rows; r += kSimtThreads) {
+        const int b = r / W, wr = r - b * W;
+        float mm = -INFINITY;
+        for (int x = 0; x < TG; ++x) mm = fmaxf(mm, red[(x * GB + b) * WP + wr].x);
+        const float ms = mm == -INFINITY ? 0.f : mm;
+        float ll = 0.f;
+        for (int x = 0; x < TG; ++x) {
+            const float2 v = red[(x * GB + b) * WP + wr];
+            ll += v.y * exp2f(v.x - ms);
+        }
+        dst[r] = make_float2(mm, ll);
+    }
+    __shared__ int s_last;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(sb.arrive + blk, 1) == nch - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const float2* src = sb.part + blk * sb.n_chunks * rows;
+    for (int r = tid; r < nh * W; r += kSimtThreads) {
+        float mm = -INFINITY;
+        for (int c = 0; c < nch; ++c) mm = fmaxf(mm, __ldcg(&src[(size_t)c * rows + r].x));
+        float ll = 0.f;
+        for (int c = 0; c < nch; ++c) {
+            const float2 v = __ldcg(&src[(size_t)c * rows + r]);
+            ll += v.y * exp2f(v.x - mm);
+        }
+        sb.lse2[((size_t)p * g.H + j * g.G + b0) * W + r] = mm + log2f(ll);
     }
 }
 
-// lse2[row] = log2 sum_j exp2(x2_j) from the per-chunk partials, merged in chunk order.
-__global__ void lse_merge_simt(Geo g, ScoreBufs sb)
+// Pass 2.  grid = (token tiles * split, problems), cluster = (split, 1, 1): the CTAs of a cluster
+// take the KV heads of one token tile in turn and add their head sums through distributed shared
+// memory, in rank order; each finishes its share of the tile's tokens.  `split` is 1 where the token
+// tiles alone fill the device.
+template <typename T, int GB, int kTok>
+__global__ void __launch_bounds__(kSimtThreads, 2)
+score_p2_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict__ k, long long ks_tok, long long ks_head,
+              long long ks_layer, float c2, float eps, ScoreBufs sb, float* __restrict__ s_out, float* __restrict__ e_out)
 {
-    const int p = blockIdx.y, seq = p % g.n_seqs;
-    if (geo_identity(g, seq)) return;
-    const int rows = g.H * g.window;
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= rows) return;
-    const int L = geo_L(g, seq);
-    const int nch = (L + kSimtThreads - 1) / kSimtThreads;
-    const float2* pr = sb.part + ((size_t)p * rows + row) * sb.n_chunks;
-    float m = -INFINITY;
-    for (int c = 0; c < nch; ++c) m = fmaxf(m, pr[c].x);
-    float l = 0.f;
-    for (int c = 0; c < nch; ++c) l += pr[c].y * exp2f(pr[c].x - m);
-    sb.lse2[(size_t)p * rows + row] = m + log2f(l);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kSimtThreads)
-score_p2_simt(Geo g, const T* __restrict__ q, const T* __restrict__ k, long long ks_tok, long long ks_head,
-              long long ks_layer, float c2, float eps, ScoreBufs sb, float* __restrict__ s_out,
-              float* __restrict__ e_out)
-{
+    pdl_wait();
+    pdl_launch();
     const int p = blockIdx.y, layer = p / g.n_seqs, seq = p % g.n_seqs;
     if (geo_identity(g, seq)) return;
-    const int L = geo_L(g, seq), Tn = L - g.window, W = g.window, D = g.D, H = g.H;
-    if (blockIdx.x * kSimtThreads >= Tn) return;
+    const int L = geo_L(g, seq), Tn = L - g.window, W = g.window, D = g.D;
+    const int split = sp.split, rank = blockIdx.x % split;
+    const int t0 = (int)(blockIdx.x / split) * sp.tile;
+    if (t0 >= Tn) return;
+    extern __shared__ __align__(16) float smem[];
+    float* qs = smem;
+    float* ks = smem + GB * W * (D + 4);
+    const int WP = 1 << sp.wp_log2, TG = kSimtThreads >> sp.wp_log2;
     const int tid = threadIdx.x;
-    const int t = blockIdx.x * kSimtThreads + tid;
-    const bool live = t < Tn;
-    extern __shared__ float smem[];
-    float* qs = smem;                                   // [kSimtWChunk][D]
-    float* ls = smem + kSimtWChunk * D;                 // [kSimtWChunk]
-    const float* lse = sb.lse2 + (size_t)p * H * W;
-    const size_t tok = (size_t)g.cu[seq] + (live ? t : 0);
-    float abar[kSimtMaxW];
+    int wi, tg;
+    simt_place(tid, sp.wp_log2, wi, tg);
+    const int w = min(wi, W - 1);
+    const float* lse = sb.lse2 + (size_t)p * g.H * W;
+    float abar[kTok];
 #pragma unroll
-    for (int w = 0; w < kSimtMaxW; ++w) abar[w] = 0.f;
+    for (int i = 0; i < kTok; ++i) abar[i] = 0.f;
+    for (int unit = rank; unit < g.Hkv * sp.batches; unit += split) {
+        const int j = unit / sp.batches, b0 = (unit - j * sp.batches) * GB;
+        const int nh = min(GB, g.G - b0);
+        __syncthreads();
+        if (b0 == 0 || split > 1)
+            simt_load_rows(ks, k + (size_t)layer * ks_layer + (size_t)j * ks_head + ((size_t)g.cu[seq] + t0) * ks_tok, ks_tok,
+                           sp.tile, L - t0, D, sp.vec_k != 0);
+        simt_load_rows(qs, q + ((size_t)p * g.H + j * g.G + b0) * W * D, (long long)D, GB * W, nh * W, D, sp.vec_q != 0);
+        float ls[GB];
 #pragma unroll
-    for (int wc = 0; wc < kSimtMaxW / kSimtWChunk; ++wc) {
-        const int w0 = wc * kSimtWChunk;
-        if (w0 >= W) break;
-        float a16[kSimtWChunk];
+        for (int b = 0; b < GB; ++b) ls[b] = b < nh ? lse[(j * g.G + b0 + b) * W + w] : INFINITY;     // exp2(-inf) = 0
+        simt_load_wait();
+        float x[kTok][GB];
+        simt_logits<GB, kTok>(ks, qs, D, TG, tg, w, W, c2, x);
 #pragma unroll
-        for (int u = 0; u < kSimtWChunk; ++u) a16[u] = 0.f;
-        for (int h = 0; h < H; ++h) {
-            __syncthreads();
-            const T* qh = q + (((size_t)p * H + h) * W + w0) * D;
-            const int nw = min(kSimtWChunk, W - w0);
-            for (int i = tid; i < nw * D; i += kSimtThreads) qs[i] = ld_as_float(qh + i);
-            if (tid < nw) ls[tid] = lse[h * W + w0 + tid];
-            __syncthreads();
-            const T* kr = k + (size_t)layer * ks_layer + tok * ks_tok + (size_t)(h / g.G) * ks_head;
-            float acc[kSimtWChunk];
+        for (int i = 0; i < kTok; ++i)
 #pragma unroll
-            for (int u = 0; u < kSimtWChunk; ++u) acc[u] = 0.f;
-            for (int d = 0; d < D; ++d) {
-                const float kd = ld_as_float(kr + d);
-#pragma unroll
-                for (int u = 0; u < kSimtWChunk; ++u)
-                    if (u < nw) acc[u] = fmaf(qs[u * D + d], kd, acc[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < kSimtWChunk; ++u)
-                if (u < nw) a16[u] += exp2f(acc[u] * c2 - ls[u]);      // A[h, w, t]
-        }
-#pragma unroll
-        for (int u = 0; u < kSimtWChunk; ++u) abar[w0 + u] = a16[u];
+            for (int b = 0; b < GB; ++b) abar[i] += exp2f(x[i][b] - ls[b]);        // A[h, w, t], summed over the heads
     }
-    if (!live) return;
-    float tot = 0.f;
+    __syncthreads();
+    // \bar A of this CTA's heads: [token][W + 1], over the key tile and, where that is short, the query rows
+    float* ab = smem;
+    const int ldw = W + 1;
+    if (wi < W)
 #pragma unroll
-    for (int w = 0; w < kSimtMaxW; ++w)
-        if (w < W) tot += abar[w];
-    float ent = 0.f;
-    if (tot > 0.f) {
-        const float inv = 1.f / tot;
-#pragma unroll
-        for (int w = 0; w < kSimtMaxW; ++w)
-            if (w < W) {
-                const float ah = abar[w] * inv;                          // \hat A (Eq. 6)
-                ent -= ah * logf(ah + eps);
-            }
-    }
+        for (int i = 0; i < kTok; ++i) ab[(tg + TG * i) * ldw + w] = abar[i];
+    if (split > 1) cluster_sync(); else __syncthreads();
+    const int lane = tid & 31, warp = tid >> 5;
     const size_t off = (size_t)layer * g.total_tokens + g.cu[seq];
-    s_out[off + t] = tot / (float)H;                                     // Eqs. 3, 4
-    e_out[off + t] = ent;
+    for (int tk = rank + split * warp; tk < sp.tile; tk += split * (kSimtThreads / 32)) {
+        if (t0 + tk >= Tn) break;
+        float a[kSimtMaxW / 32];
+        float tot = 0.f;
+#pragma unroll
+        for (int u = 0; u < kSimtMaxW / 32; ++u) {
+            const int ww = lane + 32 * u;
+            a[u] = 0.f;
+            if (ww < W) {
+                const float* at = ab + tk * ldw + ww;
+                for (int r = 0; r < split; ++r) a[u] += split > 1 ? ld_cluster_f32(at, r) : *at;
+            }
+            tot += a[u];
+        }
+        tot = warp_sum(tot);
+        float ent = 0.f;
+        if (tot > 0.f) {
+            const float inv = 1.f / tot;
+#pragma unroll
+            for (int u = 0; u < kSimtMaxW / 32; ++u)
+                if (lane + 32 * u < W) {
+                    const float ah = a[u] * inv;                         // \hat A (Eq. 6)
+                    ent -= ah * logf(ah + eps);
+                }
+        }
+        ent = warp_sum(ent);
+        if (lane == 0) {
+            s_out[off + t0 + tk] = tot / (float)g.H;                     // Eqs. 3, 4
+            e_out[off + t0 + tk] = ent;
+        }
+    }
+    if (split > 1) cluster_sync();                      // the other CTAs may still read this one's sums
 }
 
 }  // namespace sab

@@ -149,25 +149,6 @@ __global__ void pool_kernel(Geo g, const float* __restrict__ s_in, float* __rest
 // stride over the segment's tokens and combine with a butterfly, so the summation order is
 // fixed and every lane ends with the same value.
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ float warp_sum(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ int warp_sum(int v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 __global__ void __launch_bounds__(256)
 refine_kernel(Geo g, const float* __restrict__ s, const float* __restrict__ e,
               const int* __restrict__ seg_start, const int* __restrict__ n_seg, float alpha, float eta,
