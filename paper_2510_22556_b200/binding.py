@@ -113,11 +113,14 @@ def use_library(path: str):
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    """Device address as an integer: the argument types declared in _load() make a pointer of it."""
+    return None if t is None else t.data_ptr()
 
 
-def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    """Handle of torch's current stream on the current device (the stream object that
+    torch.cuda.current_stream() builds around it costs more than the launch of a kernel)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _check(code: int, where: str):
@@ -125,8 +128,15 @@ def _check(code: int, where: str):
         raise SablockError(code, where)
 
 
+_INT_ARRAYS = {n: C.c_int * n for n in range(1, 66)}       # ctypes builds a class per array length: once each
+
+
 def _iarr(xs: Sequence[int]):
-    return (C.c_int * len(xs))(*[int(x) for x in xs])
+    t = _INT_ARRAYS.get(len(xs)) or C.c_int * len(xs)
+    try:
+        return t(*xs)
+    except TypeError:
+        return t(*[int(x) for x in xs])
 
 
 def make_params(n_q_heads: int, n_kv_heads: int, head_dim: int, window: int, dtype: torch.dtype,
@@ -208,7 +218,7 @@ def segment(p: Params, token_ids: torch.Tensor, ws: torch.Tensor):
     T = L - p.window
     seg_id = torch.empty(max(T, 1), dtype=torch.int32, device=token_ids.device)
     seg_start = torch.empty(max(T, 1) + 1, dtype=torch.int32, device=token_ids.device)
-    n_seg = torch.zeros(1, dtype=torch.int32, device=token_ids.device)
+    n_seg = torch.empty(1, dtype=torch.int32, device=token_ids.device)   # always written
     _check(lib().sablock_segment(C.addressof(p), _ptr(token_ids), L, _ptr(seg_id), _ptr(seg_start), _ptr(n_seg),
                                  _ptr(ws), ws.numel(), _stream()), "sablock_segment")
     return seg_id, seg_start, n_seg
@@ -276,7 +286,7 @@ def compress(p: Params, q_win: torch.Tensor, k: torch.Tensor, v: torch.Tensor, t
     out_k = torch.empty((n,) + tuple(k.shape[1:]), dtype=k.dtype, device=k.device)
     out_v = torch.empty_like(out_k)
     out_idx = torch.empty(n, dtype=torch.int32, device=k.device)
-    n_keep = torch.zeros(1, dtype=torch.int32, device=k.device)
+    n_keep = torch.empty(1, dtype=torch.int32, device=k.device)          # always written
     cand = _iarr(candidates)
     _check(lib().sablock_compress(C.addressof(p), _ptr(q_win), _ptr(k), _ptr(v), _ptr(token_ids), L, budget, cand,
                                   len(candidates), _ptr(out_k), _ptr(out_v), _ptr(out_idx), _ptr(n_keep), _ptr(ws),
