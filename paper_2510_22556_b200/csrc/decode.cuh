@@ -1,8 +1,9 @@
 // Decoding over a (compacted) cache: attention of one new query token per problem against the
 // cache rows, grouped-query attention (Eqs. 1-2 with a single query row; Sec. 4.4 measures
 // decoding over the compressed cache against the full one).  The work is a stream over K and V
-// with 2 * G flops per loaded element (G = query heads per KV head, 4 for Llama-3-8B), far below
-// the tensor-core ridge, so it runs on plain FMAs with 16-byte coalesced loads.
+// with 2 * G flops per loaded element (G = query heads per KV head, 4 for Llama-3-8B).  fp32 caches
+// run on plain FMAs (decode_partial_kernel), bf16 caches on warp-level matrix instructions
+// (decode_mma_kernel, further down); everything below up to there is the fp32 kernel.
 //
 // grid = (splits, KV heads, problems).  Inside a CTA a row of K or V is read by the 8, 16 or 32
 // lanes that together hold its 128, 256 or 512 bytes; each such group of lanes runs an online
@@ -18,6 +19,8 @@ constexpr int kDecThreads = 256;
 constexpr int kDecMaxSplits = 512;
 constexpr int kDecMaxD = 256;
 constexpr int kDecMaxG = 4;
+constexpr int kDecClusterRows = 8192;
+constexpr int kDecMaxCluster = 8;                    // CTAs that merge through distributed shared memory
 
 struct DecodeArgs {
     const void* q;                                   // [n_prob][H][D]
@@ -35,15 +38,6 @@ struct DecodeArgs {
 
 // A 16-byte piece of a row as packed fp32 pairs.
 template <typename T> struct DecVec;
-template <> struct DecVec<__nv_bfloat16> {
-    static constexpr int kElems = 8;
-    __device__ static void unpack(const uint4 u, uint64_t (&x)[4])
-    {
-        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) x[i] = pack2u(w[i] << 16, w[i] & 0xffff0000u);   // bf16 -> fp32 is a shift of the bit pattern
-    }
-};
 template <> struct DecVec<float> {
     static constexpr int kElems = 4;
     __device__ static void unpack(const uint4 u, uint64_t (&x)[2])
@@ -76,6 +70,8 @@ decode_partial_kernel(DecodeArgs a)
     static_assert(LPK == 8 || LPK == 16 || LPK == 32, "row of 128, 256 or 512 bytes");
     const int split = blockIdx.x, j = blockIdx.y, p = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_wait();
+    pdl_launch();
     const int n = a.n_valid ? min(a.n_valid[p], a.n_rows) : a.n_rows;
     const int r0 = split * a.rows_per_split, r1 = min(r0 + a.rows_per_split, n);
     const int group = tid / LPK, piece = tid % LPK;
@@ -249,6 +245,249 @@ decode_partial_kernel(DecodeArgs a)
     }
 }
 
+// ---- bf16 caches ------------------------------------------------------------------------------------
+// The products run as warp-level matrix instructions (m16n8k16, bf16 inputs, fp32 accumulation): the
+// plain-FMA kernel above spends about 20 instructions per 16-byte piece on unpacking, multiply-adds
+// and the shuffles of the dot products, which held a full 128K cache at 53 % of the measured copy
+// bandwidth; here a 16-row chunk of K and V (8 KB at D = 128) costs a warp about 110.  The tile is far
+// too small for tcgen05 (four query rows) and the kernel is bound by DRAM.
+//
+// No precision is given up for it.  The logits are fp32 sums of exact bf16 products as before.  The
+// weights stay fp32: each is split into three bf16 pieces (24 bits, the whole fp32 mantissa) that go
+// through the same instruction in different rows of its 16-row A operand.  Row r of A belongs to head
+// r & 3: rows 0-3 carry the leading pieces, rows 8-11 the middle ones (same thread), rows 4-7 the last
+// ones (lanes 16-31, which see the same logits because the query rows are loaded twice); the three
+// partial sums are added at the end.
+//
+// A warp walks the 16-row chunks warp, warp + 4, ... of its CTA's rows on its own: cp.async into a
+// private ring of kDecMmaStages chunks (swizzled so that ldmatrix is free of bank conflicts), its own
+// online softmax, no barrier in the loop.  The running maximum only moves when a logit exceeds it by
+// 2^8, so that rescaling is rare and costs one vote otherwise.
+//
+// CL = true: the CTAs of a (problem, KV head) are a cluster and merge through distributed shared
+// memory; one launch, no scratch.  CL = false: partials to scratch, merged by decode_merge_kernel.
+constexpr int kDecMmaThreads = 128;
+constexpr int kDecMmaWarps = kDecMmaThreads / 32;
+constexpr int kDecMmaStages = 3;
+__host__ __device__ constexpr int dec_mma_smem(int D) { return kDecMmaWarps * kDecMmaStages * 2 * 16 * D * 2; }
+
+__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4])
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4])
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
+{
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+template <int G, int D, bool CL>
+__global__ void __launch_bounds__(kDecMmaThreads, D == 256 ? 1 : 2)
+decode_mma_kernel(DecodeArgs a)
+{
+    constexpr int PR = D / 8;                        // 16-byte pieces of a row
+    constexpr int KS = D / 16;                       // k-steps of the logits
+    constexpr uint32_t kOp = 16 * D * 2;             // bytes of a chunk of K or V
+    const int split = blockIdx.x, j = blockIdx.y, p = blockIdx.z;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_wait();
+    pdl_launch();
+    const int n = a.n_valid ? min(a.n_valid[p], a.n_rows) : a.n_rows;
+    const int r0 = split * a.rows_per_split, r1 = min(r0 + a.rows_per_split, n);
+    const int n_it = r1 > r0 ? ((r1 - r0 + 15) / 16 - warp + kDecMmaWarps - 1) / kDecMmaWarps : 0;
+
+    extern __shared__ __align__(128) uint8_t dec_ring[];
+    const uint32_t ring = smem_u32(dec_ring) + warp * kDecMmaStages * 2 * kOp;
+    using bf16 = __nv_bfloat16;
+    const bf16* kb = static_cast<const bf16*>(a.k) + (size_t)p * a.k_prob + (size_t)j * a.k_head;
+    const bf16* vb = static_cast<const bf16*>(a.v) + (size_t)p * a.v_prob + (size_t)j * a.v_head;
+
+    // chunk `it` of this warp into its stage; rows beyond the split read its last row and are masked later
+    auto issue = [&](int it) {
+        if (it < n_it) {
+            const int b = r0 + (it * kDecMmaWarps + warp) * 16;
+            const uint32_t dst = ring + (uint32_t)(it % kDecMmaStages) * 2 * kOp;
+            const int pc = lane % PR;
+#pragma unroll
+            for (int i = 0; i < PR / 2; ++i) {
+                const int r = lane / PR + i * (32 / PR);
+                const long long row = min(b + r, r1 - 1);
+                const uint32_t o = dst + (uint32_t)(r * PR + (pc ^ (r & 7))) * 16;
+                cp_async16(o, kb + row * a.k_row + pc * 8);
+                cp_async16(o + kOp, vb + row * a.v_row + pc * 8);
+            }
+        }
+        cp_async_commit();
+    };
+#pragma unroll
+    for (int t = 0; t < kDecMmaStages - 1; ++t) issue(t);
+
+    const int hh = (lane >> 2) & 3;                  // head of this thread's row of A
+    uint32_t qa[KS][2];
+    {
+        const bf16* qg = static_cast<const bf16*>(a.q) + ((size_t)p * a.H + (size_t)j * G + min(hh, G - 1)) * D + 2 * (lane & 3);
+        const bool vec = (reinterpret_cast<uintptr_t>(a.q) & 3) == 0;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                const bf16* s = qg + ks * 16 + x * 8;
+                qa[ks][x] = vec ? *reinterpret_cast<const uint32_t*>(s)
+                                : (uint32_t)__bfloat16_as_ushort(s[0]) | ((uint32_t)__bfloat16_as_ushort(s[1]) << 16);
+            }
+    }
+    float m = -INFINITY, l = 0.f;
+    float acc[D / 8][4];
+#pragma unroll
+    for (int i = 0; i < D / 8; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
+
+    const int lr = lane & 7, mat = lane >> 3;
+    for (int it = 0; it < n_it; ++it) {
+        issue(it + kDecMmaStages - 1);
+        cp_async_wait<kDecMmaStages - 1>();
+        __syncwarp();
+        const uint32_t ks_base = ring + (uint32_t)(it % kDecMmaStages) * 2 * kOp, vs_base = ks_base + kOp;
+        float c[2][4];
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) c[x][e] = 0.f;
+        {
+            const int row = lr + 8 * (mat >> 1);
+            const uint32_t base = ks_base + (uint32_t)row * PR * 16;
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) {
+                uint32_t b[4];
+                ldsm_x4(base + (uint32_t)((2 * ks + (mat & 1)) ^ lr) * 16, b);
+                mma_bf16(c[0], qa[ks][0], 0u, qa[ks][1], 0u, b[0], b[1]);
+                mma_bf16(c[1], qa[ks][0], 0u, qa[ks][1], 0u, b[2], b[3]);
+            }
+        }
+        // logits of head hh, rows row0, row0 + 1, row0 + 8, row0 + 9 of the chunk
+        const int left = r1 - (r0 + (it * kDecMmaWarps + warp) * 16) - 2 * (lane & 3);
+        float s[4];
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) s[2 * x + e] = 8 * x + e < left ? c[x][e] * a.c2 : -INFINITY;
+        const float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
+        if (__any_sync(0xffffffffu, mx > m + 8.f)) {
+            float q = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            q = fmaxf(q, __shfl_xor_sync(0xffffffffu, q, 2));
+            const float mn = fmaxf(m, q);
+            const float sc = m == -INFINITY ? 0.f : exp2f(m - mn);
+            m = mn;
+            l *= sc;
+#pragma unroll
+            for (int i = 0; i < D / 8; ++i)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[i][e] *= sc;
+        }
+        const float mr = m == -INFINITY ? 0.f : m;
+        uint32_t pa[4];
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const float p0 = exp2f(s[2 * x] - mr), p1 = exp2f(s[2 * x + 1] - mr);
+            l += p0 + p1;
+            const uint32_t hi = pack_bf16(p0, p1);
+            const float q0 = p0 - __uint_as_float(hi << 16), q1 = p1 - __uint_as_float(hi & 0xffff0000u);
+            const uint32_t mid = pack_bf16(q0, q1);
+            const uint32_t lo = pack_bf16(q0 - __uint_as_float(mid << 16), q1 - __uint_as_float(mid & 0xffff0000u));
+            pa[2 * x] = lane < 16 ? hi : lo;
+            pa[2 * x + 1] = lane < 16 ? mid : 0u;
+        }
+        {
+            const int row = lr + 8 * (mat & 1);
+            const uint32_t base = vs_base + (uint32_t)row * PR * 16;
+#pragma unroll
+            for (int i = 0; i < D / 8; i += 2) {
+                uint32_t b[4];
+                ldsm_x4_trans(base + (uint32_t)((i + (mat >> 1)) ^ lr) * 16, b);
+                mma_bf16(acc[i], pa[0], pa[1], pa[2], pa[3], b[0], b[1]);
+                mma_bf16(acc[i + 1], pa[0], pa[1], pa[2], pa[3], b[2], b[3]);
+            }
+        }
+        __syncwarp();                                // the stage may be refilled
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    // ---- merge: the pieces, the warps (over the ring), then the splits
+    __shared__ float ms[kDecMmaWarps][G], ls[kDecMmaWarps][G];
+    __shared__ float cm[G], cl[G];
+    float (*accs)[G][D] = reinterpret_cast<float (*)[G][D]>(dec_ring);
+    float (*csum)[D] = reinterpret_cast<float (*)[D]>(dec_ring + kDecMmaWarps * G * D * sizeof(float));
+    static_assert((kDecMmaWarps + 1) * G * D * (int)sizeof(float) <= dec_mma_smem(D), "accumulators fit in the ring");
+    l += __shfl_xor_sync(0xffffffffu, l, 1);
+    l += __shfl_xor_sync(0xffffffffu, l, 2);
+#pragma unroll
+    for (int i = 0; i < D / 8; ++i) {
+        const float t0 = __shfl_down_sync(0xffffffffu, acc[i][0], 16), t1 = __shfl_down_sync(0xffffffffu, acc[i][1], 16);
+        if (lane < 16 && hh < G)
+            *reinterpret_cast<float2*>(&accs[warp][hh][i * 8 + 2 * (lane & 3)]) =
+                make_float2(acc[i][0] + (acc[i][2] + t0), acc[i][1] + (acc[i][3] + t1));
+    }
+    if (lane < 16 && (lane & 3) == 0 && hh < G) { ms[warp][hh] = m; ls[warp][hh] = l; }
+    __syncthreads();
+    for (int i = tid; i < G * D; i += kDecMmaThreads) {
+        const int h = i / D, d = i - h * D;
+        float mx = -INFINITY;
+#pragma unroll
+        for (int w = 0; w < kDecMmaWarps; ++w) mx = fmaxf(mx, ms[w][h]);
+        float sum = 0.f, lsum = 0.f;
+#pragma unroll
+        for (int w = 0; w < kDecMmaWarps; ++w) {
+            const float wt = ms[w][h] == -INFINITY ? 0.f : exp2f(ms[w][h] - mx);
+            sum += accs[w][h][d] * wt;
+            lsum += ls[w][h] * wt;
+        }
+        if constexpr (CL) {
+            csum[h][d] = sum;
+            if (d == 0) { cm[h] = mx; cl[h] = lsum; }
+        } else {
+            float* dst = a.part + (((size_t)p * a.H + (size_t)j * G + h) * a.n_splits + split) * (D + 2);
+            dst[d] = sum;
+            if (d == 0) { dst[D] = mx; dst[D + 1] = lsum; }
+        }
+    }
+    if constexpr (CL) {
+        cluster_sync();
+        for (int i = split * kDecMmaThreads + tid; i < G * D; i += a.n_splits * kDecMmaThreads) {
+            const int h = i / D, d = i - h * D;
+            float mr[kDecMaxCluster], M = -INFINITY;
+#pragma unroll
+            for (int r = 0; r < kDecMaxCluster; ++r) {
+                mr[r] = r < a.n_splits ? ld_cluster_f32(&cm[h], r) : -INFINITY;
+                M = fmaxf(M, mr[r]);
+            }
+            float num = 0.f, den = 0.f;
+#pragma unroll
+            for (int r = 0; r < kDecMaxCluster; ++r) {
+                if (r >= a.n_splits) break;
+                const float wt = mr[r] == -INFINITY ? 0.f : exp2f(mr[r] - M);
+                num = fmaf(ld_cluster_f32(&csum[h][d], r), wt, num);
+                den = fmaf(ld_cluster_f32(&cl[h], r), wt, den);
+            }
+            const size_t row = (size_t)p * a.H + (size_t)j * G + h;
+            a.out[row * D + d] = den > 0.f ? num / den : 0.f;
+            if (a.lse && d == 0) a.lse[row] = den > 0.f ? (M + log2f(den)) * 0.6931471805599453f : -INFINITY;
+        }
+        cluster_sync();                              // the other CTAs may still read this one's sums
+    }
+}
+
 // out[p][h][:] = sum over the splits of acc * 2^(m - M) / sum over the splits of l * 2^(m - M).  The
 // weights go through shared memory so that the loads of the D-wide sums are independent of one
 // another; four slices of threads take every fourth split each and are added in slice order, so
@@ -262,6 +501,8 @@ decode_merge_kernel(DecodeArgs a)
     const int D = a.D, ns = a.n_splits;
     const int dpad = blockDim.x / kDecMergeSlices, slice = tid / dpad, d = tid - slice * dpad;
     const float* base = a.part + ((size_t)p * a.H + h) * ns * (D + 2);
+    pdl_wait();
+    pdl_launch();
     __shared__ float w_s[kDecMaxSplits], lw_s[kDecMaxSplits];
     __shared__ float red[kDecMergeSlices * kDecMaxD / 32];
     __shared__ float num_s[kDecMergeSlices][kDecMaxD];

@@ -695,7 +695,7 @@ sablock_status_t run_compact(const Geo& g, int n_prob, const sablock_params_t* p
 }
 
 // ---- decoding over a cache: launch plan ----------------------------------------------------
-struct DecodePlan { int n_splits, rows_per_split; size_t bytes; };
+struct DecodePlan { int n_splits, rows_per_split; bool cluster; size_t bytes; };
 
 sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, DecodePlan* dp)
 {
@@ -705,50 +705,73 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
     const int row_bytes = p->head_dim * elem_size(p);
     if ((G != 1 && G != 2 && G != 4) || p->head_dim > kDecMaxD || (row_bytes != 128 && row_bytes != 256 && row_bytes != 512))
         return SABLOCK_ERR_UNSUPPORTED;
-    // Row splits: at least 256 rows each, and no more CTAs than two waves of the device (two CTAs
-    // per SM are resident): the merge that follows reads one partial result per split.
-    int splits = (n_rows + kDecThreads - 1) / kDecThreads;
-    const long long ctas_wanted = 4LL * sm_count();
     const long long per_split = (long long)p->n_kv_heads * n_prob;
-    const int cap = (int)fmax(1.0, (double)(ctas_wanted / per_split));
-    if (splits > cap) splits = cap;
+    dp->cluster = false;
+    long long splits;
+    if (p->dtype == SABLOCK_BF16) {
+        // One wave of two CTAs per SM, at least 64 rows (one chunk per warp) each.  Up to eight splits
+        // are a cluster that merges on chip.  Beyond that a short cache still goes to clusters of
+        // eight: the rows that a CTA then reads more take less time than the second launch and
+        // the trip through scratch (kDecClusterRows: where the two cost the same).
+        splits = 2LL * sm_count() / per_split;
+        const long long by_rows = (n_rows + 63) / 64;
+        if (splits > by_rows) splits = by_rows;
+        if (splits < 1) splits = 1;
+        if (splits <= kDecMaxCluster || n_rows <= kDecClusterRows) {
+            dp->cluster = true;
+            int c = 1;
+            while (c < splits && c < kDecMaxCluster) c *= 2;
+            splits = c;
+        }
+    } else {
+        // Row splits: at least 256 rows each, and no more CTAs than two waves of the device (two CTAs
+        // per SM are resident): the merge that follows reads one partial result per split.
+        splits = (n_rows + kDecThreads - 1) / kDecThreads;
+        const long long cap = 4LL * sm_count() / per_split;
+        if (splits > cap) splits = cap < 1 ? 1 : cap;
+    }
     if (splits > kDecMaxSplits) splits = kDecMaxSplits;
-    dp->n_splits = splits;
-    dp->rows_per_split = (n_rows + splits - 1) / splits;
-    dp->bytes = align_up(sizeof(float) * (size_t)n_prob * p->n_q_heads * splits * (p->head_dim + 2));
+    dp->n_splits = (int)splits;
+    dp->rows_per_split = (int)((n_rows + splits - 1) / splits);
+    // the scratch of the clustered form is none; a caller's buffer may not be empty
+    dp->bytes = dp->cluster ? 256 : align_up(sizeof(float) * (size_t)n_prob * p->n_q_heads * splits * (p->head_dim + 2));
     return SABLOCK_OK;
 }
 
-template <typename T, int D>
-sablock_status_t launch_decode_d(const DecodeArgs& a, int G, dim3 grid, cudaStream_t st)
+template <int G, int D>
+sablock_status_t launch_decode_f32(const DecodeArgs& a, dim3 grid, cudaStream_t st)
 {
-    void (*kern)(DecodeArgs) = nullptr;
-    switch (G) {
-        case 1: kern = decode_partial_kernel<T, 1, D>; break;
-        case 2: kern = decode_partial_kernel<T, 2, D>; break;
-        case 4: kern = decode_partial_kernel<T, 4, D>; break;
-        default: return SABLOCK_ERR_UNSUPPORTED;
-    }
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecSmemBytes) != cudaSuccess)
-        return note_cuda_error(cudaGetLastError(), "shared memory of the decode kernel");
-    kern<<<grid, kDecThreads, kDecSmemBytes, st>>>(a);
-    return check_launch();
+    SAB_TRY(allow_smem<decode_partial_kernel<float, G, D>>(kDecSmemBytes));
+    return launch(decode_partial_kernel<float, G, D>, grid, kDecThreads, kDecSmemBytes, st, 1, a);
 }
 
-// head_dim * element size is 128, 256 or 512 bytes (checked by decode_plan)
-sablock_status_t launch_decode(const DecodeArgs& a, bool bf16, int G, dim3 grid, cudaStream_t st)
+template <int G, int D>
+sablock_status_t launch_decode_bf16(const DecodeArgs& a, bool cluster, dim3 grid, cudaStream_t st)
+{
+    constexpr int smem = dec_mma_smem(D);
+    if (cluster) {
+        SAB_TRY(allow_smem<decode_mma_kernel<G, D, true>>(smem));
+        return launch(decode_mma_kernel<G, D, true>, grid, kDecMmaThreads, smem, st, a.n_splits, a);
+    }
+    SAB_TRY(allow_smem<decode_mma_kernel<G, D, false>>(smem));
+    return launch(decode_mma_kernel<G, D, false>, grid, kDecMmaThreads, smem, st, 1, a);
+}
+
+// head_dim * element size is 128, 256 or 512 bytes and G is 1, 2 or 4 (checked by decode_plan)
+template <int G>
+sablock_status_t launch_decode(const DecodeArgs& a, bool bf16, bool cluster, dim3 grid, cudaStream_t st)
 {
     if (bf16) {
         switch (a.D) {
-            case 64: return launch_decode_d<__nv_bfloat16, 64>(a, G, grid, st);
-            case 128: return launch_decode_d<__nv_bfloat16, 128>(a, G, grid, st);
-            case 256: return launch_decode_d<__nv_bfloat16, 256>(a, G, grid, st);
+            case 64: return launch_decode_bf16<G, 64>(a, cluster, grid, st);
+            case 128: return launch_decode_bf16<G, 128>(a, cluster, grid, st);
+            case 256: return launch_decode_bf16<G, 256>(a, cluster, grid, st);
         }
     } else {
         switch (a.D) {
-            case 32: return launch_decode_d<float, 32>(a, G, grid, st);
-            case 64: return launch_decode_d<float, 64>(a, G, grid, st);
-            case 128: return launch_decode_d<float, 128>(a, G, grid, st);
+            case 32: return launch_decode_f32<G, 32>(a, grid, st);
+            case 64: return launch_decode_f32<G, 64>(a, grid, st);
+            case 128: return launch_decode_f32<G, 128>(a, grid, st);
         }
     }
     return SABLOCK_ERR_UNSUPPORTED;
@@ -1104,10 +1127,12 @@ sablock_status_t sablock_decode_attention(const sablock_params_t* p, int n_prob,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const dim3 grid(dp.n_splits, p->n_kv_heads, n_prob);
     const int G = p->n_q_heads / p->n_kv_heads;
-    SAB_TRY(launch_decode(a, p->dtype == SABLOCK_BF16, G, grid, st));
+    const bool bf16 = p->dtype == SABLOCK_BF16;
+    SAB_TRY(G == 1 ? launch_decode<1>(a, bf16, dp.cluster, grid, st)
+                   : G == 2 ? launch_decode<2>(a, bf16, dp.cluster, grid, st) : launch_decode<4>(a, bf16, dp.cluster, grid, st));
+    if (dp.cluster) return SABLOCK_OK;
     const int mt = kDecMergeSlices * ((p->head_dim + 31) / 32 * 32);
-    decode_merge_kernel<<<dim3(p->n_q_heads, n_prob), mt, 0, st>>>(a);
-    return check_launch();
+    return launch(decode_merge_kernel, dim3(p->n_q_heads, n_prob), mt, 0, st, 1, a);
 }
 
 sablock_status_t sablock_compress_layers_host(const sablock_params_t* p, int n_layers, int n_seqs, const void* h_q_win,
