@@ -10,6 +10,7 @@
 
 #include "common.cuh"
 #include "stages.cuh"
+#include "select.cuh"
 #include "score_simt.cuh"
 #include "score_tc.cuh"
 #include "score_fused.cuh"
@@ -66,11 +67,10 @@ struct Plan {
     SimtShape simt;            // shape of the SIMT passes
     int n_chunks;              // pass-1 partials per row
     int units;                 // row blocks of pass 1 per problem
-    int keep_words, long_cap, seg_tiles;
+    int keep_words, seg_tiles;
     // workspace offsets
-    size_t o_status, o_ticket, o_long_count, o_tile_state, o_keep, o_arrive, o_done, o_top, control_bytes;
-    size_t o_seg_id, o_seg_start, o_n_seg, o_s_raw, o_s, o_e, o_sr, o_part, o_lse, o_neg_lse, o_thr, o_cut, o_long_list,
-        o_phi, o_fpart, total;
+    size_t o_status, o_ticket, o_tile_state, o_keep, o_arrive, o_done, control_bytes;
+    size_t o_seg_id, o_seg_start, o_n_seg, o_s_raw, o_s, o_e, o_sr, o_part, o_lse, o_neg_lse, o_phi, o_fpart, total;
 };
 
 bool tc_eligible(const sablock_params_t* p)
@@ -235,20 +235,16 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
         pl->n_chunks = (int)((tl + sp.tpc - 1) / sp.tpc);
         pl->units = (int)units;
     }
-    pl->keep_words = (max_L + 31) / 32;
-    pl->long_cap = max_L / kSegShort + 1;
+    pl->keep_words = (max_L + 31) / 32 + kSelMaxCluster + 1;       // every CTA of a problem starts at a word of its own
     pl->seg_tiles = (max_L + kSegTile - 1) / kSegTile;
 
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes); return r; };
     pl->o_status = take(64);
     pl->o_ticket = take(sizeof(int) * n_seqs);
-    pl->o_long_count = take(sizeof(int) * pl->n_prob);
     pl->o_tile_state = take(sizeof(unsigned long long) * (size_t)n_seqs * pl->seg_tiles);
-    pl->o_keep = take(sizeof(unsigned) * (size_t)pl->n_prob * pl->keep_words);
     pl->o_arrive = take(sizeof(int) * (size_t)pl->n_prob * pl->units);
     pl->o_done = take(sizeof(int) * (size_t)pl->n_prob * g.Hkv);
-    pl->o_top = take(sizeof(TopScratch) * (size_t)pl->n_prob);
     pl->control_bytes = o;
     const size_t ntok = (size_t)n_layers * total_tokens;
     pl->o_seg_id = take(sizeof(int) * total_tokens);
@@ -263,9 +259,7 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     pl->o_part = take(sizeof(float2) * part_n);
     pl->o_lse = take(sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
     pl->o_neg_lse = take(sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
-    pl->o_thr = take(sizeof(unsigned) * pl->n_prob);
-    pl->o_cut = take(sizeof(int) * pl->n_prob);
-    pl->o_long_list = take(sizeof(int) * (size_t)pl->n_prob * pl->long_cap);
+    pl->o_keep = take(sizeof(unsigned) * (size_t)pl->n_prob * pl->keep_words);
     pl->o_phi = take(sizeof(double) * ntok);
     pl->o_fpart = take(pl->use_fused ? sizeof(float2) * (size_t)kFuMaxCtas * kFuPartSlots * 128 : 0);
     pl->total = o;
@@ -281,13 +275,6 @@ sablock_status_t note_cuda_error(cudaError_t err, const char* where)
 {
     snprintf(t_cuda_error, sizeof(t_cuda_error), "%s after launch %d: %s", where, t_launches, cudaGetErrorString(err));
     return SABLOCK_ERR_CUDA;
-}
-
-sablock_status_t check_launch()
-{
-    ++t_launches;
-    const cudaError_t err = cudaGetLastError();
-    return err == cudaSuccess ? SABLOCK_OK : note_cuda_error(err, "kernel launch");
 }
 
 // Launches a kernel with programmatic stream serialisation (see pdl_wait in common.cuh); `cluster` > 1
@@ -353,11 +340,9 @@ sablock_status_t run_segment(const Plan& pl, const sablock_params_t* p, const in
     if (!token_ids || !seg_id || !seg_start || !n_seg || !p->delim_bitmap || p->vocab_size <= 0)
         return SABLOCK_ERR_INVALID_ARG;
     dim3 grid(pl.seg_tiles, pl.geo.n_seqs);
-    segment_kernel<<<grid, kSegThreads, 0, stream>>>(pl.geo, token_ids, p->delim_bitmap, p->vocab_size, seg_id,
-                                                     seg_start, n_seg, at<unsigned long long>(ws, pl.o_tile_state),
-                                                     at<int>(ws, pl.o_ticket), pl.seg_tiles, at<int>(ws, pl.o_status),
-                                                     at<int>(ws, pl.o_status) + 1);
-    return check_launch();
+    return launch(segment_kernel, grid, kSegThreads, 0, stream, 1, pl.geo, token_ids, p->delim_bitmap, p->vocab_size, seg_id,
+                  seg_start, n_seg, at<unsigned long long>(ws, pl.o_tile_state), at<int>(ws, pl.o_ticket), pl.seg_tiles,
+                  at<int>(ws, pl.o_status), at<int>(ws, pl.o_status) + 1);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -419,12 +404,10 @@ sablock_status_t launch_p2_tc(const Plan& pl, const CUtensorMap& tmQ, const CUte
     const int n_atoms = pl.geo.D / 64;
     const int smem = 1024 + NST * 2 * n_atoms * kAtomBytes;
     auto kern = score_p2_tc<W, NST>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-        return SABLOCK_ERR_CUDA;
+    SAB_TRY(allow_smem<score_p2_tc<W, NST>>(smem));
     const int tiles = (pl.max_L + kTcTile - 1) / kTcTile;
     dim3 grid((tiles + pl.tpc2 - 1) / pl.tpc2, pl.n_prob);
-    kern<<<grid, kTcThreads, smem, stream>>>(tmQ, tmK, pl.geo, c2, eps, sb, pl.tpc2, s, e, status);
-    return check_launch();
+    return launch(kern, grid, kTcThreads, smem, stream, 1, tmQ, tmK, pl.geo, c2, eps, sb, pl.tpc2, s, e, status);
 }
 
 template <typename T, int GB, int TOK>
@@ -466,8 +449,7 @@ sablock_status_t run_score(const Plan& pl, const sablock_params_t* p, const void
     if (have_lse) {
         if (reinterpret_cast<uintptr_t>(p->row_lse) & 3) return SABLOCK_ERR_INVALID_ARG;
         const size_t n = (size_t)pl.n_prob * g.H * g.window;
-        lse_import_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(p->row_lse, sb.lse2, neg_lse2, n);
-        SAB_TRY(check_launch());
+        SAB_TRY(launch(lse_import_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, stream, 1, p->row_lse, sb.lse2, neg_lse2, n));
     }
     if (pl.use_tc) {
         CUtensorMap tmQ, tmK;
@@ -519,6 +501,10 @@ sablock_status_t run_score(const Plan& pl, const sablock_params_t* p, const void
                 int cpp = n_cta / groups;
                 if (cpp > cls_tiles) cpp = cls_tiles;
                 fa.cpp = cpp; fa.n_groups = groups;
+                if (have_lse) {        // no CTA waits for another: an ordinary launch
+                    SAB_TRY(launch(score_fused_tc, dim3(groups * cpp), kFuThreads, kFuSmemBytes, stream, 1, tmQ, tmK, g, fa));
+                    continue;
+                }
                 Geo geo = g;
                 void* args[] = {&tmQ, &tmK, &geo, &fa};
                 const cudaError_t err = cudaLaunchCooperativeKernel((const void*)score_fused_tc, dim3(groups * cpp),
@@ -538,17 +524,14 @@ sablock_status_t run_score(const Plan& pl, const sablock_params_t* p, const void
         const int n_atoms = g.D / 64;
         const int smem1 = 1024 + (1 + NST1) * n_atoms * kAtomBytes;
         auto k1 = score_p1_tc<NST1>;
-        if (cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1) != cudaSuccess)
-            return SABLOCK_ERR_CUDA;
+        SAB_TRY(allow_smem<score_p1_tc<NST1>>(smem1));
         dim3 grid1(pl.n_chunks, g.Hkv, pl.n_prob);
         if (!have_lse) {
-            k1<<<grid1, kTcThreads, smem1, stream>>>(tmQ, tmK, g, c2, sb, pl.tpc1, status);
-            SAB_TRY(check_launch());
+            SAB_TRY(launch(k1, grid1, kTcThreads, smem1, stream, 1, tmQ, tmK, g, c2, sb, pl.tpc1, status));
         }
         prof_mark(1, stream);
         if (!have_lse) {
-            lse_merge_tc<<<dim3(g.Hkv, pl.n_prob), 128, 0, stream>>>(g, sb, pl.tpc1);
-            SAB_TRY(check_launch());
+            SAB_TRY(launch(lse_merge_tc, dim3(g.Hkv, pl.n_prob), 128, 0, stream, 1, g, sb, pl.tpc1));
         }
         prof_mark(2, stream);
         switch (g.window) {
@@ -580,21 +563,22 @@ sablock_status_t run_score(const Plan& pl, const sablock_params_t* p, const void
 constexpr int kSegGridPer2K = SABLOCK_SEG_GRID_PER_2K;   // CTAs of the per-segment kernels per 2048 tokens of a sequence
 constexpr int kSegGridMax = 32 * kSegGridPer2K;
 
-sablock_status_t run_refine(const Plan& pl, const sablock_params_t* p, const float* s_raw, float* s, const float* e,
+sablock_status_t run_pool(const Plan& pl, const sablock_params_t* p, const float* s_raw, float* s, cudaStream_t stream)
+{
+    if (p->pool_kernel <= 1) return SABLOCK_OK;
+    const int gx = (int)fmin(32.0, fmax(1.0, (double)((pl.max_L + 2047) / 2048)));
+    return launch(pool_kernel, dim3(gx * 4, pl.n_prob), 256, 0, stream, 1, pl.geo, s_raw, s, p->pool_kernel, p->pool_mode);
+}
+
+sablock_status_t run_refine(const Plan& pl, const sablock_params_t* p, const float* s, const float* e,
                             const int* seg_start, const int* n_seg, float* s_ref, float* stats, int stats_stride,
                             cudaStream_t stream)
 {
-    const int gx = (int)fmin(32.0, fmax(1.0, (double)((pl.max_L + 2047) / 2048)));
-    if (p->pool_kernel > 1) {
-        pool_kernel<<<dim3(gx * 4, pl.n_prob), 256, 0, stream>>>(pl.geo, s_raw, s, p->pool_kernel, p->pool_mode);
-        SAB_TRY(check_launch());
-    }
     // one warp per segment, a few dependent loads each: the kernel is latency-bound, so it gets
     // enough warps to keep every SM's warp slots full (about ten segments per warp)
     const int gr = (int)fmin((double)kSegGridMax, fmax(1.0, (double)((pl.max_L + 2047) / 2048) * kSegGridPer2K));
-    refine_kernel<<<dim3(gr, pl.n_prob), 256, 0, stream>>>(pl.geo, s, e, seg_start, n_seg, p->alpha, p->eta, s_ref,
-                                                           stats, stats_stride);
-    return check_launch();
+    return launch(refine_kernel, dim3(gr, pl.n_prob), 256, 0, stream, 1, pl.geo, s, e, seg_start, n_seg, p->alpha, p->eta, s_ref,
+                  stats, stats_stride);
 }
 
 sablock_status_t check_candidates(const int* cand, int n, Cands* out)
@@ -607,67 +591,49 @@ sablock_status_t check_candidates(const int* cand, int n, Cands* out)
     return SABLOCK_OK;
 }
 
-// Stage 4 + index list.
-sablock_status_t run_select(const Plan& pl, const sablock_params_t* p, const float* s_ref, const int* seg_start,
-                            const int* n_seg, const Cands& cands, int* out_idx, int* out_n_keep, int* seg_g,
+// Clusters of c CTAs of the selection kernel that the current device holds at once (SMs come in groups
+// that a cluster cannot straddle, so this is less than SMs / c).
+int select_clusters(int c)
+{
+    static std::atomic<int> cached[64][kSelMaxCluster + 1];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int n = cached[dev][c].load(std::memory_order_relaxed);
+    if (n) return n - 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c, 1024); cfg.blockDim = dim3(kSelThreads); cfg.dynamicSmemBytes = kSelSmemBytes;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = c; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, select_kernel, &cfg) != cudaSuccess || n < 0) {
+        cudaGetLastError();
+        n = sm_count() / (2 * c);
+    }
+    cached[dev][c].store(n + 1, std::memory_order_relaxed);
+    return n;
+}
+
+// Stages 3 and 4 and the index list.  s == NULL: s_ref holds refined scores already.
+sablock_status_t run_select(const Plan& pl, const sablock_params_t* p, const float* s, const float* e, float* s_ref,
+                            const int* seg_start, const int* n_seg, const Cands& cands, int* out_idx, int* out_n_keep, int* seg_g,
                             int* seg_b, int seg_stride, void* ws, cudaStream_t stream)
 {
-    const Geo& g = pl.geo;
-    unsigned* thr = at<unsigned>(ws, pl.o_thr);
-    int* cut = at<int>(ws, pl.o_cut);
-    {
-        // Several CTAs per problem when the problems are few and long; they wait for one another,
-        // hence the cooperative launch (all CTAs co-resident or an error).
-        int ctas = 1;
-        int dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) {
-            // all CTAs of the launch must be co-resident: as many per SM as the kernel's occupancy allows
-            int per_sm = 1;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, topb_kernel, kTopThreads, 0) != cudaSuccess || per_sm < 1)
-                per_sm = 1;
-            ctas = sms * per_sm / pl.n_prob;
-            const int by_len = (pl.max_L + 4 * kTopThreads - 1) / (4 * kTopThreads);      // at least four rounds each
-            if (ctas > by_len) ctas = by_len;
-            if (ctas > kTopMaxCtas) ctas = kTopMaxCtas;
-            if (ctas < 1) ctas = 1;
-        }
-        TopScratch* tsc = at<TopScratch>(ws, pl.o_top);
-        int* status = at<int>(ws, pl.o_status);
-        if (ctas > 1) {
-            Geo geo = g;
-            const float* sr = s_ref;
-            void* args[] = {&geo, &sr, &thr, &cut, &tsc, &status};
-            const cudaError_t err =
-                cudaLaunchCooperativeKernel((const void*)topb_kernel, dim3(ctas, pl.n_prob), dim3(kTopThreads), args, 0, stream);
-            if (err != cudaSuccess) {
-                cudaGetLastError();
-                return note_cuda_error(err, "cooperative launch of the top-B kernel");
-            }
-            ++t_launches;
-        } else {
-            topb_kernel<<<dim3(1, pl.n_prob), kTopThreads, 0, stream>>>(g, s_ref, thr, cut, tsc, status);
-            SAB_TRY(check_launch());
-        }
-    }
-    prof_mark(5, stream);
-    SearchOut so;
-    so.keep = at<unsigned>(ws, pl.o_keep);
-    so.keep_words = pl.keep_words;
-    so.seg_g = seg_g; so.seg_b = seg_b; so.seg_stride = seg_stride;
-    so.long_list = at<int>(ws, pl.o_long_list);
-    so.long_count = at<int>(ws, pl.o_long_count);
-    so.long_cap = pl.long_cap;
-    const int gx = (int)fmin((double)kSegGridMax, fmax(1.0, (double)((pl.max_L + 2047) / 2048) * kSegGridPer2K));
-    search_kernel<<<dim3(gx, pl.n_prob), kSearchWarps * 32, 0, stream>>>(g, cands, s_ref, seg_start, n_seg, thr, cut,
-                                                                        p->tau, so);
-    SAB_TRY(check_launch());
-    search_long_kernel<<<dim3(8, pl.n_prob), kLongThreads, 0, stream>>>(g, cands, s_ref, seg_start, thr, cut, p->tau, so,
-                                                                       at<double>(ws, pl.o_phi));
-    SAB_TRY(check_launch());
-    prof_mark(6, stream);
-    index_kernel<<<pl.n_prob, kIdxThreads, 0, stream>>>(g, so.keep, pl.keep_words, out_idx, out_n_keep,
-                                                        at<int>(ws, pl.o_status));
-    return check_launch();
+    SelectArgs a;
+    a.s = s; a.e = e; a.s_ref = s_ref;
+    a.seg_start = seg_start; a.n_seg = n_seg;
+    a.alpha = p->alpha; a.eta = p->eta; a.tau = p->tau;
+    a.keep = at<unsigned>(ws, pl.o_keep); a.keep_words = pl.keep_words;
+    a.phi = at<double>(ws, pl.o_phi);
+    a.out_idx = out_idx; a.out_n_keep = out_n_keep;
+    a.seg_g = seg_g; a.seg_b = seg_b; a.seg_stride = seg_stride;
+    a.status = at<int>(ws, pl.o_status);
+    SAB_TRY(allow_smem<select_kernel>(kSelSmemBytes));
+    // CTAs per problem: as many as leave all problems' clusters resident at once, at least a thousand
+    // tokens each
+    int c = 1;
+    while (c < kSelMaxCluster && pl.max_L >= 1024 * c * 2 && pl.n_prob <= select_clusters(c * 2)) c *= 2;
+    return launch(select_kernel, dim3(c, pl.n_prob), kSelThreads, kSelSmemBytes, stream, c, pl.geo, cands, a);
 }
 
 sablock_status_t run_compact(const Geo& g, int n_prob, const sablock_params_t* p, const void* k, const void* v,
@@ -690,8 +656,7 @@ sablock_status_t run_compact(const Geo& g, int n_prob, const sablock_params_t* p
          reinterpret_cast<uintptr_t>(out_v)) & 15)
         return SABLOCK_ERR_UNSUPPORTED;
     dim3 grid((g.n_out + c.rows_per_cta - 1) / c.rows_per_cta, n_prob, 2);
-    compact_kernel<<<grid, 256, 0, stream>>>(g, c, out_idx, out_n_keep, n_keep_fixed);
-    return check_launch();
+    return launch(compact_kernel, grid, 256, 0, stream, 1, g, c, out_idx, out_n_keep, n_keep_fixed);
 }
 
 // ---- decoding over a cache: launch plan ----------------------------------------------------
@@ -967,10 +932,8 @@ sablock_status_t sablock_segment_static(const sablock_params_t* p, const int* to
     g.n_layers = g.n_seqs = 1; g.total_tokens = L; g.window = p->window;
     g.H = p->n_q_heads; g.Hkv = p->n_kv_heads; g.D = p->head_dim; g.G = g.H / g.Hkv;
     g.cu[0] = 0; g.cu[1] = L;
-    segment_kernel<<<dim3(n_tiles, 1), kSegThreads, 0, st>>>(g, token_ids, p->delim_bitmap, p->vocab_size, seg_id, seg_start,
-                                                             n_seg, scratch, ticket, n_tiles, status ? status : own_status,
-                                                             nullptr);
-    return check_launch();
+    return launch(segment_kernel, dim3(n_tiles, 1), kSegThreads, 0, st, 1, g, token_ids, p->delim_bitmap, p->vocab_size, seg_id,
+                  seg_start, n_seg, scratch, ticket, n_tiles, status ? status : own_status, nullptr);
 }
 
 sablock_status_t sablock_score(const sablock_params_t* p, const void* q_win, const void* k, int L, const int* seg_start,
@@ -989,7 +952,8 @@ sablock_status_t sablock_score(const sablock_params_t* p, const void* q_win, con
     float* e_buf = e ? e : at<float>(ws, pl.o_e);
     float* s_raw = p->pool_kernel > 1 ? at<float>(ws, pl.o_s_raw) : s;
     SAB_TRY(run_score(pl, p, q_win, k, s_raw, e_buf, ws, st));
-    return run_refine(pl, p, s_raw, s, e_buf, seg_start, n_seg, s_refined, seg_stats, L - p->window, st);
+    SAB_TRY(run_pool(pl, p, s_raw, s, st));
+    return run_refine(pl, p, s, e_buf, seg_start, n_seg, s_refined, seg_stats, L - p->window, st);
 }
 
 sablock_status_t sablock_select(const sablock_params_t* p, const float* s_refined, int L, const int* seg_start,
@@ -1008,8 +972,8 @@ sablock_status_t sablock_select(const sablock_params_t* p, const float* s_refine
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     SAB_TRY(zero_control(pl, ws, st));
     // the retained count is written to workspace (n_seg slot is free here)
-    return run_select(pl, p, s_refined, seg_start, n_seg, cands, out_idx, at<int>(ws, pl.o_n_seg), out_seg_block,
-                      out_seg_budget, L > p->window ? L - p->window : 1, ws, st);
+    return run_select(pl, p, nullptr, nullptr, const_cast<float*>(s_refined), seg_start, n_seg, cands, out_idx,
+                      at<int>(ws, pl.o_n_seg), out_seg_block, out_seg_budget, L > p->window ? L - p->window : 1, ws, st);
 }
 
 sablock_status_t sablock_compact(const sablock_params_t* p, const void* k, const void* v, int L, const int* out_idx,
@@ -1065,11 +1029,10 @@ sablock_status_t sablock_compress_layers(const sablock_params_t* p, int n_layers
     SAB_TRY(run_score(pl, p, q_win, k, s_raw, e, ws, st));
     prof_mark(3, st);
     SAB_TRY(debug_sync(p, "stage score", st));
-    SAB_TRY(run_refine(pl, p, s_raw, s, e, seg_start, n_seg, sr, nullptr, 0, st));
-    prof_mark(4, st);
-    SAB_TRY(debug_sync(p, "stage refine", st));
-    SAB_TRY(run_select(pl, p, sr, seg_start, n_seg, cands, out_idx, out_n_keep, nullptr, nullptr, 0, ws, st));
-    prof_mark(7, st);
+    SAB_TRY(run_pool(pl, p, s_raw, s, st));
+    for (int i = 4; i <= 5; ++i) prof_mark(i, st);       // refinement and Top-B are part of the selection kernel: intervals of zero
+    SAB_TRY(run_select(pl, p, s, e, sr, seg_start, n_seg, cands, out_idx, out_n_keep, nullptr, nullptr, 0, ws, st));
+    for (int i = 6; i <= 7; ++i) prof_mark(i, st);
     SAB_TRY(debug_sync(p, "stage select", st));
     sablock_status_t rc = run_compact(pl.geo, pl.n_prob, p, k, v, out_idx, out_n_keep, 0, out_k, out_v, st);
     prof_mark(8, st);

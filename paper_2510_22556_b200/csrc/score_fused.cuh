@@ -766,6 +766,8 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         tmem_alloc(smem_u32(&sh.tmem_base), kFuTmemCols);
         tmem_relinquish();
     }
+    pdl_wait();
+    pdl_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

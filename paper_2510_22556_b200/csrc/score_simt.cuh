@@ -239,7 +239,7 @@ score_p1_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
     }
     __syncthreads();
     // merge over the token groups, in order
-    float2* red = reinterpret_cast<float2*>(ks);        // [TG][GB][WP]: at most 512 entries, the key tile is larger
+    float2* red = reinterpret_cast<float2*>(ks);        // [TG][GB][WP]: the space is sized for it
 #pragma unroll
     for (int b = 0; b < GB; ++b) red[(tg * GB + b) * WP + wi] = make_float2(m[b], l[b]);
     __syncthreads();
@@ -298,7 +298,7 @@ score_p2_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
     extern __shared__ __align__(16) float smem[];
     float* qs = smem;
     float* ks = smem + GB * W * (D + 4);
-    const int WP = 1 << sp.wp_log2, TG = kSimtThreads >> sp.wp_log2;
+    const int TG = kSimtThreads >> sp.wp_log2;
     const int tid = threadIdx.x;
     int wi, tg;
     simt_place(tid, sp.wp_log2, wi, tg);

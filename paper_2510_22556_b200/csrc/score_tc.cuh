@@ -99,6 +99,8 @@ __global__ void __launch_bounds__(kTcThreads)
 score_p1_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, Geo g, float c2,
             ScoreBufs sb, int tiles_per_cta, int* status)
 {
+    pdl_wait();
+    pdl_launch();
     const int p = blockIdx.z, layer = p / g.n_seqs, seq = p % g.n_seqs;
     if (geo_identity(g, seq)) return;
     const int L = geo_L(g, seq), Tn = L - g.window;
@@ -204,6 +206,8 @@ score_p1_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 // Merge of the per-chunk row statistics into lse2[p][h*W + w] (log2 units), in chunk order.
 __global__ void lse_merge_tc(Geo g, ScoreBufs sb, int tiles_per_cta)
 {
+    pdl_wait();
+    pdl_launch();
     const int p = blockIdx.y, seq = p % g.n_seqs, j = blockIdx.x;
     if (geo_identity(g, seq)) return;
     const int R = g.G * g.window;
@@ -233,6 +237,8 @@ score_p2_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             float eps, ScoreBufs sb, int tiles_per_cta, float* __restrict__ s_out, float* __restrict__ e_out,
             int* status)
 {
+    pdl_wait();
+    pdl_launch();
     const int p = blockIdx.y, layer = p / g.n_seqs, seq = p % g.n_seqs;
     if (geo_identity(g, seq)) return;
     const int L = geo_L(g, seq), Tn = L - W;

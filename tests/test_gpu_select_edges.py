@@ -1,0 +1,69 @@
+"""The selection kernel where its bookkeeping changes: segments around the longest that one warp
+searches, more long segments than its list holds, more segments than shared memory holds starts for, more
+segments to search than one round takes, ranges that do not fit shared memory, prompts that get 1, 2,
+4 or 8 CTAs, and many problems in one call.  Exact against the oracle (integers)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+from paper_2510_22556_b200 import binding as B
+from test_gpu_stages import _select_case, _sync_ok
+
+pytestmark = pytest.mark.gpu
+CANDS = [1, 2, 4, 8, 16, 32]
+
+
+def _lens(total, draw):
+    out, left = [], total
+    while left > 0:
+        n = min(left, int(draw()))
+        out.append(n)
+        left -= n
+    return np.array(out, np.int64)
+
+
+@pytest.mark.parametrize("T,lens,B_tok", [
+    (1024 * 5, [255, 256, 257, 512] * 4, 1500),                     # around the warp's longest segment
+    (60000, [300] * 200, 9000),                                      # two hundred long segments over eight CTAs
+    (30000, [400] * 75, 9000),                                       # more of them in a CTA than its list holds
+    (9000, [1] * 9000, 700),                                         # more segments than starts in shared memory
+    (40000, [4] * 10000, 20000),                                     # thousands of segments to search
+    (40000, [30000, 10000], 3000),                                   # ranges of very different length
+    (33280 + 1, [33280, 1], 2000),                                   # exactly what shared memory holds, and a token more
+    (33281, [33281], 2000),
+    (300000, [25] * 12000, 4000),                                    # longer than eight CTAs hold: scores stay in global memory
+])
+@pytest.mark.parametrize("quantised", [False, True])
+def test_select_bookkeeping(T, lens, B_tok, quantised):
+    lens = np.array(lens, np.int64)
+    if lens.sum() < T:
+        rng = np.random.default_rng(T)
+        lens = np.concatenate([lens, _lens(T - int(lens.sum()), lambda: rng.geometric(1 / 25.0))])
+    _select_case(T, 32, lens, B_tok, CANDS, 0.85, quantised, T + B_tok)
+
+
+@pytest.mark.parametrize("T", [2, 31, 33, 1023, 2015, 2016, 4063, 4064, 8160, 16352])
+def test_select_cluster_sizes(T):
+    rng = np.random.default_rng(T)
+    _select_case(T, 32, _lens(T, lambda: rng.geometric(1 / 25.0)), max(1, T // 7), CANDS, 0.85, False, T)
+
+
+@pytest.mark.parametrize("n_layers,L", [(40, 2500), (20, 9001), (150, 700)])
+def test_select_many_problems(n_layers, L):
+    """One call over many layers: each layer's list equals the oracle's on the library's own scores."""
+    cfg = synth.Config("t", n_layers, 8, 2, 64, 16, (L,), (128,), (1, 2, 4, 8), "bf16", 5000, 8, 2.0, 20, (0.4,), 3)
+    b = synth.make_batch(cfg, device="cuda")
+    p = B.make_params(8, 2, 64, 16, torch.bfloat16, b.bitmap, cfg.vocab)
+    ws = B.alloc_workspace(p, L, L, 1, n_layers)
+    out = B.compress_layers(p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, 128, cfg.candidates, ws)
+    _sync_ok(ws)
+    sr = B.workspace_view(p, ws, "s_refined", L, L, 1, n_layers).cpu().numpy()
+    ns = int(B.workspace_view(p, ws, "n_seg", L, L, 1, n_layers)[0])
+    st = B.workspace_view(p, ws, "seg_start", L, L, 1, n_layers)[: ns + 1].cpu().numpy()
+    T = L - 16
+    for l in range(0, n_layers, 7):
+        r = oracle.select(sr[l, :T].astype(np.float64), st, 112, cfg.candidates, tau=float(np.float32(0.85)))
+        assert out.out_idx[l, 0, :112].cpu().numpy().tolist() == r["keep"].tolist()
+        assert out.out_idx[l, 0, 112:].cpu().numpy().tolist() == list(range(T, L))
