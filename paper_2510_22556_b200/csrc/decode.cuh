@@ -103,7 +103,7 @@ decode_partial_kernel(DecodeArgs a)
     // Every lane of the CTA makes the same number of turns (the shuffles below involve whole warps);
     // a group whose turn lies beyond the split's last row works on masked rows.
     const int n_turns = r1 > r0 ? (r1 - r0 + kGroups * R - 1) / (kGroups * R) : 0;
-    extern __shared__ __align__(16) uint8_t dec_ring[];
+    extern __shared__ __align__(128) uint8_t dec_ring[];
     uint4* ring = reinterpret_cast<uint4*>(dec_ring);      // [stage][piece 0 .. 2R)[thread] x 16 bytes
     // Copies of turn t into its stage of the ring (rows beyond the split read its last row and are
     // masked later); an empty group once the turns are used up keeps the group count in step.

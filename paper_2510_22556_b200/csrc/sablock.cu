@@ -14,6 +14,7 @@
 #include "score_simt.cuh"
 #include "score_tc.cuh"
 #include "score_fused.cuh"
+#include "score_flow.cuh"
 #include "decode.cuh"
 
 using namespace sab;
@@ -62,14 +63,15 @@ struct Plan {
     int n_prob, max_L;
     bool use_tc;
     bool use_fused;            // the persistent two-sweep kernel (Llama-shaped problems)
-    int fu_cpp, fu_groups;     // its CTAs per problem group and number of groups
+    bool use_flow;             // the unit-flow kernel
+    int fl_groups, fl_heads, fl_m, fl_parts, fl_tiles;   // its head groups, heads of a group, tiles per set of an A unit, partials, tiles
     int tpc1, tpc2;            // tiles per CTA of the tensor-core passes
     SimtShape simt;            // shape of the SIMT passes
     int n_chunks;              // pass-1 partials per row
     int units;                 // row blocks of pass 1 per problem
     int keep_words, seg_tiles;
     // workspace offsets
-    size_t o_status, o_ticket, o_tile_state, o_keep, o_arrive, o_done, control_bytes;
+    size_t o_status, o_ticket, o_tile_state, o_keep, o_arrive, o_done, o_fl_ticket, o_bdone, o_carry, control_bytes;
     size_t o_seg_id, o_seg_start, o_n_seg, o_s_raw, o_s, o_e, o_sr, o_part, o_lse, o_neg_lse, o_phi, o_fpart, total;
 };
 
@@ -196,6 +198,27 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     pl->use_tc = p->score_impl == SABLOCK_SCORE_TENSOR || p->score_impl == SABLOCK_SCORE_FUSED ||
                  (p->score_impl == SABLOCK_SCORE_AUTO && tc_eligible(p) && tc_rows_ok);
     const long long tiles = (max_L + kTcTile - 1) / kTcTile;
+    bool flow_ok = pl->use_tc && p->score_impl == SABLOCK_SCORE_AUTO;
+    pl->fl_tiles = (int)tiles;
+    pl->fl_m = tiles <= 256 ? 1 : tiles <= 512 ? 2 : 4;
+    pl->fl_parts = (int)((tiles + 4 * pl->fl_m - 1) / (4 * pl->fl_m));
+    {
+        // head groups: their keys stay at kFlGroupBytes (two sweeps), their window rows at kFlMaxRows
+        const long long head_bytes = (long long)max_L * p->head_dim * 2;
+        // (the workspace is laid out for two sweeps, whether or not the log-sum-exps are given this time)
+        int h = (int)fmax(1.0, (double)(kFlGroupBytes / head_bytes));
+        if (h > kFlMaxRows / (g.G * p->window)) h = kFlMaxRows / (g.G * p->window);
+        if (h > g.Hkv) h = g.Hkv;
+        pl->fl_groups = (g.Hkv + h - 1) / h;
+        pl->fl_heads = (g.Hkv + pl->fl_groups - 1) / pl->fl_groups;
+        pl->fl_groups = (g.Hkv + pl->fl_heads - 1) / pl->fl_heads;
+        if ((long long)pl->fl_groups * n_seqs > kFlMaxSlots) flow_ok = false;
+    }
+    // Two sweeps: only where one group holds all heads.  Longer sequences, whose groups have to wait for one another's
+    // row sums every few microseconds, are faster on the kernels with fixed shares (128K tokens, 32 layers: 3.3
+    // against 4.7 ms).
+    pl->use_flow = flow_ok && (p->row_lse != nullptr || pl->fl_groups == 1);
+    const bool carries = flow_ok && g.Hkv * g.G * p->window > kFlMaxRows;      // (head groups in the single sweep)
     pl->use_fused = pl->use_tc && p->score_impl != SABLOCK_SCORE_TENSOR && fused_eligible(p);
     if (pl->use_tc) {
         long long work1 = tiles * g.Hkv * pl->n_prob, work2 = tiles * pl->n_prob;
@@ -203,7 +226,7 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
         pl->tpc1 = (int)fmin(8.0, fmax(1.0, (double)(work1 / (sms * 4))));
         pl->tpc2 = (int)fmin(4.0, fmax(1.0, (double)(work2 / (sms * 4))));
         pl->n_chunks = (int)((tiles + pl->tpc1 - 1) / pl->tpc1);
-        pl->units = g.Hkv;
+        pl->units = g.Hkv * (flow_ok ? 1 + (pl->fl_parts + kFlMerge - 1) / kFlMerge : 1);
     } else {
         // SIMT passes: as many heads per thread as the KV head has (up to four) and shared memory holds;
         // pass 1 gets one wave of two CTAs per SM (what shared memory holds at D = 128) and at most
@@ -245,6 +268,8 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     pl->o_tile_state = take(sizeof(unsigned long long) * (size_t)n_seqs * pl->seg_tiles);
     pl->o_arrive = take(sizeof(int) * (size_t)pl->n_prob * pl->units);
     pl->o_done = take(sizeof(int) * (size_t)pl->n_prob * g.Hkv);
+    pl->o_fl_ticket = take(sizeof(int));
+    pl->o_bdone = take(carries ? sizeof(int) * (size_t)pl->n_prob * pl->fl_tiles : 0);
     pl->control_bytes = o;
     const size_t ntok = (size_t)n_layers * total_tokens;
     pl->o_seg_id = take(sizeof(int) * total_tokens);
@@ -256,7 +281,9 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     pl->o_sr = take(sizeof(float) * ntok);
     const size_t part_n = pl->use_tc ? (size_t)pl->n_prob * g.Hkv * pl->n_chunks * 128
                                      : (size_t)pl->n_prob * pl->units * pl->n_chunks * pl->simt.gb * g.window;
-    pl->o_part = take(sizeof(float2) * part_n);
+    const size_t flow_n = flow_ok ? (size_t)pl->n_prob * g.Hkv * (pl->fl_parts + (pl->fl_parts + kFlMerge - 1) / kFlMerge) * g.G * g.window : 0;
+    pl->o_part = take(sizeof(float2) * (part_n > flow_n ? part_n : flow_n));
+    pl->o_carry = take(carries ? sizeof(float) * (size_t)kFlCarryRing * pl->fl_tiles * g.window * 128 : 0);
     pl->o_lse = take(sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
     pl->o_neg_lse = take(sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
     pl->o_keep = take(sizeof(unsigned) * (size_t)pl->n_prob * pl->keep_words);
@@ -363,7 +390,7 @@ EncodeTiledFn encode_fn()
 }
 
 sablock_status_t make_tensor_maps(const Plan& pl, const sablock_params_t* p, const void* q, const void* k,
-                                  CUtensorMap* tmQ, CUtensorMap* tmK)
+                                  int q_rows, CUtensorMap* tmQ, CUtensorMap* tmK)
 {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return SABLOCK_ERR_CUDA;
@@ -376,7 +403,7 @@ sablock_status_t make_tensor_maps(const Plan& pl, const sablock_params_t* p, con
     {   // queries as rows: [n_prob * H * W, D]
         cuuint64_t dims[2] = {(cuuint64_t)g.D, (cuuint64_t)pl.n_prob * g.H * g.window};
         cuuint64_t strides[1] = {(cuuint64_t)g.D * 2};
-        cuuint32_t box[2] = {64, 128};
+        cuuint32_t box[2] = {64, (cuuint32_t)q_rows};
         cuuint32_t estr[2] = {1, 1};
         if (enc(tmQ, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(q), dims, strides, box, estr,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -408,6 +435,58 @@ sablock_status_t launch_p2_tc(const Plan& pl, const CUtensorMap& tmQ, const CUte
     const int tiles = (pl.max_L + kTcTile - 1) / kTcTile;
     dim3 grid((tiles + pl.tpc2 - 1) / pl.tpc2, pl.n_prob);
     return launch(kern, grid, kTcThreads, smem, stream, 1, tmQ, tmK, pl.geo, c2, eps, sb, pl.tpc2, s, e, status);
+}
+
+template <int W, int D>
+sablock_status_t run_flow(const Plan& pl, const sablock_params_t* p, const CUtensorMap& tmQ, const CUtensorMap& tmK, float c2,
+                          const ScoreBufs& sb, float* s, float* e, void* ws, cudaStream_t stream)
+{
+    const Geo& g = pl.geo;
+    FlowArgs fa;
+    memset(&fa, 0, sizeof(fa));
+    fa.c2 = c2; fa.eps = p->eps;
+    fa.part = sb.part; fa.max_part_units = pl.fl_parts; fa.max_grp = (pl.fl_parts + kFlMerge - 1) / kFlMerge;
+    fa.two_sweep = p->row_lse == nullptr;
+    fa.neg_lse2 = at<float>(ws, pl.o_neg_lse);
+    fa.row_lse = p->row_lse;
+    fa.arrive = at<int>(ws, pl.o_arrive);
+    fa.done = at<int>(ws, pl.o_done);
+    fa.bdone = at<int>(ws, pl.o_bdone);
+    fa.carry = at<float>(ws, pl.o_carry);
+    fa.max_tiles = pl.fl_tiles;
+    fa.ticket = at<int>(ws, pl.o_fl_ticket);
+    fa.s_out = s; fa.e_out = e; fa.status = at<int>(ws, pl.o_status);
+    long long tiles = 0, units_b = 0;
+    for (int i = 0; i < g.n_seqs; ++i) {
+        const int L = g.cu[i + 1] - g.cu[i];
+        if (L <= g.n_out) continue;                                  // returned unchanged: no scores needed
+        fa.sel[fa.n_sel++] = (unsigned char)i;
+        const int tb = (L - W + kTcTile - 1) / kTcTile;
+        tiles += (L + kTcTile - 1) / kTcTile;
+        units_b += (tb + 3) / 4;
+    }
+    prof_mark(1, stream);
+    prof_mark(2, stream);
+    if (fa.n_sel == 0) return SABLOCK_OK;
+    fa.n_prob = g.n_layers * fa.n_sel;
+    fa.group_heads = pl.fl_heads; fa.n_groups = pl.fl_groups;
+    if (!fa.two_sweep) {                                             // nothing is read twice: as many heads as fit
+        const int h = kFlMaxRows / (g.G * W) < g.Hkv ? kFlMaxRows / (g.G * W) : g.Hkv;
+        fa.n_groups = (g.Hkv + h - 1) / h;
+        fa.group_heads = (g.Hkv + fa.n_groups - 1) / fa.n_groups;
+        fa.n_groups = (g.Hkv + fa.group_heads - 1) / fa.group_heads;
+    }
+    fa.m = pl.fl_m;
+    // A units run ahead of the B units of the same (problem, head group) by about two units per SM
+    const int sms = sm_count();
+    const long long ua = tiles * fa.group_heads / (4LL * fa.m * fa.n_sel) + 1;       // on average
+    fa.lag = fa.two_sweep ? (int)fmin(16.0, (double)((2LL * sms + ua - 1) / ua)) : 0;
+    // four tiles per B unit, or one with the heads spread over the sets where that takes fewer rounds
+    units_b *= g.n_layers;
+    const long long rounds = (units_b + sms - 1) / sms * fa.group_heads * 4, split = (units_b * 4 + sms - 1) / sms * (fa.group_heads + 1);
+    fa.head_split = fa.n_groups == 1 && fa.group_heads >= 4 && split < rounds;
+    SAB_TRY(allow_smem<score_flow_tc<W, D>>(fl_smem(D)));
+    return launch(score_flow_tc<W, D>, dim3(sms), kFlThreads, fl_smem(D), stream, 1, tmQ, tmK, g, fa);
 }
 
 template <typename T, int GB, int TOK>
@@ -446,14 +525,25 @@ sablock_status_t run_score(const Plan& pl, const sablock_params_t* p, const void
     // log of Eq. 2's normaliser per query row): no pass over K for the row statistics.
     const bool have_lse = p->row_lse != nullptr;
     float* neg_lse2 = at<float>(ws, pl.o_neg_lse);
-    if (have_lse) {
-        if (reinterpret_cast<uintptr_t>(p->row_lse) & 3) return SABLOCK_ERR_INVALID_ARG;
+    if (have_lse && (reinterpret_cast<uintptr_t>(p->row_lse) & 3)) return SABLOCK_ERR_INVALID_ARG;
+    if (have_lse && !pl.use_flow) {
         const size_t n = (size_t)pl.n_prob * g.H * g.window;
         SAB_TRY(launch(lse_import_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, stream, 1, p->row_lse, sb.lse2, neg_lse2, n));
     }
     if (pl.use_tc) {
         CUtensorMap tmQ, tmK;
-        SAB_TRY(make_tensor_maps(pl, p, q, k, &tmQ, &tmK));
+        SAB_TRY(make_tensor_maps(pl, p, q, k, pl.use_flow ? (g.G * g.window + 15) / 16 * 16 : 128, &tmQ, &tmK));
+        if (pl.use_flow) {
+            switch (g.window * 256 + g.D) {
+                case 8 * 256 + 64: return run_flow<8, 64>(pl, p, tmQ, tmK, c2, sb, s, e, ws, stream);
+                case 16 * 256 + 64: return run_flow<16, 64>(pl, p, tmQ, tmK, c2, sb, s, e, ws, stream);
+                case 32 * 256 + 64: return run_flow<32, 64>(pl, p, tmQ, tmK, c2, sb, s, e, ws, stream);
+                case 8 * 256 + 128: return run_flow<8, 128>(pl, p, tmQ, tmK, c2, sb, s, e, ws, stream);
+                case 16 * 256 + 128: return run_flow<16, 128>(pl, p, tmQ, tmK, c2, sb, s, e, ws, stream);
+                case 32 * 256 + 128: return run_flow<32, 128>(pl, p, tmQ, tmK, c2, sb, s, e, ws, stream);
+            }
+            return SABLOCK_ERR_UNSUPPORTED;
+        }
         // Persistent two-sweep kernel: groups of CTAs each walk their share of the problems.
         const int tiles_max = (pl.max_L + kTcTile - 1) / kTcTile;
         const int min_cpp = (tiles_max + kFuMaxTilesPerCta - 1) / kFuMaxTilesPerCta;
