@@ -200,7 +200,11 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     const long long tiles = (max_L + kTcTile - 1) / kTcTile;
     bool flow_ok = pl->use_tc && p->score_impl == SABLOCK_SCORE_AUTO;
     pl->fl_tiles = (int)tiles;
-    pl->fl_m = tiles <= 256 ? 1 : tiles <= 512 ? 2 : 4;
+    // A units of sixteen tiles of a head (a query block is loaded per unit, and its partial sums are handed over per
+    // unit: 16 prompts of 4K-16K tokens take 5.3, 4.97 and 4.75 ms with four, eight and sixteen), fewer where that would
+    // leave less than two units per SM
+    const long long m = tiles * g.Hkv * pl->n_prob / (8LL * sm_count());
+    pl->fl_m = (int)(m < 1 ? 1 : m > 4 ? 4 : m);
     pl->fl_parts = (int)((tiles + 4 * pl->fl_m - 1) / (4 * pl->fl_m));
     {
         // head groups: their keys stay at kFlGroupBytes (two sweeps), their window rows at kFlMaxRows
@@ -214,11 +218,14 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
         pl->fl_groups = (g.Hkv + pl->fl_heads - 1) / pl->fl_heads;
         if ((long long)pl->fl_groups * n_seqs > kFlMaxSlots) flow_ok = false;
     }
-    // Two sweeps: only where one group holds all heads.  Longer sequences, whose groups have to wait for one another's
-    // row sums every few microseconds, are faster on the kernels with fixed shares (128K tokens, 32 layers: 3.3
-    // against 4.7 ms).
-    pl->use_flow = flow_ok && (p->row_lse != nullptr || pl->fl_groups == 1);
-    const bool carries = flow_ok && g.Hkv * g.G * p->window > kFlMaxRows;      // (head groups in the single sweep)
+    // Two sweeps with 128 window rows per KV head: only where one group holds all heads.  Between groups the head-summed
+    // attention goes through L2 (16 KB per tile each way, next to 32 KB of keys per head), and the kernel with
+    // fixed shares, which keeps it in tensor memory, is faster: 1.05 against 1.13 ms at 32K, 1.95 against 2.25 ms at
+    // 64K tokens (32 layers).  With 64 rows or fewer that kernel does not apply and the traffic is a quarter or less:
+    // 1.09 -> 0.88 ms against the two-launch kernels at window 8, 1.16 -> 0.99 ms at window 16 (32K, 32 layers).
+    const bool flow_two = pl->fl_groups == 1 || g.G * p->window <= 64;
+    pl->use_flow = flow_ok && (p->row_lse != nullptr || flow_two);
+    const bool carries = flow_ok && (g.Hkv * g.G * p->window > kFlMaxRows || (flow_two && pl->fl_groups > 1));
     pl->use_fused = pl->use_tc && p->score_impl != SABLOCK_SCORE_TENSOR && fused_eligible(p);
     if (pl->use_tc) {
         long long work1 = tiles * g.Hkv * pl->n_prob, work2 = tiles * pl->n_prob;
@@ -477,10 +484,11 @@ sablock_status_t run_flow(const Plan& pl, const sablock_params_t* p, const CUten
         fa.n_groups = (g.Hkv + fa.group_heads - 1) / fa.group_heads;
     }
     fa.m = pl.fl_m;
-    // A units run ahead of the B units of the same (problem, head group) by about two units per SM
+    // A units run ahead of the B units of the same (problem, head group) by about a unit per SM: enough that the row sums
+    // are there in time (what is late is put aside), little enough that the keys are still in L2
     const int sms = sm_count();
     const long long ua = tiles * fa.group_heads / (4LL * fa.m * fa.n_sel) + 1;       // on average
-    fa.lag = fa.two_sweep ? (int)fmin(16.0, (double)((2LL * sms + ua - 1) / ua)) : 0;
+    fa.lag = fa.two_sweep ? (int)fmin(16.0, (double)((sms + ua - 1) / ua)) : 0;
     // four tiles per B unit, or one with the heads spread over the sets where that takes fewer rounds
     units_b *= g.n_layers;
     const long long rounds = (units_b + sms - 1) / sms * fa.group_heads * 4, split = (units_b * 4 + sms - 1) / sms * (fa.group_heads + 1);

@@ -613,13 +613,18 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                         const bool mask = tok0 + kTcTile - 1 > Tn;
                         const int lim = Tn + (r0 & (W - 1));     // causal: key index <= T + w (Eq. 2)
 #pragma unroll 1
-                        for (int c = 0; c < 4; ++c) {
-                            uint32_t r[32];
-                            tmem_ld32_issue(acc_addr + c * 32, r);
+                        for (int c = 0; c < 4; c += 2) {         // the accumulator is given back with half of the tile still to do
+                            uint32_t ra[32], rb[32];
+                            tmem_ld32_issue(acc_addr + c * 32, ra);
+                            tmem_ld32_issue(acc_addr + c * 32 + 32, rb);
                             tmem_ld_wait();
-                            if (c == 3) release();
-                            if (mask) chunk_mask(r, tok0 + c * 32, lim);
-                            rs.add(r, c2);
+                            if (c == 2) release();
+                            if (mask) {
+                                chunk_mask(ra, tok0 + c * 32, lim);
+                                chunk_mask(rb, tok0 + c * 32 + 32, lim);
+                            }
+                            rs.add(ra, c2);
+                            rs.add(rb, c2);
                         }
                     } else {
                         release();
