@@ -69,9 +69,9 @@ struct Plan {
     SimtShape simt;            // shape of the SIMT passes
     int n_chunks;              // pass-1 partials per row
     int units;                 // row blocks of pass 1 per problem
-    int keep_words, seg_tiles;
+    int keep_words;
     // workspace offsets
-    size_t o_status, o_ticket, o_tile_state, o_keep, o_arrive, o_done, o_fl_ticket, o_bdone, o_carry, control_bytes;
+    size_t o_status, o_keep, o_arrive, o_done, o_fl_ticket, o_bdone, o_carry, control_bytes;
     size_t o_seg_id, o_seg_start, o_n_seg, o_s_raw, o_s, o_e, o_sr, o_part, o_lse, o_neg_lse, o_phi, o_fpart, total;
 };
 
@@ -266,13 +266,10 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
         pl->units = (int)units;
     }
     pl->keep_words = (max_L + 31) / 32 + kSelMaxCluster + 1;       // every CTA of a problem starts at a word of its own
-    pl->seg_tiles = (max_L + kSegTile - 1) / kSegTile;
 
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes); return r; };
     pl->o_status = take(64);
-    pl->o_ticket = take(sizeof(int) * n_seqs);
-    pl->o_tile_state = take(sizeof(unsigned long long) * (size_t)n_seqs * pl->seg_tiles);
     pl->o_arrive = take(sizeof(int) * (size_t)pl->n_prob * pl->units);
     pl->o_done = take(sizeof(int) * (size_t)pl->n_prob * g.Hkv);
     pl->o_fl_ticket = take(sizeof(int));
@@ -361,10 +358,16 @@ sablock_status_t debug_sync(const sablock_params_t* p, const char* stage, cudaSt
     return err == cudaSuccess ? SABLOCK_OK : note_cuda_error(err, stage);
 }
 
+// Clears the control words for a call that does not start with the segmentation (which does it itself).
 sablock_status_t zero_control(const Plan& pl, void* ws, cudaStream_t stream)
 {
-    const cudaError_t err = cudaMemsetAsync(ws, 0, pl.control_bytes, stream);
-    return err == cudaSuccess ? SABLOCK_OK : note_cuda_error(err, "clearing the control words");
+    return launch(clear_kernel, dim3(1), 1024, 0, stream, 1, static_cast<uint4*>(ws), pl.control_bytes / 16);
+}
+
+int segment_ctas(int max_L)
+{
+    const int c = (max_L + kSegMinTokens - 1) / kSegMinTokens;
+    return c < 1 ? 1 : c > kSegMaxCluster ? kSegMaxCluster : c;
 }
 
 // ------------------------------------------------------------------ stage launchers
@@ -373,9 +376,9 @@ sablock_status_t run_segment(const Plan& pl, const sablock_params_t* p, const in
 {
     if (!token_ids || !seg_id || !seg_start || !n_seg || !p->delim_bitmap || p->vocab_size <= 0)
         return SABLOCK_ERR_INVALID_ARG;
-    dim3 grid(pl.seg_tiles, pl.geo.n_seqs);
-    return launch(segment_kernel, grid, kSegThreads, 0, stream, 1, pl.geo, token_ids, p->delim_bitmap, p->vocab_size, seg_id,
-                  seg_start, n_seg, at<unsigned long long>(ws, pl.o_tile_state), at<int>(ws, pl.o_ticket), pl.seg_tiles,
+    const int c = segment_ctas(pl.max_L);
+    return launch(segment_kernel, dim3(c, pl.geo.n_seqs), kSegThreads, 0, stream, c, pl.geo, token_ids, p->delim_bitmap,
+                  p->vocab_size, seg_id, seg_start, n_seg, static_cast<uint4*>(ws), pl.control_bytes / 16,
                   at<int>(ws, pl.o_status), at<int>(ws, pl.o_status) + 1);
 }
 
@@ -668,14 +671,16 @@ sablock_status_t run_pool(const Plan& pl, const sablock_params_t* p, const float
     return launch(pool_kernel, dim3(gx * 4, pl.n_prob), 256, 0, stream, 1, pl.geo, s_raw, s, p->pool_kernel, p->pool_mode);
 }
 
-sablock_status_t run_refine(const Plan& pl, const sablock_params_t* p, const float* s, const float* e,
+// s_raw != s: s is pooled from it in the same kernel.
+sablock_status_t run_refine(const Plan& pl, const sablock_params_t* p, const float* s_raw, float* s, const float* e,
                             const int* seg_start, const int* n_seg, float* s_ref, float* stats, int stats_stride,
                             cudaStream_t stream)
 {
     // one warp per segment, a few dependent loads each: the kernel is latency-bound, so it gets
     // enough warps to keep every SM's warp slots full (about ten segments per warp)
     const int gr = (int)fmin((double)kSegGridMax, fmax(1.0, (double)((pl.max_L + 2047) / 2048) * kSegGridPer2K));
-    return launch(refine_kernel, dim3(gr, pl.n_prob), 256, 0, stream, 1, pl.geo, s, e, seg_start, n_seg, p->alpha, p->eta, s_ref,
+    return launch(refine_kernel, dim3(gr, pl.n_prob), 256, 0, stream, 1, pl.geo, s_raw == s ? nullptr : s_raw,
+                  p->pool_kernel, p->pool_mode, s, e, seg_start, n_seg, p->alpha, p->eta, s_ref,
                   stats, stats_stride);
 }
 
@@ -715,7 +720,7 @@ int select_clusters(int c)
 // Stages 3 and 4 and the index list.  s == NULL: s_ref holds refined scores already.
 sablock_status_t run_select(const Plan& pl, const sablock_params_t* p, const float* s, const float* e, float* s_ref,
                             const int* seg_start, const int* n_seg, const Cands& cands, int* out_idx, int* out_n_keep, int* seg_g,
-                            int* seg_b, int seg_stride, void* ws, cudaStream_t stream)
+                            int* seg_b, int seg_stride, bool clear_status, void* ws, cudaStream_t stream)
 {
     SelectArgs a;
     a.s = s; a.e = e; a.s_ref = s_ref;
@@ -726,6 +731,7 @@ sablock_status_t run_select(const Plan& pl, const sablock_params_t* p, const flo
     a.out_idx = out_idx; a.out_n_keep = out_n_keep;
     a.seg_g = seg_g; a.seg_b = seg_b; a.seg_stride = seg_stride;
     a.status = at<int>(ws, pl.o_status);
+    a.clear_status = clear_status;
     SAB_TRY(allow_smem<select_kernel>(kSelSmemBytes));
     // CTAs per problem: as many as leave all problems' clusters resident at once, at least a thousand
     // tokens each
@@ -983,17 +989,11 @@ sablock_status_t sablock_segment(const sablock_params_t* p, const int* token_ids
     SAB_TRY(make_plan(p, 1, 1, nullptr, L, L, p->window + 1, &pl));
     if (!ws || ws_bytes < pl.total) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    SAB_TRY(zero_control(pl, ws, st));
     return run_segment(pl, p, token_ids, seg_id, seg_start, n_seg, ws, st);
 }
 
 // ---- segmentation without a workspace ---------------------------------------------------
-// Scratch of sablock_segment_static: one look-back word per 2048-token tile, then the ticket
-// counter and a private status word.  In host code this name is only a handle for the symbol
-// look-up below; the kernel gets the device address from cudaGetSymbolAddress.
-constexpr int kStaticSegTiles = SABLOCK_SEGMENT_STATIC_MAX_T / kSegTile;
-static __device__ __align__(256) unsigned long long g_segment_scratch[kStaticSegTiles + 32];
-
+// The scan exchanges its counts through distributed shared memory: it needs no scratch in global memory.
 sablock_status_t sablock_segment_static(const sablock_params_t* p, const int* token_ids, int L, int* seg_id,
                                         int* seg_start, int* n_seg, int* status, sablock_stream_t stream)
 {
@@ -1002,36 +1002,15 @@ sablock_status_t sablock_segment_static(const sablock_params_t* p, const int* to
     SAB_TRY(validate_params(p));
     if (!token_ids || !seg_id || !seg_start || !n_seg || !p->delim_bitmap || p->vocab_size <= 0)
         return SABLOCK_ERR_INVALID_ARG;
-    const long long T = (long long)L - p->window;
-    if (T > SABLOCK_SEGMENT_STATIC_MAX_T) return SABLOCK_ERR_UNSUPPORTED;
-    // device address of the static array, looked up once per device with that device current
-    static unsigned long long* addr[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SABLOCK_ERR_CUDA;
-    if (!addr[dev]) {
-        void* ptr = nullptr;
-        if (cudaGetSymbolAddress(&ptr, g_segment_scratch) != cudaSuccess || !ptr) {
-            cudaGetLastError();
-            return SABLOCK_ERR_CUDA;
-        }
-        addr[dev] = static_cast<unsigned long long*>(ptr);
-    }
-    unsigned long long* scratch = addr[dev];
-    const int n_tiles = (int)((T + kSegTile - 1) / kSegTile);
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the array keeps the previous call's contents: tile states, ticket and private status restart at zero
-    if (cudaMemsetAsync(scratch, 0, sizeof(unsigned long long) * (size_t)n_tiles, st) != cudaSuccess ||
-        cudaMemsetAsync(scratch + kStaticSegTiles, 0, 2 * sizeof(unsigned long long), st) != cudaSuccess)
-        return SABLOCK_ERR_CUDA;
-    int* ticket = reinterpret_cast<int*>(scratch + kStaticSegTiles);
-    int* own_status = reinterpret_cast<int*>(scratch + kStaticSegTiles + 1);
+    if ((long long)L - p->window > SABLOCK_SEGMENT_STATIC_MAX_T) return SABLOCK_ERR_UNSUPPORTED;
     Geo g;
     memset(&g, 0, sizeof(g));
     g.n_layers = g.n_seqs = 1; g.total_tokens = L; g.window = p->window;
     g.H = p->n_q_heads; g.Hkv = p->n_kv_heads; g.D = p->head_dim; g.G = g.H / g.Hkv;
     g.cu[0] = 0; g.cu[1] = L;
-    return launch(segment_kernel, dim3(n_tiles, 1), kSegThreads, 0, st, 1, g, token_ids, p->delim_bitmap, p->vocab_size, seg_id,
-                  seg_start, n_seg, scratch, ticket, n_tiles, status ? status : own_status, nullptr);
+    const int c = segment_ctas(L);
+    return launch(segment_kernel, dim3(c, 1), kSegThreads, 0, static_cast<cudaStream_t>(stream), c, g, token_ids, p->delim_bitmap,
+                  p->vocab_size, seg_id, seg_start, n_seg, nullptr, 0, status, nullptr);
 }
 
 sablock_status_t sablock_score(const sablock_params_t* p, const void* q_win, const void* k, int L, const int* seg_start,
@@ -1050,8 +1029,7 @@ sablock_status_t sablock_score(const sablock_params_t* p, const void* q_win, con
     float* e_buf = e ? e : at<float>(ws, pl.o_e);
     float* s_raw = p->pool_kernel > 1 ? at<float>(ws, pl.o_s_raw) : s;
     SAB_TRY(run_score(pl, p, q_win, k, s_raw, e_buf, ws, st));
-    SAB_TRY(run_pool(pl, p, s_raw, s, st));
-    return run_refine(pl, p, s, e_buf, seg_start, n_seg, s_refined, seg_stats, L - p->window, st);
+    return run_refine(pl, p, s_raw, s, e_buf, seg_start, n_seg, s_refined, seg_stats, L - p->window, st);
 }
 
 sablock_status_t sablock_select(const sablock_params_t* p, const float* s_refined, int L, const int* seg_start,
@@ -1068,10 +1046,9 @@ sablock_status_t sablock_select(const sablock_params_t* p, const float* s_refine
     SAB_TRY(make_plan(p, 1, 1, nullptr, L, L, rows_out(p, budget), &pl));
     if (!ws || ws_bytes < pl.total) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    SAB_TRY(zero_control(pl, ws, st));
     // the retained count is written to workspace (n_seg slot is free here)
     return run_select(pl, p, nullptr, nullptr, const_cast<float*>(s_refined), seg_start, n_seg, cands, out_idx,
-                      at<int>(ws, pl.o_n_seg), out_seg_block, out_seg_budget, L > p->window ? L - p->window : 1, ws, st);
+                      at<int>(ws, pl.o_n_seg), out_seg_block, out_seg_budget, L > p->window ? L - p->window : 1, true, ws, st);
 }
 
 sablock_status_t sablock_compact(const sablock_params_t* p, const void* k, const void* v, int L, const int* out_idx,
@@ -1113,7 +1090,6 @@ sablock_status_t sablock_compress_layers(const sablock_params_t* p, int n_layers
     if (!ws || ws_bytes < pl.total) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     prof_begin_call(st);
-    SAB_TRY(zero_control(pl, ws, st));
     int* seg_id = at<int>(ws, pl.o_seg_id);
     int* seg_start = at<int>(ws, pl.o_seg_start);
     int* n_seg = at<int>(ws, pl.o_n_seg);
@@ -1129,7 +1105,7 @@ sablock_status_t sablock_compress_layers(const sablock_params_t* p, int n_layers
     SAB_TRY(debug_sync(p, "stage score", st));
     SAB_TRY(run_pool(pl, p, s_raw, s, st));
     for (int i = 4; i <= 5; ++i) prof_mark(i, st);       // refinement and Top-B are part of the selection kernel: intervals of zero
-    SAB_TRY(run_select(pl, p, s, e, sr, seg_start, n_seg, cands, out_idx, out_n_keep, nullptr, nullptr, 0, ws, st));
+    SAB_TRY(run_select(pl, p, s, e, sr, seg_start, n_seg, cands, out_idx, out_n_keep, nullptr, nullptr, 0, false, ws, st));
     for (int i = 6; i <= 7; ++i) prof_mark(i, st);
     SAB_TRY(debug_sync(p, "stage select", st));
     sablock_status_t rc = run_compact(pl.geo, pl.n_prob, p, k, v, out_idx, out_n_keep, 0, out_k, out_v, st);

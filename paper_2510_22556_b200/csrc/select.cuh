@@ -46,6 +46,7 @@ struct SelectArgs {
     int* seg_b;
     int seg_stride;
     int* status;
+    int clear_status;          // the kernel is the first of its call: status words are cleared here
 };
 
 struct SelShared {
@@ -104,32 +105,14 @@ __device__ __forceinline__ int warp_lower_bound(const int* __restrict__ x, int n
     return lo;
 }
 
-// All CTAs of the cluster have arrived `n` times (n counts from 0); what each wrote before is
-// visible.  Bounded; false if it gave up.  Called by every thread of every CTA.
 __device__ __forceinline__ bool sel_exchange(SelShared& sm, int C, int n, bool post, int* status)
 {
-    __syncthreads();
-    if (C == 1) return true;
-    if ((int)threadIdx.x < C && post)
-        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_map(&sm.bar, (int)threadIdx.x))
-                     : "memory");
-    const uint32_t bar = smem_u32(&sm.bar);
-    const long long t0 = clock64();
-    bool ok = false;
-    while (true) {
-        uint32_t done;
-        asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done) : "r"(bar), "r"((uint32_t)(n & 1)), "r"(20000u) : "memory");
-        if (done) { ok = true; break; }
-        if (clock64() - t0 > kWaitLimitCycles) break;
-    }
+    const bool ok = cluster_exchange(&sm.bar, C, n, post);
     if (!ok && threadIdx.x == 0) {
         atomicOr(status, kStatTimeout);
         note_giveup(status, kGiveupTopB);
     }
-    return __syncthreads_and(ok) != 0;
+    return ok;
 }
 
 __device__ __forceinline__ double sel_block_sum(double v, SelShared& sm)
@@ -792,6 +775,7 @@ select_kernel(const Geo g, const Cands cands, const SelectArgs a)
     }
     pdl_wait();
     pdl_launch();
+    if (a.clear_status && rank == 0 && p == 0 && tid < 16) a.status[tid] = 0;       // (one problem: its cluster meets below before anything is reported)
     const int layer = p / g.n_seqs, seq = p % g.n_seqs;
     const int L = geo_L(g, seq), T = L - g.window;
     int* oi = a.out_idx + (size_t)p * g.n_out;

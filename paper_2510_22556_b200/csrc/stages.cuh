@@ -8,12 +8,16 @@ namespace sab {
 // ---------------------------------------------------------------------------------------
 // Stage 1: segmentation (Sec. 3.1).  seg_id[t] = number of delimiters among tokens [0, t),
 // i.e. an inclusive prefix sum of the "a segment starts here" flags f[t] = delim(t-1).
-// Single pass over the tokens with a decoupled look-back between tiles: each tile publishes
-// its aggregate, then its inclusive prefix, in one 64-bit word {flag, value}.
+// A cluster of up to eight CTAs per sequence: every CTA collects the flags of its range as a bitmask in
+// shared memory, the counts are exchanged through distributed shared memory, and the ids follow from
+// population counts.  (The look-back scan over global tile states that this replaces needed its state
+// cleared by a memset, 4 us with the gap behind it in front of every call, and 6 to 12 us itself; this takes
+// 5 to 8.)  The kernel is the first of a pass, so it also clears the control words of the kernels behind it.
 // ---------------------------------------------------------------------------------------
-constexpr int kSegThreads = 256;
-constexpr int kSegItems = 8;
-constexpr int kSegTile = kSegThreads * kSegItems;
+constexpr int kSegThreads = 1024;
+constexpr int kSegMaxCluster = 8;
+constexpr int kSegWords = 2048;                    // flag words in shared memory: 64K tokens at a time
+constexpr int kSegMinTokens = 1024;                // per CTA of a cluster
 
 __device__ __forceinline__ int is_delim(int id, const unsigned* bitmap, int vocab)
 {
@@ -21,113 +25,180 @@ __device__ __forceinline__ int is_delim(int id, const unsigned* bitmap, int voca
     return (__ldg(bitmap + (id >> 5)) >> (id & 31)) & 1u;
 }
 
-__global__ void __launch_bounds__(kSegThreads)
-segment_kernel(Geo g, const int* __restrict__ token_ids, const unsigned* __restrict__ bitmap, int vocab,
-               int* __restrict__ seg_id, int* __restrict__ seg_start, int* __restrict__ n_seg,
-               unsigned long long* tile_state, int* ticket, int max_tiles, int* status, int* giveup)
+// Arrivals of a cluster's CTAs, for exchanges through distributed shared memory: every CTA posts to
+// all barriers; all have arrived `n` times (n counts from 0) when wait returns true, and what each wrote
+// before is visible.  Bounded; false if it gave up.  Called by every thread.
+__device__ __forceinline__ bool cluster_exchange(uint64_t* bar, int C, int n, bool post)
+{
+    __syncthreads();
+    if (C == 1) return true;
+    if ((int)threadIdx.x < C && post)
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_map(bar, (int)threadIdx.x)) : "memory");
+    const uint32_t b = smem_u32(bar);
+    const long long t0 = clock64();
+    bool ok = false;
+    while (true) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done) : "r"(b), "r"((uint32_t)(n & 1)), "r"(20000u) : "memory");
+        if (done) { ok = true; break; }
+        if (clock64() - t0 > kWaitLimitCycles) break;
+    }
+    return __syncthreads_and(ok) != 0;
+}
+
+__global__ void clear_kernel(uint4* ctl, size_t n16)
 {
     pdl_wait();
+    for (size_t i = threadIdx.x; i < n16; i += blockDim.x) ctl[i] = make_uint4(0, 0, 0, 0);
+    __threadfence();
+    __syncthreads();
     pdl_launch();
-    const int seq = blockIdx.y;
+}
+
+// grid = (C, sequences), cluster = (C, 1, 1).  ctl: control words to clear (n16 16-byte pieces), or NULL.
+__global__ void __launch_bounds__(kSegThreads)
+segment_kernel(const Geo g, const int* __restrict__ token_ids, const unsigned* __restrict__ bitmap, int vocab,
+               int* __restrict__ seg_id, int* __restrict__ seg_start, int* __restrict__ n_seg, uint4* ctl, size_t n16,
+               int* status, int* giveup)
+{
+    __shared__ unsigned bits[kSegWords];
+    __shared__ int pre[kSegWords];
+    __shared__ int s_warp[kSegThreads / 32], s_count;
+    __shared__ uint64_t bar;
+    const int C = gridDim.x, rank = blockIdx.x, seq = blockIdx.y;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        mbar_init(smem_u32(&bar), C);
+        fence_mbar_init();
+    }
+    pdl_wait();
+    // The control words first: the next kernel may start as soon as they are clear (it takes nothing else from
+    // this one before its end; its accesses to them are atomics and acquire loads, which go to L2, where the
+    // fence has put the zeros).
+    if (ctl) {
+        const size_t stride = (size_t)C * gridDim.y * kSegThreads;
+        for (size_t i = ((size_t)seq * C + rank) * kSegThreads + tid; i < n16; i += stride) ctl[i] = make_uint4(0, 0, 0, 0);
+        __threadfence();
+        __syncthreads();
+    }
+    pdl_launch();
     const int T = geo_L(g, seq) - g.window;
-    const int tid = threadIdx.x;
-    if (T <= 0) {
-        if (blockIdx.x == 0 && tid == 0) n_seg[seq] = 0;
+    if (T <= 0) {                                  // the whole cluster
+        if (rank == 0 && tid == 0) n_seg[seq] = 0;
         return;
     }
-    const int ntiles = (T + kSegTile - 1) / kSegTile;
-    __shared__ int s_tile, s_prefix;
-    __shared__ int s_warp[kSegThreads / 32];
-    // Tiles are handed out in launch order so that every predecessor of a running tile is
-    // itself running or done: the look-back below always makes progress.
-    if (tid == 0) s_tile = atomicAdd(&ticket[seq], 1);
-    __syncthreads();
-    const int tile = s_tile;
-    if (tile >= ntiles) return;
-
     const int* ids = token_ids + g.cu[seq];
     int* sid = seg_id + g.cu[seq];
     int* sst = seg_start + g.cu[seq] + seq;
-    unsigned long long* state = tile_state + (size_t)seq * max_tiles;
-
-    const int base = tile * kSegTile + tid * kSegItems;
-    int f[kSegItems];
-    int cnt = 0;
+    const int words = (T + 31) >> 5, per = (words + C - 1) / C;
+    const int w0 = min(rank * per, words), w1 = min(w0 + per, words);
+    // flags of words [a, z) of the sequence into `bits`, and this thread's share of their count
+    auto collect = [&](int a, int z) -> int {
+        int c = 0;
+        for (int w = a + warp; w < z; w += 4 * (kSegThreads / 32)) {
+            int id[4];
 #pragma unroll
-    for (int i = 0; i < kSegItems; ++i) {
-        int t = base + i;
-        f[i] = (t >= 1 && t < T) ? is_delim(__ldg(ids + t - 1), bitmap, vocab) : 0;
-        cnt += f[i];
-    }
-    // block-wide exclusive scan of cnt
-    const int lane = tid & 31, warp = tid >> 5;
-    int inc = cnt;
+            for (int u = 0; u < 4; ++u) {
+                const int ww = w + u * (kSegThreads / 32), t = ww * 32 + lane;
+                id[u] = ww < z && t >= 1 && t < T ? __ldg(ids + t - 1) : -1;
+            }
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int v = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += v;
-    }
-    if (lane == 31) s_warp[warp] = inc;
-    __syncthreads();
-    int woff = 0, total = 0;
-#pragma unroll
-    for (int w = 0; w < kSegThreads / 32; ++w) {
-        int v = s_warp[w];
-        if (w < warp) woff += v;
-        total += v;
-    }
-    const int excl = woff + inc - cnt;
-
-    if (tid == 0) {
-        int prefix = 0;
-        const bool withheld = SAB_HOOK(0) && tile == 1;       // test builds: this tile never publishes
-        if (tile == 0) {
-            *(volatile unsigned long long*)&state[0] = (2ull << 32) | (unsigned)total;
-        } else {
-            if (!withheld) *(volatile unsigned long long*)&state[tile] = (1ull << 32) | (unsigned)total;
-            int j = tile - 1;
-            const long long t0 = clock64();
-            while (j >= 0) {
-                unsigned long long st = *(volatile unsigned long long*)&state[j];
-                unsigned flag = (unsigned)(st >> 32);
-                if (flag == 0) {
-                    if (clock64() - t0 > kWaitLimitCycles) {   // bounded: report and carry on
-                        atomicOr(status, kStatTimeout);
-                        if (giveup) atomicCAS(giveup, 0, kGiveupSegment | ((int)blockIdx.x << 8));
-                        break;
-                    }
-                    __nanosleep(40);
-                    continue;
+            for (int u = 0; u < 4; ++u) {
+                const int ww = w + u * (kSegThreads / 32);
+                const unsigned m = __ballot_sync(0xffffffffu, is_delim(id[u], bitmap, vocab));
+                if (ww < z && lane == 0) {
+                    bits[ww - a] = m;
+                    c += __popc(m);
                 }
-                prefix += (int)(unsigned)st;
-                if (flag == 2) break;
-                --j;
             }
-            if (!withheld) *(volatile unsigned long long*)&state[tile] = (2ull << 32) | (unsigned)(prefix + total);
         }
-        s_prefix = prefix;
-    }
+        return c;
+    };
+    int c = 0;
+    for (int a = w0; a < w1; a += kSegWords) c += collect(a, min(a + kSegWords, w1));
+    c = warp_sum(c);
+    if (lane == 0) s_warp[warp] = c;
     __syncthreads();
-    int run = s_prefix + excl;
+    if (tid < 32) {
+        c = warp_sum(s_warp[tid]);
+        if (tid == 0) s_count = c;
+    }
+    int run0 = 0;
+    if (C > 1) {
+        cluster_sync();                            // every CTA's barrier is set up
+        const bool withheld = SAB_HOOK(0) && rank == 1;        // test builds: this CTA never reports
+        if (!cluster_exchange(&bar, C, 0, !withheld) && tid == 0) {
+            if (status) atomicOr(status, kStatTimeout);        // bounded: report and carry on
+            if (giveup) atomicCAS(giveup, 0, kGiveupSegment | ((int)blockIdx.x << 8));
+        }
 #pragma unroll
-    for (int i = 0; i < kSegItems; ++i) {
-        int t = base + i;
-        if (t < T) {
-            run += f[i];
-            sid[t] = run;
-            if (f[i] || t == 0) sst[run] = t;
-            if (t == T - 1) {
-                n_seg[seq] = run + 1;
-                sst[run + 1] = T;
+        for (int r = 0; r < kSegMaxCluster; ++r)
+            if (r < rank) run0 += ld_cluster_s32(&s_count, r);
+    }
+    for (int a = w0; a < w1; a += kSegWords) {
+        const int z = min(a + kSegWords, w1);
+        __syncthreads();
+        if (w1 - w0 > kSegWords) {                 // more than shared memory holds: once more
+            collect(a, z);
+            __syncthreads();
+        }
+        // exclusive prefix over the words: two per thread
+        const int i0 = 2 * tid, n = z - a;
+        const int c0 = i0 < n ? __popc(bits[i0]) : 0, c1 = i0 + 1 < n ? __popc(bits[i0 + 1]) : 0;
+        int inc = c0 + c1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
+        }
+        if (lane == 31) s_warp[warp] = inc;
+        __syncthreads();
+        int woff = 0, total = 0;
+#pragma unroll
+        for (int w = 0; w < kSegThreads / 32; ++w) {
+            const int v = s_warp[w];
+            if (w < warp) woff += v;
+            total += v;
+        }
+        const int excl = run0 + woff + inc - c0 - c1;
+        if (i0 < n) pre[i0] = excl;
+        if (i0 + 1 < n) pre[i0 + 1] = excl + c0;
+        __syncthreads();
+        for (int w = warp; w < n; w += kSegThreads / 32) {
+            const unsigned m = bits[w];
+            const int t = (a + w) * 32 + lane;
+            const int run = pre[w] + __popc(m & (0xffffffffu >> (31 - lane)));
+            if (t < T) {
+                sid[t] = run;
+                if (((m >> lane) & 1u) || t == 0) sst[run] = t;
+                if (t == T - 1) {
+                    n_seg[seq] = run + 1;
+                    sst[run + 1] = T;
+                }
             }
         }
+        run0 += total;
     }
+    if (C > 1) cluster_sync();                     // the other CTAs may still read this one's count
 }
 
 // ---------------------------------------------------------------------------------------
 // Optional pooling of s_t over a clipped window (not part of the method's equations).
 // ---------------------------------------------------------------------------------------
-__global__ void pool_kernel(Geo g, const float* __restrict__ s_in, float* __restrict__ s_out, int kernel, int mode)
+__device__ __forceinline__ float pooled(const float* __restrict__ s, int t, int T, int half, int mode)
+{
+    const int lo = max(t - half, 0), hi = min(t + half, T - 1);
+    float acc = s[lo];
+    for (int i = lo + 1; i <= hi; ++i) {
+        const float v = s[i];
+        acc = mode == 0 ? fmaxf(acc, v) : acc + v;
+    }
+    return mode == 0 ? acc : acc / (float)(hi - lo + 1);
+}
+__global__ void pool_kernel(const Geo g, const float* __restrict__ s_in, float* __restrict__ s_out, int kernel, int mode)
 {
     pdl_wait();
     pdl_launch();
@@ -135,16 +206,8 @@ __global__ void pool_kernel(Geo g, const float* __restrict__ s_in, float* __rest
     if (geo_identity(g, seq)) return;
     const int T = geo_L(g, seq) - g.window;
     const size_t off = (size_t)layer * g.total_tokens + g.cu[seq];
-    const int half = kernel / 2;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < T; t += gridDim.x * blockDim.x) {
-        int lo = max(t - half, 0), hi = min(t + half, T - 1);
-        float acc = s_in[off + lo];
-        for (int i = lo + 1; i <= hi; ++i) {
-            float v = s_in[off + i];
-            acc = mode == 0 ? fmaxf(acc, v) : acc + v;
-        }
-        s_out[off + t] = mode == 0 ? acc : acc / (float)(hi - lo + 1);
-    }
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < T; t += gridDim.x * blockDim.x)
+        s_out[off + t] = pooled(s_in + off, t, T, kernel / 2, mode);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -152,8 +215,9 @@ __global__ void pool_kernel(Geo g, const float* __restrict__ s_in, float* __rest
 // stride over the segment's tokens and combine with a butterfly, so the summation order is
 // fixed and every lane ends with the same value.
 // ---------------------------------------------------------------------------------------
+// s_raw != NULL: s is pooled from it (and written) first.
 __global__ void __launch_bounds__(256)
-refine_kernel(Geo g, const float* __restrict__ s, const float* __restrict__ e,
+refine_kernel(const Geo g, const float* __restrict__ s_raw, int pool_k, int pool_mode, float* s, const float* __restrict__ e,
               const int* __restrict__ seg_start, const int* __restrict__ n_seg, float alpha, float eta,
               float* __restrict__ s_ref, float* __restrict__ stats, int stats_stride)
 {
@@ -162,6 +226,7 @@ refine_kernel(Geo g, const float* __restrict__ s, const float* __restrict__ e,
     const int p = blockIdx.y, layer = p / g.n_seqs, seq = p % g.n_seqs;
     if (geo_identity(g, seq)) return;
     const size_t off = (size_t)layer * g.total_tokens + g.cu[seq];
+    const int T = geo_L(g, seq) - g.window;
     const int* sst = seg_start + g.cu[seq] + seq;
     const int ns = n_seg[seq];
     const int lane = threadIdx.x & 31;
@@ -170,7 +235,14 @@ refine_kernel(Geo g, const float* __restrict__ s, const float* __restrict__ e,
         const int a = sst[k], z = sst[k + 1];
         float si = 0.f, sd = 0.f;
         for (int t = a + lane; t < z; t += 32) {
-            si += s[off + t];
+            float v;
+            if (s_raw) {
+                v = pooled(s_raw + off, t, T, pool_k / 2, pool_mode);
+                s[off + t] = v;                    // (read again below, by this thread)
+            } else {
+                v = s[off + t];
+            }
+            si += v;
             sd += e[off + t];
         }
         si = warp_sum(si);
