@@ -73,6 +73,9 @@ struct Plan {
     // workspace offsets
     size_t o_status, o_keep, o_arrive, o_done, o_fl_ticket, o_bdone, o_carry, control_bytes;
     size_t o_seg_id, o_seg_start, o_n_seg, o_s_raw, o_s, o_e, o_sr, o_part, o_lse, o_neg_lse, o_phi, o_fpart, total;
+    struct Region { size_t Plan::*field; size_t bytes; } regions[24];      // the same in layout order
+    int n_regions;
+    size_t clear_from;         // the control words from here on are cleared by the call
 };
 
 bool tc_eligible(const sablock_params_t* p)
@@ -268,31 +271,35 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     pl->keep_words = (max_L + 31) / 32 + kSelMaxCluster + 1;       // every CTA of a problem starts at a word of its own
 
     size_t o = 0;
-    auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes); return r; };
-    pl->o_status = take(64);
-    pl->o_arrive = take(sizeof(int) * (size_t)pl->n_prob * pl->units);
-    pl->o_done = take(sizeof(int) * (size_t)pl->n_prob * g.Hkv);
-    pl->o_fl_ticket = take(sizeof(int));
-    pl->o_bdone = take(carries ? sizeof(int) * (size_t)pl->n_prob * pl->fl_tiles : 0);
+    auto take = [&](size_t Plan::*field, size_t bytes) {
+        pl->*field = o;
+        pl->regions[pl->n_regions++] = {field, bytes};
+        o = align_up(o + bytes);
+    };
+    take(&Plan::o_status, 64);
+    take(&Plan::o_arrive, sizeof(int) * (size_t)pl->n_prob * pl->units);
+    take(&Plan::o_done, sizeof(int) * (size_t)pl->n_prob * g.Hkv);
+    take(&Plan::o_fl_ticket, sizeof(int));
+    take(&Plan::o_bdone, carries ? sizeof(int) * (size_t)pl->n_prob * pl->fl_tiles : 0);
     pl->control_bytes = o;
     const size_t ntok = (size_t)n_layers * total_tokens;
-    pl->o_seg_id = take(sizeof(int) * total_tokens);
-    pl->o_seg_start = take(sizeof(int) * (total_tokens + n_seqs));
-    pl->o_n_seg = take(sizeof(int) * n_seqs);
-    pl->o_s_raw = take(p->pool_kernel > 1 ? sizeof(float) * ntok : 0);
-    pl->o_s = take(sizeof(float) * ntok);
-    pl->o_e = take(sizeof(float) * ntok);
-    pl->o_sr = take(sizeof(float) * ntok);
+    take(&Plan::o_seg_id, sizeof(int) * total_tokens);
+    take(&Plan::o_seg_start, sizeof(int) * (total_tokens + n_seqs));
+    take(&Plan::o_n_seg, sizeof(int) * n_seqs);
+    take(&Plan::o_s_raw, p->pool_kernel > 1 ? sizeof(float) * ntok : 0);
+    take(&Plan::o_s, sizeof(float) * ntok);
+    take(&Plan::o_e, sizeof(float) * ntok);
+    take(&Plan::o_sr, sizeof(float) * ntok);
     const size_t part_n = pl->use_tc ? (size_t)pl->n_prob * g.Hkv * pl->n_chunks * 128
                                      : (size_t)pl->n_prob * pl->units * pl->n_chunks * pl->simt.gb * g.window;
     const size_t flow_n = flow_ok ? (size_t)pl->n_prob * g.Hkv * (pl->fl_parts + (pl->fl_parts + kFlMerge - 1) / kFlMerge) * g.G * g.window : 0;
-    pl->o_part = take(sizeof(float2) * (part_n > flow_n ? part_n : flow_n));
-    pl->o_carry = take(carries ? sizeof(float) * (size_t)kFlCarryRing * pl->fl_tiles * g.window * 128 : 0);
-    pl->o_lse = take(sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
-    pl->o_neg_lse = take(sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
-    pl->o_keep = take(sizeof(unsigned) * (size_t)pl->n_prob * pl->keep_words);
-    pl->o_phi = take(sizeof(double) * ntok);
-    pl->o_fpart = take(pl->use_fused ? sizeof(float2) * (size_t)kFuMaxCtas * kFuPartSlots * 128 : 0);
+    take(&Plan::o_part, sizeof(float2) * (part_n > flow_n ? part_n : flow_n));
+    take(&Plan::o_carry, carries ? sizeof(float) * (size_t)kFlCarryRing * pl->fl_tiles * g.window * 128 : 0);
+    take(&Plan::o_lse, sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
+    take(&Plan::o_neg_lse, sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
+    take(&Plan::o_keep, sizeof(unsigned) * (size_t)pl->n_prob * pl->keep_words);
+    take(&Plan::o_phi, sizeof(double) * ntok);
+    take(&Plan::o_fpart, pl->use_fused ? sizeof(float2) * (size_t)kFuMaxCtas * kFuPartSlots * 128 : 0);
     pl->total = o;
     return SABLOCK_OK;
 }
@@ -378,7 +385,7 @@ sablock_status_t run_segment(const Plan& pl, const sablock_params_t* p, const in
         return SABLOCK_ERR_INVALID_ARG;
     const int c = segment_ctas(pl.max_L);
     return launch(segment_kernel, dim3(c, pl.geo.n_seqs), kSegThreads, 0, stream, c, pl.geo, token_ids, p->delim_bitmap,
-                  p->vocab_size, seg_id, seg_start, n_seg, static_cast<uint4*>(ws), pl.control_bytes / 16,
+                  p->vocab_size, seg_id, seg_start, n_seg, at<uint4>(ws, pl.clear_from), (pl.control_bytes - pl.clear_from) / 16,
                   at<int>(ws, pl.o_status), at<int>(ws, pl.o_status) + 1);
 }
 
@@ -763,6 +770,91 @@ sablock_status_t run_compact(const Geo& g, int n_prob, const sablock_params_t* p
     return launch(compact_kernel, grid, 256, 0, stream, 1, g, c, out_idx, out_n_keep, n_keep_fixed);
 }
 
+// All stages of the pass.
+sablock_status_t run_pass(const Plan& pl, const sablock_params_t* p, const Cands& cands, const void* q_win, const void* k,
+                          const void* v, const int* token_ids, void* out_k, void* out_v, int* out_idx, int* out_n_keep, void* ws,
+                          cudaStream_t st)
+{
+    prof_begin_call(st);
+    int* seg_id = at<int>(ws, pl.o_seg_id);
+    int* seg_start = at<int>(ws, pl.o_seg_start);
+    int* n_seg = at<int>(ws, pl.o_n_seg);
+    float* s = at<float>(ws, pl.o_s);
+    float* e = at<float>(ws, pl.o_e);
+    float* sr = at<float>(ws, pl.o_sr);
+    float* s_raw = p->pool_kernel > 1 ? at<float>(ws, pl.o_s_raw) : s;
+    SAB_TRY(run_segment(pl, p, token_ids, seg_id, seg_start, n_seg, ws, st));
+    prof_mark(0, st);
+    SAB_TRY(debug_sync(p, "stage segment", st));
+    SAB_TRY(run_score(pl, p, q_win, k, s_raw, e, ws, st));
+    prof_mark(3, st);
+    SAB_TRY(debug_sync(p, "stage score", st));
+    SAB_TRY(run_pool(pl, p, s_raw, s, st));
+    for (int i = 4; i <= 5; ++i) prof_mark(i, st);       // refinement and Top-B are part of the selection kernel: intervals of zero
+    SAB_TRY(run_select(pl, p, s, e, sr, seg_start, n_seg, cands, out_idx, out_n_keep, nullptr, nullptr, 0, false, ws, st));
+    for (int i = 6; i <= 7; ++i) prof_mark(i, st);
+    SAB_TRY(debug_sync(p, "stage select", st));
+    sablock_status_t rc = run_compact(pl.geo, pl.n_prob, p, k, v, out_idx, out_n_keep, 0, out_k, out_v, st);
+    prof_mark(8, st);
+    prof_end_call();
+    if (rc == SABLOCK_OK) rc = debug_sync(p, "stage compact", st);
+    return rc;
+}
+
+// ---- host buffers ---------------------------------------------------------------------------
+#define SAB_CUDA(call, what) do { const cudaError_t _e = (call); if (_e != cudaSuccess) { cudaGetLastError(); return note_cuda_error(_e, what); } } while (0)
+
+// Two streams and the events between them, kept per host thread and device (so that threads never share
+// them) and given back when the thread ends.
+struct HostStreams {
+    int dev = -1;
+    cudaStream_t in = nullptr, out = nullptr;
+    cudaEvent_t ev[20] = {};
+    void release()
+    {
+        for (cudaEvent_t& e : ev) { if (e) cudaEventDestroy(e); e = nullptr; }
+        if (in) cudaStreamDestroy(in);
+        if (out) cudaStreamDestroy(out);
+        in = out = nullptr;
+        dev = -1;
+    }
+    ~HostStreams() { release(); }
+};
+
+HostStreams* host_streams()
+{
+    thread_local HostStreams hs;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    if (hs.dev == dev) return &hs;
+    hs.release();                                    // (a thread that changes its device keeps one set)
+    bool ok = cudaStreamCreateWithFlags(&hs.in, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&hs.out, cudaStreamNonBlocking) == cudaSuccess;
+    for (cudaEvent_t& e : hs.ev) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
+        hs.release();
+        return nullptr;
+    }
+    hs.dev = dev;
+    return &hs;
+}
+
+// The plan of n_layers of a larger call's layers inside that call's workspace; false if a region would not
+// hold what it needs.
+bool plan_inside(const Plan& whole, const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, int max_L, int n_out,
+                 Plan* pl)
+{
+    if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, pl) != SABLOCK_OK || pl->n_regions != whole.n_regions) return false;
+    for (int i = 0; i < pl->n_regions; ++i) {
+        if (pl->regions[i].bytes > whole.regions[i].bytes) return false;
+        pl->*(pl->regions[i].field) = whole.*(whole.regions[i].field);
+    }
+    pl->control_bytes = whole.control_bytes;
+    pl->total = whole.total;
+    return true;
+}
+
 // ---- decoding over a cache: launch plan ----------------------------------------------------
 struct DecodePlan { int n_splits, rows_per_split; bool cluster; size_t bytes; };
 
@@ -1088,31 +1180,7 @@ sablock_status_t sablock_compress_layers(const sablock_params_t* p, int n_layers
     Plan pl;
     SAB_TRY(make_plan(p, n_layers, n_seqs, cu_seqlens, cu_seqlens[n_seqs], max_L, rows_out(p, budget), &pl));
     if (!ws || ws_bytes < pl.total) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    prof_begin_call(st);
-    int* seg_id = at<int>(ws, pl.o_seg_id);
-    int* seg_start = at<int>(ws, pl.o_seg_start);
-    int* n_seg = at<int>(ws, pl.o_n_seg);
-    float* s = at<float>(ws, pl.o_s);
-    float* e = at<float>(ws, pl.o_e);
-    float* sr = at<float>(ws, pl.o_sr);
-    float* s_raw = p->pool_kernel > 1 ? at<float>(ws, pl.o_s_raw) : s;
-    SAB_TRY(run_segment(pl, p, token_ids, seg_id, seg_start, n_seg, ws, st));
-    prof_mark(0, st);
-    SAB_TRY(debug_sync(p, "stage segment", st));
-    SAB_TRY(run_score(pl, p, q_win, k, s_raw, e, ws, st));
-    prof_mark(3, st);
-    SAB_TRY(debug_sync(p, "stage score", st));
-    SAB_TRY(run_pool(pl, p, s_raw, s, st));
-    for (int i = 4; i <= 5; ++i) prof_mark(i, st);       // refinement and Top-B are part of the selection kernel: intervals of zero
-    SAB_TRY(run_select(pl, p, s, e, sr, seg_start, n_seg, cands, out_idx, out_n_keep, nullptr, nullptr, 0, false, ws, st));
-    for (int i = 6; i <= 7; ++i) prof_mark(i, st);
-    SAB_TRY(debug_sync(p, "stage select", st));
-    sablock_status_t rc = run_compact(pl.geo, pl.n_prob, p, k, v, out_idx, out_n_keep, 0, out_k, out_v, st);
-    prof_mark(8, st);
-    prof_end_call();
-    if (rc == SABLOCK_OK) rc = debug_sync(p, "stage compact", st);
-    return rc;
+    return run_pass(pl, p, cands, q_win, k, v, token_ids, out_k, out_v, out_idx, out_n_keep, ws, static_cast<cudaStream_t>(stream));
 }
 
 sablock_status_t sablock_compress(const sablock_params_t* p, const void* q_win, const void* k, const void* v,
@@ -1190,19 +1258,17 @@ sablock_status_t sablock_compress_layers_host(const sablock_params_t* p, int n_l
     // Everything the copies below are sized from is checked first: nothing is enqueued on bad arguments.
     if (budget <= (p->budget_includes_window ? p->window : 0)) return SABLOCK_ERR_INVALID_ARG;
     if (cu_seqlens[0] != 0) return SABLOCK_ERR_INVALID_ARG;
-    {
-        int max_L = 0;
-        for (int i = 0; i < n_seqs; ++i) {
-            const int L = cu_seqlens[i + 1] - cu_seqlens[i];
-            if (L < 1) return SABLOCK_ERR_INVALID_ARG;
-            if (L > max_L) max_L = L;
-        }
-        Cands cands;
-        SAB_TRY(check_candidates(block_candidates, n_candidates, &cands));
-        Plan pl;
-        SAB_TRY(make_plan(p, n_layers, n_seqs, cu_seqlens, cu_seqlens[n_seqs], max_L, rows_out(p, budget), &pl));
-        if (!ws || ws_bytes < pl.total) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
+    int max_L = 0;
+    for (int i = 0; i < n_seqs; ++i) {
+        const int L = cu_seqlens[i + 1] - cu_seqlens[i];
+        if (L < 1) return SABLOCK_ERR_INVALID_ARG;
+        if (L > max_L) max_L = L;
     }
+    Cands cands;
+    SAB_TRY(check_candidates(block_candidates, n_candidates, &cands));
+    Plan pl;
+    SAB_TRY(make_plan(p, n_layers, n_seqs, cu_seqlens, cu_seqlens[n_seqs], max_L, rows_out(p, budget), &pl));
+    if (!ws || ws_bytes < pl.total) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const size_t es = elem_size(p);
     const size_t total = (size_t)cu_seqlens[n_seqs];
@@ -1214,28 +1280,86 @@ sablock_status_t sablock_compress_layers_host(const sablock_params_t* p, int n_l
     // The pass reads every key but only the retained rows of V.  If h_v is pinned (page-locked,
     // device-accessible) memory the gather reads those rows from it in place; otherwise V is staged
     // like the rest.
-    const void* v_src = dev_v;
+    const char* v_src = static_cast<const char*>(dev_v);
     {
         cudaPointerAttributes attr;
         if (cudaPointerGetAttributes(&attr, h_v) == cudaSuccess && attr.type == cudaMemoryTypeHost && attr.devicePointer)
-            v_src = attr.devicePointer;
+            v_src = static_cast<const char*>(attr.devicePointer);
         else
             cudaGetLastError();
     }
-    if (cudaMemcpyAsync(dev_token_ids, h_token_ids, total * sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(dev_q_win, h_q_win, q_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(dev_k, h_k, kv_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        (v_src == dev_v && cudaMemcpyAsync(dev_v, h_v, kv_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess))
-        return SABLOCK_ERR_CUDA;
-    SAB_TRY(sablock_compress_layers(p, n_layers, n_seqs, dev_q_win, dev_k, v_src, dev_token_ids, cu_seqlens, budget,
-                                    block_candidates, n_candidates, dev_out_k, dev_out_v, dev_out_idx, dev_out_n_keep,
-                                    ws, ws_bytes, stream));
-    if (cudaMemcpyAsync(h_out_k, dev_out_k, okv_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(h_out_v, dev_out_v, okv_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(h_out_idx, dev_out_idx, n_prob * n_out * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(h_out_n_keep, dev_out_n_keep, n_prob * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        return SABLOCK_ERR_CUDA;
-    return cudaStreamSynchronize(st) == cudaSuccess ? SABLOCK_OK : SABLOCK_ERR_CUDA;
+    const bool stage_v = v_src == dev_v;
+    // The copies take longer than everything else together (PCIe), so the layers go through in chunks, a chunk's compute and
+    // the copies of its results behind the next chunk's copies: 4 layers of 8K tokens 1.49 -> 1.33 ms.  The
+    // chunks use the workspace as one call over all layers would (same places for what a caller may look at
+    // afterwards); chunks of less than 4 MB of keys are not worth their launches.
+    int per = n_layers;
+    Plan part;
+    const size_t layer_kv = kv_bytes / n_layers;
+    const int by_size = (int)(((4u << 20) + layer_kv - 1) / layer_kv), by_count = (n_layers + 7) / 8;
+    const int want = by_size > by_count ? by_size : by_count;
+    HostStreams* hs = want < n_layers ? host_streams() : nullptr;
+    if (hs && plan_inside(pl, p, want, n_seqs, cu_seqlens, max_L, n_out, &part) &&
+        (n_layers % want == 0 || plan_inside(pl, p, n_layers % want, n_seqs, cu_seqlens, max_L, n_out, &part)))
+        per = want;
+    cudaStream_t s_in = st, s_out = st;
+    if (per < n_layers) {
+        s_in = hs->in; s_out = hs->out;
+        SAB_CUDA(cudaEventRecord(hs->ev[0], st), "host pass: event");              // what the caller has enqueued comes first
+        SAB_CUDA(cudaStreamWaitEvent(s_in, hs->ev[0], 0), "host pass: wait");
+        SAB_CUDA(cudaStreamWaitEvent(s_out, hs->ev[0], 0), "host pass: wait");
+    }
+    const size_t lq = q_bytes / n_layers, lo = okv_bytes / n_layers, n_idx = (size_t)n_seqs * n_out;
+    int launches = 0, n_ev = 1;
+    SAB_CUDA(cudaMemcpyAsync(dev_token_ids, h_token_ids, total * sizeof(int), cudaMemcpyHostToDevice, s_in), "host pass: copy in");
+    for (int l0 = 0; l0 < n_layers; l0 += per) {
+        const int nl = l0 + per <= n_layers ? per : n_layers - l0;
+        auto in = [&](const void* d, const void* h, size_t layer) {
+            return cudaMemcpyAsync((char*)const_cast<void*>(d) + l0 * layer, (const char*)h + l0 * layer, nl * layer,
+                                   cudaMemcpyHostToDevice, s_in);
+        };
+        auto out = [&](void* h, const void* d, size_t layer) {
+            return cudaMemcpyAsync((char*)h + l0 * layer, (const char*)d + l0 * layer, nl * layer, cudaMemcpyDeviceToHost, s_out);
+        };
+        SAB_CUDA(in(dev_q_win, h_q_win, lq), "host pass: copy in");
+        SAB_CUDA(in(dev_k, h_k, layer_kv), "host pass: copy in");
+        if (stage_v) SAB_CUDA(in(dev_v, h_v, layer_kv), "host pass: copy in");
+        if (per < n_layers) {
+            SAB_CUDA(cudaEventRecord(hs->ev[n_ev], s_in), "host pass: event");
+            SAB_CUDA(cudaStreamWaitEvent(st, hs->ev[n_ev++], 0), "host pass: wait");
+        }
+        const Plan* run = &pl;
+        sablock_params_t pp = *p;
+        if (per < n_layers) {
+            if (!plan_inside(pl, p, nl, n_seqs, cu_seqlens, max_L, n_out, &part)) return SABLOCK_ERR_INVALID_ARG;   // (checked above)
+            const size_t tok0 = (size_t)l0 * total * sizeof(float);
+            part.o_s += tok0; part.o_e += tok0; part.o_sr += tok0;
+            if (p->pool_kernel > 1) part.o_s_raw += tok0;
+            part.clear_from = l0 > 0 ? pl.o_arrive : 0;                    // the status words of the earlier chunks stay
+            if (p->row_lse) pp.row_lse = p->row_lse + (size_t)l0 * n_seqs * p->n_q_heads * p->window;
+            run = &part;
+        }
+        t_launches = 0;
+        SAB_TRY(run_pass(*run, &pp, cands, (const char*)dev_q_win + l0 * lq, (const char*)dev_k + l0 * layer_kv, v_src + l0 * layer_kv,
+                         dev_token_ids, (char*)dev_out_k + l0 * lo, (char*)dev_out_v + l0 * lo, dev_out_idx + l0 * n_idx,
+                         dev_out_n_keep + (size_t)l0 * n_seqs, ws, st));
+        launches += t_launches;
+        if (per < n_layers) {
+            SAB_CUDA(cudaEventRecord(hs->ev[n_ev], st), "host pass: event");
+            SAB_CUDA(cudaStreamWaitEvent(s_out, hs->ev[n_ev++], 0), "host pass: wait");
+        }
+        SAB_CUDA(out(h_out_k, dev_out_k, lo), "host pass: copy out");
+        SAB_CUDA(out(h_out_v, dev_out_v, lo), "host pass: copy out");
+        SAB_CUDA(out(h_out_idx, dev_out_idx, n_idx * sizeof(int)), "host pass: copy out");
+        SAB_CUDA(out(h_out_n_keep, dev_out_n_keep, n_seqs * sizeof(int)), "host pass: copy out");
+    }
+    t_launches = launches;
+    if (per < n_layers) {
+        SAB_CUDA(cudaEventRecord(hs->ev[0], s_out), "host pass: event");
+        SAB_CUDA(cudaStreamWaitEvent(st, hs->ev[0], 0), "host pass: wait");
+    }
+    SAB_CUDA(cudaStreamSynchronize(st), "host pass");
+    return SABLOCK_OK;
 }
 
 }  // extern "C"
