@@ -209,26 +209,23 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     const long long m = tiles * g.Hkv * pl->n_prob / (8LL * sm_count());
     pl->fl_m = (int)(m < 1 ? 1 : m > 4 ? 4 : m);
     pl->fl_parts = (int)((tiles + 4 * pl->fl_m - 1) / (4 * pl->fl_m));
-    {
-        // head groups: their keys stay at kFlGroupBytes (two sweeps), their window rows at kFlMaxRows
-        const long long head_bytes = (long long)max_L * p->head_dim * 2;
-        // (the workspace is laid out for two sweeps, whether or not the log-sum-exps are given this time)
-        int h = (int)fmax(1.0, (double)(kFlGroupBytes / head_bytes));
-        if (h > kFlMaxRows / (g.G * p->window)) h = kFlMaxRows / (g.G * p->window);
+    {   // head groups: as many heads as have room for their log-sum-exps
+        int h = kFlMaxRows / (g.G * p->window);
         if (h > g.Hkv) h = g.Hkv;
         pl->fl_groups = (g.Hkv + h - 1) / h;
         pl->fl_heads = (g.Hkv + pl->fl_groups - 1) / pl->fl_groups;
         pl->fl_groups = (g.Hkv + pl->fl_heads - 1) / pl->fl_heads;
         if ((long long)pl->fl_groups * n_seqs > kFlMaxSlots) flow_ok = false;
     }
-    // Two sweeps with 128 window rows per KV head: only where one group holds all heads.  Between groups the head-summed
-    // attention goes through L2 (16 KB per tile each way, next to 32 KB of keys per head), and the kernel with
-    // fixed shares, which keeps it in tensor memory, is faster: 1.05 against 1.13 ms at 32K, 1.95 against 2.25 ms at
-    // 64K tokens (32 layers).  With 64 rows or fewer that kernel does not apply and the traffic is a quarter or less:
-    // 1.09 -> 0.88 ms against the two-launch kernels at window 8, 1.16 -> 0.99 ms at window 16 (32K, 32 layers).
-    const bool flow_two = pl->fl_groups == 1 || g.G * p->window <= 64;
-    pl->use_flow = flow_ok && (p->row_lse != nullptr || flow_two);
-    const bool carries = flow_ok && (g.Hkv * g.G * p->window > kFlMaxRows || (flow_two && pl->fl_groups > 1));
+    const bool carries = flow_ok && pl->fl_groups > 1;
+    // Two sweeps over a long sequence: the flow kernel reads the keys of a problem that L2 does not hold twice from
+    // memory, the kernel with fixed shares (one KV head of all CTAs at a time) once, but idles at every
+    // head.  Under the power cap the two meet at about 48 MB of keys per problem: 20K tokens 678 against 710 us, 32K
+    // 1048 against 1035 us, 64K 1.98 against 1.93 ms, 128K 3.86 against 3.74 ms (32 layers, 8 KV heads of 128).
+    const bool fixed_shares = fused_eligible(p) && tiles <= (long long)kFuMaxTilesPerCta * sm_count() &&
+                              (long long)n_layers * total_tokens < 0x7fffffffLL &&
+                              (long long)max_L * g.Hkv * p->head_dim * 2 > (48LL << 20);
+    pl->use_flow = flow_ok && (p->row_lse != nullptr || !fixed_shares);
     pl->use_fused = pl->use_tc && p->score_impl != SABLOCK_SCORE_TENSOR && fused_eligible(p);
     if (pl->use_tc) {
         long long work1 = tiles * g.Hkv * pl->n_prob, work2 = tiles * pl->n_prob;
@@ -487,12 +484,6 @@ sablock_status_t run_flow(const Plan& pl, const sablock_params_t* p, const CUten
     if (fa.n_sel == 0) return SABLOCK_OK;
     fa.n_prob = g.n_layers * fa.n_sel;
     fa.group_heads = pl.fl_heads; fa.n_groups = pl.fl_groups;
-    if (!fa.two_sweep) {                                             // nothing is read twice: as many heads as fit
-        const int h = kFlMaxRows / (g.G * W) < g.Hkv ? kFlMaxRows / (g.G * W) : g.Hkv;
-        fa.n_groups = (g.Hkv + h - 1) / h;
-        fa.group_heads = (g.Hkv + fa.n_groups - 1) / fa.n_groups;
-        fa.n_groups = (g.Hkv + fa.group_heads - 1) / fa.group_heads;
-    }
     fa.m = pl.fl_m;
     // A units run ahead of the B units of the same (problem, head group) by about a unit per SM: enough that the row sums
     // are there in time (what is late is put aside), little enough that the keys are still in L2

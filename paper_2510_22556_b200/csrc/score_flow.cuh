@@ -10,9 +10,11 @@
 // A B unit needs the log-sum-exps of its problem, i.e. A units with smaller numbers: whoever holds those
 // is running, so waiting for them always ends and no CTA has to be resident for another's sake.  The
 // order is A(v + lag), B(v) for v = 0, 1, ...: by the time a B unit is handed out the A units it needs are
-// long done, and the keys they read are still in L2.  v counts (problem, group of KV heads); a group is
-// as many heads as keep its keys at about 34 MB (a quarter of L2: measured, a chunk of that size read again one
-// chunk later costs no DRAM traffic, 48 MB does).  With the row log-sum-exps given there are B units only.
+// done or nearly so (a CTA puts a B unit that is early aside and goes on with A units), and as little more
+// as possible has been read since, so that the keys of a problem of up to about 48 MB are read from L2 the
+// second time.  v counts (problem, group of KV heads); a group is as many heads as have room for their
+// log-sum-exps (1024 window rows), for the usual shapes all of them.  With the row log-sum-exps given there
+// are B units only.
 //
 // Both are 128 x N x D products with the operand roles swapped (A: tensor-memory lane = window row, so row sums
 // are thread-local; B: lane = token, so the sums over heads and window positions are).  CTA = 20 warps.
@@ -43,7 +45,6 @@ constexpr int kFlMerge = 8;
 constexpr int kFlCarryRing = 4;
 constexpr int kFlMaxRows = 1024;             // window rows of a head group
 constexpr int kFlMaxSlots = 512;             // (sequence, head group) pairs of a launch
-constexpr long long kFlGroupBytes = 34LL << 20;
 __host__ __device__ constexpr int fl_kstages(int D) { return D == 128 ? 4 : 8; }
 __host__ __device__ constexpr int fl_smem(int D) { return 1024 + (kFlQStages + fl_kstages(D)) * 128 * D * 2; }
 
