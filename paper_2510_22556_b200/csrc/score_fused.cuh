@@ -499,23 +499,23 @@ __device__ __forceinline__ void fu_issue_tile(uint32_t d, uint32_t a_lo, uint32_
 // ---- arithmetic of the epilogue ---------------------------------------------------------------
 // Packed fp32 pairs (one instruction for two lanes of arithmetic: the epilogue is short of issue
 // slots, not of fp32 throughput).
-// Sum of exp2(v * c2 - m) over 32 logits of one window row.  (The additions are scalar: packing the
-// results of the special-function unit for a paired addition costs moves.)
+// Sum of exp2(v * c2 - m) over 32 logits of one window row.
 __device__ __forceinline__ float chunk_expsum(const uint32_t (&r)[32], float c2, float m)
 {
     const uint64_t cc = pack2(c2, c2), mm = pack2(-m, -m);
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+    uint64_t s0 = pack2(0.f, 0.f), s1 = s0;
 #pragma unroll
     for (int i = 0; i < 32; i += 4) {
         float a, b, c, d;
         unpack2(fma2(pack2u(r[i + 0], r[i + 1]), cc, mm), a, b);
         unpack2(fma2(pack2u(r[i + 2], r[i + 3]), cc, mm), c, d);
-        s0 += ex2_approx(a);
-        s1 += ex2_approx(b);
-        s2 += ex2_approx(c);
-        s3 += ex2_approx(d);
+        s0 = add2(s0, pack2(ex2_approx(a), ex2_approx(b)));
+        s1 = add2(s1, pack2(ex2_approx(c), ex2_approx(d)));
     }
-    return (s0 + s1) + (s2 + s3);
+    float a, b, c, d;
+    unpack2(s0, a, b);
+    unpack2(s1, c, d);
+    return (a + b) + (c + d);
 }
 __device__ __forceinline__ float chunk_max(const uint32_t (&r)[32])
 {
