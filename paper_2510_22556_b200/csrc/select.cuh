@@ -629,29 +629,48 @@ __device__ bool sel_body(const Geo& g, const Cands& cands, const SelectArgs& a, 
     // the searches of the segments listed so far
     auto flush = [&]() {
         __syncthreads();
-        const int n_items = sm.n_active * n_cand;
+        const int n_act = sm.n_active, n_items = n_act * n_cand;
+        // Where the range leaves room behind its scores, an item leaves the tokens it would retain there (eight words), and the
+        // segment's winner need not be evaluated again.
+        unsigned* masks = reinterpret_cast<unsigned*>(dyn + (size_t)((len + 3) & ~3) * 4);
+        const bool keep_masks = kSm && n_items <= (kSelCap - ((len + 3) & ~3)) / 8;
         while (true) {
             int it = 0;
             if (lane == 0) it = atomicAdd(&sm.next, 1);
             it = __shfl_sync(0xffffffffu, it, 0);
             if (it >= n_items) break;
-            const int x = it / n_cand, ci = n_cand - (it - x * n_cand);
+            const int y = it / n_act, x = it - y * n_act, ci = n_cand - y;         // large block sizes first
             const SelActive& s = active[x];
             const int gs = cands.g[ci], pos = s.pos, n = s.n, b = s.b;
             if (gs > min(n, b)) continue;
+            unsigned passed = 0;
+            if (lane == 0) passed = *(volatile const unsigned*)&s.passed;
+            if (__shfl_sync(0xffffffffu, passed, 0) >> ci) continue;               // a larger one has passed
             unsigned bits;
             const bool pass = kSm ? sel_candidate(sv + pos, ta + pos, n, b, gs, thr, cut, a.tau, phi, rk, bits)
                                   : sel_candidate(s_ref + ta + pos, ta + pos, n, b, gs, thr, cut, a.tau, phi, rk, bits);
-            if (pass && lane == 0) atomicOr(&active[x].passed, 1u << ci);
+            if (!pass) continue;
+            if (keep_masks)
+                for (int q = 0; q * 32 < n; ++q) {
+                    const unsigned m = __ballot_sync(0xffffffffu, (bits >> q) & 1u);
+                    if (lane == 0) masks[(size_t)it * 8 + q] = m;
+                }
+            if (lane == 0) atomicOr(&active[x].passed, 1u << ci);
         }
         __syncthreads();
-        for (int x = warp; x < sm.n_active; x += kSelWarps) {
+        for (int x = warp; x < n_act; x += kSelWarps) {
             const SelActive& s = active[x];
             if (!s.passed) continue;
-            const int gs = cands.g[31 - __clz(s.passed)], pos = s.pos, n = s.n;
-            unsigned bits;
-            if (kSm) sel_candidate(sv + pos, ta + pos, n, s.b, gs, thr, cut, a.tau, phi, rk, bits);
-            else sel_candidate(s_ref + ta + pos, ta + pos, n, s.b, gs, thr, cut, a.tau, phi, rk, bits);
+            const int ci = 31 - __clz(s.passed), gs = cands.g[ci], pos = s.pos, n = s.n;
+            unsigned bits = 0;
+            if (keep_masks) {
+                const unsigned* m = masks + (size_t)((n_cand - ci) * n_act + x) * 8;
+                for (int q = 0; q * 32 < n; ++q) bits |= ((m[q] >> lane) & 1u) << q;
+            } else if (kSm) {
+                sel_candidate(sv + pos, ta + pos, n, s.b, gs, thr, cut, a.tau, phi, rk, bits);
+            } else {
+                sel_candidate(s_ref + ta + pos, ta + pos, n, s.b, gs, thr, cut, a.tau, phi, rk, bits);
+            }
             for (int i = lane, q = 0; i < n; i += 32, ++q) sel_set_bit(keep, pos + i, (bits >> q) & 1u);
             if (seg_g && lane == 0) seg_g[s.k] = gs;
         }
