@@ -13,6 +13,11 @@ from typing import Optional, Sequence
 
 import torch
 
+try:
+    from . import _fastcall
+except ImportError:                        # not built: ctypes marshals
+    _fastcall = None
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libsablock.so")
 
@@ -85,6 +90,12 @@ def _load(path: str):
     l.sablock_compress_layers.argtypes = [vp, ci, ci, vp, vp, vp, vp, vp, ci, vp, ci, vp, vp, vp, vp, vp, sz, vp]
     l.sablock_compress_layers_host.argtypes = [vp, ci, ci, vp, vp, vp, vp, vp, ci, vp, ci, vp, vp, vp, vp,
                                                vp, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp]
+    # The entry points that enqueue work, by their short names: through the C module where it is built.  A
+    # sequence argument is a tuple or list there and a ctypes array here.
+    for name in ("segment", "segment_static", "score", "select", "compact", "compress", "compress_layers", "compress_layers_host",
+                 "decode_attention"):
+        fn = getattr(l, "sablock_" + name)
+        setattr(l, name, _fastcall.bind(C.cast(fn, C.c_void_p).value) if _fastcall else fn)
     l.sablock_decode_workspace_bytes.restype = C.c_size_t
     l.sablock_decode_workspace_bytes.argtypes = [vp, ci, ci]
     l.sablock_decode_attention.argtypes = [vp, ci, vp, vp, vp, ci, vp, vp, vp, vp, sz, vp]
@@ -128,15 +139,11 @@ def _check(code: int, where: str):
         raise SablockError(code, where)
 
 
-_INT_ARRAYS = {n: C.c_int * n for n in range(1, 66)}       # ctypes builds a class per array length: once each
-
-
 def _iarr(xs: Sequence[int]):
-    t = _INT_ARRAYS.get(len(xs)) or C.c_int * len(xs)
-    try:
-        return t(*xs)
-    except TypeError:
-        return t(*[int(x) for x in xs])
+    """A sequence of ints as an argument of an entry point."""
+    if _fastcall is not None:
+        return xs if type(xs) is tuple or type(xs) is list else [int(x) for x in xs]
+    return (C.c_int * len(xs))(*[int(x) for x in xs])
 
 
 def make_params(n_q_heads: int, n_kv_heads: int, head_dim: int, window: int, dtype: torch.dtype,
@@ -219,7 +226,7 @@ def segment(p: Params, token_ids: torch.Tensor, ws: torch.Tensor):
     seg_id = torch.empty(max(T, 1), dtype=torch.int32, device=token_ids.device)
     seg_start = torch.empty(max(T, 1) + 1, dtype=torch.int32, device=token_ids.device)
     n_seg = torch.empty(1, dtype=torch.int32, device=token_ids.device)   # always written
-    _check(lib().sablock_segment(C.addressof(p), _ptr(token_ids), L, _ptr(seg_id), _ptr(seg_start), _ptr(n_seg),
+    _check(lib().segment(C.addressof(p), _ptr(token_ids), L, _ptr(seg_id), _ptr(seg_start), _ptr(n_seg),
                                  _ptr(ws), ws.numel(), _stream()), "sablock_segment")
     return seg_id, seg_start, n_seg
 
@@ -231,7 +238,7 @@ def segment_static(p: Params, token_ids: torch.Tensor, seg_id: torch.Tensor, seg
                    n_seg: torch.Tensor, status: Optional[torch.Tensor] = None) -> None:
     """sablock_segment without a workspace: the caller supplies every buffer (outputs included),
     the scan's scratch is a fixed array inside the library.  Nothing is allocated here."""
-    _check(lib().sablock_segment_static(C.addressof(p), _ptr(token_ids), token_ids.numel(), _ptr(seg_id),
+    _check(lib().segment_static(C.addressof(p), _ptr(token_ids), token_ids.numel(), _ptr(seg_id),
                                         _ptr(seg_start), _ptr(n_seg), _ptr(status), _stream()),
            "sablock_segment_static")
 
@@ -245,7 +252,7 @@ def score(p: Params, q_win: torch.Tensor, k: torch.Tensor, seg_start: torch.Tens
     e = torch.empty(T, dtype=torch.float32, device=dev)
     sr = torch.empty(T, dtype=torch.float32, device=dev)
     stats = torch.zeros(3 * T, dtype=torch.float32, device=dev) if want_stats else None
-    _check(lib().sablock_score(C.addressof(p), _ptr(q_win), _ptr(k), L, _ptr(seg_start), _ptr(n_seg), _ptr(s), _ptr(e),
+    _check(lib().score(C.addressof(p), _ptr(q_win), _ptr(k), L, _ptr(seg_start), _ptr(n_seg), _ptr(s), _ptr(e),
                                _ptr(sr), _ptr(stats), _ptr(ws), ws.numel(), _stream()), "sablock_score")
     return s, e, sr, (stats.view(3, T) if want_stats else None)
 
@@ -263,7 +270,7 @@ def select(p: Params, s_refined: torch.Tensor, L: int, seg_start: torch.Tensor, 
     seg_g = torch.zeros(max(T, 1), dtype=torch.int32, device=dev) if want_segments else None
     seg_b = torch.zeros(max(T, 1), dtype=torch.int32, device=dev) if want_segments else None
     cand = _iarr(candidates)
-    _check(lib().sablock_select(C.addressof(p), _ptr(s_refined), L, _ptr(seg_start), _ptr(n_seg), budget, cand,
+    _check(lib().select(C.addressof(p), _ptr(s_refined), L, _ptr(seg_start), _ptr(n_seg), budget, cand,
                                 len(candidates), _ptr(out_idx), _ptr(seg_g), _ptr(seg_b), _ptr(ws), ws.numel(),
                                 _stream()), "sablock_select")
     return out_idx, seg_g, seg_b
@@ -273,7 +280,7 @@ def compact(p: Params, k: torch.Tensor, v: torch.Tensor, out_idx: torch.Tensor):
     n = out_idx.numel()
     out_k = torch.empty((n,) + tuple(k.shape[1:]), dtype=k.dtype, device=k.device)
     out_v = torch.empty_like(out_k)
-    _check(lib().sablock_compact(C.addressof(p), _ptr(k), _ptr(v), k.shape[0], _ptr(out_idx), n, _ptr(out_k),
+    _check(lib().compact(C.addressof(p), _ptr(k), _ptr(v), k.shape[0], _ptr(out_idx), n, _ptr(out_k),
                                  _ptr(out_v), _stream()), "sablock_compact")
     return out_k, out_v
 
@@ -288,7 +295,7 @@ def compress(p: Params, q_win: torch.Tensor, k: torch.Tensor, v: torch.Tensor, t
     out_idx = torch.empty(n, dtype=torch.int32, device=k.device)
     n_keep = torch.empty(1, dtype=torch.int32, device=k.device)          # always written
     cand = _iarr(candidates)
-    _check(lib().sablock_compress(C.addressof(p), _ptr(q_win), _ptr(k), _ptr(v), _ptr(token_ids), L, budget, cand,
+    _check(lib().compress(C.addressof(p), _ptr(q_win), _ptr(k), _ptr(v), _ptr(token_ids), L, budget, cand,
                                   len(candidates), _ptr(out_k), _ptr(out_v), _ptr(out_idx), _ptr(n_keep), _ptr(ws),
                                   ws.numel(), _stream()), "sablock_compress")
     return out_k, out_v, out_idx, n_keep
@@ -315,7 +322,7 @@ def compress_layers(p: Params, q_win: torch.Tensor, k: torch.Tensor, v: torch.Te
         out = LayersOut(p, n_layers, n_seqs, budget, k.dtype, k.device)
     cu = _iarr(cu_seqlens)
     cand = _iarr(candidates)
-    _check(lib().sablock_compress_layers(C.addressof(p), n_layers, n_seqs, _ptr(q_win), _ptr(k), _ptr(v),
+    _check(lib().compress_layers(C.addressof(p), n_layers, n_seqs, _ptr(q_win), _ptr(k), _ptr(v),
                                          _ptr(token_ids), cu, budget, cand, len(candidates), _ptr(out.out_k),
                                          _ptr(out.out_v), _ptr(out.out_idx), _ptr(out.n_keep), _ptr(ws), ws.numel(),
                                          _stream()), "sablock_compress_layers")
@@ -328,7 +335,7 @@ def compress_layers_host(p: Params, h_q, h_k, h_v, h_ids, cu_seqlens, budget, ca
     n_layers, n_seqs = h_q.shape[0], h_q.shape[1]
     cu = _iarr(cu_seqlens)
     cand = _iarr(candidates)
-    _check(lib().sablock_compress_layers_host(
+    _check(lib().compress_layers_host(
         C.addressof(p), n_layers, n_seqs, _ptr(h_q), _ptr(h_k), _ptr(h_v), _ptr(h_ids), cu, budget, cand,
         len(candidates), _ptr(h_out.out_k), _ptr(h_out.out_v), _ptr(h_out.out_idx), _ptr(h_out.n_keep),
         _ptr(d_q), _ptr(d_k), _ptr(d_v), _ptr(d_ids), _ptr(d_out.out_k), _ptr(d_out.out_v), _ptr(d_out.out_idx),
@@ -350,7 +357,7 @@ def decode_attention(p: Params, q: torch.Tensor, k_cache: torch.Tensor, v_cache:
         ws = torch.empty(nb, dtype=torch.uint8, device=q.device)
     out = torch.empty(n_prob, H, D, dtype=torch.float32, device=q.device)
     lse = torch.empty(n_prob, H, dtype=torch.float32, device=q.device) if want_lse else None
-    _check(lib().sablock_decode_attention(C.addressof(p), n_prob, _ptr(q), _ptr(k_cache), _ptr(v_cache), n_rows,
+    _check(lib().decode_attention(C.addressof(p), n_prob, _ptr(q), _ptr(k_cache), _ptr(v_cache), n_rows,
                                           _ptr(n_valid), _ptr(out), _ptr(lse), _ptr(ws), ws.numel(), _stream()),
            "sablock_decode_attention")
     return (out, lse) if want_lse else out

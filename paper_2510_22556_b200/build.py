@@ -4,10 +4,12 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsablock.so")
+FASTCALL = os.path.join(HERE, "_fastcall.so")
 SOURCES = ["sablock.cu"]
 HEADERS = ["common.cuh", "stages.cuh", "select.cuh", "score_simt.cuh", "score_tc.cuh", "score_fused.cuh", "score_flow.cuh", "decode.cuh"]
 
@@ -32,7 +34,19 @@ def _compile(out: str, defines=(), verbose: bool = False) -> None:
     subprocess.run(cmd, check=True)
 
 
+def _build_fastcall(force: bool = False) -> None:
+    """The marshalling module of the binding (plain C, Python's own headers; optional: without them the
+    binding stays with ctypes)."""
+    src = os.path.join(CSRC, "fastcall.c")
+    inc = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(inc, "Python.h")):
+        return
+    if force or not os.path.exists(FASTCALL) or os.path.getmtime(src) > os.path.getmtime(FASTCALL):
+        subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", inc, src, "-o", FASTCALL], check=True)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    _build_fastcall(force)
     if not force and not _stale():
         return LIB
     _compile(LIB, verbose=verbose)
