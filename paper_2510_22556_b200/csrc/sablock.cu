@@ -239,9 +239,10 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
         // pass 1 gets one wave of two CTAs per SM (what shared memory holds at D = 128) and at most
         // kSimtMaxChunks partials per row.
         SimtShape& sp = pl->simt;
-        sp.wp_log2 = 0;
-        while ((1 << sp.wp_log2) < p->window) ++sp.wp_log2;
+        int w_log2 = 0;
+        while ((1 << w_log2) < p->window) ++w_log2;
         sp.tok = kSimtTokLarge;
+        sp.wp_log2 = w_log2 > 0 ? w_log2 - 1 : 0;                    // (two window positions per thread)
         sp.tile = (kSimtThreads >> sp.wp_log2) * sp.tok;
         sp.gb = g.G >= 3 ? 4 : g.G;
         while (sp.gb > 1 && simt_smem_bytes(sp.gb, p->window, g.D, sp.tile) > kSimtSmemMax) sp.gb /= 2;
@@ -249,6 +250,7 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
         const long long units = (long long)g.Hkv * sp.batches;
         if ((max_L + sp.tile - 1) / sp.tile * units * pl->n_prob < sm_count()) {
             sp.tok = kSimtTokSmall;
+            sp.wp_log2 = w_log2;
             sp.tile = (kSimtThreads >> sp.wp_log2) * sp.tok;
         }
         sp.smem = simt_smem_bytes(sp.gb, p->window, g.D, sp.tile);

@@ -4,23 +4,23 @@
 // reduces over heads and window positions per token (Eqs. 3, 4 and the inner sum of Eq. 6).
 // Logits are kept in log2 units: x2 = (q . k) * log2(e) / sqrt(D).
 //
-// Both passes are the same register-tiled product.  A CTA of 256 threads holds a tile of key rows
+// Both passes are the same register-tiled product.  A CTA of 128 threads holds a tile of key rows
 // and the window rows of GB query heads of one KV head in shared memory (fp32, rows padded by 16
 // bytes so that the eight lanes of a 16-byte shared-memory phase hit different banks).  A thread
-// owns one window position w and eight tokens and computes GB x 8 logits: the GB heads of a w are
-// summed inside the thread (Eq. 3), and per four elements of D the thread's 8 + GB shared-memory
-// loads feed 16 GB packed multiply-adds, so that with GB = 4 the FMA pipes and not the
-// shared-memory port are the busier unit.  Problems too small to give every SM a tile of that size
-// take two tokens per thread (four times the CTAs, a quarter of the serial work in each).  (One thread per token reading its key row straight from
-// global memory, the way this path used to work, took 225 + 1406 us for the two passes on a
-// 4096-token fp32 layer with 32 / 8 heads of 128; the tiled passes take 50 + 49 us, of which 2 x 17 us
-// are the multiply-adds at full rate and the rest loads that nothing overlaps and the merges.)
+// owns two window positions and eight tokens and computes 2 x GB x 8 logits: the GB heads of a position are
+// summed inside the thread (Eq. 3).  What bounds it is the 128 bytes per cycle at which shared memory
+// fills registers (a broadcast counts in full): per four elements of D a warp's 8 + 2 GB vector loads take as
+// long as their 64 GB multiply-adds with GB = 4, and half as long again with one position per thread (8192 tokens:
+// 204 -> 175 us a call).  Problems too small to give every SM a tile of that size take two tokens and one
+// position per thread (more CTAs, less serial work in each).  (One thread per token reading its key
+// row straight from global memory, the way this path used to work, took 225 + 1406 us for the two
+// passes on a 4096-token fp32 layer with 32 / 8 heads of 128: 1.70 ms a call against 0.12 now.)
 #pragma once
 #include "common.cuh"
 
 namespace sab {
 
-constexpr int kSimtThreads = 256;
+constexpr int kSimtThreads = 128;
 constexpr int kSimtTokLarge = 8, kSimtTokSmall = 2;     // tokens per thread
 constexpr int kSimtMaxW = 64;
 constexpr int kSimtMaxD = 256;
@@ -53,7 +53,7 @@ struct SimtShape {
 // Query rows, then the key tile; the end of each pass reuses the space for its merge.
 __host__ __device__ inline int simt_smem_bytes(int gb, int W, int D, int tile)
 {
-    const int keys = tile * (D + 4), red = kSimtThreads * gb * 2, sums = tile * (W + 1);
+    const int keys = tile * (D + 4), red = kSimtThreads * 2 * gb * 2, sums = tile * (W + 1);
     int n = gb * W * (D + 4) + (keys > red ? keys : red);
     if (sums > n) n = sums;
     return n * (int)sizeof(float);
@@ -142,43 +142,49 @@ __device__ __forceinline__ void simt_place(int tid, int wp_log2, int& wi, int& t
 }
 
 // x2[i][b] = c2 * (key row tg + TG i) . (window row of head b at position w)
+// Window positions per thread: two (w and w + threads along w) in the large tiles.
+template <int kTok> constexpr int kSimtNw = kTok == kSimtTokLarge ? 2 : 1;
+
 template <int GB, int kTok>
-__device__ __forceinline__ void simt_logits(const float* ks, const float* qs, int D, int TG, int tg, int w, int W, float c2,
-                                            float (&x)[kTok][GB])
+__device__ __forceinline__ void simt_logits(const float* ks, const float* qs, int D, int TG, int tg, const int (&w)[kSimtNw<kTok>],
+                                            int W, float c2, float (&x)[kTok][kSimtNw<kTok>][GB])
 {
-    const int ld = D + 4;
-    uint64_t acc[kTok][GB];
+    constexpr int NW = kSimtNw<kTok>;
+    const int ld = D + 4, q_step = W * ld, k_step = TG * ld;
 #pragma unroll
     for (int i = 0; i < kTok; ++i)
 #pragma unroll
-        for (int b = 0; b < GB; ++b) acc[i][b] = pack2(0.f, 0.f);
-    const float* qw = qs + w * ld;
+        for (int y = 0; y < NW; ++y)
+#pragma unroll
+            for (int b = 0; b < GB; ++b) x[i][y][b] = 0.f;
     const float* kt = ks + tg * ld;
 #pragma unroll 1
     for (int d = 0; d < D; d += 4) {
-        uint64_t q0[GB], q1[GB];
+        float4 q[NW][GB];
 #pragma unroll
-        for (int b = 0; b < GB; ++b) {
-            const float4 v = *reinterpret_cast<const float4*>(qw + b * W * ld + d);
-            q0[b] = pack2(v.x, v.y);
-            q1[b] = pack2(v.z, v.w);
-        }
+        for (int y = 0; y < NW; ++y)
+#pragma unroll
+            for (int b = 0; b < GB; ++b) q[y][b] = *reinterpret_cast<const float4*>(qs + w[y] * ld + b * q_step + d);
 #pragma unroll
         for (int i = 0; i < kTok; ++i) {
-            const float4 v = *reinterpret_cast<const float4*>(kt + i * TG * ld + d);
-            const uint64_t k0 = pack2(v.x, v.y), k1 = pack2(v.z, v.w);
+            const float4 v = *reinterpret_cast<const float4*>(kt + i * k_step + d);
 #pragma unroll
-            for (int b = 0; b < GB; ++b) acc[i][b] = fma2(q1[b], k1, fma2(q0[b], k0, acc[i][b]));
+            for (int y = 0; y < NW; ++y)
+#pragma unroll
+                for (int b = 0; b < GB; ++b) {
+                    x[i][y][b] = fmaf(q[y][b].x, v.x, x[i][y][b]);
+                    x[i][y][b] = fmaf(q[y][b].y, v.y, x[i][y][b]);
+                    x[i][y][b] = fmaf(q[y][b].z, v.z, x[i][y][b]);
+                    x[i][y][b] = fmaf(q[y][b].w, v.w, x[i][y][b]);
+                }
         }
     }
 #pragma unroll
     for (int i = 0; i < kTok; ++i)
 #pragma unroll
-        for (int b = 0; b < GB; ++b) {
-            float lo, hi;
-            unpack2(acc[i][b], lo, hi);
-            x[i][b] = (lo + hi) * c2;
-        }
+        for (int y = 0; y < NW; ++y)
+#pragma unroll
+            for (int b = 0; b < GB; ++b) x[i][y][b] *= c2;
 }
 
 // Pass 1.  grid = (chunks, Hkv * batches, problems): row statistics of GB * W window rows over
@@ -206,11 +212,16 @@ score_p1_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
     const int tid = threadIdx.x;
     int wi, tg;
     simt_place(tid, sp.wp_log2, wi, tg);
-    const int w = min(wi, W - 1);
-    simt_load_rows(qs, q + ((size_t)p * g.H + j * g.G + b0) * W * D, (long long)D, GB * W, nh * W, D, sp.vec_q != 0);
-    float m[GB], l[GB];
+    constexpr int NW = kSimtNw<kTok>;
+    int w[NW];
 #pragma unroll
-    for (int b = 0; b < GB; ++b) { m[b] = -INFINITY; l[b] = 0.f; }
+    for (int y = 0; y < NW; ++y) w[y] = min(wi + y * (1 << sp.wp_log2), W - 1);
+    simt_load_rows(qs, q + ((size_t)p * g.H + j * g.G + b0) * W * D, (long long)D, GB * W, nh * W, D, sp.vec_q != 0);
+    float m[NW][GB], l[NW][GB];
+#pragma unroll
+    for (int y = 0; y < NW; ++y)
+#pragma unroll
+        for (int b = 0; b < GB; ++b) { m[y][b] = -INFINITY; l[y][b] = 0.f; }
     const int t_end = min(ntiles, (chunk + 1) * sp.tpc);
     for (int tl = chunk * sp.tpc; tl < t_end; ++tl) {
         const int t0 = tl * sp.tile;
@@ -218,30 +229,36 @@ score_p1_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
         simt_load_rows(ks, k + (size_t)layer * ks_layer + (size_t)j * ks_head + ((size_t)g.cu[seq] + t0) * ks_tok, ks_tok,
                        sp.tile, L - t0, D, sp.vec_k != 0);
         simt_load_wait();
-        float x[kTok][GB];
+        float x[kTok][NW][GB];
         simt_logits<GB, kTok>(ks, qs, D, TG, tg, w, W, c2, x);
-        const int lim = min(L - 1, Tn + w) - t0;        // causal (Eq. 2): tokens of the tile up to here are visible
 #pragma unroll
-        for (int b = 0; b < GB; ++b) {
-            float mx = m[b];
+        for (int y = 0; y < NW; ++y) {
+            const int lim = min(L - 1, Tn + w[y]) - t0;         // causal (Eq. 2): tokens of the tile up to here are visible
 #pragma unroll
-            for (int i = 0; i < kTok; ++i) {
-                if (tg + TG * i > lim) x[i][b] = -INFINITY;
-                mx = fmaxf(mx, x[i][b]);
+            for (int b = 0; b < GB; ++b) {
+                float mx = m[y][b];
+#pragma unroll
+                for (int i = 0; i < kTok; ++i) {
+                    if (tg + TG * i > lim) x[i][y][b] = -INFINITY;
+                    mx = fmaxf(mx, x[i][y][b]);
+                }
+                const float ms = mx == -INFINITY ? 0.f : mx;
+                float s = 0.f;
+#pragma unroll
+                for (int i = 0; i < kTok; ++i) s += exp2f(x[i][y][b] - ms);
+                l[y][b] = l[y][b] * exp2f(m[y][b] - ms) + s;
+                m[y][b] = mx;
             }
-            const float ms = mx == -INFINITY ? 0.f : mx;
-            float s = 0.f;
-#pragma unroll
-            for (int i = 0; i < kTok; ++i) s += exp2f(x[i][b] - ms);
-            l[b] = l[b] * exp2f(m[b] - ms) + s;
-            m[b] = mx;
         }
     }
     __syncthreads();
     // merge over the token groups, in order
-    float2* red = reinterpret_cast<float2*>(ks);        // [TG][GB][WP]: the space is sized for it
+    const int RP = NW * WP;                             // window positions, rounded
+    float2* red = reinterpret_cast<float2*>(ks);        // [TG][GB][RP]: the space is sized for it
 #pragma unroll
-    for (int b = 0; b < GB; ++b) red[(tg * GB + b) * WP + wi] = make_float2(m[b], l[b]);
+    for (int y = 0; y < NW; ++y)
+#pragma unroll
+        for (int b = 0; b < GB; ++b) red[(tg * GB + b) * RP + wi + y * WP] = make_float2(m[y][b], l[y][b]);
     __syncthreads();
     const int rows = GB * W;
     const size_t blk = (size_t)p * gridDim.y + unit;
@@ -249,11 +266,11 @@ score_p1_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
     for (int r = tid; r < rows; r += kSimtThreads) {
         const int b = r / W, wr = r - b * W;
         float mm = -INFINITY;
-        for (int x = 0; x < TG; ++x) mm = fmaxf(mm, red[(x * GB + b) * WP + wr].x);
+        for (int x = 0; x < TG; ++x) mm = fmaxf(mm, red[(x * GB + b) * RP + wr].x);
         const float ms = mm == -INFINITY ? 0.f : mm;
         float ll = 0.f;
         for (int x = 0; x < TG; ++x) {
-            const float2 v = red[(x * GB + b) * WP + wr];
+            const float2 v = red[(x * GB + b) * RP + wr];
             ll += v.y * exp2f(v.x - ms);
         }
         dst[r] = make_float2(mm, ll);
@@ -267,12 +284,19 @@ score_p1_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
     __threadfence();
     const float2* src = sb.part + blk * sb.n_chunks * rows;
     for (int r = tid; r < nh * W; r += kSimtThreads) {
-        float mm = -INFINITY;
-        for (int c = 0; c < nch; ++c) mm = fmaxf(mm, __ldcg(&src[(size_t)c * rows + r].x));
-        float ll = 0.f;
-        for (int c = 0; c < nch; ++c) {
-            const float2 v = __ldcg(&src[(size_t)c * rows + r]);
-            ll += v.y * exp2f(v.x - mm);
+        float mm = -INFINITY, ll = 0.f;
+        for (int c0 = 0; c0 < nch; c0 += 16) {          // sixteen loads in flight
+            float2 v[16];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) v[c] = c0 + c < nch ? __ldcg(&src[(size_t)(c0 + c) * rows + r]) : make_float2(-INFINITY, 0.f);
+            float mn = mm;
+#pragma unroll
+            for (int c = 0; c < 16; ++c) mn = fmaxf(mn, v[c].x);
+            const float ms = mn == -INFINITY ? 0.f : mn;
+            ll *= exp2f(mm - ms);
+#pragma unroll
+            for (int c = 0; c < 16; ++c) ll += v[c].y * exp2f(v[c].x - ms);
+            mm = mn;
         }
         sb.lse2[((size_t)p * g.H + j * g.G + b0) * W + r] = mm + log2f(ll);
     }
@@ -302,11 +326,16 @@ score_p2_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
     const int tid = threadIdx.x;
     int wi, tg;
     simt_place(tid, sp.wp_log2, wi, tg);
-    const int w = min(wi, W - 1);
-    const float* lse = sb.lse2 + (size_t)p * g.H * W;
-    float abar[kTok];
+    constexpr int NW = kSimtNw<kTok>;
+    int w[NW];
 #pragma unroll
-    for (int i = 0; i < kTok; ++i) abar[i] = 0.f;
+    for (int y = 0; y < NW; ++y) w[y] = min(wi + y * (1 << sp.wp_log2), W - 1);
+    const float* lse = sb.lse2 + (size_t)p * g.H * W;
+    float abar[NW][kTok];
+#pragma unroll
+    for (int y = 0; y < NW; ++y)
+#pragma unroll
+        for (int i = 0; i < kTok; ++i) abar[y][i] = 0.f;
     for (int unit = rank; unit < g.Hkv * sp.batches; unit += split) {
         const int j = unit / sp.batches, b0 = (unit - j * sp.batches) * GB;
         const int nh = min(GB, g.G - b0);
@@ -315,24 +344,30 @@ score_p2_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
             simt_load_rows(ks, k + (size_t)layer * ks_layer + (size_t)j * ks_head + ((size_t)g.cu[seq] + t0) * ks_tok, ks_tok,
                            sp.tile, L - t0, D, sp.vec_k != 0);
         simt_load_rows(qs, q + ((size_t)p * g.H + j * g.G + b0) * W * D, (long long)D, GB * W, nh * W, D, sp.vec_q != 0);
-        float ls[GB];
+        float ls[NW][GB];
 #pragma unroll
-        for (int b = 0; b < GB; ++b) ls[b] = b < nh ? lse[(j * g.G + b0 + b) * W + w] : INFINITY;     // exp2(-inf) = 0
+        for (int y = 0; y < NW; ++y)
+#pragma unroll
+            for (int b = 0; b < GB; ++b) ls[y][b] = b < nh ? lse[(j * g.G + b0 + b) * W + w[y]] : INFINITY;     // exp2(-inf) = 0
         simt_load_wait();
-        float x[kTok][GB];
+        float x[kTok][NW][GB];
         simt_logits<GB, kTok>(ks, qs, D, TG, tg, w, W, c2, x);
 #pragma unroll
-        for (int i = 0; i < kTok; ++i)
+        for (int y = 0; y < NW; ++y)
 #pragma unroll
-            for (int b = 0; b < GB; ++b) abar[i] += exp2f(x[i][b] - ls[b]);        // A[h, w, t], summed over the heads
+            for (int i = 0; i < kTok; ++i)
+#pragma unroll
+                for (int b = 0; b < GB; ++b) abar[y][i] += exp2f(x[i][y][b] - ls[y][b]);    // A[h, w, t], summed over the heads
     }
     __syncthreads();
     // \bar A of this CTA's heads: [token][W + 1], over the key tile and, where that is short, the query rows
     float* ab = smem;
     const int ldw = W + 1;
-    if (wi < W)
 #pragma unroll
-        for (int i = 0; i < kTok; ++i) ab[(tg + TG * i) * ldw + w] = abar[i];
+    for (int y = 0; y < NW; ++y)
+        if (wi + y * (1 << sp.wp_log2) < W)
+#pragma unroll
+            for (int i = 0; i < kTok; ++i) ab[(tg + TG * i) * ldw + w[y]] = abar[y][i];
     if (split > 1) cluster_sync(); else __syncthreads();
     const int lane = tid & 31, warp = tid >> 5;
     const size_t off = (size_t)layer * g.total_tokens + g.cu[seq];

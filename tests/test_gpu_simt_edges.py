@@ -1,0 +1,53 @@
+"""The fp32 score path on either side of its launch rules: one tile and its remainders, tiles of both sizes,
+KV heads spread over clusters of 1 to 8 CTAs, group sizes that do not divide the heads of a thread, odd
+windows, rows that only allow scalar loads.  Reference: float64 on the stored values.
+
+Tolerance: a logit is an fp32 sum of D <= 128 rounded products, partial sums below 64 in log2 units: error
+about 2 * sqrt(128) * 2^-24 * 64 = 8e-5, times ln 2 the relative error of a weight and as much again of
+the normaliser: 1.2e-4; taken as 2e-4 for scores, 4e-4 for entropies."""
+import pytest
+import torch
+
+import synth
+from paper_2510_22556_b200 import binding as B
+from test_gpu_flow_edges import _reference
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("H,Hkv,D,W,L", [
+    (4, 1, 64, 16, 129), (4, 1, 64, 16, 512), (32, 8, 128, 32, 700), (32, 8, 128, 32, 4097), (8, 8, 64, 8, 2500), (6, 2, 32, 5, 333),
+    (10, 2, 48, 32, 1000), (3, 3, 128, 1, 200), (2, 1, 128, 64, 900), (16, 8, 64, 7, 6001), (32, 8, 128, 32, 9000),
+])
+@pytest.mark.parametrize("layers", [1, 5])
+def test_fp32_scores(H, Hkv, D, W, L, layers):
+    cfg = synth.Config("t", layers, H, Hkv, D, W, (L,), (W + 20,), (1, 2, 4), "f32", 5000, 8, 2.0, 20, (), 3)
+    b = synth.make_batch(cfg, device="cuda")
+    p = B.make_params(H, Hkv, D, W, torch.float32, b.bitmap, cfg.vocab)
+    ws = B.alloc_workspace(p, L, L, 1, layers)
+    B.compress_layers(p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, W + 20, cfg.candidates, ws)
+    torch.cuda.synchronize()
+    assert B.read_status(ws) == 0
+    s = B.workspace_view(p, ws, "s", L, L, 1, layers)
+    e = B.workspace_view(p, ws, "e", L, L, 1, layers)
+    for l in range(layers):
+        rs, re = _reference(b.q_win[l, 0], b.k[l], W)
+        assert float(((s[l, :L - W].double() - rs).abs() / rs).max()) <= 2e-4
+        assert float((e[l, :L - W].double() - re).abs().max()) <= 4e-4
+
+
+def test_fp32_unaligned_rows():
+    """Keys whose address is a multiple of 4 bytes only."""
+    H, Hkv, D, W, L = 8, 2, 64, 16, 777
+    g = torch.Generator(device="cuda").manual_seed(1)
+    buf = torch.randn(L * Hkv * D + 1, generator=g, device="cuda")
+    k = buf[1:].view(L, Hkv, D)
+    q = torch.randn(H, W, D, generator=g, device="cuda")
+    p = B.make_params(H, Hkv, D, W, torch.float32)
+    ws = B.alloc_workspace(p, L, L)
+    st = torch.arange(0, L - W + 1, L - W, dtype=torch.int32, device="cuda")
+    seg_start = torch.zeros(L - W + 1, dtype=torch.int32, device="cuda")
+    seg_start[: st.numel()] = st
+    s, e, _, _ = B.score(p, q, k, seg_start, torch.ones(1, dtype=torch.int32, device="cuda"), ws)
+    rs, re = _reference(q, k, W)
+    assert float(((s.double() - rs).abs() / rs).max()) <= 2e-4 and float((e.double() - re).abs().max()) <= 4e-4
