@@ -205,19 +205,24 @@ def run_ours(args):
         return {"ms_step": ms_total / steps, "steps": steps, "clocks": clocks, "launches": launches,
                 "stage_avg": {k: sum(v) / len(v) for k, v in stage_ms.items()}}
 
-    def score_kernel(stage_avg):
+    def score_kernel(stage_avg, mode):
         """(name, ms per launch) of the dominant kernel: the score stage's largest interval."""
         dom = max(("score_pass1", "score_pass2"), key=lambda k: stage_avg.get(k, 0.0))
         dom_ms = stage_avg.get(dom, float("nan"))
         fused = cfg.dtype == "bf16" and stage_avg.get("score_pass2", 0.0) < 0.02 * dom_ms
-        # the persistent kernel: the whole score stage in one launch, timed in the first interval
-        return ("score_fused_tc" if fused else dom), dom_ms
+        # the tensor-core kernels that are the whole score stage in one launch, timed in the first interval: with
+        # fixed shares for two sweeps over more than 48 MB of keys per problem, the unit flow otherwise
+        long = max_L * cfg.n_kv_heads * cfg.head_dim * 2 > 48 << 20
+        name = "score_fused_tc" if mode == "two_sweep" and long else "score_flow_tc"
+        return (name if fused else dom), dom_ms
 
     def summary(r, traffic_key):
         """Time, throughput and the two roofline fractions of one timed loop."""
-        kern, kern_ms = score_kernel(r["stage_avg"])
+        kern, kern_ms = score_kernel(r["stage_avg"], traffic_key)
         achieved = ab["k_read"] / (kern_ms * 1e-3) / 1e9
-        cap = TRAFFIC_CAPTURES.get(traffic_key) if kern == "score_fused_tc" else None
+        cap = TRAFFIC_CAPTURES.get(traffic_key)
+        if cap is not None and kern != cap["kernel"]:
+            cap = None
         traffic = None if cap is None else cap["bytes"] * (nl * total) / cap["token_layers"]
         roofline = {"bound": "hbm", "kernel": kern, "achieved": round(achieved, 1), "peak": hbm_peak, "unit": "GB/s",
                     "frac": round(achieved / hbm_peak, 4), "traffic": traffic,
@@ -284,15 +289,15 @@ def run_ours(args):
         dist.destroy_process_group()
 
 
-# DRAM bytes (read + write) of one launch of the persistent score kernel, from the ncu captures
+# DRAM bytes (read + write) of one launch of the score kernel, from the ncu captures
 # summarised under profiles/ (taken on fewer layers; the traffic grows in proportion to layers x
 # tokens because every (layer, KV head) streams its own keys).  A capture is quoted only while
 # the kernel is the one it was taken on: otherwise its entry is None.
 TRAFFIC_CAPTURES = {
-    "two_sweep": {"bytes": 546839296 + 6333440, "token_layers": 2 * 131072,
-                  "source": "profiles/score_fused_tc_headline128k_2layers.txt (2 layers, scaled by layers x tokens)"},
-    "single_sweep": {"bytes": 537501184 + 4266496, "token_layers": 2 * 131072,
-                     "source": "profiles/score_fused_tc_single_sweep_headline128k_2layers.txt (2 layers, scaled by layers x tokens)"},
+    "two_sweep": {"kernel": "score_fused_tc", "bytes": 547387904 + 6991872, "token_layers": 2 * 131072,
+                  "source": "profiles/score_kernels_headline128k_2layers.txt (2 layers, scaled by layers x tokens)"},
+    "single_sweep": {"kernel": "score_flow_tc", "bytes": 537498112 + 4051968, "token_layers": 2 * 131072,
+                     "source": "profiles/score_kernels_headline128k_2layers.txt (2 layers, scaled by layers x tokens)"},
 }
 
 

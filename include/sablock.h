@@ -43,12 +43,13 @@ typedef enum {
 
 typedef enum { SABLOCK_F32 = 0, SABLOCK_BF16 = 1 } sablock_dtype_t;
 
-/* Which kernel family computes the attention scores.  AUTO picks, in this order, the
- * persistent tensor-core kernel (bf16, head_dim 128, window 32, four query heads per KV head,
- * at most 7 token tiles of 128 per CTA; two sweeps over K, or one when row_lse is given), the
- * two-launch tensor-core kernels (bf16, head_dim 64/128, window 8/16/32), and the SIMT kernels
- * otherwise (with row_lse these run their second pass only).  FUSED and TENSOR force the first
- * and the second and fail with SABLOCK_ERR_UNSUPPORTED where they cannot run. */
+/* Which kernel family computes the attention scores.  AUTO picks, for bf16, head_dim 64/128, window
+ * 8/16/32 and at most 128 window rows per KV head, the unit-flow tensor-core kernel, except for two sweeps
+ * (row_lse not given) over more than 48 MB of keys per sequence and layer in the shape of the persistent
+ * tensor-core kernel (head_dim 128, window 32, four query heads per KV head, at most 7 token tiles of 128
+ * per CTA), which takes those; everything else runs on the SIMT kernels (with row_lse these run their
+ * second pass only).  FUSED forces the persistent kernel, TENSOR the two-launch tensor-core kernels; both
+ * fail with SABLOCK_ERR_UNSUPPORTED where they cannot run. */
 typedef enum { SABLOCK_SCORE_AUTO = 0, SABLOCK_SCORE_SIMT = 1, SABLOCK_SCORE_TENSOR = 2, SABLOCK_SCORE_FUSED = 3 }
     sablock_score_impl_t;
 
@@ -140,12 +141,13 @@ sablock_status_t sablock_read_status(const void *ws, sablock_stream_t stream, in
 
 /* The same, with the word that follows the status word: raw2 (host int[2]) receives the status
  * word and, if a bounded wait ran out, which one gave up first:
- * code | (CTA index << 8) | (warp index << 20).  Codes 1-29 are waits of the persistent score kernel
+ * code | (CTA index << 8) | (warp index << 20).  Codes 1-29 are waits of the score kernels
  * (1 query-block buffer free, 2 K stage free, 3 query block loaded, 4 accumulator free, 5 K tile
  * loaded, 6 row sums of a phase in shared memory, 7 accumulator complete, 8 log-sum-exps fetched,
  * 9 turn at the exponentials, 11 partial-sum slot free, 12 row sums of all CTAs, 13 merged
- * log-sum-exps, 20 / 21 exchanges inside the epilogue, 22 the other epilogue set's previous step), 30 the look-back of the segmentation scan,
- * 31 the CTAs of one problem in the Top-B select.  Every such wait is limited to about a second of
+ * log-sum-exps, 20 / 21 exchanges inside the epilogue, 22 the other epilogue set's previous step; in the
+ * unit flow also 11 row sums taken, 14 / 15 / 17 a unit posted, 16 log-sum-exps taken, 18 / 19 carry of a tile, 21 unit record free), 30 the CTAs of a sequence in the segmentation,
+ * 31 the CTAs of one problem in the selection.  Every such wait is limited to about a second of
  * device time; the kernel that gave up returns, the later stages still run on whatever was
  * produced and stay inside their buffers. */
 sablock_status_t sablock_read_status_detail(const void *ws, sablock_stream_t stream, int *raw2);
@@ -164,20 +166,14 @@ sablock_status_t sablock_segment(const sablock_params_t *p, const int *token_ids
  * code may not allocate: an inference server whose memory pool is sized once and then frozen, a
  * plug-in that is handed only its input and output buffers, a latency-critical loop in which
  * cudaMalloc's implicit device synchronisation is not acceptable.  This variant needs no
- * workspace: the look-back state of the segmentation scan lives in a fixed 8.25 KB array inside the
- * library's device image (every GPU that loads the library holds it until the process exits).
+ * workspace: the CTAs of the scan exchange their counts on chip.
  * Same arguments and results as sablock_segment, minus the workspace.
  *  - Limit: T = L - W <= SABLOCK_SEGMENT_STATIC_MAX_T tokens; longer inputs are rejected with
  *    SABLOCK_ERR_UNSUPPORTED and nothing is enqueued.
  *  - status: dev int32[1] or NULL.  If given it must be zero before the call; a bounded wait that
- *    ran out sets bit 0 (as in the workspace status word).  With NULL the word is kept inside the
- *    static array and cannot be read back.
- *  - The first call on each device looks up the array's device address (no allocation); make
- *    that first call outside any stream capture.
- *  - Every call on a device shares the one array.  The call clears what it needs on `stream`
- *    before the kernel, so back-to-back calls on one stream are fine; two calls whose device work
- *    overlaps (different streams, or different host threads on different streams) race on it and
- *    give wrong segment ids.
+ *    ran out sets bit 0 (as in the workspace status word).  With NULL it is not
+ *    reported.
+ *  - Calls share nothing: any number of them may overlap, on any streams and threads.
  *  - Calls no cudaMalloc / cudaFree and no allocating library routine. */
 #define SABLOCK_SEGMENT_STATIC_MAX_T (1024 * 2048)
 sablock_status_t sablock_segment_static(const sablock_params_t *p, const int *token_ids, int L,

@@ -481,9 +481,11 @@ sablock_status_t run_flow(const Plan& pl, const sablock_params_t* p, const CUten
         tiles += (L + kTcTile - 1) / kTcTile;
         units_b += (tb + 3) / 4;
     }
-    prof_mark(1, stream);
-    prof_mark(2, stream);
-    if (fa.n_sel == 0) return SABLOCK_OK;
+    if (fa.n_sel == 0) {
+        prof_mark(1, stream);
+        prof_mark(2, stream);
+        return SABLOCK_OK;
+    }
     fa.n_prob = g.n_layers * fa.n_sel;
     fa.group_heads = pl.fl_heads; fa.n_groups = pl.fl_groups;
     fa.m = pl.fl_m;
@@ -497,7 +499,10 @@ sablock_status_t run_flow(const Plan& pl, const sablock_params_t* p, const CUten
     const long long rounds = (units_b + sms - 1) / sms * fa.group_heads * 4, split = (units_b * 4 + sms - 1) / sms * (fa.group_heads + 1);
     fa.head_split = fa.n_groups == 1 && fa.group_heads >= 4 && split < rounds;
     SAB_TRY(allow_smem<score_flow_tc<W, D>>(fl_smem(D)));
-    return launch(score_flow_tc<W, D>, dim3(sms), kFlThreads, fl_smem(D), stream, 1, tmQ, tmK, g, fa);
+    SAB_TRY(launch(score_flow_tc<W, D>, dim3(sms), kFlThreads, fl_smem(D), stream, 1, tmQ, tmK, g, fa));
+    prof_mark(1, stream);
+    prof_mark(2, stream);
+    return SABLOCK_OK;
 }
 
 template <typename T, int GB, int TOK>
