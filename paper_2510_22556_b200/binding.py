@@ -355,7 +355,9 @@ def decode_attention(p: Params, q: torch.Tensor, k_cache: torch.Tensor, v_cache:
         if nb == 0:
             raise SablockError(2, "sablock_decode_workspace_bytes")
         ws = torch.empty(nb, dtype=torch.uint8, device=q.device)
-    out = torch.empty(n_prob, H, D, dtype=torch.float32, device=q.device)
+    # (empty_like is the cheaper call; it keeps the strides of a dense input, so it is for contiguous ones)
+    out = (torch.empty_like(q, dtype=torch.float32) if q.is_contiguous()
+           else torch.empty(n_prob, H, D, dtype=torch.float32, device=q.device))
     lse = torch.empty(n_prob, H, dtype=torch.float32, device=q.device) if want_lse else None
     _check(lib().decode_attention(C.addressof(p), n_prob, _ptr(q), _ptr(k_cache), _ptr(v_cache), n_rows,
                                           _ptr(n_valid), _ptr(out), _ptr(lse), _ptr(ws), ws.numel(), _stream()),

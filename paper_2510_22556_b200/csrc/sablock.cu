@@ -729,7 +729,7 @@ sablock_status_t run_select(const Plan& pl, const sablock_params_t* p, const flo
 {
     SelectArgs a;
     a.s = s; a.e = e; a.s_ref = s_ref;
-    a.seg_start = seg_start; a.n_seg = n_seg;
+    a.seg_start = seg_start; a.n_seg = n_seg; a.seg_id = s ? at<int>(ws, pl.o_seg_id) : nullptr;
     a.alpha = p->alpha; a.eta = p->eta; a.tau = p->tau;
     a.keep = at<unsigned>(ws, pl.o_keep); a.keep_words = pl.keep_words;
     a.phi = at<double>(ws, pl.o_phi);

@@ -36,6 +36,7 @@ struct SelectArgs {
     float* s_ref;              // refined scores, written (or read, see s)
     const int* seg_start;
     const int* n_seg;
+    const int* seg_id;         // segment of every token, or NULL (sablock_select)
     float alpha, eta, tau;
     unsigned* keep;            // scratch of ranges beyond kSelCap: [n_prob][keep_words]
     int keep_words;
@@ -809,7 +810,9 @@ select_kernel(const Geo g, const Cands cands, const SelectArgs a)
     const int ns = a.n_seg[seq];
     if (warp < 2) {                                // the segments that start in this CTA's share of the tokens
         const int v = (int)((long long)T * (rank + warp) / C);
-        const int kk = rank + warp == C ? ns : rank + warp == 0 ? 0 : warp_lower_bound(sst, ns, v);
+        int kk = rank + warp == C ? ns : 0;
+        if (rank + warp > 0 && rank + warp < C)    // segments that start before v = the segment of token v - 1, and those before it
+            kk = a.seg_id ? a.seg_id[g.cu[seq] + v - 1] + 1 : warp_lower_bound(sst, ns, v);
         if ((tid & 31) == 0) (warp ? sm.kz : sm.ka) = kk;
     }
     if (C > 1) cluster_sync(); else __syncthreads();           // barriers and counters of all CTAs are set up
