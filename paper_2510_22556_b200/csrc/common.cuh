@@ -26,8 +26,8 @@ constexpr int kStatInternal = 2;   // an internal consistency check failed
 constexpr long long kWaitLimitCycles = SABLOCK_WAIT_LIMIT_CYCLES;
 
 // The first wait of a launch that gave up leaves (code | CTA << 8 | warp << 20) in the word after
-// the status word.  Codes 1-29: waits of the persistent score kernel; 30: look-back of the
-// segmentation scan; 31: CTAs of a problem in the Top-B select.
+// the status word.  Codes 1-29: waits of the tensor-core score kernels; 30: CTAs of a
+// sequence in the segmentation; 31: CTAs of a problem in the selection.
 constexpr int kGiveupSegment = 30;
 constexpr int kGiveupTopB = 31;
 __device__ __forceinline__ void note_giveup(int* status, int code)
@@ -36,9 +36,10 @@ __device__ __forceinline__ void note_giveup(int* status, int code)
 }
 
 // Test builds only (-DSABLOCK_TEST_HOOKS): a word, set from the host, that makes one producer skip
-// its post so that the waiting side runs into its limit.  bit 0: the second tile of the segmentation
-// scan never publishes its state; bit 1: CTA 0 of every Top-B problem never reports its first
-// histogram; bit 2: CTA 0 of the persistent score kernel never reports its row sums of phase 0.
+// its post so that the waiting side runs into its limit.  bit 0: CTA 1 of a segmentation cluster never
+// reports its count; bit 1: CTA 0 of every selection cluster never reports its first digit counts; bit
+// 2: CTA 0 of the persistent score kernel never reports its row sums of phase 0, the first unit of the
+// unit flow not its own.
 // Production builds compile none of this.
 #ifdef SABLOCK_TEST_HOOKS
 __device__ int g_test_hooks;
