@@ -702,8 +702,9 @@ __device__ bool sel_body(const Geo& g, const Cands& cands, const SelectArgs& a, 
             }
             search = any && n <= kSegShort;
         }
+        const int n_old = sm.n_active;             // read before the barrier: behind it the first warps already count themselves in
         const int n_new = __syncthreads_count(search);
-        if (sm.n_active + n_new > kSelMaxActive) flush();
+        if (n_old + n_new > kSelMaxActive) flush();
         if (search) {
             SelActive& s = active[atomicAdd(&sm.n_active, 1)];
             s.pos = pos; s.k = kk; s.n = (unsigned short)n; s.b = (unsigned short)b; s.passed = 0u;

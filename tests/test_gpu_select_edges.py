@@ -67,3 +67,15 @@ def test_select_many_problems(n_layers, L):
         r = oracle.select(sr[l, :T].astype(np.float64), st, 112, cfg.candidates, tau=float(np.float32(0.85)))
         assert out.out_idx[l, 0, :112].cpu().numpy().tolist() == r["keep"].tolist()
         assert out.out_idx[l, 0, 112:].cpu().numpy().tolist() == list(range(T, L))
+
+
+@pytest.mark.parametrize("T,seg,B_tok", [
+    (1800, 3, 1500),           # one CTA, 600 segments to search: one round, although a count read late looks like two
+    (2014, 2, 2000),           # 1007 of them: a round's list all but full
+    (33280, 2, 33000),         # eight CTAs with 2080 each: the list is emptied in between
+])
+def test_select_counts_the_segments_of_a_round_once(T, seg, B_tok):
+    """More than 512 segments to search in a round: whether the list of segments has to be emptied first is decided by
+    every thread alike."""
+    for rep in range(4):
+        _select_case(T, 32, np.full(T // seg, seg, np.int64), B_tok, CANDS, 0.85, False, T + rep)
