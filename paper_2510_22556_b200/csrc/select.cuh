@@ -812,7 +812,9 @@ select_kernel(const Geo g, const Cands cands, const SelectArgs a)
     if (warp < 2) {                                // the segments that start in this CTA's share of the tokens
         const int v = (int)((long long)T * (rank + warp) / C);
         int kk = rank + warp == C ? ns : 0;
-        if (rank + warp > 0 && rank + warp < C)    // segments that start before v = the segment of token v - 1, and those before it
+        // segments that start before v = the segment of token v - 1, and those before it; none before v = 0, which a
+        // sequence of fewer tokens than CTAs has at inner boundaries too
+        if (v > 0 && rank + warp < C)
             kk = a.seg_id ? a.seg_id[g.cu[seq] + v - 1] + 1 : warp_lower_bound(sst, ns, v);
         if ((tid & 31) == 0) (warp ? sm.kz : sm.ka) = kk;
     }

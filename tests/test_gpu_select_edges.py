@@ -79,3 +79,32 @@ def test_select_counts_the_segments_of_a_round_once(T, seg, B_tok):
     every thread alike."""
     for rep in range(4):
         _select_case(T, 32, np.full(T // seg, seg, np.int64), B_tok, CANDS, 0.85, False, T + rep)
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("B_tok", [1, 2, 4])
+def test_select_sequences_shorter_than_a_cluster(B_tok, order):
+    """A few compressible tokens beside a long prompt, whose cluster size they get: most shares are empty."""
+    W = 16
+    lens = [9000] + [W + t for t in range(2, 10)] + [W + 1, 9000]
+    if order:
+        lens = lens[1:] + lens[:1]                               # a short sequence comes first in the packed rows
+    cfg = synth.Config("t", 2, 8, 2, 64, W, tuple(lens), (W + B_tok,), (1, 2, 4), "bf16", 5000, 8, 2.0, 3, (), 3)
+    b = synth.make_batch(cfg, device="cuda")
+    p = B.make_params(8, 2, 64, W, torch.bfloat16, b.bitmap, cfg.vocab)
+    cu, total = b.cu_seqlens, b.cu_seqlens[-1]
+    ws = B.alloc_workspace(p, total, 9000, len(lens), 2)
+    ws.fill_(0x7f)                                               # what the pass does not write holds large numbers
+    out = B.compress_layers(p, b.q_win, b.k, b.v, b.token_ids, cu, W + B_tok, cfg.candidates, ws)
+    _sync_ok(ws)
+    sr = B.workspace_view(p, ws, "s_refined", total, 9000, len(lens), 2).cpu().numpy()
+    for l in range(2):
+        for i, L in enumerate(lens):
+            idx = out.out_idx[l, i].cpu().numpy()
+            if L <= W + B_tok:
+                assert int(out.n_keep[l, i]) == L and idx[:L].tolist() == list(range(L))
+                continue
+            T = L - W
+            _, st = oracle.segment(b.token_ids[cu[i]:cu[i + 1]], W, b.bitmap, cfg.vocab)
+            r = oracle.select(sr[l, cu[i]:cu[i] + T].astype(np.float64), st, B_tok, cfg.candidates, tau=float(np.float32(0.85)))
+            assert idx[:B_tok].tolist() == r["keep"].tolist() and idx[B_tok:].tolist() == list(range(T, L))
