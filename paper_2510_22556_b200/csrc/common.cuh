@@ -64,7 +64,7 @@ struct Cands {
     int g[kMaxCand];
 };
 
-__device__ __forceinline__ int geo_L(const Geo& g, int seq) { return g.cu[seq + 1] - g.cu[seq]; }
+__host__ __device__ __forceinline__ int geo_L(const Geo& g, int seq) { return g.cu[seq + 1] - g.cu[seq]; }
 // A sequence is returned unchanged when it already fits in the output rows.
 __device__ __forceinline__ bool geo_identity(const Geo& g, int seq) { return geo_L(g, seq) <= g.n_out; }
 

@@ -1068,6 +1068,19 @@ int sablock_test_set_hooks(int hooks)
 {
     return (int)cudaMemcpyToSymbol(sab::g_test_hooks, &hooks, sizeof(int));
 }
+
+// The problem that a problem of a flow launch waits for before it writes the carry of a tile (host only).
+int sablock_test_carry_tenant(int n_seqs, const int* cu, int window, int n_out, int index, int tile)
+{
+    static Geo g;
+    static FlowArgs fa;
+    memset(&fa, 0, sizeof(fa));
+    g.n_seqs = n_seqs; g.window = window; g.n_out = n_out;
+    for (int i = 0; i <= n_seqs; ++i) g.cu[i] = cu[i];
+    for (int i = 0; i < n_seqs; ++i)
+        if (cu[i + 1] - cu[i] > n_out) fa.sel[fa.n_sel++] = (unsigned char)i;
+    return fl_carry_tenant(g, fa, index, tile);
+}
 #endif
 
 sablock_status_t sablock_segment(const sablock_params_t* p, const int* token_ids, int L, int* seg_id, int* seg_start,

@@ -60,7 +60,7 @@ struct FlowArgs {
     int* done;               // [problem][n_groups] heads of the group whose log-sum-exps are there
     int* bdone;              // [problem][tile] warps that have left the carry of the tile, all head groups together
     float* carry;            // [kFlCarryRing][tile][W][128]: head-summed attention between two head groups; problem i of the
-                             // launch has slot i % kFlCarryRing
+                             // launch has slot i % kFlCarryRing once the previous tenant of the tile (fl_carry_tenant) is through
     int max_tiles;           // per problem, for bdone and carry
     int* ticket;
     int n_sel, n_prob;       // sequences of the launch (the ones not returned unchanged) and problems = layers * n_sel
@@ -81,8 +81,6 @@ struct FlUnit {
     int tok_base, Tn;        // first packed token row and compressible length of the sequence
     int layer, group;
     int index;               // A: which partial of the row block.  B: number of the problem in the launch
-    int prev, prev_tiles;    // B: the problem whose carry slot this one takes over (-1: none), and its tiles
-    int pad;
 };
 
 struct FlShared {
@@ -128,6 +126,19 @@ __device__ __forceinline__ void fl_tiles(const Geo& g, int seq, int& ta, int& tb
     tb = (L - g.window + kTcTile - 1) / kTcTile;
 }
 
+// The problem of the call that used the carry of `tile` before problem `index` of the launch does: the nearest one before
+// it in the same slot that has this tile (sequences differ in length), or -1.  Whoever waits for all head groups of that one
+// has waited for all earlier ones, since each waited for its own predecessor.  At most n_sel steps back: there
+// the slot has the same sequence.
+__host__ __device__ inline int fl_carry_tenant(const Geo& g, const FlowArgs& fa, int index, int tile)
+{
+    for (int pi = index - kFlCarryRing; pi >= 0; pi -= kFlCarryRing) {
+        const int layer = pi / fa.n_sel, seq = fa.sel[pi - layer * fa.n_sel];
+        if (tile * kTcTile < geo_L(g, seq) - g.window) return layer * g.n_seqs + seq;
+    }
+    return -1;
+}
+
 // Lane quarter at which set s has its window rows in an A unit.
 __device__ __forceinline__ int fl_shift(int R, int s) { return R <= 32 ? s : R <= 64 ? (s & 1) * 2 : 0; }
 
@@ -136,8 +147,7 @@ __device__ __forceinline__ FlUnit fl_decode(const Geo& g, const FlowArgs& fa, co
 {
     FlUnit u;
     u.kind = 2;
-    u.prob = u.j0 = u.nh = u.tile0 = u.nt = u.tok_base = u.Tn = u.layer = u.group = u.index = u.prev_tiles = u.pad = 0;
-    u.prev = -1;
+    u.prob = u.j0 = u.nh = u.tile0 = u.nt = u.tok_base = u.Tn = u.layer = u.group = u.index = 0;
     const int ng = fa.n_groups, period = fa.n_sel * ng, n_v = fa.n_prob * ng;
     int v = -1, off = 0;
     bool is_a = false;
@@ -188,11 +198,6 @@ __device__ __forceinline__ FlUnit fl_decode(const Geo& g, const FlowArgs& fa, co
         u.tile0 = fa.head_split ? off : off * 4;
         u.nt = min(fa.head_split ? 1 : 4, tb - u.tile0);
         u.index = pi;
-        if (pi >= kFlCarryRing) {
-            const int lp = (pi - kFlCarryRing) / fa.n_sel, sp = fa.sel[pi - kFlCarryRing - lp * fa.n_sel];
-            u.prev = lp * g.n_seqs + sp;
-            fl_tiles(g, sp, ta, u.prev_tiles);
-        }
     }
     return u;
 }
@@ -710,9 +715,10 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                     if (split && set > 0) {
                         // set 0 goes on with the tokens
                     } else if (u.group < fa.n_groups - 1) {
-                        if (u.group == 0 && u.prev >= 0 && tile < u.prev_tiles) {        // the slot's previous tenant is through
-                            if (lane == 0)
-                                ok = FL_WAIT(19, wait_counter(fa.bdone + (size_t)u.prev * fa.max_tiles + tile, 4 * fa.n_groups,
+                        if (u.group == 0) {                      // the slot's previous tenant is through
+                            const int prev = lane == 0 ? fl_carry_tenant(g, fa, u.index, tile) : -1;
+                            if (prev >= 0)
+                                ok = FL_WAIT(19, wait_counter(fa.bdone + (size_t)prev * fa.max_tiles + tile, 4 * fa.n_groups,
                                                               abort_flag, fa.status));
                             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
                             if (!ok) break;
@@ -740,7 +746,8 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                             fa.s_out[o] = tot / (float)g.H;      // Eqs. 3, 4
                             fa.e_out[o] = ent;
                         }
-                        if (fa.n_groups > 1) {
+                        if (fa.n_groups > 1) {                   // the carry is read: the slot may be written again
+                            __threadfence();
                             __syncwarp();
                             if (lane == 0) atomicAdd(bdone, 1);
                         }

@@ -92,3 +92,16 @@ def test_packed(lse):
 @pytest.mark.parametrize("lens,n_layers", [([3000], 6), ([900, 2500, 40], 4)])
 def test_single_sweep_with_two_groups(lens, n_layers):
     _run(64, 16, 128, 32, lens, n_layers, 64, True)
+
+
+@pytest.mark.parametrize("H,Hkv,D,W", [(64, 16, 128, 32),        # two groups of eight heads, 128 window rows each
+                                       (35, 35, 64, 32),         # 18 and 17 heads of 32 rows: a smaller last group
+                                       (255, 17, 64, 8)])        # 6, 6 and 5 heads of 120 rows: a group between two others
+@pytest.mark.parametrize("lens,n_layers", [([3000, 300, 3000], 4),
+                                           ([12800] + [129] * 7, 3),
+                                           ([700, 40, 2500, 900, 130, 1300], 4)])
+@pytest.mark.parametrize("lse", [False, True])
+def test_carry_between_head_groups(H, Hkv, D, W, lens, n_layers, lse):
+    """More than 1024 window rows: the head groups hand their sums on through scratch that problems of other lengths have
+    used before."""
+    _run(H, Hkv, D, W, lens, n_layers, 64, lse)
