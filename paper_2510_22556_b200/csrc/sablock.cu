@@ -209,7 +209,7 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     const long long m = tiles * g.Hkv * pl->n_prob / (8LL * sm_count());
     pl->fl_m = (int)(m < 1 ? 1 : m > 4 ? 4 : m);
     pl->fl_parts = (int)((tiles + 4 * pl->fl_m - 1) / (4 * pl->fl_m));
-    {   // head groups: as many heads as have room for their log-sum-exps
+    if (flow_ok) {   // head groups: as many heads as have room for their log-sum-exps (at most 128 window rows each)
         int h = kFlMaxRows / (g.G * p->window);
         if (h > g.Hkv) h = g.Hkv;
         pl->fl_groups = (g.Hkv + h - 1) / h;

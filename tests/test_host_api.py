@@ -54,6 +54,15 @@ def test_workspace_bytes(lib):
     assert lib.sablock_workspace_bytes(C.addressof(p), 100, 100, 65, 1) == 0
 
 
+@pytest.mark.parametrize("kw", [dict(n_q_heads=64, n_kv_heads=1, window=32), dict(n_q_heads=64, n_kv_heads=1, window=17),
+                                dict(n_q_heads=256, n_kv_heads=1, window=8), dict(n_q_heads=64, n_kv_heads=1, dtype=torch.float32)])
+def test_workspace_bytes_with_many_window_rows_per_kv_head(lib, kw):
+    """More than 1024 window rows of one KV head (multi-query attention): sized like any other shape of the plain score
+    kernels."""
+    n = B.workspace_bytes(_params(**kw), 8192, 8192)
+    assert B.workspace_bytes(_params(), 8192, 8192) // 4 < n < 1024 ** 3
+
+
 @pytest.mark.parametrize("kw,code", [
     (dict(n_q_heads=30), 1), (dict(window=0), 1), (dict(pool_kernel=4), 1), (dict(score_impl=7), 1),
     (dict(window=128), 2), (dict(head_dim=512), 2), (dict(head_dim=100, score_impl=B.SCORE_TENSOR), 2),
