@@ -60,7 +60,7 @@ def test_workspace_bytes_with_many_window_rows_per_kv_head(lib, kw):
     """More than 1024 window rows of one KV head (multi-query attention): sized like any other shape of the plain score
     kernels."""
     n = B.workspace_bytes(_params(**kw), 8192, 8192)
-    assert B.workspace_bytes(_params(), 8192, 8192) // 4 < n < 1024 ** 3
+    assert 28 * 8192 < n < 1024 ** 3                             # segment ids and starts, s, e, refined s, block scores: 28 bytes a token
 
 
 @pytest.mark.parametrize("kw,code", [
