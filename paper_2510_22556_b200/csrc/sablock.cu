@@ -235,25 +235,13 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
         pl->n_chunks = (int)((tiles + pl->tpc1 - 1) / pl->tpc1);
         pl->units = g.Hkv * (flow_ok ? 1 + (pl->fl_parts + kFlMerge - 1) / kFlMerge : 1);
     } else {
-        // SIMT passes: as many heads per thread as the KV head has (up to four) and shared memory holds;
-        // pass 1 gets one wave of two CTAs per SM (what shared memory holds at D = 128) and at most
+        // SIMT passes: pass 1 gets one wave of two CTAs per SM (what shared memory holds at D = 128) and at most
         // kSimtMaxChunks partials per row.
         SimtShape& sp = pl->simt;
-        int w_log2 = 0;
-        while ((1 << w_log2) < p->window) ++w_log2;
-        sp.tok = kSimtTokLarge;
-        sp.wp_log2 = w_log2 > 0 ? w_log2 - 1 : 0;                    // (two window positions per thread)
-        sp.tile = (kSimtThreads >> sp.wp_log2) * sp.tok;
-        sp.gb = g.G >= 3 ? 4 : g.G;
-        while (sp.gb > 1 && simt_smem_bytes(sp.gb, p->window, g.D, sp.tile) > kSimtSmemMax) sp.gb /= 2;
-        sp.batches = (g.G + sp.gb - 1) / sp.gb;
+        simt_tile(sp, g.G, p->window, g.D, false);
+        if ((long long)((max_L + sp.tile - 1) / sp.tile) * g.Hkv * sp.batches * pl->n_prob < sm_count())
+            simt_tile(sp, g.G, p->window, g.D, true);
         const long long units = (long long)g.Hkv * sp.batches;
-        if ((max_L + sp.tile - 1) / sp.tile * units * pl->n_prob < sm_count()) {
-            sp.tok = kSimtTokSmall;
-            sp.wp_log2 = w_log2;
-            sp.tile = (kSimtThreads >> sp.wp_log2) * sp.tok;
-        }
-        sp.smem = simt_smem_bytes(sp.gb, p->window, g.D, sp.tile);
         const long long tl = (max_L + sp.tile - 1) / sp.tile;
         long long tpc = (tl * units * pl->n_prob + sm_count() * 2 - 1) / (sm_count() * 2);
         if (tpc < (tl + kSimtMaxChunks - 1) / kSimtMaxChunks) tpc = (tl + kSimtMaxChunks - 1) / kSimtMaxChunks;
@@ -1067,6 +1055,14 @@ sablock_status_t sablock_read_status_detail(const void* ws, sablock_stream_t str
 int sablock_test_set_hooks(int hooks)
 {
     return (int)cudaMemcpyToSymbol(sab::g_test_hooks, &hooks, sizeof(int));
+}
+
+// Dynamic shared memory of the SIMT score passes of a call, 0 where the tensor cores take it (host only).
+int sablock_test_simt_smem(const sablock_params_t* p, int max_L, int n_layers)
+{
+    Plan pl;
+    if (make_plan(p, n_layers, 1, nullptr, max_L, max_L, p->window + 1, &pl) != SABLOCK_OK) return -1;
+    return pl.use_tc ? 0 : pl.simt.smem;
 }
 
 // The problem that a problem of a flow launch waits for before it writes the carry of a tile (host only).

@@ -26,7 +26,8 @@ constexpr int kSimtMaxW = 64;
 constexpr int kSimtMaxD = 256;
 constexpr int kSimtMaxSplit = 8;                        // CTAs of a cluster that share the KV heads of a token tile
 constexpr int kSimtMaxChunks = 64;                      // pass-1 partials per window row
-constexpr int kSimtSmemMax = 200 * 1024;
+constexpr int kSimtSmemMax = 200 * 1024;                // heads per thread are given up above this
+constexpr int kSimtSmemLimit = 226 * 1024;              // what a CTA may have beside its few static words
 
 // Partial row statistics of pass 1: (m, l) with m the running maximum (log2 units) and
 // l = sum exp2(x2 - m) over the keys seen.
@@ -57,6 +58,30 @@ __host__ __device__ inline int simt_smem_bytes(int gb, int W, int D, int tile)
     int n = gb * W * (D + 4) + (keys > red ? keys : red);
     if (sums > n) n = sums;
     return n * (int)sizeof(float);
+}
+
+// Heads per thread and tile of a parameter block: as many heads as the KV head has (up to four) and shared memory holds.
+// Eight tokens a thread, two where `few` (the large tiles would not give every SM one) or where rows are so long
+// and window positions so few that the large tile does not fit (fewer threads along the window are
+// more token rows: 274 KB for rows of 256 at window 8, 540 KB for rows of 128 at window 1).  For a single window position and
+// rows of more than 220 even the small one is halved, by threads along the window that have no position.
+__host__ inline void simt_tile(SimtShape& sp, int G, int W, int D, bool few)
+{
+    int w_log2 = 0;
+    while ((1 << w_log2) < W) ++w_log2;
+    auto fit = [&](int tok, int wp_log2) {
+        sp.tok = tok;
+        sp.wp_log2 = wp_log2;
+        sp.tile = (kSimtThreads >> wp_log2) * tok;
+        sp.gb = G >= 3 ? 4 : G;
+        while (sp.gb > 1 && simt_smem_bytes(sp.gb, W, D, sp.tile) > kSimtSmemMax) sp.gb /= 2;
+        return simt_smem_bytes(sp.gb, W, D, sp.tile) <= kSimtSmemLimit;
+    };
+    const bool large = !few && fit(kSimtTokLarge, w_log2 > 0 ? w_log2 - 1 : 0);       // (two window positions per thread)
+    if (!large)
+        for (int wp = w_log2; !fit(kSimtTokSmall, wp); ++wp) { }
+    sp.batches = (G + sp.gb - 1) / sp.gb;
+    sp.smem = simt_smem_bytes(sp.gb, W, D, sp.tile);
 }
 
 // Single-sweep mode: the caller knows ln sum_j exp(logit_j) of every window row (the prefill's

@@ -36,6 +36,31 @@ def test_fp32_scores(H, Hkv, D, W, L, layers):
         assert float((e[l, :L - W].double() - re).abs().max()) <= 4e-4
 
 
+@pytest.mark.parametrize("H,Hkv,D,W", [(16, 8, 256, 8), (4, 4, 256, 4), (6, 2, 256, 1), (8, 8, 128, 1), (8, 2, 128, 2), (8, 2, 128, 4),
+                                       (8, 4, 192, 3), (4, 4, 64, 2), (3, 1, 112, 4)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("L,layers", [(9000, 1), (1500, 10)])
+@pytest.mark.parametrize("lse", [False, True])
+def test_long_rows_and_few_window_positions(H, Hkv, D, W, dtype, L, layers, lse):
+    """Shapes whose tile of eight tokens a thread would not fit shared memory."""
+    dt = synth.torch_dtype(dtype)
+    cfg = synth.Config("t", layers, H, Hkv, D, W, (L,), (W + 20,), (1, 2, 4), dtype, 5000, 8, 2.0, 20, (), 3)
+    b = synth.make_batch(cfg, device="cuda")
+    kw = dict(row_lse=synth.prefill_row_lse(b.q_win, b.k, b.cu_seqlens)) if lse else {}
+    p = B.make_params(H, Hkv, D, W, dt, b.bitmap, cfg.vocab, **kw)
+    ws = B.alloc_workspace(p, L, L, 1, layers)
+    B.compress_layers(p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, W + 20, cfg.candidates, ws)
+    torch.cuda.synchronize()
+    assert B.read_status(ws) == 0
+    s = B.workspace_view(p, ws, "s", L, L, 1, layers)
+    e = B.workspace_view(p, ws, "e", L, L, 1, layers)
+    scale = max(1.0, (D / 128) ** 0.5)                           # the bound above grows with the root of D
+    for l in range(layers):
+        rs, re = _reference(b.q_win[l, 0], b.k[l], W)
+        assert float(((s[l, :L - W].double() - rs).abs() / rs).max()) <= 2e-4 * scale
+        assert float((e[l, :L - W].double() - re).abs().max()) <= 4e-4 * scale
+
+
 def test_fp32_unaligned_rows():
     """Keys whose address is a multiple of 4 bytes only."""
     H, Hkv, D, W, L = 8, 2, 64, 16, 777

@@ -3,7 +3,9 @@ that the device code uses."""
 import ctypes as C
 
 import pytest
+import torch
 
+from paper_2510_22556_b200 import binding as B
 from paper_2510_22556_b200.build import build_test_hooks
 
 
@@ -31,3 +33,18 @@ def test_a_carry_slot_is_taken_over_from_the_last_tenant_that_has_the_tile(rules
             assert got == last.get((index % 4, tile), -1), (index, tile)
         for tile in range((lens[i] - W + 127) // 128):
             last[index % 4, tile] = layer * len(lens) + i
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("H,Hkv", [(1, 1), (2, 1), (3, 1), (8, 8), (16, 8), (32, 8), (14, 2), (64, 1)])
+def test_the_plain_score_passes_fit_shared_memory(rules, dtype, H, Hkv):
+    """Every head dimension and window that the parameter check accepts, few and many tiles."""
+    p = B.make_params(H, Hkv, 64, 8, dtype)
+    p.score_impl = B.SCORE_SIMT
+    at = C.c_void_p(C.addressof(p))
+    for D in range(4 if dtype == torch.float32 else 8, 257, 4 if dtype == torch.float32 else 8):
+        for W in range(1, min(64, 2048 // H) + 1):
+            p.head_dim, p.window = D, W
+            for L, layers in ((W + 5, 1), (9000, 1), (9000, 32)):
+                n = rules.sablock_test_simt_smem(at, L, layers)
+                assert 0 < n <= 226 * 1024, (D, W, L, layers, n)
