@@ -1057,6 +1057,9 @@ int sablock_test_set_hooks(int hooks)
     return (int)cudaMemcpyToSymbol(sab::g_test_hooks, &hooks, sizeof(int));
 }
 
+// Barrier (bit 1) and parity (bit 0) of the n-th exchange of a cluster (host only).
+int sablock_test_exchange(int n) { return exchange_barrier(n) * 2 + exchange_parity(n); }
+
 // Dynamic shared memory of the SIMT score passes of a call, 0 where the tensor cores take it (host only).
 int sablock_test_simt_smem(const sablock_params_t* p, int max_L, int n_layers)
 {

@@ -62,7 +62,7 @@ struct SelShared {
     int long_list[64];         // segments left to the whole CTA
     int scan[kSelWarps];
     double red[kSelWarps];
-    uint64_t bar;              // arrivals of the cluster's CTAs
+    uint64_t bars[2];          // arrivals of the cluster's CTAs, one exchange each in turn
 };
 
 // A segment to search: position (relative to the CTA's range), number, length, implicit budget, and
@@ -108,7 +108,7 @@ __device__ __forceinline__ int warp_lower_bound(const int* __restrict__ x, int n
 
 __device__ __forceinline__ bool sel_exchange(SelShared& sm, int C, int n, bool post, int* status)
 {
-    const bool ok = cluster_exchange(&sm.bar, C, n, post);
+    const bool ok = cluster_exchange(sm.bars, C, n, post);
     if (!ok && threadIdx.x == 0) {
         atomicOr(status, kStatTimeout);
         note_giveup(status, kGiveupTopB);
@@ -791,7 +791,8 @@ select_kernel(const Geo g, const Cands cands, const SelectArgs a)
         sm.n_active = 0;
         sm.next = 0;
         sm.n_long = 0;
-        mbar_init(smem_u32(&sm.bar), C);
+        mbar_init(smem_u32(&sm.bars[0]), C);
+        mbar_init(smem_u32(&sm.bars[1]), C);
         fence_mbar_init();
     }
     pdl_wait();

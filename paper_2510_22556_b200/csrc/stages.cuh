@@ -21,13 +21,20 @@ constexpr int kSegMinTokens = 1024;                // per CTA of a cluster
 constexpr int kSegMapWords = 6144;                 // delimiter bitmap in shared memory: 196608 ids
 constexpr int kSegMapTokens = 4096;                // tokens per CTA from which that pays
 
+// Barrier and parity of the n-th exchange of a cluster (n counts from 0).  Two barriers take turns: a CTA that has seen
+// exchange n complete may post n + 1 to a CTA that still lacks a third one's arrival for n, and on one barrier that
+// post would complete n there.  A post for n + 2 comes after exchange n + 1, for which that CTA has posted, so after its n.
+__host__ __device__ constexpr int exchange_barrier(int n) { return n & 1; }
+__host__ __device__ constexpr int exchange_parity(int n) { return (n >> 1) & 1; }
+
 // Arrivals of a cluster's CTAs, for exchanges through distributed shared memory: every CTA posts to
-// all barriers; all have arrived `n` times (n counts from 0) when wait returns true, and what each wrote
-// before is visible.  Bounded; false if it gave up.  Called by every thread.
-__device__ __forceinline__ bool cluster_exchange(uint64_t* bar, int C, int n, bool post)
+// all of them; all have arrived for exchange `n` when wait returns true, and what each wrote
+// before is visible.  `bars`: two barriers (one, if there is one exchange).  Bounded; false if it gave up.  Called by every thread.
+__device__ __forceinline__ bool cluster_exchange(uint64_t* bars, int C, int n, bool post)
 {
     __syncthreads();
     if (C == 1) return true;
+    uint64_t* bar = bars + exchange_barrier(n);
     if ((int)threadIdx.x < C && post)
         asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_map(bar, (int)threadIdx.x)) : "memory");
     const uint32_t b = smem_u32(bar);
@@ -38,7 +45,7 @@ __device__ __forceinline__ bool cluster_exchange(uint64_t* bar, int C, int n, bo
         asm volatile("{\n\t.reg .pred p;\n\t"
                      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
                      "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done) : "r"(b), "r"((uint32_t)(n & 1)), "r"(20000u) : "memory");
+                     : "=r"(done) : "r"(b), "r"((uint32_t)exchange_parity(n)), "r"(20000u) : "memory");
         if (done) { ok = true; break; }
         if (clock64() - t0 > kWaitLimitCycles) break;
     }

@@ -48,3 +48,37 @@ def test_the_plain_score_passes_fit_shared_memory(rules, dtype, H, Hkv):
             for L, layers in ((W + 5, 1), (9000, 1), (9000, 32)):
                 n = rules.sablock_test_simt_smem(at, L, layers)
                 assert 0 < n <= 226 * 1024, (D, W, L, layers, n)
+
+
+@pytest.mark.parametrize("n_ctas,n_exchanges", [(2, 6), (3, 4)])
+def test_an_exchange_is_complete_when_every_cta_has_posted(rules, n_ctas, n_exchanges):
+    """Every order in which the posts of a cluster can arrive: a CTA that leaves exchange n does so after all CTAs have posted n.
+    A barrier counts arrivals and flips its phase at every n_ctas of them; a wait on a parity ends once the phase of that parity
+    is over."""
+    where = [divmod(rules.sablock_test_exchange(n), 2) for n in range(n_exchanges)]
+    # state: per CTA the exchange it waits for (its post is out); posts under way (exchange, to); arrivals per CTA and barrier
+    start = (tuple([0] * n_ctas), frozenset((c, 0, to) for c in range(n_ctas) for to in range(n_ctas)), tuple([(0, 0)] * n_ctas))
+    seen, todo = {start}, [start]
+    while todo:
+        at, flying, got = todo.pop()
+        nxt = []
+        for post in flying:
+            _, n, to = post
+            bar = where[n][0]
+            g = list(map(list, got))
+            g[to][bar] += 1
+            nxt.append((at, flying - {post}, tuple(map(tuple, g))))
+        for c in range(n_ctas):
+            n = at[c]
+            if n == n_exchanges:
+                continue
+            bar, parity = where[n]
+            if (got[c][bar] // n_ctas) % 2 != parity:            # the phase with that parity has completed
+                assert all(a >= n for a in at) and not any(m == n and to == c for _, m, to in flying), (at, flying, got)
+                a2 = tuple(a + 1 if i == c else a for i, a in enumerate(at))
+                more = frozenset((c, n + 1, to) for to in range(n_ctas)) if n + 1 < n_exchanges else frozenset()
+                nxt.append((a2, flying | more, got))
+        for s in nxt:
+            if s not in seen:
+                seen.add(s)
+                todo.append(s)
