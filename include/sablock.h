@@ -7,7 +7,8 @@
  * Conventions (all entry points):
  *  - "dev" pointers are CUDA device pointers owned by the caller; "host" pointers are
  *    ordinary host memory.  The library never allocates or frees device memory: all
- *    scratch comes from the caller's workspace `ws` (size from sablock_workspace_bytes).
+ *    scratch comes from the caller's workspace `ws` (size from sablock_workspace_bytes; any address that
+ *    is a multiple of 8, a multiple of 16 where score_impl asks for the persistent kernel with row_lse).
  *  - Device work is enqueued asynchronously on `stream` (a cudaStream_t passed as void*).
  *    The return code reports host-side validation and launch errors only; on any error
  *    nothing further is enqueued.  Conditions detected on the device (a bounded wait that

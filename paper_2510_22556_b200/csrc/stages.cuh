@@ -52,10 +52,20 @@ __device__ __forceinline__ bool cluster_exchange(uint64_t* bars, int C, int n, b
     return __syncthreads_and(ok) != 0;
 }
 
+// This thread's share (`first`, `first` + `stride`, ...) of n16 16-byte pieces of control words.  A workspace may start on
+// any boundary that its elements allow: by words where that is not one of 16 bytes.
+__device__ __forceinline__ void clear_control(uint4* ctl, size_t n16, size_t first, size_t stride)
+{
+    if ((reinterpret_cast<uintptr_t>(ctl) & 15) == 0)
+        for (size_t i = first; i < n16; i += stride) ctl[i] = make_uint4(0, 0, 0, 0);
+    else
+        for (size_t i = first; i < 4 * n16; i += stride) reinterpret_cast<unsigned*>(ctl)[i] = 0u;
+}
+
 __global__ void clear_kernel(uint4* ctl, size_t n16)
 {
     pdl_wait();
-    for (size_t i = threadIdx.x; i < n16; i += blockDim.x) ctl[i] = make_uint4(0, 0, 0, 0);
+    clear_control(ctl, n16, threadIdx.x, blockDim.x);
     __threadfence();
     __syncthreads();
     pdl_launch();
@@ -83,8 +93,7 @@ segment_kernel(const Geo g, const int* __restrict__ token_ids, const unsigned* _
     // this one before its end; its accesses to them are atomics and acquire loads, which go to L2, where the
     // fence has put the zeros).
     if (ctl) {
-        const size_t stride = (size_t)C * gridDim.y * kSegThreads;
-        for (size_t i = ((size_t)seq * C + rank) * kSegThreads + tid; i < n16; i += stride) ctl[i] = make_uint4(0, 0, 0, 0);
+        clear_control(ctl, n16, ((size_t)seq * C + rank) * kSegThreads + tid, (size_t)C * gridDim.y * kSegThreads);
         __threadfence();
         __syncthreads();
     }
