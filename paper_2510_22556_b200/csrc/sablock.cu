@@ -827,11 +827,14 @@ HostStreams* host_streams()
 }
 
 // The plan of n_layers of a larger call's layers inside that call's workspace; false if a region would not
-// hold what it needs.
+// hold what it needs, or if so few layers would go to other kernels than the whole call (the tensor maps need 128
+// rows of queries).
 bool plan_inside(const Plan& whole, const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, int max_L, int n_out,
                  Plan* pl)
 {
     if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, pl) != SABLOCK_OK || pl->n_regions != whole.n_regions) return false;
+    if (pl->use_tc != whole.use_tc || pl->use_flow != whole.use_flow || pl->use_fused != whole.use_fused) return false;
+    if (pl->use_tc && (long long)pl->n_prob * pl->geo.H * pl->geo.window < kTcTile) return false;
     for (int i = 0; i < pl->n_regions; ++i) {
         if (pl->regions[i].bytes > whole.regions[i].bytes) return false;
         pl->*(pl->regions[i].field) = whole.*(whole.regions[i].field);
@@ -839,6 +842,21 @@ bool plan_inside(const Plan& whole, const sablock_params_t* p, int n_layers, int
     pl->control_bytes = whole.control_bytes;
     pl->total = whole.total;
     return true;
+}
+
+// Layers that go through a host-buffer pass at a time.  The copies take longer than everything else together (PCIe), so the
+// layers go through in chunks, a chunk's compute and the copies of its results behind the next chunk's copies: 4 layers
+// of 8K tokens 1.56 -> 1.43 ms.  At most eight chunks, and none of less than 4 MB of keys, which are not worth
+// their launches.  All layers at once where a chunk would not fit the plan of the whole call.
+int host_chunk(const Plan& whole, const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, int max_L, int n_out)
+{
+    const size_t layer_kv = (size_t)cu[n_seqs] * p->n_kv_heads * p->head_dim * elem_size(p);
+    const int by_size = (int)(((4u << 20) + layer_kv - 1) / layer_kv), by_count = (n_layers + 7) / 8;
+    const int want = by_size > by_count ? by_size : by_count;
+    Plan part;
+    if (want >= n_layers || !plan_inside(whole, p, want, n_seqs, cu, max_L, n_out, &part)) return n_layers;
+    if (n_layers % want && !plan_inside(whole, p, n_layers % want, n_seqs, cu, max_L, n_out, &part)) return n_layers;
+    return want;
 }
 
 // ---- decoding over a cache: launch plan ----------------------------------------------------
@@ -1055,6 +1073,14 @@ sablock_status_t sablock_read_status_detail(const void* ws, sablock_stream_t str
 int sablock_test_set_hooks(int hooks)
 {
     return (int)cudaMemcpyToSymbol(sab::g_test_hooks, &hooks, sizeof(int));
+}
+
+// Layers at a time of a host-buffer pass (host only).
+int sablock_test_host_chunk(const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, int max_L, int n_out)
+{
+    Plan pl;
+    if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, &pl) != SABLOCK_OK) return -1;
+    return host_chunk(pl, p, n_layers, n_seqs, cu, max_L, n_out);
 }
 
 // Barrier (bit 1) and parity (bit 0) of the n-th exchange of a cluster (host only).
@@ -1299,19 +1325,13 @@ sablock_status_t sablock_compress_layers_host(const sablock_params_t* p, int n_l
             cudaGetLastError();
     }
     const bool stage_v = v_src == dev_v;
-    // The copies take longer than everything else together (PCIe), so the layers go through in chunks, a chunk's compute and
-    // the copies of its results behind the next chunk's copies: 4 layers of 8K tokens 1.49 -> 1.33 ms.  The
-    // chunks use the workspace as one call over all layers would (same places for what a caller may look at
-    // afterwards); chunks of less than 4 MB of keys are not worth their launches.
-    int per = n_layers;
+    int per = host_chunk(pl, p, n_layers, n_seqs, cu_seqlens, max_L, n_out);
+    HostStreams* hs = per < n_layers ? host_streams() : nullptr;
+    if (!hs) per = n_layers;
     Plan part;
     const size_t layer_kv = kv_bytes / n_layers;
-    const int by_size = (int)(((4u << 20) + layer_kv - 1) / layer_kv), by_count = (n_layers + 7) / 8;
-    const int want = by_size > by_count ? by_size : by_count;
-    HostStreams* hs = want < n_layers ? host_streams() : nullptr;
-    if (hs && plan_inside(pl, p, want, n_seqs, cu_seqlens, max_L, n_out, &part) &&
-        (n_layers % want == 0 || plan_inside(pl, p, n_layers % want, n_seqs, cu_seqlens, max_L, n_out, &part)))
-        per = want;
+    // (The chunks use the workspace as one call over all layers would: same places for what a caller may look at
+    // afterwards.)
     cudaStream_t s_in = st, s_out = st;
     if (per < n_layers) {
         s_in = hs->in; s_out = hs->out;

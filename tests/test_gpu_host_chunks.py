@@ -13,11 +13,11 @@ from paper_2510_22556_b200 import binding as B
 pytestmark = pytest.mark.gpu
 
 
-def _case(n_layers, lens, budget=128, pinned=True, lse=False, pool=1, W=32):
-    cfg = synth.Config("t", n_layers, 32, 8, 128, W, tuple(lens), (budget,), (1, 2, 4, 8), "bf16", 128256, 16, 2.0, 25, (0.4,), 11)
+def _case(n_layers, lens, budget=128, pinned=True, lse=False, pool=1, W=32, H=32, impl=B.SCORE_AUTO):
+    cfg = synth.Config("t", n_layers, H, 8, 128, W, tuple(lens), (budget,), (1, 2, 4, 8), "bf16", 128256, 16, 2.0, 25, (0.4,), 11)
     b = synth.make_batch(cfg, device="cuda")
     kw = dict(row_lse=synth.prefill_row_lse(b.q_win, b.k, b.cu_seqlens)) if lse else {}
-    p = B.make_params(32, 8, 128, W, torch.bfloat16, b.bitmap, cfg.vocab, pool_kernel=pool, **kw)
+    p = B.make_params(H, 8, 128, W, torch.bfloat16, b.bitmap, cfg.vocab, pool_kernel=pool, score_impl=impl, **kw)
     total, max_L, ns = b.cu_seqlens[-1], max(lens), len(lens)
     ws, ws2 = (B.alloc_workspace(p, total, max_L, ns, n_layers) for _ in range(2))
     ref = B.compress_layers(p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, budget, cfg.candidates, ws2)
@@ -48,6 +48,7 @@ def _case(n_layers, lens, budget=128, pinned=True, lse=False, pool=1, W=32):
 @pytest.mark.parametrize("n_layers,lens,kw", [
     (1, [8192], {}), (2, [2049], {}), (3, [2049], {}), (4, [8192], {}), (5, [1500], {}), (9, [2100, 300, 100], {}),
     (17, [2500], dict(lse=True)), (4, [4096], dict(pool=7)), (4, [3000], dict(pinned=False)), (6, [5000], dict(W=8)),
+    (9, [2100], dict(W=8, H=8)), (9, [2100], dict(W=8, H=8, impl=B.SCORE_TENSOR)),       # a last layer alone would have 64 query rows
 ])
 def test_host_pass_in_chunks(n_layers, lens, kw):
     _case(n_layers, lens, **kw)

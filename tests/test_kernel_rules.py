@@ -82,3 +82,21 @@ def test_an_exchange_is_complete_when_every_cta_has_posted(rules, n_ctas, n_exch
             if s not in seen:
                 seen.add(s)
                 todo.append(s)
+
+
+@pytest.mark.parametrize("impl", [B.SCORE_AUTO, B.SCORE_TENSOR])
+@pytest.mark.parametrize("n_layers,lens,H,Hkv,W", [(9, [2100], 8, 8, 8), (9, [2100], 32, 8, 32), (17, [700, 1500], 8, 8, 8),
+                                                  (3, [2100], 8, 8, 8), (33, [4100], 8, 8, 8), (5, [4100, 90, 300], 16, 8, 8)])
+def test_chunks_of_a_host_pass_run_like_the_whole(rules, impl, n_layers, lens, H, Hkv, W):
+    """Either all layers at once or chunks of which each, the last one too, has the 128 query rows that the tensor maps
+    need."""
+    p = B.make_params(H, Hkv, 128, W, torch.bfloat16, score_impl=impl)
+    cu = (C.c_int * (len(lens) + 1))(0)
+    for i, n in enumerate(lens):
+        cu[i + 1] = cu[i] + n
+    per = rules.sablock_test_host_chunk(C.c_void_p(C.addressof(p)), n_layers, len(lens), cu, max(lens), 64)
+    assert 1 <= per <= n_layers
+    for at in range(0, n_layers, per):
+        assert min(per, n_layers - at) * len(lens) * H * W >= 128
+    if (H, W) == (32, 32):                                       # the rule itself, where nothing stands against it
+        assert per == max((n_layers + 7) // 8, -(-(4 << 20) // (cu[len(lens)] * Hkv * 256)))
