@@ -242,7 +242,8 @@ sablock_status_t sablock_compress_layers(const sablock_params_t *p, int n_layers
  * (pinned) host memory the gather reads those rows from it in place and dev_v is not written;
  * otherwise v is copied to dev_v first.  Pinned host memory also makes the copies asynchronous
  * with respect to each other; pageable memory works too.  All arguments are validated before the
- * first copy is enqueued. */
+ * first copy is enqueued; if a launch is refused after that (an alignment that the kernels need, a runtime error) the
+ * call waits for what it has enqueued before it returns the error. */
 sablock_status_t sablock_compress_layers_host(const sablock_params_t *p, int n_layers, int n_seqs,
                                               const void *h_q_win, const void *h_k, const void *h_v,
                                               const int *h_token_ids, const int *cu_seqlens, int budget,

@@ -1333,60 +1333,71 @@ sablock_status_t sablock_compress_layers_host(const sablock_params_t* p, int n_l
     // (The chunks use the workspace as one call over all layers would: same places for what a caller may look at
     // afterwards.)
     cudaStream_t s_in = st, s_out = st;
-    if (per < n_layers) {
-        s_in = hs->in; s_out = hs->out;
-        SAB_CUDA(cudaEventRecord(hs->ev[0], st), "host pass: event");              // what the caller has enqueued comes first
-        SAB_CUDA(cudaStreamWaitEvent(s_in, hs->ev[0], 0), "host pass: wait");
-        SAB_CUDA(cudaStreamWaitEvent(s_out, hs->ev[0], 0), "host pass: wait");
-    }
-    const size_t lq = q_bytes / n_layers, lo = okv_bytes / n_layers, n_idx = (size_t)n_seqs * n_out;
-    int launches = 0, n_ev = 1;
-    SAB_CUDA(cudaMemcpyAsync(dev_token_ids, h_token_ids, total * sizeof(int), cudaMemcpyHostToDevice, s_in), "host pass: copy in");
-    for (int l0 = 0; l0 < n_layers; l0 += per) {
-        const int nl = l0 + per <= n_layers ? per : n_layers - l0;
-        auto in = [&](const void* d, const void* h, size_t layer) {
-            return cudaMemcpyAsync((char*)const_cast<void*>(d) + l0 * layer, (const char*)h + l0 * layer, nl * layer,
-                                   cudaMemcpyHostToDevice, s_in);
-        };
-        auto out = [&](void* h, const void* d, size_t layer) {
-            return cudaMemcpyAsync((char*)h + l0 * layer, (const char*)d + l0 * layer, nl * layer, cudaMemcpyDeviceToHost, s_out);
-        };
-        SAB_CUDA(in(dev_q_win, h_q_win, lq), "host pass: copy in");
-        SAB_CUDA(in(dev_k, h_k, layer_kv), "host pass: copy in");
-        if (stage_v) SAB_CUDA(in(dev_v, h_v, layer_kv), "host pass: copy in");
+    if (per < n_layers) { s_in = hs->in; s_out = hs->out; }
+    const sablock_status_t rc = [&]() -> sablock_status_t {
         if (per < n_layers) {
-            SAB_CUDA(cudaEventRecord(hs->ev[n_ev], s_in), "host pass: event");
-            SAB_CUDA(cudaStreamWaitEvent(st, hs->ev[n_ev++], 0), "host pass: wait");
+            SAB_CUDA(cudaEventRecord(hs->ev[0], st), "host pass: event");              // what the caller has enqueued comes first
+            SAB_CUDA(cudaStreamWaitEvent(s_in, hs->ev[0], 0), "host pass: wait");
+            SAB_CUDA(cudaStreamWaitEvent(s_out, hs->ev[0], 0), "host pass: wait");
         }
-        const Plan* run = &pl;
-        sablock_params_t pp = *p;
+        const size_t lq = q_bytes / n_layers, lo = okv_bytes / n_layers, n_idx = (size_t)n_seqs * n_out;
+        int launches = 0, n_ev = 1;
+        SAB_CUDA(cudaMemcpyAsync(dev_token_ids, h_token_ids, total * sizeof(int), cudaMemcpyHostToDevice, s_in), "host pass: copy in");
+        for (int l0 = 0; l0 < n_layers; l0 += per) {
+            const int nl = l0 + per <= n_layers ? per : n_layers - l0;
+            auto in = [&](const void* d, const void* h, size_t layer) {
+                return cudaMemcpyAsync((char*)const_cast<void*>(d) + l0 * layer, (const char*)h + l0 * layer, nl * layer,
+                                       cudaMemcpyHostToDevice, s_in);
+            };
+            auto out = [&](void* h, const void* d, size_t layer) {
+                return cudaMemcpyAsync((char*)h + l0 * layer, (const char*)d + l0 * layer, nl * layer, cudaMemcpyDeviceToHost, s_out);
+            };
+            SAB_CUDA(in(dev_q_win, h_q_win, lq), "host pass: copy in");
+            SAB_CUDA(in(dev_k, h_k, layer_kv), "host pass: copy in");
+            if (stage_v) SAB_CUDA(in(dev_v, h_v, layer_kv), "host pass: copy in");
+            if (per < n_layers) {
+                SAB_CUDA(cudaEventRecord(hs->ev[n_ev], s_in), "host pass: event");
+                SAB_CUDA(cudaStreamWaitEvent(st, hs->ev[n_ev++], 0), "host pass: wait");
+            }
+            const Plan* run = &pl;
+            sablock_params_t pp = *p;
+            if (per < n_layers) {
+                if (!plan_inside(pl, p, nl, n_seqs, cu_seqlens, max_L, n_out, &part)) return SABLOCK_ERR_INVALID_ARG;   // (checked above)
+                const size_t tok0 = (size_t)l0 * total * sizeof(float);
+                part.o_s += tok0; part.o_e += tok0; part.o_sr += tok0;
+                if (p->pool_kernel > 1) part.o_s_raw += tok0;
+                part.clear_from = l0 > 0 ? pl.o_arrive : 0;                    // the status words of the earlier chunks stay
+                if (p->row_lse) pp.row_lse = p->row_lse + (size_t)l0 * n_seqs * p->n_q_heads * p->window;
+                run = &part;
+            }
+            t_launches = 0;
+            SAB_TRY(run_pass(*run, &pp, cands, (const char*)dev_q_win + l0 * lq, (const char*)dev_k + l0 * layer_kv, v_src + l0 * layer_kv,
+                             dev_token_ids, (char*)dev_out_k + l0 * lo, (char*)dev_out_v + l0 * lo, dev_out_idx + l0 * n_idx,
+                             dev_out_n_keep + (size_t)l0 * n_seqs, ws, st));
+            launches += t_launches;
+            if (per < n_layers) {
+                SAB_CUDA(cudaEventRecord(hs->ev[n_ev], st), "host pass: event");
+                SAB_CUDA(cudaStreamWaitEvent(s_out, hs->ev[n_ev++], 0), "host pass: wait");
+            }
+            SAB_CUDA(out(h_out_k, dev_out_k, lo), "host pass: copy out");
+            SAB_CUDA(out(h_out_v, dev_out_v, lo), "host pass: copy out");
+            SAB_CUDA(out(h_out_idx, dev_out_idx, n_idx * sizeof(int)), "host pass: copy out");
+            SAB_CUDA(out(h_out_n_keep, dev_out_n_keep, n_seqs * sizeof(int)), "host pass: copy out");
+        }
+        t_launches = launches;
         if (per < n_layers) {
-            if (!plan_inside(pl, p, nl, n_seqs, cu_seqlens, max_L, n_out, &part)) return SABLOCK_ERR_INVALID_ARG;   // (checked above)
-            const size_t tok0 = (size_t)l0 * total * sizeof(float);
-            part.o_s += tok0; part.o_e += tok0; part.o_sr += tok0;
-            if (p->pool_kernel > 1) part.o_s_raw += tok0;
-            part.clear_from = l0 > 0 ? pl.o_arrive : 0;                    // the status words of the earlier chunks stay
-            if (p->row_lse) pp.row_lse = p->row_lse + (size_t)l0 * n_seqs * p->n_q_heads * p->window;
-            run = &part;
+            SAB_CUDA(cudaEventRecord(hs->ev[0], s_out), "host pass: event");
+            SAB_CUDA(cudaStreamWaitEvent(st, hs->ev[0], 0), "host pass: wait");
         }
-        t_launches = 0;
-        SAB_TRY(run_pass(*run, &pp, cands, (const char*)dev_q_win + l0 * lq, (const char*)dev_k + l0 * layer_kv, v_src + l0 * layer_kv,
-                         dev_token_ids, (char*)dev_out_k + l0 * lo, (char*)dev_out_v + l0 * lo, dev_out_idx + l0 * n_idx,
-                         dev_out_n_keep + (size_t)l0 * n_seqs, ws, st));
-        launches += t_launches;
-        if (per < n_layers) {
-            SAB_CUDA(cudaEventRecord(hs->ev[n_ev], st), "host pass: event");
-            SAB_CUDA(cudaStreamWaitEvent(s_out, hs->ev[n_ev++], 0), "host pass: wait");
-        }
-        SAB_CUDA(out(h_out_k, dev_out_k, lo), "host pass: copy out");
-        SAB_CUDA(out(h_out_v, dev_out_v, lo), "host pass: copy out");
-        SAB_CUDA(out(h_out_idx, dev_out_idx, n_idx * sizeof(int)), "host pass: copy out");
-        SAB_CUDA(out(h_out_n_keep, dev_out_n_keep, n_seqs * sizeof(int)), "host pass: copy out");
-    }
-    t_launches = launches;
-    if (per < n_layers) {
-        SAB_CUDA(cudaEventRecord(hs->ev[0], s_out), "host pass: event");
-        SAB_CUDA(cudaStreamWaitEvent(st, hs->ev[0], 0), "host pass: wait");
+        return SABLOCK_OK;
+    }();
+    if (rc != SABLOCK_OK) {
+        // what was enqueued before the error still reads and writes the caller's buffers, some of it on streams that the
+        // caller cannot wait for
+        if (per < n_layers) { cudaStreamSynchronize(s_in); cudaStreamSynchronize(s_out); }
+        cudaStreamSynchronize(st);
+        cudaGetLastError();
+        return rc;
     }
     SAB_CUDA(cudaStreamSynchronize(st), "host pass");
     return SABLOCK_OK;

@@ -54,6 +54,32 @@ def test_host_pass_in_chunks(n_layers, lens, kw):
     _case(n_layers, lens, **kw)
 
 
+@pytest.mark.parametrize("n_layers", [1, 8])
+def test_host_pass_that_is_refused_leaves_nothing_in_flight(n_layers):
+    """An output address that the gather cannot take shows after the copies and the other stages are enqueued."""
+    L, budget = 16384, 128
+    cfg = synth.Config("t", n_layers, 32, 8, 128, 32, (L,), (budget,), (1, 2, 4, 8), "bf16", 128256, 16, 2.0, 25, (0.4,), 11)
+    b = synth.make_batch(cfg, device="cuda")
+    p = B.make_params(32, 8, 128, 32, torch.bfloat16, b.bitmap, cfg.vocab)
+    ws = B.alloc_workspace(p, L, L, 1, n_layers)
+    host = [t.cpu().pin_memory() for t in (b.q_win, b.k, b.v, b.token_ids)]
+    dev = [torch.zeros_like(t) for t in (b.q_win, b.k, b.v, b.token_ids)]
+    h_out = B.LayersOut(p, n_layers, 1, budget, torch.bfloat16, pinned_host=True)
+    d_out = B.LayersOut(p, n_layers, 1, budget, torch.bfloat16)
+    good = d_out.out_k
+    d_out.out_k = torch.empty(good.numel() + 1, dtype=good.dtype, device="cuda")[1:]
+    torch.cuda.synchronize()
+    with pytest.raises(B.SablockError) as err:
+        B.compress_layers_host(p, *host, b.cu_seqlens, budget, cfg.candidates, h_out, *dev, d_out, ws)
+    assert err.value.code == 2 and torch.cuda.current_stream().query()
+    d_out.out_k = good                                           # and the next call is as good as any
+    B.compress_layers_host(p, *host, b.cu_seqlens, budget, cfg.candidates, h_out, *dev, d_out, ws)
+    assert B.read_status(ws) == 0
+    at = h_out.out_idx[:, 0].long()
+    for l in range(n_layers):
+        assert torch.equal(h_out.out_k[l, 0], host[1][l, at[l]]) and torch.equal(h_out.out_v[l, 0], host[2][l, at[l]])
+
+
 def test_host_pass_from_several_threads():
     err = []
 
