@@ -279,7 +279,11 @@ sablock_status_t sablock_decode_attention(const sablock_params_t *p, int n_prob,
  * sablock_profile_read(slot, ...) waits for that slot's last event and stores the
  * milliseconds of each stage interval; it returns the number of intervals (0 if the slot
  * was never used).  sablock_profile_stage_name(i) names interval i.  The stages are:
- * segment, score_pass1, score_merge, score_pass2, refine, topb, search, index, compact. */
+ * segment, score_pass1, score_merge, score_pass2, refine, topb, search, index, compact.  Where one kernel is several
+ * stages the first of them has its time and the others are zero: score_pass1 for the tensor kernels in one launch,
+ * score_pass2 for the single sweep of the others, search for everything from the refinement to the index list.
+ * sablock_compress_layers_host takes all layers at once while timing is enabled (one slot, like the device call; its
+ * copies then do not overlap with its kernels). */
 #define SABLOCK_PROFILE_MAX_SLOTS 512
 sablock_status_t sablock_profile_enable(int slots);   /* 0 disables; resets the slot counter */
 int sablock_profile_read(int slot, float *ms_out, int max_n);

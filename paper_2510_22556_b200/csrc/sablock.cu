@@ -1325,7 +1325,9 @@ sablock_status_t sablock_compress_layers_host(const sablock_params_t* p, int n_l
             cudaGetLastError();
     }
     const bool stage_v = v_src == dev_v;
-    int per = host_chunk(pl, p, n_layers, n_seqs, cu_seqlens, max_L, n_out);
+    // (A call has one set of profile events: while they are recorded, all layers go through at once.)
+    const bool profiled = t_prof && t_prof->slots > 0;
+    int per = profiled ? n_layers : host_chunk(pl, p, n_layers, n_seqs, cu_seqlens, max_L, n_out);
     HostStreams* hs = per < n_layers ? host_streams() : nullptr;
     if (!hs) per = n_layers;
     Plan part;

@@ -80,6 +80,28 @@ def test_host_pass_that_is_refused_leaves_nothing_in_flight(n_layers):
         assert torch.equal(h_out.out_k[l, 0], host[1][l, at[l]]) and torch.equal(h_out.out_v[l, 0], host[2][l, at[l]])
 
 
+def test_host_pass_takes_one_profile_slot():
+    """Stage times of a call that would go through in chunks: one slot per call, and no stage of it missing."""
+    L, n_layers, budget = 8192, 4, 128
+    cfg = synth.Config("t", n_layers, 32, 8, 128, 32, (L,), (budget,), (1, 2, 4, 8), "bf16", 128256, 16, 2.0, 25, (0.4,), 11)
+    b = synth.make_batch(cfg, device="cuda")
+    p = B.make_params(32, 8, 128, 32, torch.bfloat16, b.bitmap, cfg.vocab)
+    ws = B.alloc_workspace(p, L, L, 1, n_layers)
+    host = [t.cpu().pin_memory() for t in (b.q_win, b.k, b.v, b.token_ids)]
+    dev = [torch.zeros_like(t) for t in (b.q_win, b.k, b.v, b.token_ids)]
+    h_out = B.LayersOut(p, n_layers, 1, budget, torch.bfloat16, pinned_host=True)
+    d_out = B.LayersOut(p, n_layers, 1, budget, torch.bfloat16)
+    B.profile_enable(3)
+    try:
+        for _ in range(2):
+            B.compress_layers_host(p, *host, b.cu_seqlens, budget, cfg.candidates, h_out, *dev, d_out, ws)
+        used = [B.profile_read(i) for i in range(3)]
+    finally:
+        B.profile_enable(0)
+    assert used[0] and used[1] and not used[2]
+    assert all(u[stage] > 0 for u in used[:2] for stage in ("segment", "score_pass1", "search", "compact"))
+
+
 def test_host_pass_from_several_threads():
     err = []
 
