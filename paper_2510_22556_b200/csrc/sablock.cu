@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include <atomic>
+#include <mutex>
 
 #include "common.cuh"
 #include "stages.cuh"
@@ -324,22 +325,33 @@ sablock_status_t launch(void (*kern)(KArgs...), dim3 grid, int threads, size_t s
     return note_cuda_error(err, "kernel launch");
 }
 
-// Raises a kernel's limit of dynamic shared memory, once per device for as long as it suffices.
+// A limit that is only ever raised: set(bytes) runs once for as long as it suffices, and one thread at a time, so that a call
+// that needs less never sets it below what another was told it may use.
+struct RaisedLimit {
+    std::mutex mu;
+    std::atomic<int> allowed{0};
+    template <typename Set> cudaError_t raise(int bytes, Set&& set)
+    {
+        if (bytes <= allowed.load(std::memory_order_acquire)) return cudaSuccess;
+        std::lock_guard<std::mutex> lock(mu);
+        if (bytes <= allowed.load(std::memory_order_relaxed)) return cudaSuccess;
+        const cudaError_t err = set(bytes);
+        if (err == cudaSuccess) allowed.store(bytes, std::memory_order_release);
+        return err;
+    }
+};
+
+// Raises a kernel's limit of dynamic shared memory on the current device.
 template <auto Kern>
 sablock_status_t allow_smem(int bytes)
 {
-    static std::atomic<int> allowed[64];
+    static RaisedLimit limit[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return note_cuda_error(cudaGetLastError(), "current device");
-    if (bytes <= allowed[dev].load(std::memory_order_acquire)) return SABLOCK_OK;
-    const cudaError_t err = cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (err != cudaSuccess) {
-        cudaGetLastError();
-        return note_cuda_error(err, "shared memory of a kernel");
-    }
-    int seen = allowed[dev].load();
-    while (seen < bytes && !allowed[dev].compare_exchange_weak(seen, bytes)) { }
-    return SABLOCK_OK;
+    const cudaError_t err = limit[dev].raise(bytes, [](int n) { return cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, n); });
+    if (err == cudaSuccess) return SABLOCK_OK;
+    cudaGetLastError();
+    return note_cuda_error(err, "shared memory of a kernel");
 }
 #define SAB_TRY(...) do { sablock_status_t _s = (__VA_ARGS__); if (_s != SABLOCK_OK) return _s; } while (0)
 
@@ -1073,6 +1085,13 @@ sablock_status_t sablock_read_status_detail(const void* ws, sablock_stream_t str
 int sablock_test_set_hooks(int hooks)
 {
     return (int)cudaMemcpyToSymbol(sab::g_test_hooks, &hooks, sizeof(int));
+}
+
+// A limit of dynamic shared memory with `set` in the runtime's place (host only).
+int sablock_test_raise_limit(int bytes, int (*set)(int))
+{
+    static RaisedLimit limit;
+    return (int)limit.raise(bytes, [set](int n) { return (cudaError_t)set(n); });
 }
 
 // Layers at a time of a host-buffer pass (host only).

@@ -1,6 +1,8 @@
 """Rules that kernels and launches follow, on the CPU: the test build of the library exports the functions
 that the device code uses."""
 import ctypes as C
+import threading
+import time
 
 import pytest
 import torch
@@ -100,3 +102,29 @@ def test_chunks_of_a_host_pass_run_like_the_whole(rules, impl, n_layers, lens, H
         assert min(per, n_layers - at) * len(lens) * H * W >= 128
     if (H, W) == (32, 32):                                       # the rule itself, where nothing stands against it
         assert per == max((n_layers + 7) // 8, -(-(4 << 20) // (cu[len(lens)] * Hkv * 256)))
+
+
+def test_a_limit_is_never_lowered_by_another_thread(rules):
+    """Two threads raise one kernel's limit of shared memory at the same time, the one that needs less being slower: what each
+    was granted holds from then on."""
+    now, set_to = [0], []
+
+    @C.CFUNCTYPE(C.c_int, C.c_int)
+    def setter(n):
+        if n == 50:
+            time.sleep(0.2)
+        now[0] = n
+        set_to.append(n)
+        return 0
+
+    threads = [threading.Thread(target=rules.sablock_test_raise_limit, args=(n, setter)) for n in (50, 100)]
+    for t in threads:
+        t.start()
+        time.sleep(0.05)
+    for t in threads:
+        t.join()
+    assert now[0] == 100, set_to
+    assert rules.sablock_test_raise_limit(70, setter) == 0 and now[0] == 100
+    failing = C.CFUNCTYPE(C.c_int, C.c_int)(lambda n: 1)
+    assert rules.sablock_test_raise_limit(200, failing) == 1     # a refusal is passed on and not remembered
+    assert rules.sablock_test_raise_limit(200, setter) == 0 and now[0] == 200
