@@ -1,6 +1,7 @@
 /* Calls of the C ABI from Python without ctypes' per-argument objects: bind(address) returns a builtin
  * that takes integers (device or host addresses, sizes, handles), None (a null pointer) and tuples
- * or lists of integers (passed as int arrays that live for the call), and returns the status code.
+ * or lists of numbers (passed as int arrays that live for the call), and returns the status code.  What counts as an
+ * integer is what the ctypes declarations take.
  * Marshalling only, like the ctypes declarations in binding.py, which are used where this module has not
  * been built; a decode call's share of host time goes from 1.0 to 0.3 us.
  *
@@ -16,33 +17,57 @@ enum { kMaxArgs = 26, kMaxInts = 256 };
 typedef uint64_t u;
 typedef int (*entry)(u, u, u, u, u, u, u, u, u, u, u, u, u, u, u, u, u, u, u, u, u, u, u, u, u, u);
 
+/* What ctypes makes of an int argument: anything with an index (numpy and torch integers too), its low bits. */
+static int take_scalar(PyObject* x, u* out)
+{
+    if (PyLong_Check(x)) {
+        *out = PyLong_AsUnsignedLongLongMask(x);
+    } else {
+        PyObject* v = PyNumber_Index(x);
+        if (!v) return -1;
+        *out = PyLong_AsUnsignedLongLongMask(v);
+        Py_DECREF(v);
+    }
+    return PyErr_Occurred() ? -1 : 0;
+}
+
+/* What c_int makes of int(x). */
+static int take_element(PyObject* x, int* out)
+{
+    PyObject* v = PyLong_Check(x) ? Py_NewRef(x) : PyNumber_Long(x);
+    if (!v) return -1;
+    *out = (int)(unsigned)PyLong_AsUnsignedLongMask(v);
+    Py_DECREF(v);
+    return PyErr_Occurred() ? -1 : 0;
+}
+
 static PyObject* invoke(PyObject* self, PyObject* const* args, Py_ssize_t n)
 {
     u a[kMaxArgs] = {0};
-    int ints[kMaxInts];
+    int stack[kMaxInts], *ints = stack;
+    PyObject* seq[kMaxArgs] = {0};                     /* sequence arguments as tuples of this call's own */
+    PyObject* result = NULL;
     Py_ssize_t used = 0;
     if (n > kMaxArgs) return PyErr_Format(PyExc_TypeError, "%zd arguments, at most %d", n, kMaxArgs);
-    for (Py_ssize_t i = 0; i < n; ++i) {
-        PyObject* x = args[i];
-        if (PyLong_Check(x)) {
-            a[i] = PyLong_AsUnsignedLongLongMask(x);
-        } else if (x == Py_None) {
-            a[i] = 0;
-        } else if (PyTuple_Check(x) || PyList_Check(x)) {
-            const Py_ssize_t m = PySequence_Fast_GET_SIZE(x);
-            PyObject** it = PySequence_Fast_ITEMS(x);
-            if (used + m > kMaxInts) return PyErr_Format(PyExc_ValueError, "too many values in sequence arguments");
-            a[i] = (u)(uintptr_t)(ints + used);
-            for (Py_ssize_t k = 0; k < m; ++k) {
-                const long v = PyLong_AsLong(it[k]);
-                if (v == -1 && PyErr_Occurred()) return NULL;
-                if (v > INT32_MAX || v < INT32_MIN) return PyErr_Format(PyExc_OverflowError, "%ld does not fit an int", v);
-                ints[used++] = (int)v;
-            }
-        } else {
-            return PyErr_Format(PyExc_TypeError, "argument %zd: an integer, None or a sequence of integers", i);
+    for (Py_ssize_t i = 0; i < n; ++i)
+        if (PyTuple_Check(args[i]) || PyList_Check(args[i])) {
+            seq[i] = PySequence_Tuple(args[i]);
+            if (!seq[i]) goto done;
+            used += PyTuple_GET_SIZE(seq[i]);
         }
-        if (PyErr_Occurred()) return NULL;
+    if (used > kMaxInts && !(ints = PyMem_Malloc(used * sizeof(int)))) {
+        PyErr_NoMemory();
+        goto done;
+    }
+    used = 0;
+    for (Py_ssize_t i = 0; i < n; ++i) {
+        if (seq[i]) {
+            a[i] = (u)(uintptr_t)(ints + used);
+            for (Py_ssize_t k = 0; k < PyTuple_GET_SIZE(seq[i]); ++k)
+                if (take_element(PyTuple_GET_ITEM(seq[i], k), ints + used++) < 0) goto done;
+        } else if (args[i] != Py_None && take_scalar(args[i], &a[i]) < 0) {
+            goto done;
+        }
     }
     const entry f = (entry)(uintptr_t)PyLong_AsUnsignedLongLong(self);
     int rc;
@@ -50,7 +75,11 @@ static PyObject* invoke(PyObject* self, PyObject* const* args, Py_ssize_t n)
     rc = f(a[0], a[1], a[2], a[3], a[4], a[5], a[6], a[7], a[8], a[9], a[10], a[11], a[12], a[13], a[14], a[15], a[16], a[17],
            a[18], a[19], a[20], a[21], a[22], a[23], a[24], a[25]);
     Py_END_ALLOW_THREADS
-    return PyLong_FromLong(rc);
+    result = PyLong_FromLong(rc);
+done:
+    for (Py_ssize_t i = 0; i < n; ++i) Py_XDECREF(seq[i]);
+    if (ints != stack) PyMem_Free(ints);
+    return result;
 }
 
 static PyMethodDef invoke_def = {"entry", (PyCFunction)(void (*)(void))invoke, METH_FASTCALL, "calls one entry point of the C ABI"};
