@@ -210,13 +210,14 @@ __device__ __forceinline__ void warp_count_digit(int* hist, int bin)
 // A warp owns consecutive segments and takes them in batches of at most kSelBatch tokens: the batch's
 // scores and entropies arrive by coalesced loads, all in flight at once, and the per-segment sums are then
 // made from shared memory by groups of eight lanes (a warp per segment reading global memory directly
-// spends its time on the latency of two or three dependent loads per segment).  Lanes stride over
-// a segment's tokens and combine with a butterfly: the summation order is fixed.
+// spends its time on the latency of two or three dependent loads per segment).  The summation order is the
+// one of refine_kernel, whatever the batch: token t of a segment belongs to accumulator t % 32, and the 32 are
+// combined with a butterfly, so that a call's refined scores are those of sablock_score bit for bit.  A lane of a
+// group of eight has four of the accumulators, 8 apart, and does the first two steps of the butterfly by itself.
 __device__ __forceinline__ float sel_factor(const SelectArgs& a, float si, float sd, int n)
 {
-    const float inv = 1.f / (float)n;
-    const float I = si * inv;                      // Eq. 5
-    const float Dk = sd * inv;                     // Eq. 6
+    const float I = si / (float)n;                 // Eq. 5
+    const float Dk = sd / (float)n;                // Eq. 6
     const float om = I * (1.f + a.eta * Dk);       // Eq. 7
     return 1.f + a.alpha * om;                     // Eq. 8
 }
@@ -268,8 +269,12 @@ __device__ __forceinline__ void sel_refine(const SelectArgs& a, const float* __r
         // eight lanes per segment, four segments at a time
         for (int i = lane >> 3; i < ((m + 3) & ~3); i += 4) {
             const int b0 = __shfl_sync(0xffffffffu, bound, min(i, m)) - p0, b1 = __shfl_sync(0xffffffffu, bound, min(i + 1, m)) - p0;
-            float si = 0.f, sd = 0.f;
-            for (int t = b0 + (lane & 7); t < b1; t += 8) { si += sb[t]; sd += eb[t]; }
+            float as[4] = {0.f, 0.f, 0.f, 0.f}, ad[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int t = b0 + (lane & 7); t < b1; t += 32)
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+                    if (t + 8 * x < b1) { as[x] += sb[t + 8 * x]; ad[x] += eb[t + 8 * x]; }
+            float si = (as[0] + as[2]) + (as[1] + as[3]), sd = (ad[0] + ad[2]) + (ad[1] + ad[3]);
 #pragma unroll
             for (int o = 4; o > 0; o >>= 1) {
                 si += __shfl_xor_sync(0xffffffffu, si, o);
