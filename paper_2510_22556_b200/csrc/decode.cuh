@@ -435,9 +435,12 @@ decode_mma_kernel(DecodeArgs a)
 #pragma unroll
     for (int i = 0; i < D / 8; ++i) {
         const float t0 = __shfl_down_sync(0xffffffffu, acc[i][0], 16), t1 = __shfl_down_sync(0xffffffffu, acc[i][1], 16);
+        // an infinite value times a smaller piece is an infinity of either sign or, where the piece is zero, no number: the
+        // leading piece alone says what the weight times the value is
         if (lane < 16 && hh < G)
             *reinterpret_cast<float2*>(&accs[warp][hh][i * 8 + 2 * (lane & 3)]) =
-                make_float2(acc[i][0] + (acc[i][2] + t0), acc[i][1] + (acc[i][3] + t1));
+                make_float2(isinf(acc[i][0]) ? acc[i][0] : acc[i][0] + (acc[i][2] + t0),
+                            isinf(acc[i][1]) ? acc[i][1] : acc[i][1] + (acc[i][3] + t1));
     }
     if (lane < 16 && (lane & 3) == 0 && hh < G) { ms[warp][hh] = m; ls[warp][hh] = l; }
     __syncthreads();

@@ -68,3 +68,23 @@ def test_decode_strided_cache_and_odd_query_address():
     out = B.decode_attention(p, q, k, v)
     ref, _ = _reference(q, k, v, [n, n])
     assert float((out.double() - ref).abs().max()) <= 2e-5 * float(v.double().abs().max())
+
+
+@pytest.mark.parametrize("H,Hkv,D", [(8, 2, 128), (4, 4, 64), (4, 2, 256)])
+@pytest.mark.parametrize("n_rows", [64, 1024, 20000])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_decode_infinite_values(H, Hkv, D, n_rows, dtype):
+    """An infinity in a row of V is one in its column of the output, of its sign, and nowhere else."""
+    if dtype == torch.float32:
+        D = min(D, 128)
+    g = torch.Generator(device="cuda").manual_seed(n_rows + D)
+    q = torch.randn(1, H, D, generator=g, device="cuda").to(dtype)
+    k, v = (torch.randn(1, n_rows, Hkv, D, generator=g, device="cuda").to(dtype) for _ in range(2))
+    v[0, 5, :, 3], v[0, 40, :, 10], v[0, n_rows // 2, :, 33] = float("inf"), float("-inf"), float("inf")
+    p = B.make_params(H, Hkv, D, 8, dtype)
+    ref, _ = _reference(q, k, v, [n_rows])
+    out = B.decode_attention(p, q, k, v).double()
+    assert torch.equal(torch.isinf(ref), torch.isinf(out)) and bool((out[torch.isinf(ref)] == ref[torch.isinf(ref)]).all())
+    fin = ~torch.isinf(ref)
+    assert int(fin.sum()) == H * (D - 3)
+    assert float((out - ref)[fin].abs().max()) <= 2e-5 * float(v.double()[torch.isfinite(v)].abs().max())
