@@ -315,7 +315,7 @@ __device__ __forceinline__ bool sel_candidate(const float* x, int a, int n, int 
     }
     double base = 0.0;                             // Score_base: the segment's tokens of the Top-B set
     for (int i = lane; i < n; i += 32)
-        if (in_topb(x[i], a + i, thr, cut)) base += (double)x[i];
+        if (counts_in_topb(x[i], a + i, thr, cut)) base += (double)x[i];
     __syncwarp();
     // rank by (Phi desc, index asc).  Rounding to fp32 keeps the order, so the ranks follow from fp32
     // comparisons unless two blocks round to the same value: only then are the doubles compared.
@@ -621,12 +621,16 @@ __device__ bool sel_body(const Geo& g, const Cands& cands, const SelectArgs& a, 
     // segments with large budgets, needles, was the longest chain of the stage.)  The largest candidate
     // that passed is the segment's block size.
     auto kept = [&](int w) -> unsigned { return kSm ? keep[w] : __ldcg(keep + w); };       // (global bits are changed by atomics in L2)
+    bool nan = false;
     for (int i0 = 0; i0 < len; i0 += kSelThreads) {
         const int i = i0 + tid;
-        const unsigned w = __ballot_sync(0xffffffffu, i < len && in_topb(val(min(i, len - 1)), ta + i, thr, cut));
+        const float v = val(min(i, len - 1));
+        const bool in = i < len && in_topb(v, ta + i, thr, cut);
+        nan |= in && is_nan_key(order_key(v));
+        const unsigned w = __ballot_sync(0xffffffffu, in);
         if (lane == 0 && i < len) keep[i >> 5] = w;
     }
-    __syncthreads();
+    const bool any_nan = __syncthreads_or(nan) != 0;
     double* phi = reinterpret_cast<double*>(scratch);
     unsigned char* rk = scratch + (kSegShort / 2) * 12;
     int* seg_g = a.seg_g ? a.seg_g + (size_t)p * a.seg_stride : nullptr;
@@ -698,6 +702,13 @@ __device__ bool sel_body(const Geo& g, const Cands& cands, const SelectArgs& a, 
                 if (w == w1) m &= 0xffffffffu >> (31 - ((pos + n - 1) & 31));
                 b += __popc(m);
             }
+            if (any_nan && b > 0) {                // a segment whose share of the Top-B set is NaN alone retains nothing
+                int n_nan = 0;
+                for (int i = pos; i < pos + n; ++i) n_nan += ((kept(i >> 5) >> (i & 31)) & 1u) && is_nan_key(order_key(val(i)));
+                b -= n_nan;
+                if (b == 0)
+                    for (int i = pos; i < pos + n; ++i) sel_set_bit(keep, i, false);
+            }
             if (seg_b) seg_b[kk] = b;
             if (seg_g) seg_g[kk] = b > 0 ? 1 : 0;
             const bool any = n_cand > 0 && cands.g[1] <= min(n, b);
@@ -726,7 +737,7 @@ __device__ bool sel_body(const Geo& g, const Cands& cands, const SelectArgs& a, 
         double base = 0.0;
         for (int i = tid; i < n; i += kSelThreads) {
             const float v = val(sa - ta + i);
-            if (in_topb(v, sa + i, thr, cut)) { ++bl; base += (double)v; }
+            if (counts_in_topb(v, sa + i, thr, cut)) { ++bl; base += (double)v; }
         }
         const int b = sel_block_sum(bl, sm);
         base = sel_block_sum(base, sm);
@@ -772,8 +783,8 @@ __device__ bool sel_body(const Geo& g, const Cands& cands, const SelectArgs& a, 
     }
     if (rank == C - 1) {
         for (int i = tid; i < g.window; i += kSelThreads) oi[g.B + i] = T + i;
-        // |T*| = B (Eq. 13) whenever the scores are finite.  If the search retained fewer (scores that do
-        // not order, e.g. NaN), the rest of the list still gets valid positions, so that the gather that
+        // |T*| = B (Eq. 13) whenever the scores are numbers.  If the search retained fewer (segments whose share of
+        // the Top-B is NaN), the rest of the list still gets valid positions, so that the gather that
         // follows stays inside the cache, and the status word reports it.
         for (int i = all + tid; i < g.B; i += kSelThreads) oi[i] = 0;
         if (tid == 0) {

@@ -284,10 +284,12 @@ refine_kernel(const Geo g, const float* __restrict__ s_raw, int pool_k, int pool
 }
 
 // ---- shared by the selection kernel (select.cuh) --------------------------------------------------
-// Order-preserving integer image of an fp32 score.
+// Order-preserving integer image of an fp32 score.  The bits are taken by an instruction of their own: where a score is also
+// used as a number the compiler may otherwise compare numbers, which NaN does not take part in, and where it is not, bits.
 __device__ __forceinline__ unsigned order_key(float f)
 {
-    unsigned u = __float_as_uint(f);
+    unsigned u;
+    asm("mov.b32 %0, %1;" : "=r"(u) : "f"(f));
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
@@ -295,6 +297,13 @@ __device__ __forceinline__ bool in_topb(float v, int t, unsigned thr, int cut)
 {
     unsigned u = order_key(v);
     return u > thr || (u == thr && t <= cut);
+}
+// The keys of numbers run from that of minus infinity to that of infinity.  A NaN of the Top-B set does not count towards a
+// segment's budget and baseline.
+__device__ __forceinline__ bool is_nan_key(unsigned u) { return u - 0x007fffffu > 0xff800000u - 0x007fffffu; }
+__device__ __forceinline__ bool counts_in_topb(float v, int t, unsigned thr, int cut)
+{
+    return in_topb(v, t, thr, cut) && !is_nan_key(order_key(v));
 }
 
 // Greedy fill of Alg. 2 for block size g, evaluated in closed form from the block ranks:

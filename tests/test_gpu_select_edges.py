@@ -108,3 +108,36 @@ def test_select_sequences_shorter_than_a_cluster(B_tok, order):
             _, st = oracle.segment(b.token_ids[cu[i]:cu[i + 1]], W, b.bitmap, cfg.vocab)
             r = oracle.select(sr[l, cu[i]:cu[i] + T].astype(np.float64), st, B_tok, cfg.candidates, tau=float(np.float32(0.85)))
             assert idx[:B_tok].tolist() == r["keep"].tolist() and idx[B_tok:].tolist() == list(range(T, L))
+
+
+@pytest.mark.parametrize("T,seg", [(640, 4), (20000, 4), (6000, 300), (300000, 25)])
+def test_select_reports_scores_that_do_not_order(T, seg):
+    """NaN ranks above every number but is no budget: segments whose share of the Top-B is NaN retain nothing, the
+    status says so, and the list holds valid positions; beside other numbers a NaN only does not count."""
+    W, B_tok = 32, T // 8 // seg * seg
+    rng = np.random.default_rng(T)
+    sr = rng.random(T).astype(np.float32)
+    st = np.arange(0, T + 1, seg).astype(np.int32)
+    seg_start = torch.zeros(T + 1, dtype=torch.int32, device="cuda")
+    seg_start[: len(st)] = torch.from_numpy(st).cuda()
+    n_seg = torch.tensor([len(st) - 1], dtype=torch.int32, device="cuda")
+    p = B.make_params(4, 1, 64, W, torch.bfloat16)
+    ws = B.alloc_workspace(p, T + W, T + W)
+
+    def run(x):
+        idx, g, b = B.select(p, torch.from_numpy(x).cuda(), T + W, seg_start, n_seg, B_tok + W, [1, 2, 4], ws, want_segments=True)
+        torch.cuda.synchronize()
+        return idx.cpu().numpy(), g.cpu().numpy()[: len(st) - 1], b.cpu().numpy()[: len(st) - 1], B.read_status(ws)
+
+    whole = sr.copy()
+    whole[seg: 2 * seg] = np.nan                                 # the second segment
+    idx, g, b, status = run(whole)
+    assert status == 6 and b[1] == 0 and g[1] == 0 and b.sum() == B_tok - seg
+    assert ((idx >= 0) & (idx < T + W)).all() and not ((idx >= seg) & (idx < 2 * seg)).any()
+    one = sr.copy()
+    one[:seg] = 2.0                                              # a segment that is retained whole ...
+    one[1] = np.nan                                              # ... with one NaN in it
+    idx, g, b, status = run(one)
+    assert status == 0 and b[0] == seg - 1 and b.sum() == B_tok - 1 and idx[:seg].tolist() == list(range(seg))
+    idx, g, b, status = run(np.full(T, np.nan, np.float32))
+    assert status == 6 and b.sum() == 0 and ((idx >= 0) & (idx < T + W)).all()
