@@ -264,7 +264,8 @@ __device__ __forceinline__ bool fl_last(int* ctr, int n, bool withheld)
     return true;
 }
 
-// Merges n partials [n][R], in order: into one, or into minus the rows' log-sum-exps.  A lane has R / 32 rows.
+// Merges n partials [n][R], in order: into one, or into minus the rows' log-sum-exps.  A lane has R / 32 rows.  A sum of zero has
+// seen no key; one that is no number (a key that is none) makes the row's log-sum-exp none.
 template <bool kFinal>
 __device__ __forceinline__ void fl_merge(const float2* part, int n, int R, float2* out, float* neg_lse)
 {
@@ -286,11 +287,11 @@ __device__ __forceinline__ void fl_merge(const float2* part, int n, int R, float
             float mn = m[y];
 #pragma unroll
             for (int x = 0; x < 4; ++x)
-                if (v[x][y].y > 0.f) mn = fmaxf(mn, v[x][y].x);
+                if (v[x][y].y != 0.f) mn = fmaxf(mn, v[x][y].x);
             l[y] = m[y] == -INFINITY ? 0.f : l[y] * pow2_nonpos((int)(m[y] - mn));
 #pragma unroll
             for (int x = 0; x < 4; ++x)
-                if (v[x][y].y > 0.f) l[y] += v[x][y].y * pow2_nonpos((int)(v[x][y].x - mn));
+                if (v[x][y].y != 0.f) l[y] += v[x][y].y * pow2_nonpos((int)(v[x][y].x - mn));
             m[y] = mn;
         }
     }
@@ -547,11 +548,11 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                 float m = -INFINITY, l = 0.f;
 #pragma unroll
                 for (int x = 0; x < 4; ++x)
-                    if (sh.sums[b][x][r].y > 0.f) m = fmaxf(m, sh.sums[b][x][r].x);
+                    if (sh.sums[b][x][r].y != 0.f) m = fmaxf(m, sh.sums[b][x][r].x);
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
                     const float2 v = sh.sums[b][x][r];
-                    if (v.y > 0.f) l += v.y * pow2_nonpos((int)(v.x - m));
+                    if (v.y != 0.f) l += v.y * pow2_nonpos((int)(v.x - m));
                 }
                 __stcg(part + (size_t)index * R + r, make_float2(l > 0.f ? m : 0.f, l));
             }

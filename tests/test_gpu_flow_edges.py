@@ -105,3 +105,22 @@ def test_carry_between_head_groups(H, Hkv, D, W, lens, n_layers, lse):
     """More than 1024 window rows: the head groups hand their sums on through scratch that problems of other lengths have
     used before."""
     _run(H, Hkv, D, W, lens, n_layers, 64, lse)
+
+
+@pytest.mark.parametrize("H,Hkv,D,W", [(32, 8, 128, 32), (8, 2, 64, 8), (6, 2, 128, 16), (64, 16, 64, 32)])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("L", [700, 5000, 9000])
+def test_a_key_that_is_no_number(H, Hkv, D, W, value, L):
+    """A NaN or infinite element of one key makes the softmax of every window row of its head NaN, and with it all scores, as
+    the definition has it; the status word says so."""
+    cfg = synth.Config("t", 1, H, Hkv, D, W, (L,), (64,), (1, 2, 4), "bf16", 5000, 8, 2.0, 20, (0.4,), 9)
+    b = synth.make_batch(cfg, device="cuda")
+    b.k[0, L // 3, 0, 5] = value
+    p = B.make_params(H, Hkv, D, W, torch.bfloat16, b.bitmap, cfg.vocab)
+    ws = B.alloc_workspace(p, L, L)
+    B.compress_layers(p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, 64, cfg.candidates, ws)
+    torch.cuda.synchronize()
+    rs, _ = _reference(b.q_win[0, 0], b.k[0], W)
+    s = B.workspace_view(p, ws, "s", L, L)[0, :L - W]
+    assert bool(torch.isnan(rs).all()) and bool(torch.isnan(s).all())
+    assert B.read_status(ws) == 6
