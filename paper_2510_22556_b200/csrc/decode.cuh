@@ -384,7 +384,7 @@ decode_mma_kernel(DecodeArgs a)
 #pragma unroll
             for (int e = 0; e < 2; ++e) s[2 * x + e] = 8 * x + e < left ? c[x][e] * a.c2 : -INFINITY;
         const float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
-        if (__any_sync(0xffffffffu, mx > m + 8.f)) {
+        if (__any_sync(0xffffffffu, mx > m)) {
             float q = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
             q = fmaxf(q, __shfl_xor_sync(0xffffffffu, q, 2));
             const float mn = fmaxf(m, q);

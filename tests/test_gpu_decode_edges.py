@@ -88,3 +88,21 @@ def test_decode_infinite_values(H, Hkv, D, n_rows, dtype):
     fin = ~torch.isinf(ref)
     assert int(fin.sum()) == H * (D - 3)
     assert float((out - ref)[fin].abs().max()) <= 2e-5 * float(v.double()[torch.isfinite(v)].abs().max())
+
+
+@pytest.mark.parametrize("H,Hkv,D", [(32, 8, 128), (16, 16, 64), (16, 8, 256)])
+@pytest.mark.parametrize("n_rows,n_prob", [(128, 64), (20000, 1)])
+def test_decode_values_near_the_end_of_the_range(H, Hkv, D, n_rows, n_prob):
+    """Values of 1e38 under logits that rise along the cache: no weight above one, no sum above the largest value."""
+    g = torch.Generator(device="cuda").manual_seed(n_rows + D)
+    q = torch.randn(n_prob, H, D, generator=g, device="cuda").to(torch.bfloat16)
+    k = torch.randn(n_prob, n_rows, Hkv, D, generator=g, device="cuda").to(torch.bfloat16)
+    k[:, 64:] += q.view(n_prob, 1, Hkv, H // Hkv, D)[:, :, :, 0] * 0.3                # about 5 in log2 units above the first rows
+    v = torch.zeros(n_prob, n_rows, Hkv, D, device="cuda").to(torch.bfloat16)
+    v[:, 70] = 1e38
+    v[:, n_rows - 3] = -3e37
+    p = B.make_params(H, Hkv, D, 8, torch.bfloat16)
+    ref, _ = _reference(q, k, v, [n_rows] * n_prob)
+    out = B.decode_attention(p, q, k, v).double()
+    assert bool(torch.isfinite(out).all())
+    assert float((out - ref).abs().max()) <= 2e-5 * 4 * 1e38                        # logits up to four times those above
