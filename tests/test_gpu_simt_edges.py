@@ -76,3 +76,23 @@ def test_fp32_unaligned_rows():
     s, e, _, _ = B.score(p, q, k, seg_start, torch.ones(1, dtype=torch.int32, device="cuda"), ws)
     rs, re = _reference(q, k, W)
     assert float(((s.double() - rs).abs() / rs).max()) <= 2e-4 and float((e.double() - re).abs().max()) <= 4e-4
+
+
+@pytest.mark.parametrize("H,Hkv", [(5, 1), (6, 2), (7, 1), (8, 2)])
+@pytest.mark.parametrize("layers,L", [(1, 300), (8, 6000)])
+def test_an_infinite_key_under_given_normalisers(H, Hkv, layers, L):
+    """Heads that a thread has room for but the KV head has not add nothing, not even where a logit is infinite."""
+    D, W = 64, 12
+    cfg = synth.Config("t", layers, H, Hkv, D, W, (L,), (W + 20,), (1, 2, 4), "f32", 5000, 8, 2.0, 20, (), 3)
+    b = synth.make_batch(cfg, device="cuda")
+    lse = synth.prefill_row_lse(b.q_win, b.k, b.cu_seqlens)      # of the keys before one becomes infinite
+    t = L // 2
+    b.k[:, t, 0, 5] = float("inf")
+    b.q_win[..., 5] = b.q_win[..., 5].abs() + 0.1                # every logit of that key is plus infinity
+    p = B.make_params(H, Hkv, D, W, torch.float32, b.bitmap, cfg.vocab, row_lse=lse)
+    ws = B.alloc_workspace(p, L, L, 1, layers)
+    B.compress_layers(p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, W + 20, cfg.candidates, ws)
+    torch.cuda.synchronize()
+    s = B.workspace_view(p, ws, "s", L, L, 1, layers)[:, :L - W]
+    assert bool((s[:, t] == float("inf")).all())
+    assert int(torch.isfinite(s).sum()) == s.numel() - layers
