@@ -261,8 +261,9 @@ decode_partial_kernel(DecodeArgs a)
 //
 // A warp walks the 16-row chunks warp, warp + 4, ... of its CTA's rows on its own: cp.async into a
 // private ring of kDecMmaStages chunks (swizzled so that ldmatrix is free of bank conflicts), its own
-// online softmax, no barrier in the loop.  The running maximum only moves when a logit exceeds it by
-// 2^8, so that rescaling is rare and costs one vote otherwise.
+// online softmax, no barrier in the loop.  The running maximum moves as soon as one of the chunk's logits exceeds it, and
+// costs one vote otherwise: no weight is above one, and no sum beyond what the values allow.  (Letting weights grow to 2^8
+// before it moves was no faster: 96.8 and 96.7 us on a layer of 128K rows, the kernel waits for memory.)
 //
 // CL = true: the CTAs of a (problem, KV head) are a cluster and merge through distributed shared
 // memory; one launch, no scratch.  CL = false: partials to scratch, merged by decode_merge_kernel.
