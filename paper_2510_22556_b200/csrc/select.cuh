@@ -24,7 +24,11 @@ constexpr int kSelThreads = 1024;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelMaxCluster = 8;
 constexpr int kSelCap = 33280;                 // tokens of a CTA's range that shared memory holds
-constexpr int kSegShort = 256;                 // longest segment that one warp searches
+constexpr int kSegShort = 256;                 // longest segment that one warp searches, and tokens per warp of a team
+constexpr int kSelTeam = 4;                    // warps of a team that searches a longer one
+constexpr int kSelTeams = kSelWarps / kSelTeam;
+constexpr int kSegMid = kSelTeam * kSegShort;  // longest segment that a team searches
+constexpr int kSelMaxMid = 192;                // of which a CTA's list holds so many (all that shared memory holds the scores of)
 constexpr int kSelMaxActive = 1024;            // segments of a CTA whose candidates are searched side by side
 constexpr int kSelSegs = 4096;                 // segment starts that shared memory holds
 constexpr int kSelBatch = 320;                 // tokens of a warp's batch of segments in the refinement
@@ -58,8 +62,10 @@ struct SelShared {
     int ka, kz;                // segments of this CTA
     int k, neq, digit, mp, b;
     int n_active, next;        // segments to search, next (segment, candidate) to hand out
-    int n_long;
+    int n_long, n_mid;
+    int team_item[kSelTeams];
     int long_list[64];         // segments left to the whole CTA
+    unsigned long long key;
     int scan[kSelWarps];
     double red[kSelWarps];
     uint64_t bars[2];          // arrivals of the cluster's CTAs, one exchange each in turn
@@ -74,7 +80,7 @@ struct SelActive {
 };
 
 // Dynamic shared memory: refined scores | retained bits | active segments | segment starts | per-warp
-// scratch.  The scratch of a warp holds the entropies of its batch in the refinement, the
+// scratch | segments for the teams.  The scratch of a warp holds the entropies of its batch in the refinement, the
 // copies of the digit counters in the radix passes (over all warps' scratch), block scores and ranks
 // in the search.
 constexpr int kSelOffKeep = kSelCap * 4;
@@ -82,7 +88,8 @@ constexpr int kSelOffActive = (kSelOffKeep + (kSelCap / 32 + 1) * 4 + 15) / 16 *
 constexpr int kSelOffSegs = kSelOffActive + kSelMaxActive * (int)sizeof(SelActive);
 constexpr int kSelOffScratch = (kSelOffSegs + (kSelSegs + 1) * 2 + 15) / 16 * 16;
 constexpr int kSelScratch = (kSegShort / 2) * 13;              // bytes per warp: a double, a float and a byte per block
-constexpr int kSelSmemBytes = kSelOffScratch + kSelWarps * kSelScratch;
+constexpr int kSelOffMid = kSelOffScratch + kSelWarps * kSelScratch;
+constexpr int kSelSmemBytes = kSelOffMid + kSelMaxMid * (int)sizeof(SelActive);
 static_assert(kSelBatch * 4 <= kSelScratch && kSelScratch % 8 == 0, "entropies of a batch; alignment of the block scores");
 static_assert(kSelCopies * 512 * 4 <= kSelWarps * kSelScratch, "copies of the digit counters");
 static_assert(kSegShort / 2 < 256, "ranks are bytes");
@@ -373,11 +380,184 @@ __device__ __forceinline__ bool sel_candidate(const float* x, int a, int n, int 
     return score >= (double)tau * base;            // R_k(g) >= tau (Eqs. 11, 12)
 }
 
+// ---- the same for a segment of at most kSegShort tokens per warp, by a team of warps -------------------
+// Neighbouring warps with a barrier of their own; their scratch put together holds the blocks of a segment four times as
+// long.  Teams work side by side, on the candidates of a segment too.  (The whole CTA on one segment after the other, by the
+// search for long ones below, costs seven barriers and a radix select per candidate: 32 x 32K tokens in segments of 200 on
+// average, the whole selection, took 561 us that way and takes 154 now; a warp per segment in a kernel of its own took 288.
+// Teams of eight for segments up to 2048 tokens were slower than the whole CTA, their ranks are quadratic.)
+__device__ __forceinline__ void team_sync(int team)
+{
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kSelTeam * 32) : "memory");
+}
+
+// `bits`: bit q = token lane-of-team + 32 kSelTeam q is retained.
+__device__ __forceinline__ bool sel_candidate_team(const float* x, int a, int n, int b, int gs, unsigned thr, int cut, float tau,
+                                                   uint8_t* scratch, int team, unsigned& bits)
+{
+    constexpr int nl = kSelTeam * 32, kBlocks = kSegMid / 2, kPer = kBlocks / nl;              // blocks in all and of a lane
+    const int lt = threadIdx.x & (nl - 1), lane = threadIdx.x & 31;
+    const int nb = (n + gs - 1) / gs, rem = n - (nb - 1) * gs;
+    double* phi = reinterpret_cast<double*>(scratch);
+    float* phif = reinterpret_cast<float*>(phi + kBlocks);
+    int* rank = reinterpret_cast<int*>(phif);      // once the scores in fp32 are read
+    double* red = reinterpret_cast<double*>(phif + kBlocks);
+    int* redi = reinterpret_cast<int*>(red);
+    static_assert(kBlocks * 12 + kSelTeam * 16 <= kSelTeam * kSelScratch, "blocks and sums in the team's scratch");
+    for (int m = lt; m < nb; m += nl) {            // block scores Phi, tokens in index order
+        const int t0 = m * gs, t1 = min(t0 + gs, n);
+        double acc = 0.0;
+#pragma unroll 4
+        for (int t = t0; t < t1; ++t) acc += (double)x[t];
+        phi[m] = acc;
+        phif[m] = (float)acc;
+    }
+    double base = 0.0;                             // Score_base: the segment's tokens of the Top-B set
+    for (int i = lt; i < n; i += nl)
+        if (counts_in_topb(x[i], a + i, thr, cut)) base += (double)x[i];
+    team_sync(team);
+    // rank by (Phi desc, index asc), on fp32 unless two blocks round to the same value: the ranks then are not 0 .. nb - 1, and
+    // their sum is smaller
+    float pm[kPer];
+    int r[kPer], sum = 0;
+#pragma unroll
+    for (int y = 0; y < kPer; ++y) {
+        r[y] = 0;
+        pm[y] = lt + nl * y < nb ? phif[lt + nl * y] : INFINITY;
+    }
+#pragma unroll 4
+    for (int m2 = 0; m2 < nb; ++m2) {
+        const float q = phif[m2];
+#pragma unroll
+        for (int y = 0; y < kPer; ++y) r[y] += q > pm[y];
+    }
+#pragma unroll
+    for (int y = 0; y < kPer; ++y) sum += r[y];
+    sum = warp_sum(sum);
+    if (lane == 0) redi[lt >> 5] = sum;
+    team_sync(team);
+    sum = 0;
+#pragma unroll
+    for (int w = 0; w < kSelTeam; ++w) sum += redi[w];
+    if (sum != nb * (nb - 1) / 2) {
+#pragma unroll
+        for (int y = 0; y < kPer; ++y) {
+            const int m = lt + nl * y;
+            if (m < nb) {
+                const double p = phi[m];
+                int c = 0;
+                for (int m2 = 0; m2 < nb; ++m2) {
+                    const double q = phi[m2];
+                    c += (q > p) || (q == p && m2 < m);
+                }
+                r[y] = c;
+            }
+        }
+    }
+#pragma unroll
+    for (int y = 0; y < kPer; ++y)
+        if (lt + nl * y < nb) rank[lt + nl * y] = r[y];
+    team_sync(team);
+    int r_star, m_take;
+    greedy_cut(nb, gs, rem, rank[nb - 1], b, r_star, m_take);
+    int mp = -1;                                   // the block that is truncated
+    if (m_take > 0)
+        for (int m0 = 0; m0 < nb; m0 += 32) {
+            const unsigned hit = __ballot_sync(0xffffffffu, m0 + lane < nb && rank[min(m0 + lane, nb - 1)] == r_star);
+            if (hit) { mp = m0 + __ffs(hit) - 1; break; }
+        }
+    double score = 0.0;
+    bits = 0;
+    for (int i = lt, q = 0; i < n; i += nl, ++q) {
+        const int m = i / gs;
+        bool take = rank[m] < r_star;
+        if (m == mp) {                             // top m_take tokens of the block, (score desc, index asc)
+            const int t0 = mp * gs, t1 = min(t0 + gs, n);
+            const float vi = x[i];
+            int tr = 0;
+#pragma unroll 4
+            for (int t = t0; t < t1; ++t) tr += (x[t] > vi) || (x[t] == vi && t < i);
+            take = tr < m_take;
+        }
+        if (take) { bits |= 1u << q; score += (double)x[i]; }
+    }
+    __syncwarp();
+    base = warp_sum(base);
+    score = warp_sum(score);
+    if (lane == 0) { red[2 * (lt >> 5)] = base; red[2 * (lt >> 5) + 1] = score; }
+    team_sync(team);
+    base = score = 0.0;
+#pragma unroll
+    for (int w = 0; w < kSelTeam; ++w) { base += red[2 * w]; score += red[2 * w + 1]; }
+    team_sync(team);                               // the scratch may be used again
+    return score >= (double)tau * base;            // R_k(g) >= tau (Eqs. 11, 12)
+}
+
 // Bit range of a segment in the CTA's bitmask: bit i of `keep` := take.
 __device__ __forceinline__ void sel_set_bit(unsigned* keep, int i, bool take)
 {
     if (take) atomicOr(&keep[i >> 5], 1u << (i & 31));
     else atomicAnd(&keep[i >> 5], ~(1u << (i & 31)));
+}
+
+// The searches of the segments listed for teams: the items are handed out as those of the warps are.  `x`: the scores of
+// the CTA's range, from position ta on.  (Not inlined: most calls have no such segment, and its registers are not theirs.)
+template <bool kSm>
+__device__ __noinline__ void sel_teams(SelShared& sm, uint8_t* dyn, const Cands& cands, const float* x, int ta, int len, unsigned thr,
+                                       int cut, float tau, unsigned* keep, int* seg_g)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_cand = cands.n - 1;
+    const int team = warp / kSelTeam, wt = warp % kSelTeam;
+    const int n_mid = min(sm.n_mid, kSelMaxMid), n_items = n_mid * n_cand;
+    SelActive* list = reinterpret_cast<SelActive*>(dyn + kSelOffMid);
+    uint8_t* ts = dyn + kSelOffScratch + team * kSelTeam * kSelScratch;
+    unsigned* masks = reinterpret_cast<unsigned*>(dyn + (size_t)((len + 3) & ~3) * 4);
+    constexpr int kMask = kSegMid / 32;            // words of an item's mask
+    const bool keep_masks = kSm && n_items <= (kSelCap - ((len + 3) & ~3)) / kMask;
+    __syncthreads();                               // (sm.next is zero: set up so, or left so by the searches before)
+    while (true) {
+        if (wt == 0 && lane == 0) {                // the next item that needs to be looked at
+            int it;
+            while ((it = atomicAdd(&sm.next, 1)) < n_items) {
+                const int c = it / n_mid, ci = n_cand - c;                         // large block sizes first
+                const SelActive& s = list[it - c * n_mid];
+                if (cands.g[ci] <= min((int)s.n, (int)s.b) && !(*(volatile const unsigned*)&s.passed >> ci)) break;
+            }
+            sm.team_item[team] = it;
+        }
+        team_sync(team);
+        const int it = *(volatile const int*)&sm.team_item[team];
+        if (it >= n_items) break;
+        const int c = it / n_mid, ci = n_cand - c;
+        SelActive& s = list[it - c * n_mid];
+        unsigned bits;
+        if (!sel_candidate_team(x + s.pos, ta + s.pos, s.n, s.b, cands.g[ci], thr, cut, tau, ts, team, bits)) continue;
+        if (keep_masks)
+            for (int q = 0; q < kMask / kSelTeam; ++q) {
+                const unsigned m = __ballot_sync(0xffffffffu, (bits >> q) & 1u);
+                if (lane == 0) masks[(size_t)it * kMask + q * kSelTeam + wt] = m;
+            }
+        if (wt == 0 && lane == 0) atomicOr(&s.passed, 1u << ci);
+    }
+    __syncthreads();
+    for (int y = team; y < n_mid; y += kSelTeams) {
+        const SelActive& s = list[y];
+        if (!s.passed) continue;
+        const int ci = 31 - __clz(s.passed), gs = cands.g[ci], pos = s.pos, n = s.n;
+        unsigned bits = 0;
+        if (keep_masks) {
+            const unsigned* m = masks + (size_t)((n_cand - ci) * n_mid + y) * kMask;
+            for (int q = 0; q < kMask / kSelTeam; ++q) bits |= ((m[q * kSelTeam + wt] >> lane) & 1u) << q;
+        } else {
+            sel_candidate_team(x + pos, ta + pos, n, s.b, gs, thr, cut, tau, ts, team, bits);
+        }
+        for (int i = wt * 32 + lane, q = 0; i < n; i += kSelTeam * 32, ++q) sel_set_bit(keep, pos + i, (bits >> q) & 1u);
+        if (seg_g && wt == 0 && lane == 0) seg_g[s.k] = gs;
+    }
+    __syncthreads();
+    if (tid == 0) sm.next = 0;
+    __syncthreads();
 }
 
 // ---- the same for a longer segment, by the whole CTA --------------------------------------------------
@@ -421,6 +601,17 @@ __device__ __forceinline__ void sel_long_select(const double* phi, int nb, int k
         k = sm.k;
         prefix |= (unsigned long long)sm.digit << shift;
         mask |= 0xFFull << shift;
+        if (sm.neq == 1) {                         // one block left with these digits (after three or four, as a rule): it is the one
+            for (int m = tid; m < nb; m += kSelThreads) {
+                const unsigned long long u = order_key64(phi[m]);
+                if ((u & mask) == prefix) { sm.mp = m; sm.key = u; }
+            }
+            __syncthreads();
+            thr = sm.key;
+            mp = sm.mp;
+            __syncthreads();
+            return;
+        }
         __syncthreads();
     }
     // the k-th block, in index order, among those whose key equals the threshold
@@ -516,6 +707,7 @@ __device__ bool sel_body(const Geo& g, const Cands& cands, const SelectArgs& a, 
     // retained tokens of this CTA, bit i = position ta + i
     unsigned* keep = kSm ? reinterpret_cast<unsigned*>(dyn + kSelOffKeep) : a.keep + (size_t)p * a.keep_words + (ta >> 5) + rank;
     SelActive* active = reinterpret_cast<SelActive*>(dyn + kSelOffActive);
+    SelActive* mid = reinterpret_cast<SelActive*>(dyn + kSelOffMid);
     unsigned short* segs = reinterpret_cast<unsigned short*>(dyn + kSelOffSegs);
     uint8_t* scratch = dyn + kSelOffScratch + warp * kSelScratch;
     const bool segs_sm = kSm && kz - ka <= kSelSegs;               // segment starts in shared memory too
@@ -713,8 +905,14 @@ __device__ bool sel_body(const Geo& g, const Cands& cands, const SelectArgs& a, 
             if (seg_g) seg_g[kk] = b > 0 ? 1 : 0;
             const bool any = n_cand > 0 && cands.g[1] <= min(n, b);
             if (any && n > kSegShort) {
-                const int slot = atomicAdd(&sm.n_long, 1);
-                if (slot < 64) sm.long_list[slot] = kk;
+                int slot = n <= kSegMid ? atomicAdd(&sm.n_mid, 1) : kSelMaxMid;
+                if (slot < kSelMaxMid) {
+                    SelActive& s = mid[slot];
+                    s.pos = pos; s.k = kk; s.n = (unsigned short)n; s.b = (unsigned short)b; s.passed = 0u;
+                } else {
+                    slot = atomicAdd(&sm.n_long, 1);
+                    if (slot < 64) sm.long_list[slot] = kk;
+                }
             }
             search = any && n <= kSegShort;
         }
@@ -728,11 +926,13 @@ __device__ bool sel_body(const Geo& g, const Cands& cands, const SelectArgs& a, 
         __syncthreads();
     }
     if (sm.n_active > 0) flush();
+    if (sm.n_mid > 0)
+        sel_teams<kSm>(sm, dyn, cands, kSm ? sv : s_ref + ta, ta, len, thr, cut, a.tau, keep, seg_g);
     const int n_long = sm.n_long;
     for (int x = n_long > 64 ? ka : 0, end = n_long > 64 ? kz : n_long; x < end; ++x) {     // more than the list holds: look at all
         const int kk = n_long > 64 ? x : sm.long_list[x];
         const int sa = sst[kk], n = sst[kk + 1] - sa;
-        if (n <= kSegShort) continue;
+        if (n <= kSegShort || (n <= kSegMid && sm.n_mid <= kSelMaxMid)) continue;      // searched by a warp or a team
         int bl = 0;
         double base = 0.0;
         for (int i = tid; i < n; i += kSelThreads) {
@@ -807,6 +1007,7 @@ select_kernel(const Geo g, const Cands cands, const SelectArgs a)
         sm.n_active = 0;
         sm.next = 0;
         sm.n_long = 0;
+        sm.n_mid = 0;
         mbar_init(smem_u32(&sm.bars[0]), C);
         mbar_init(smem_u32(&sm.bars[1]), C);
         fence_mbar_init();

@@ -34,6 +34,9 @@ def _lens(total, draw):
     (33280 + 1, [33280, 1], 2000),                                   # exactly what shared memory holds, and a token more
     (33281, [33281], 2000),
     (300000, [25] * 12000, 4000),                                    # longer than eight CTAs hold: scores stay in global memory
+    (9000, [1023, 1024, 1025, 700, 2], 4000),                        # around the longest segment that a team searches
+    (33280, [257] * 129, 20000),                                     # as many of those as a CTA's shared memory holds, in one CTA's share and less
+    (450000, [257] * 1750, 90000),                                   # more of them than a CTA's list holds
 ])
 @pytest.mark.parametrize("quantised", [False, True])
 def test_select_bookkeeping(T, lens, B_tok, quantised):
