@@ -377,25 +377,20 @@ score_p2_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
         simt_load_wait();
         float x[kTok][NW][GB];
         simt_logits<GB, kTok>(ks, qs, D, TG, tg, w, W, c2, x);
-        // A[h, w, t], summed over the heads; those that the KV head does not have add nothing, not even where a logit is
-        // infinite (a branch around the whole: a condition in every term costs 5 % of the pass)
-        if (nh == GB) {
+        if (nh < GB)                                    // heads that the KV head does not have add nothing, whatever the logit
 #pragma unroll
-            for (int y = 0; y < NW; ++y)
+            for (int b = 0; b < GB; ++b)
+                if (b >= nh)
 #pragma unroll
-                for (int i = 0; i < kTok; ++i)
+                    for (int y = 0; y < NW; ++y)
 #pragma unroll
-                    for (int b = 0; b < GB; ++b) abar[y][i] += exp2f(x[i][y][b] - ls[y][b]);
-        } else {
+                        for (int i = 0; i < kTok; ++i) x[i][y][b] = -INFINITY;
 #pragma unroll
-            for (int b = 0; b < GB; ++b) {
-                if (b >= nh) break;
+        for (int y = 0; y < NW; ++y)
 #pragma unroll
-                for (int y = 0; y < NW; ++y)
+            for (int i = 0; i < kTok; ++i)
 #pragma unroll
-                    for (int i = 0; i < kTok; ++i) abar[y][i] += exp2f(x[i][y][b] - ls[y][b]);
-            }
-        }
+                for (int b = 0; b < GB; ++b) abar[y][i] += exp2f(x[i][y][b] - ls[y][b]);    // A[h, w, t], summed over the heads
     }
     __syncthreads();
     // \bar A of this CTA's heads: [token][W + 1], over the key tile and, where that is short, the query rows
