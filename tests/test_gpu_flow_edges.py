@@ -1,7 +1,7 @@
 """The unit-flow score kernel at the edges of its schedule: lengths around a token tile and a unit, every
-number of window rows per KV head, several head groups (whose sums pass through scratch, more
-problems than that has slots), packed sequences of very different length among them ones that are
-returned unchanged, and the single sweep with more window rows than one group holds.  Reference: the
+number of window rows per KV head, long sequences of few window rows, several head groups (more than 1024 window rows:
+their sums pass through scratch that has fewer slots than there are problems) in one and two sweeps, packed
+sequences of very different length among them ones that are returned unchanged.  Reference: the
 scores and entropies in float64 on the stored values.
 
 Tolerance: a logit is an fp32 sum of D <= 128 exact products, partial sums below 64 in log2 units, so its
@@ -75,13 +75,15 @@ def test_window_rows(H, Hkv, W, D, lse):
     _run(H, Hkv, D, W, [1500], 3, 64, lse)
 
 
-@pytest.mark.parametrize("H,Hkv,W,D,L,n_layers", [(32, 8, 8, 128, 20011, 9), (32, 8, 16, 128, 40000, 6), (16, 4, 8, 64, 70001, 3)])
+@pytest.mark.parametrize("H,Hkv,W,D,L,n_layers", [(32, 8, 8, 128, 20011, 9), (32, 8, 16, 128, 40000, 6), (16, 4, 8, 64, 70001, 3),     # one group
+                                                  (64, 16, 32, 128, 5000, 9), (40, 40, 32, 64, 9001, 6), (35, 35, 32, 128, 2500, 5)])   # two
 def test_head_groups(H, Hkv, W, D, L, n_layers):
     _run(H, Hkv, D, W, [L], n_layers, 128)
 
 
-def test_head_groups_packed():
-    _run(32, 8, 128, 8, [17000, 300, 60, 9000, 129, 50], 5, 64)
+@pytest.mark.parametrize("H,Hkv,W", [(32, 8, 8), (40, 40, 32), (64, 16, 32)])
+def test_head_groups_packed(H, Hkv, W):
+    _run(H, Hkv, 128, W, [17000, 300, 60, 9000, 129, 50], 5, 64)
 
 
 @pytest.mark.parametrize("lse", [False, True])

@@ -1,8 +1,8 @@
 """The give-up paths of the bounded device-side waits, exercised without hanging anything: a second
 build of the library has the waits shortened to about a millisecond and hooks that make ONE producer
-withhold its post (a tile of the segmentation scan never publishes its state; one CTA of the Top-B
-select never reports its histogram; one CTA of the persistent score kernel never reports its row
-sums).  The waiting side must run into its limit, the kernel must return, the status word must say
+withhold its post (one CTA of a segmentation cluster never reports its count; one CTA of a selection cluster
+never reports its digit counts; one CTA of the persistent score kernel never reports its row
+sums, nor does the first unit of the unit-flow kernel).  The waiting side must run into its limit, the kernel must return, the status word must say
 TIMEOUT and the word after it must name the wait.  Nothing traps or faults; the product library is
 not involved (needs a B200)."""
 import numpy as np
@@ -105,5 +105,36 @@ def test_score_kernel_handover_gives_up(hooked):
     assert ((idx >= 0) & (idx < L)).all()
     hooked.sablock_test_set_hooks(0)
     out = B.compress_layers(p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, 256, cfg.candidates, ws)
+    torch.cuda.synchronize()
+    assert B.read_status_detail(ws) == (0, 0, 0) and torch.equal(out.out_idx, good)
+
+
+@pytest.mark.parametrize("H,Hkv,D,W,lens,layers", [(32, 8, 128, 32, [8192], 1),              # few tiles: the sets share the heads
+                                                   (32, 8, 128, 32, [3000, 700, 5000], 6),   # four tiles a unit
+                                                   (64, 16, 64, 32, [900, 2500], 3)])        # head groups waiting for one another
+def test_unit_flow_gives_up(hooked, H, Hkv, D, W, lens, layers):
+    """The kernel that the default choice takes: the row sums of one unit are missing, so one problem's log-sum-exps never
+    come, and whoever waits for them runs out."""
+    cfg = synth.Config("t", layers, H, Hkv, D, W, tuple(lens), (256,), (1, 2, 4), "bf16", 5000, 8, 2.0, 20, (0.4,), 9)
+    b = synth.make_batch(cfg, device="cuda")
+    total, max_L = b.cu_seqlens[-1], max(lens)
+    p = B.make_params(H, Hkv, D, W, torch.bfloat16, b.bitmap, cfg.vocab)
+    ws = B.alloc_workspace(p, total, max_L, len(lens), layers)
+    args = (p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, 256, cfg.candidates, ws)
+    out = B.compress_layers(*args)
+    torch.cuda.synchronize()
+    assert B.read_status_detail(ws) == (0, 0, 0)
+    good = out.out_idx.clone()
+    assert hooked.sablock_test_set_hooks(HOOK_SCORE) == 0
+    out = B.compress_layers(*args)
+    torch.cuda.synchronize()                                  # every role of every CTA left its loop
+    code, raw, where = B.read_status_detail(ws)
+    assert code == TIMEOUT and raw & 1
+    assert 1 <= _code(where) <= 21
+    for i, L in enumerate(lens):
+        idx = out.out_idx[:, i].cpu().numpy()
+        assert ((idx >= 0) & (idx < L)).all()
+    hooked.sablock_test_set_hooks(0)
+    out = B.compress_layers(*args)
     torch.cuda.synchronize()
     assert B.read_status_detail(ws) == (0, 0, 0) and torch.equal(out.out_idx, good)
