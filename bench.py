@@ -231,7 +231,8 @@ def run_ours(args):
         path = {"t_roofline_ms": round(t_roof_ms, 4), "frac_of_measured_hbm": round(t_roof_ms / r["ms_step"], 4),
                 "frac_of_nominal_8TBs": round(ab["total"] / 8e12 * 1e3 / r["ms_step"], 4),
                 "algorithmic_bytes": ab["total"], "score_flops": flops,
-                "stage_ms": {k: round(v, 4) for k, v in r["stage_avg"].items()}}
+                # (stages that are part of another one's kernel have intervals of nothing but two event records)
+                "stage_ms": {k: round(v, 4) for k, v in r["stage_avg"].items() if v > 0.01 or k in ("segment", "compact")}}
         return roofline, path
 
     def sustained(params, ms_step_hint):

@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libsablock.so (include/sablock.h): argument marshalling only.
+"""Thin binding of libsablock.so (include/sablock.h), argument marshalling only: by ctypes, the entry points that
+enqueue work through the C module csrc/fastcall.c where it is built.
 
 Every function takes torch CUDA tensors (or raw pointers), passes their device pointers
 through the C ABI and enqueues on torch's current stream.  No step of the pass runs in
@@ -236,8 +237,8 @@ SEGMENT_STATIC_MAX_T = 1024 * 2048
 
 def segment_static(p: Params, token_ids: torch.Tensor, seg_id: torch.Tensor, seg_start: torch.Tensor,
                    n_seg: torch.Tensor, status: Optional[torch.Tensor] = None) -> None:
-    """sablock_segment without a workspace: the caller supplies every buffer (outputs included),
-    the scan's scratch is a fixed array inside the library.  Nothing is allocated here."""
+    """sablock_segment without a workspace: the caller supplies every buffer (outputs included), and the
+    kernel's CTAs exchange their counts on chip.  Nothing is allocated here."""
     _check(lib().segment_static(C.addressof(p), _ptr(token_ids), token_ids.numel(), _ptr(seg_id),
                                         _ptr(seg_start), _ptr(n_seg), _ptr(status), _stream()),
            "sablock_segment_static")

@@ -1,6 +1,6 @@
 // C ABI of the SABlock compression library (see include/sablock.h): argument validation,
-// workspace planning, TMA tensor maps and kernel launches.  Every step of the pass runs in
-// the kernels of stages.cuh / score_simt.cuh / score_tc.cuh; there is no host fallback.
+// workspace planning, TMA tensor maps and kernel launches.  Every step of the pass runs in the kernels of
+// stages.cuh, select.cuh and the score_*.cuh, decoding in those of decode.cuh; there is no host fallback.
 #include <math.h>
 #include <stdio.h>
 #include <stdlib.h>

@@ -27,7 +27,8 @@
 // The head-summed attention of a token is in the registers of one thread for the whole unit.  What this
 // replaces for single-sweep scoring kept it in tensor memory and worked through the KV heads one at a
 // time: it had room for two accumulators only, two sets of eight warps that took turns at the
-// special-function unit, 3050 instructions per tile and SM against 1500 here.
+// special-function unit (schedulers issuing on 49 % of the cycles of the two-sweep kernel that still works so, on 38 % of
+// this one's single sweep).
 //
 // Few tiles in all (a short prompt, one layer): a B unit is ONE tile and the sets share the heads instead of the
 // tiles; their sums meet in tensor memory at the end of the unit.
@@ -102,7 +103,7 @@ struct FlShared {
 
 // The producer and the MMA issuer run as whole warps with uniform control flow, one elected lane issuing: TMA
 // and MMA instructions take their operands from uniform registers, and in a branch of a single lane every
-// operand would have to be moved there first (about forty moves per tile).
+// operand would have to be moved there first.
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t p;
