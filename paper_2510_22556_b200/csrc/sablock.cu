@@ -8,6 +8,7 @@
 
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "stages.cuh"
@@ -517,10 +518,14 @@ sablock_status_t launch_simt(const Plan& pl, const sablock_params_t* p, const Si
     }
     prof_mark(1, stream);
     prof_mark(2, stream);
-    SAB_TRY(allow_smem<score_p2_simt<T, GB, TOK>>(sp.smem));
     const int tiles = (pl.max_L + sp.tile - 1) / sp.tile;
-    return launch(score_p2_simt<T, GB, TOK>, dim3(tiles * sp.split, pl.n_prob), kSimtThreads, sp.smem, stream, sp.split, g, sp,
-                  (const T*)q, (const T*)k, ks.tok, ks.head, ks.layer, c2, p->eps, sb, s, e);
+    auto pass2 = [&](auto part) -> sablock_status_t {
+        constexpr bool kPart = decltype(part)::value;
+        SAB_TRY(allow_smem<score_p2_simt<T, GB, TOK, kPart>>(sp.smem));
+        return launch(score_p2_simt<T, GB, TOK, kPart>, dim3(tiles * sp.split, pl.n_prob), kSimtThreads, sp.smem, stream, sp.split, g, sp,
+                      (const T*)q, (const T*)k, ks.tok, ks.head, ks.layer, c2, p->eps, sb, s, e);
+    };
+    return GB > 1 && g.G % GB ? pass2(std::integral_constant<bool, (GB > 1)>()) : pass2(std::false_type());
 }
 
 // Stage 2: window scores s (pre-pooling) and per-token entropy e.

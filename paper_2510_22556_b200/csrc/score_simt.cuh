@@ -330,8 +330,8 @@ score_p1_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
 // Pass 2.  grid = (token tiles * split, problems), cluster = (split, 1, 1): the CTAs of a cluster
 // take the KV heads of one token tile in turn and add their head sums through distributed shared
 // memory, in rank order; each finishes its share of the tile's tokens.  `split` is 1 where the token
-// tiles alone fill the device.
-template <typename T, int GB, int kTok>
+// tiles alone fill the device.  kPart: a KV head's last unit may have fewer than GB heads (GB does not divide G).
+template <typename T, int GB, int kTok, bool kPart>
 __global__ void __launch_bounds__(kSimtThreads, 2)
 score_p2_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict__ k, long long ks_tok, long long ks_head,
               long long ks_layer, float c2, float eps, ScoreBufs sb, float* __restrict__ s_out, float* __restrict__ e_out)
@@ -363,7 +363,7 @@ score_p2_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
         for (int i = 0; i < kTok; ++i) abar[y][i] = 0.f;
     for (int unit = rank; unit < g.Hkv * sp.batches; unit += split) {
         const int j = unit / sp.batches, b0 = (unit - j * sp.batches) * GB;
-        const int nh = min(GB, g.G - b0);
+        const int nh = kPart ? min(GB, g.G - b0) : GB;
         __syncthreads();
         if (b0 == 0 || split > 1)
             simt_load_rows(ks, k + (size_t)layer * ks_layer + (size_t)j * ks_head + ((size_t)g.cu[seq] + t0) * ks_tok, ks_tok,
@@ -377,7 +377,7 @@ score_p2_simt(Geo g, SimtShape sp, const T* __restrict__ q, const T* __restrict_
         simt_load_wait();
         float x[kTok][NW][GB];
         simt_logits<GB, kTok>(ks, qs, D, TG, tg, w, W, c2, x);
-        if (nh < GB)                                    // heads that the KV head does not have add nothing, whatever the logit
+        if (kPart && nh < GB)                           // heads that the KV head does not have add nothing, whatever the logit
 #pragma unroll
             for (int b = 0; b < GB; ++b)
                 if (b >= nh)
