@@ -17,6 +17,7 @@
 #include "score_tc.cuh"
 #include "score_fused.cuh"
 #include "score_flow.cuh"
+#include "score_x3.cuh"
 #include "decode.cuh"
 
 using namespace sab;
@@ -69,12 +70,14 @@ struct Plan {
     int fl_groups, fl_heads, fl_m, fl_parts, fl_tiles;   // its head groups, heads of a group, tiles per set of an A unit, partials, tiles
     int tpc1, tpc2;            // tiles per CTA of the tensor-core passes
     SimtShape simt;            // shape of the SIMT passes
+    bool use_x3;               // fp32 on the tensor cores
+    int x3_ld, x3_tpc, x3_chunks;      // its rows of logits, tiles per CTA, partials per window row
     int n_chunks;              // pass-1 partials per row
     int units;                 // row blocks of pass 1 per problem
     int keep_words;
     // workspace offsets
     size_t o_status, o_keep, o_arrive, o_done, o_fl_ticket, o_bdone, o_carry, control_bytes;
-    size_t o_seg_id, o_seg_start, o_n_seg, o_s_raw, o_s, o_e, o_sr, o_part, o_lse, o_neg_lse, o_phi, o_fpart, total;
+    size_t o_seg_id, o_seg_start, o_n_seg, o_s_raw, o_s, o_e, o_sr, o_part, o_lse, o_neg_lse, o_phi, o_fpart, o_x3, total;
     struct Region { size_t Plan::*field; size_t bytes; } regions[24];      // the same in layout order
     int n_regions;
     size_t clear_from;         // the control words from here on are cleared by the call
@@ -88,6 +91,12 @@ bool tc_eligible(const sablock_params_t* p)
     const int G = p->n_q_heads / p->n_kv_heads;
     if (G * p->window > 128) return false;
     return true;
+}
+
+bool x3_eligible(const sablock_params_t* p)
+{
+    return p->dtype == SABLOCK_F32 && p->score_impl == SABLOCK_SCORE_AUTO && (p->head_dim == 64 || p->head_dim == 128) &&
+           p->window <= kX3MaxW && p->n_q_heads / p->n_kv_heads * p->window <= 128;
 }
 
 // The persistent kernel takes the shape whose 128 window rows per KV head fill one MMA tile.
@@ -178,9 +187,12 @@ Strides v_strides(const sablock_params_t* p, long long total_tokens)
     return s;
 }
 
+// Bytes of a call's logits.
+size_t x3_logits(const Plan& pl) { return sizeof(float) * (size_t)pl.n_prob * pl.geo.H * pl.geo.window * pl.x3_ld; }
+
 // Builds geometry + workspace layout.  cu == NULL means one sequence of max_L tokens.
 sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, long long total_tokens,
-                           int max_L, int n_out, Plan* pl)
+                           int max_L, int n_out, Plan* pl, bool allow_x3 = true)
 {
     sablock_status_t st = validate_params(p);
     if (st != SABLOCK_OK) return st;
@@ -256,6 +268,12 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
         pl->tpc1 = pl->tpc2 = 1;
         pl->n_chunks = (int)((tl + sp.tpc - 1) / sp.tpc);
         pl->units = (int)units;
+        // fp32 on the tensor cores: one CTA per SM, whole tiles of one KV head each
+        pl->x3_ld = (int)(tiles * kTcTile);
+        pl->use_x3 = allow_x3 && x3_eligible(p) && x3_logits(*pl) <= kX3MaxBytes;
+        pl->x3_tpc = (int)((tiles * g.Hkv * pl->n_prob + sm_count() - 1) / sm_count());
+        if (pl->x3_tpc > tiles) pl->x3_tpc = (int)tiles;
+        pl->x3_chunks = (int)((tiles + pl->x3_tpc - 1) / pl->x3_tpc);
     }
     pl->keep_words = (max_L + 31) / 32 + kSelMaxCluster + 1;       // every CTA of a problem starts at a word of its own
 
@@ -282,13 +300,21 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     const size_t part_n = pl->use_tc ? (size_t)pl->n_prob * g.Hkv * pl->n_chunks * 128
                                      : (size_t)pl->n_prob * pl->units * pl->n_chunks * pl->simt.gb * g.window;
     const size_t flow_n = flow_ok ? (size_t)pl->n_prob * g.Hkv * (pl->fl_parts + (pl->fl_parts + kFlMerge - 1) / kFlMerge) * g.G * g.window : 0;
-    take(&Plan::o_part, sizeof(float2) * (part_n > flow_n ? part_n : flow_n));
+    // (Scratch that only calls up to some size use is kept in larger ones' plans too: a workspace that is sized for the longest
+    // prompt serves the shorter ones.)
+    const bool x3_room = !pl->use_tc && x3_eligible(p);
+    const size_t x3_n = x3_room ? ((size_t)sm_count() + (size_t)pl->n_prob * g.Hkv) * g.G * g.window : 0;
+    size_t most = part_n > flow_n ? part_n : flow_n;
+    if (x3_n > most) most = x3_n;
+    take(&Plan::o_part, sizeof(float2) * most);
     take(&Plan::o_carry, carries ? sizeof(float) * (size_t)kFlCarryRing * pl->fl_tiles * g.window * 128 : 0);
     take(&Plan::o_lse, sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
     take(&Plan::o_neg_lse, sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
     take(&Plan::o_keep, sizeof(unsigned) * (size_t)pl->n_prob * pl->keep_words);
     take(&Plan::o_phi, sizeof(double) * ntok);
     take(&Plan::o_fpart, pl->use_fused ? sizeof(float2) * (size_t)kFuMaxCtas * kFuPartSlots * 128 : 0);
+    const size_t x3_bytes = x3_room ? x3_logits(*pl) : 0;                  // (rows start on 32-byte boundaries wherever the workspace does)
+    take(&Plan::o_x3, x3_room ? (x3_bytes < kX3MaxBytes ? x3_bytes : kX3MaxBytes) + 32 : 0);
     pl->total = o;
     return SABLOCK_OK;
 }
@@ -528,6 +554,30 @@ sablock_status_t launch_simt(const Plan& pl, const sablock_params_t* p, const Si
     return GB > 1 && g.G % GB ? pass2(std::integral_constant<bool, (GB > 1)>()) : pass2(std::false_type());
 }
 
+template <int D>
+sablock_status_t run_x3(const Plan& pl, const sablock_params_t* p, const void* q, const void* k, const Strides& ks, float c2,
+                        const ScoreBufs& sb, float* s, float* e, void* ws, cudaStream_t stream)
+{
+    const Geo& g = pl.geo;
+    X3Args a;
+    a.q = static_cast<const float*>(q); a.k = static_cast<const float*>(k);
+    a.k_tok = ks.tok; a.k_head = ks.head; a.k_layer = ks.layer;
+    a.c2 = c2;
+    a.sb = sb;
+    a.sb.n_chunks = pl.x3_chunks;
+    a.x = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(at<char>(ws, pl.o_x3)) + 31) & ~(uintptr_t)31);
+    a.ld = pl.x3_ld; a.tpc = pl.x3_tpc;
+    a.stats = p->row_lse == nullptr;
+    a.status = at<int>(ws, pl.o_status);
+    SAB_TRY(allow_smem<score_x3_logits<D>>(x3_smem(D)));
+    SAB_TRY(launch(score_x3_logits<D>, dim3(pl.x3_chunks, g.Hkv, pl.n_prob), kX3Threads, x3_smem(D), stream, 1, g, a));
+    prof_mark(1, stream);
+    prof_mark(2, stream);
+    const int groups = (pl.max_L - g.window + kX3SumTokens - 1) / kX3SumTokens;
+    const int threads = g.H * g.window >= kX3SumManyRows ? kX3SumThreads : kX3SumThreads / 2;
+    return launch(score_x3_sum, dim3(groups > 0 ? groups : 1, pl.n_prob), threads, 0, stream, 1, g, a.x, a.ld, p->eps, sb.lse2, s, e);
+}
+
 // Stage 2: window scores s (pre-pooling) and per-token entropy e.
 sablock_status_t run_score(const Plan& pl, const sablock_params_t* p, const void* q, const void* k, float* s,
                            float* e, void* ws, cudaStream_t stream)
@@ -656,6 +706,8 @@ sablock_status_t run_score(const Plan& pl, const sablock_params_t* p, const void
     sp.vec_q = (reinterpret_cast<uintptr_t>(q) & 15) == 0;              // D * element size is a multiple of 16
     const int es = elem_size(p);
     sp.vec_k = ((reinterpret_cast<uintptr_t>(k) | (uintptr_t)(ks.tok * es) | (uintptr_t)(ks.head * es) | (uintptr_t)(ks.layer * es)) & 15) == 0;
+    if (pl.use_x3 && sp.vec_q && sp.vec_k)
+        return g.D == 128 ? run_x3<128>(pl, p, q, k, ks, c2, sb, s, e, ws, stream) : run_x3<64>(pl, p, q, k, ks, c2, sb, s, e, ws, stream);
     const bool bf = p->dtype == SABLOCK_BF16;
 #define SAB_SIMT(T, GB) (sp.tok == kSimtTokLarge ? launch_simt<T, GB, kSimtTokLarge>(pl, p, sp, q, k, ks, c2, sb, s, e, stream) \
                                                  : launch_simt<T, GB, kSimtTokSmall>(pl, p, sp, q, k, ks, c2, sb, s, e, stream))
@@ -849,8 +901,9 @@ HostStreams* host_streams()
 bool plan_inside(const Plan& whole, const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, int max_L, int n_out,
                  Plan* pl)
 {
-    if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, pl) != SABLOCK_OK || pl->n_regions != whole.n_regions) return false;
-    if (pl->use_tc != whole.use_tc || pl->use_flow != whole.use_flow || pl->use_fused != whole.use_fused) return false;
+    if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, pl, whole.use_x3) != SABLOCK_OK || pl->n_regions != whole.n_regions)
+        return false;
+    if (pl->use_tc != whole.use_tc || pl->use_x3 != whole.use_x3 || pl->use_flow != whole.use_flow || pl->use_fused != whole.use_fused) return false;
     if (pl->use_tc && (long long)pl->n_prob * pl->geo.H * pl->geo.window < kTcTile) return false;
     for (int i = 0; i < pl->n_regions; ++i) {
         if (pl->regions[i].bytes > whole.regions[i].bytes) return false;
