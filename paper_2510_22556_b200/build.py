@@ -11,7 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsablock.so")
 FASTCALL = os.path.join(HERE, "_fastcall.so")
 SOURCES = ["sablock.cu"]
-HEADERS = ["common.cuh", "stages.cuh", "select.cuh", "score_simt.cuh", "score_tc.cuh", "score_fused.cuh", "score_flow.cuh", "score_x3.cuh",
+HEADERS = ["common.cuh", "stages.cuh", "select.cuh", "score_simt.cuh", "score_tc.cuh", "score_fused.cuh", "score_flow.cuh", "score_pair.cuh", "score_x3.cuh",
            "decode.cuh"]
 
 

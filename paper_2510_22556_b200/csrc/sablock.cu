@@ -17,6 +17,7 @@
 #include "score_tc.cuh"
 #include "score_fused.cuh"
 #include "score_flow.cuh"
+#include "score_pair.cuh"
 #include "score_x3.cuh"
 #include "decode.cuh"
 
@@ -66,7 +67,9 @@ struct Plan {
     int n_prob, max_L;
     bool use_tc;
     bool use_fused;            // the persistent two-sweep kernel (Llama-shaped problems)
-    bool use_flow;             // the unit-flow kernel
+    bool use_flow;             // the unit-flow kernel, or for short prompts
+    bool use_pair;             // the two kernels of score_pair.cuh,
+    int pr_parts;              // with so many partials per window row
     int fl_groups, fl_heads, fl_m, fl_parts, fl_tiles;   // its head groups, heads of a group, tiles per set of an A unit, partials, tiles
     int tpc1, tpc2;            // tiles per CTA of the tensor-core passes
     SimtShape simt;            // shape of the SIMT passes
@@ -240,6 +243,11 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
                               (long long)n_layers * total_tokens < 0x7fffffffLL &&
                               (long long)max_L * g.Hkv * p->head_dim * 2 > (48LL << 20);
     pl->use_flow = flow_ok && (p->row_lse != nullptr || !fixed_shares);
+    // Short prompts: two kernels of few CTAs
+    pl->pr_parts = (int)((tiles + kPrTiles - 1) / kPrTiles);
+    const bool pair_room = flow_ok && g.Hkv <= kPrMaxHeads && (g.Hkv & (g.Hkv - 1)) == 0;
+    const long long pair_ctas = (long long)pl->pr_parts * g.Hkv * pl->n_prob, pair_max = pr_max_ctas(true) * sm_count();
+    pl->use_pair = pl->use_flow && pair_room && pair_ctas <= pr_max_ctas(p->row_lse == nullptr) * sm_count();
     pl->use_fused = pl->use_tc && p->score_impl != SABLOCK_SCORE_TENSOR && fused_eligible(p);
     if (pl->use_tc) {
         long long work1 = tiles * g.Hkv * pl->n_prob, work2 = tiles * pl->n_prob;
@@ -299,6 +307,7 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     take(&Plan::o_sr, sizeof(float) * ntok);
     const size_t part_n = pl->use_tc ? (size_t)pl->n_prob * g.Hkv * pl->n_chunks * 128
                                      : (size_t)pl->n_prob * pl->units * pl->n_chunks * pl->simt.gb * g.window;
+    const size_t pair_n = pair_room ? (size_t)(pair_ctas < pair_max ? pair_ctas : pair_max) * g.G * g.window : 0;
     const size_t flow_n = flow_ok ? (size_t)pl->n_prob * g.Hkv * (pl->fl_parts + (pl->fl_parts + kFlMerge - 1) / kFlMerge) * g.G * g.window : 0;
     // (Scratch that only calls up to some size use is kept in larger ones' plans too: a workspace that is sized for the longest
     // prompt serves the shorter ones.)
@@ -306,6 +315,7 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     const size_t x3_n = x3_room ? ((size_t)sm_count() + (size_t)pl->n_prob * g.Hkv) * g.G * g.window : 0;
     size_t most = part_n > flow_n ? part_n : flow_n;
     if (x3_n > most) most = x3_n;
+    if (pair_n > most) most = pair_n;
     take(&Plan::o_part, sizeof(float2) * most);
     take(&Plan::o_carry, carries ? sizeof(float) * (size_t)kFlCarryRing * pl->fl_tiles * g.window * 128 : 0);
     take(&Plan::o_lse, sizeof(float) * (size_t)pl->n_prob * g.H * g.window);
@@ -481,9 +491,30 @@ sablock_status_t launch_p2_tc(const Plan& pl, const CUtensorMap& tmQ, const CUte
 }
 
 template <int W, int D>
+sablock_status_t run_pair(const Plan& pl, const sablock_params_t* p, const CUtensorMap& tmQ, const CUtensorMap& tmK, float c2,
+                          const ScoreBufs& sb, float* s, float* e, void* ws, cudaStream_t stream)
+{
+    const Geo& g = pl.geo;
+    PairArgs a;
+    a.c2 = c2; a.eps = p->eps;
+    a.part = sb.part; a.n_part = pl.pr_parts;
+    a.row_lse = p->row_lse;
+    a.s_out = s; a.e_out = e; a.status = at<int>(ws, pl.o_status);
+    if (!a.row_lse) {
+        SAB_TRY(allow_smem<score_rows_tc<W, D>>(pr_smem(D)));
+        SAB_TRY(launch(score_rows_tc<W, D>, dim3(pl.pr_parts, g.Hkv, pl.n_prob), kPrThreads, pr_smem(D), stream, 1, tmQ, tmK, g, a));
+    }
+    prof_mark(1, stream);
+    prof_mark(2, stream);
+    SAB_TRY(allow_smem<score_heads_tc<W, D>>(pr_smem(D)));
+    return launch(score_heads_tc<W, D>, dim3(g.Hkv, pl.pr_parts, pl.n_prob), kPrThreads, pr_smem(D), stream, g.Hkv, tmQ, tmK, g, a);
+}
+
+template <int W, int D>
 sablock_status_t run_flow(const Plan& pl, const sablock_params_t* p, const CUtensorMap& tmQ, const CUtensorMap& tmK, float c2,
                           const ScoreBufs& sb, float* s, float* e, void* ws, cudaStream_t stream)
 {
+    if (pl.use_pair) return run_pair<W, D>(pl, p, tmQ, tmK, c2, sb, s, e, ws, stream);
     const Geo& g = pl.geo;
     FlowArgs fa;
     memset(&fa, 0, sizeof(fa));
