@@ -20,6 +20,11 @@ constexpr int kDecMaxSplits = 512;
 constexpr int kDecMaxD = 256;
 constexpr int kDecMaxG = 4;
 constexpr int kDecClusterRows = 8192;
+// Rows up to which eight splits in a cluster beat as many splits as the device has room for and a second launch, one problem of
+// 8 KV heads (us a layer, cluster / two launches): rows of 256 bytes, 4096 9.7 / 10.5, 6144 12.0 / 12.0, 8192 14.1 / 13.2;
+// rows of 128 bytes, 4096 6.9 / 6.4, 8192 10.5 / 9.0.
+__host__ __device__ constexpr int dec_cluster_rows(int row_bytes) { return row_bytes <= 128 ? 3072 : 6144; }
+constexpr int kDecClusterSplits = 9;                 // four problems, 9 splits: 4096 rows 15.1 / 17.1, 8192 25.0 / 27.4, 16384 47.0 / 48.6
 constexpr int kDecMaxCluster = 8;                    // CTAs that merge through distributed shared memory
 
 struct DecodeArgs {

@@ -963,7 +963,8 @@ int host_chunk(const Plan& whole, const sablock_params_t* p, int n_layers, int n
 // ---- decoding over a cache: launch plan ----------------------------------------------------
 struct DecodePlan { int n_splits, rows_per_split; bool cluster; size_t bytes; };
 
-sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, DecodePlan* dp)
+// The plan of a call that has ws_bytes of scratch.
+sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, size_t ws_bytes, DecodePlan* dp)
 {
     SAB_TRY(validate_params(p));
     if (n_prob < 1 || n_rows < 1) return SABLOCK_ERR_INVALID_ARG;
@@ -974,16 +975,19 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
     const long long per_split = (long long)p->n_kv_heads * n_prob;
     dp->cluster = false;
     long long splits;
+    auto scratch = [&](long long n) { return align_up(sizeof(float) * (size_t)n_prob * p->n_q_heads * n * (p->head_dim + 2)); };
     if (p->dtype == SABLOCK_BF16) {
         // One wave of two CTAs per SM, at least 64 rows (one chunk per warp) each.  Up to eight splits
         // are a cluster that merges on chip.  Beyond that a short cache still goes to clusters of
-        // eight: the rows that a CTA then reads more take less time than the second launch and
-        // the trip through scratch (kDecClusterRows: where the two cost the same).
+        // eight, and so does one that would have a single split more: the rows that a CTA then reads more take less time
+        // than the second launch and the trip through scratch (dec_cluster_rows: where the two cost the same).  And a
+        // cache of at most kDecClusterRows whose caller has brought no scratch for the other form.
         splits = 2LL * sm_count() / per_split;
         const long long by_rows = (n_rows + 63) / 64;
         if (splits > by_rows) splits = by_rows;
         if (splits < 1) splits = 1;
-        if (splits <= kDecMaxCluster || n_rows <= kDecClusterRows) {
+        if (splits <= kDecClusterSplits || n_rows <= dec_cluster_rows(row_bytes) ||
+            (n_rows <= kDecClusterRows && ws_bytes < scratch(splits))) {
             dp->cluster = true;
             int c = 1;
             while (c < splits && c < kDecMaxCluster) c *= 2;
@@ -1000,7 +1004,7 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
     dp->n_splits = (int)splits;
     dp->rows_per_split = (int)((n_rows + splits - 1) / splits);
     // the scratch of the clustered form is none; a caller's buffer may not be empty
-    dp->bytes = dp->cluster ? 256 : align_up(sizeof(float) * (size_t)n_prob * p->n_q_heads * splits * (p->head_dim + 2));
+    dp->bytes = dp->cluster ? 256 : scratch(splits);
     return SABLOCK_OK;
 }
 
@@ -1342,7 +1346,7 @@ sablock_status_t sablock_compress(const sablock_params_t* p, const void* q_win, 
 size_t sablock_decode_workspace_bytes(const sablock_params_t* p, int n_prob, int n_rows)
 {
     DecodePlan dp;
-    return decode_plan(p, n_prob, n_rows, &dp) == SABLOCK_OK ? dp.bytes : 0;
+    return decode_plan(p, n_prob, n_rows, SIZE_MAX, &dp) == SABLOCK_OK ? dp.bytes : 0;
 }
 
 sablock_status_t sablock_decode_attention(const sablock_params_t* p, int n_prob, const void* q, const void* k_cache,
@@ -1352,7 +1356,7 @@ sablock_status_t sablock_decode_attention(const sablock_params_t* p, int n_prob,
     t_launches = 0;
     if (!p || !q || !k_cache || !v_cache || !out) return SABLOCK_ERR_INVALID_ARG;
     DecodePlan dp;
-    SAB_TRY(decode_plan(p, n_prob, n_rows, &dp));
+    SAB_TRY(decode_plan(p, n_prob, n_rows, ws_bytes, &dp));
     if (!ws || ws_bytes < dp.bytes) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
     const int es = elem_size(p);
     DecodeArgs a;

@@ -106,3 +106,25 @@ def test_decode_values_near_the_end_of_the_range(H, Hkv, D, n_rows, n_prob):
     out = B.decode_attention(p, q, k, v).double()
     assert bool(torch.isfinite(out).all())
     assert float((out - ref).abs().max()) <= 2e-5 * 4 * 1e38                        # logits up to four times those above
+
+
+@pytest.mark.parametrize("H,Hkv,D,n_rows,n_prob", [(32, 8, 128, 6144, 1), (32, 8, 128, 6145, 1), (16, 8, 64, 3072, 1), (16, 8, 64, 3073, 1),
+                                                   (32, 8, 128, 9000, 4), (8, 2, 256, 6144, 2), (8, 2, 256, 6145, 2)])
+def test_decode_on_either_side_of_the_cluster_rule(H, Hkv, D, n_rows, n_prob):
+    """And with a scratch that holds no partial results, which a caller sized for a batch that needs none may bring: the cluster
+    takes what it took (8192 rows), longer caches are refused."""
+    g = torch.Generator(device="cuda").manual_seed(n_rows + D)
+    q = torch.randn(n_prob, H, D, generator=g, device="cuda").to(torch.bfloat16)
+    k, v = (torch.randn(n_prob, n_rows, Hkv, D, generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    p = B.make_params(H, Hkv, D, 8, torch.bfloat16)
+    ref, _ = _reference(q, k, v, [n_rows] * n_prob)
+    tol = 2e-5 * float(v.double().abs().max())
+    need = int(B.lib().sablock_decode_workspace_bytes(B.C.addressof(p), n_prob, n_rows))
+    for nb in {need, 256}:
+        ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+        if nb < need and n_rows > 8192:
+            with pytest.raises(B.SablockError) as err:
+                B.decode_attention(p, q, k, v, ws=ws)
+            assert err.value.code == 3
+        else:
+            assert float((B.decode_attention(p, q, k, v, ws=ws).double() - ref).abs().max()) <= tol
