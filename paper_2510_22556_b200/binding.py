@@ -97,6 +97,7 @@ def _load(path: str):
                  "decode_attention"):
         fn = getattr(l, "sablock_" + name)
         setattr(l, name, _fastcall.bind(C.cast(fn, C.c_void_p).value) if _fastcall else fn)
+    l.decode_step = _fastcall.bind_decode(C.cast(l.sablock_decode_attention, C.c_void_p).value) if _fastcall else None
     l.sablock_decode_workspace_bytes.restype = C.c_size_t
     l.sablock_decode_workspace_bytes.argtypes = [vp, ci, ci]
     l.sablock_decode_attention.argtypes = [vp, ci, vp, vp, vp, ci, vp, vp, vp, vp, sz, vp]
@@ -349,18 +350,23 @@ def decode_attention(p: Params, q: torch.Tensor, k_cache: torch.Tensor, v_cache:
                      want_lse: bool = False):
     """One decode step's attention over a cache.  q [n_prob, H, D]; k_cache, v_cache
     [n_prob, n_rows, Hkv, D] (contiguous).  Returns out f32 [n_prob, H, D] (and lse [n_prob, H])."""
-    n_prob, H, D = q.shape
-    n_rows = k_cache.shape[1]
     if ws is None:
+        n_prob, n_rows = q.shape[0], k_cache.shape[1]
         nb = int(lib().sablock_decode_workspace_bytes(C.addressof(p), n_prob, n_rows))
         if nb == 0:
             raise SablockError(2, "sablock_decode_workspace_bytes")
         ws = torch.empty(nb, dtype=torch.uint8, device=q.device)
     # (empty_like is the cheaper call; it keeps the strides of a dense input, so it is for contiguous ones)
     out = (torch.empty_like(q, dtype=torch.float32) if q.is_contiguous()
-           else torch.empty(n_prob, H, D, dtype=torch.float32, device=q.device))
-    lse = torch.empty(n_prob, H, dtype=torch.float32, device=q.device) if want_lse else None
-    _check(lib().decode_attention(C.addressof(p), n_prob, _ptr(q), _ptr(k_cache), _ptr(v_cache), n_rows,
-                                          _ptr(n_valid), _ptr(out), _ptr(lse), _ptr(ws), ws.numel(), _stream()),
-           "sablock_decode_attention")
+           else torch.empty(q.shape, dtype=torch.float32, device=q.device))
+    lse = torch.empty(q.shape[:2], dtype=torch.float32, device=q.device) if want_lse else None
+    l = lib()
+    if l.decode_step is not None:
+        code = l.decode_step(C.addressof(p), q, k_cache, v_cache, n_valid, out, lse, ws, _stream())
+    else:
+        n_prob, H, D = q.shape
+        code = l.decode_attention(C.addressof(p), n_prob, _ptr(q), _ptr(k_cache), _ptr(v_cache), k_cache.shape[1], _ptr(n_valid),
+                                  _ptr(out), _ptr(lse), _ptr(ws), ws.numel(), _stream())
+    if code != OK:
+        raise SablockError(code, "sablock_decode_attention")
     return (out, lse) if want_lse else out

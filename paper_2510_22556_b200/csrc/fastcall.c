@@ -91,6 +91,69 @@ static PyObject* bind(PyObject* module, PyObject* address)
     return PyCFunction_New(&invoke_def, address);
 }
 
-static PyMethodDef methods[] = {{"bind", bind, METH_O, "bind(address): a callable for the entry point at that address"}, {NULL, NULL, 0, NULL}};
+/* A decoding step is one short call per layer, and most of its host time is Python's: bind_decode(address) returns a builtin
+ * that takes the tensors themselves, (params, q, k_cache, v_cache, n_valid, out, lse, ws, stream), and asks them for what
+ * sablock_decode_attention wants to know. */
+static PyObject *s_data_ptr, *s_shape, *s_numel;
+
+static int take_method(PyObject* t, PyObject* name, u* out)
+{
+    if (t == Py_None) return 0;                        /* a null pointer */
+    PyObject* v = PyObject_CallMethodNoArgs(t, name);
+    if (!v) return -1;
+    const int rc = take_scalar(v, out);
+    Py_DECREF(v);
+    return rc;
+}
+
+/* Extent `dim` of a tensor; it has `rank` dimensions (0: any number). */
+static int take_extent(PyObject* t, Py_ssize_t rank, Py_ssize_t dim, u* out)
+{
+    PyObject* shape = PyObject_GetAttr(t, s_shape);
+    if (!shape) return -1;
+    int rc = -1;
+    if (!PyTuple_Check(shape)) PyErr_SetString(PyExc_TypeError, "a tensor");
+    else if (rank && PyTuple_GET_SIZE(shape) != rank) PyErr_Format(PyExc_ValueError, "%zd dimensions, not %zd", PyTuple_GET_SIZE(shape), rank);
+    else if (dim >= PyTuple_GET_SIZE(shape)) PyErr_SetString(PyExc_IndexError, "too few dimensions");
+    else rc = take_scalar(PyTuple_GET_ITEM(shape, dim), out);
+    Py_DECREF(shape);
+    return rc;
+}
+
+static PyObject* invoke_decode(PyObject* self, PyObject* const* args, Py_ssize_t n)
+{
+    typedef int (*decode)(u, u, u, u, u, u, u, u, u, u, u, u);
+    u p = 0, q = 0, k = 0, v = 0, valid = 0, out = 0, lse = 0, ws = 0, ws_bytes = 0, stream = 0, n_prob = 0, n_rows = 0;
+    if (n != 9) return PyErr_Format(PyExc_TypeError, "%zd arguments, not 9", n);
+    if (take_scalar(args[0], &p) < 0 || take_extent(args[1], 3, 0, &n_prob) < 0 || take_extent(args[2], 0, 1, &n_rows) < 0 ||
+        take_method(args[1], s_data_ptr, &q) < 0 || take_method(args[2], s_data_ptr, &k) < 0 || take_method(args[3], s_data_ptr, &v) < 0 ||
+        take_method(args[4], s_data_ptr, &valid) < 0 || take_method(args[5], s_data_ptr, &out) < 0 || take_method(args[6], s_data_ptr, &lse) < 0 ||
+        take_method(args[7], s_data_ptr, &ws) < 0 || take_method(args[7], s_numel, &ws_bytes) < 0 || take_scalar(args[8], &stream) < 0)
+        return NULL;
+    const decode f = (decode)(uintptr_t)PyLong_AsUnsignedLongLong(self);
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = f(p, n_prob, q, k, v, n_rows, valid, out, lse, ws, ws_bytes, stream);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(rc);
+}
+
+static PyMethodDef invoke_decode_def = {"decode", (PyCFunction)(void (*)(void))invoke_decode, METH_FASTCALL, "calls sablock_decode_attention"};
+
+static PyObject* bind_decode(PyObject* module, PyObject* address)
+{
+    (void)module;
+    if (!PyLong_Check(address)) return PyErr_Format(PyExc_TypeError, "an address");
+    return PyCFunction_New(&invoke_decode_def, address);
+}
+
+static PyMethodDef methods[] = {{"bind_decode", bind_decode, METH_O, "bind_decode(address): sablock_decode_attention for tensors"},
+                                {"bind", bind, METH_O, "bind(address): a callable for the entry point at that address"}, {NULL, NULL, 0, NULL}};
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_fastcall", NULL, -1, methods, NULL, NULL, NULL, NULL};
-PyMODINIT_FUNC PyInit__fastcall(void) { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__fastcall(void)
+{
+    s_data_ptr = PyUnicode_InternFromString("data_ptr");
+    s_shape = PyUnicode_InternFromString("shape");
+    s_numel = PyUnicode_InternFromString("numel");
+    return s_data_ptr && s_shape && s_numel ? PyModule_Create(&module) : NULL;
+}

@@ -73,3 +73,27 @@ def test_the_binding_takes_numpy_integers():
                                   [np.int64(1), np.int64(2)], 2, fake.data_ptr(), fake.data_ptr(), fake.data_ptr(), fake.data_ptr(),
                                   fake.data_ptr(), 4, None), "sablock_compress")
     assert err.value.code == 3
+
+
+def test_a_decoding_step_passes_what_the_tensors_say():
+    """(on the CPU: a callback in the entry point's place, tensors that are views and carry an offset)"""
+    seen = []
+    proto = C.CFUNCTYPE(C.c_int, *[C.c_uint64] * 12)
+    fn = proto(lambda *a: seen.append(a) or 7)
+    step = fastcall.bind_decode(C.cast(fn, C.c_void_p).value)
+    q = torch.zeros(5, 4, 8)[1:4]
+    k, v = torch.zeros(3, 2, 11, 2, 8).unbind(1)
+    out, ws, n = torch.zeros(3, 4, 8), torch.zeros(300, dtype=torch.uint8)[44:], torch.zeros(3, dtype=torch.int32)
+    assert step(np.int64(99), q, k, v, n, out, None, ws, 1 << 40) == 7
+    assert seen == [(99, 3, q.data_ptr(), k.data_ptr(), v.data_ptr(), 11, n.data_ptr(), out.data_ptr(), 0, ws.data_ptr(), 256, 1 << 40)]
+    with pytest.raises(ValueError):
+        step(99, q[0], k, v, None, out, None, ws, 0)
+    with pytest.raises(IndexError):
+        step(99, q, k[0, :, 0, 0], v, None, out, None, ws, 0)
+    with pytest.raises(AttributeError):
+        step(99, q, k, 5, None, out, None, ws, 0)
+    with pytest.raises(TypeError):
+        step(99, q, k, v, None, out, None, ws)
+    with pytest.raises(TypeError):
+        step(9.5, q, k, v, None, out, None, ws, 0)
+    assert len(seen) == 1
