@@ -94,8 +94,10 @@ struct FlShared {
     uint64_t afull[4], aempty[4];                // row sums of an A unit
     uint32_t tmem_base;
     int abort_flag;
-    int units_a[kMaxSeqs], units_b[kMaxSeqs];
-    int prefix[kFlMaxSlots + 1];
+    int units_a[kMaxSeqs], units_b[kMaxSeqs], per_head[kMaxSeqs];        // per sequence: A and B units of a head group, A units of a head
+    int prefix[kFlMaxSlots + 1];                 // units before each (sequence, head group) of a period,
+    int ahead_units[kFlMaxSlots];                // of which so many are A units (of the one `lag` further on)
+    int ahead;                                   // A units that come before all of them
     __align__(16) FlUnit unit[kFlUnits];
     __align__(16) float lse[2][kFlMaxRows];
     float2 sums[4][4][128];  // [A unit & 3][set][row]
@@ -143,24 +145,33 @@ __host__ __device__ inline int fl_carry_tenant(const Geo& g, const FlowArgs& fa,
 // Lane quarter at which set s has its window rows in an A unit.
 __device__ __forceinline__ int fl_shift(int R, int s) { return R <= 32 ? s : R <= 64 ? (s & 1) * 2 : 0; }
 
-// Unit of ticket t; kind 3: the number belongs to no unit.
+// Unit of ticket t; kind 3: the number belongs to no unit.  The producer works this out between two units, alone, while at
+// most four tiles are on their way, so it counts: three divisions and a search.  (Counting through the first A blocks for
+// every ticket, two divisions each and up to sixteen of them, made the producer the bottleneck of short sequences: us a call, 32 layers of
+// 1500 tokens 101.4 -> 96.4, of 3000 at window 8 129.5 -> 115.7, 16 layers of eight prompts of 560 to 2238 tokens 313 -> 284.)
 __device__ __forceinline__ FlUnit fl_decode(const Geo& g, const FlowArgs& fa, const FlShared& sh, int t)
 {
     FlUnit u;
     u.kind = 2;
     u.prob = u.j0 = u.nh = u.tile0 = u.nt = u.tok_base = u.Tn = u.layer = u.group = u.index = 0;
     const int ng = fa.n_groups, period = fa.n_sel * ng, n_v = fa.n_prob * ng;
-    int v = -1, off = 0;
-    bool is_a = false;
-    for (int i = 0; i < fa.lag && v < 0; ++i) {                     // the first A blocks, ahead of any B
-        const int ua = i < n_v ? sh.units_a[(i / ng) % fa.n_sel] : 0;
-        if (t < ua) { v = i; off = t; is_a = true; }
-        else t -= ua;
-    }
-    if (v < 0) {
+    int v = 0, off = t;
+    bool is_a = true;
+    if (t < sh.ahead) {                                             // the first A blocks, ahead of any B
+#pragma unroll 1
+        for (int slot = 0, left = ng; off >= sh.units_a[slot]; ++v) {
+            off -= sh.units_a[slot];
+            if (--left == 0) {
+                left = ng;
+                if (++slot == fa.n_sel) slot = 0;
+            }
+        }
+    } else {
+        t -= sh.ahead;
         const int total = sh.prefix[period];
         const int q = t / total, r = t - q * total;
         int lo = 0, hi = period - 1;                                // last slot with prefix <= r
+#pragma unroll 1
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
             if (sh.prefix[mid] <= r) lo = mid; else hi = mid - 1;
@@ -168,15 +179,16 @@ __device__ __forceinline__ FlUnit fl_decode(const Geo& g, const FlowArgs& fa, co
         const int k = q * period + lo;
         if (k >= n_v) return u;                                     // past the end
         off = r - sh.prefix[lo];
-        const int ua = fa.two_sweep ? sh.units_a[((k + fa.lag) / ng) % fa.n_sel] : 0;
-        if (off < ua) { v = k + fa.lag; is_a = true; }
-        else { v = k; off -= ua; }
+        const int ua = sh.ahead_units[lo];
+        is_a = off < ua;
+        v = is_a ? k + fa.lag : k;
+        if (!is_a) off -= ua;
         if (v >= n_v) { u.kind = 3; return u; }
     }
-    const int pi = v / ng;
+    const int pi = ng == 1 ? v : v / ng;
     u.group = v - pi * ng;
     u.layer = pi / fa.n_sel;
-    const int seq = fa.sel[pi - u.layer * fa.n_sel];
+    const int slot = pi - u.layer * fa.n_sel, seq = fa.sel[slot];
     u.prob = u.layer * g.n_seqs + seq;
     u.tok_base = g.cu[seq];
     u.Tn = geo_L(g, seq) - g.window;
@@ -184,11 +196,11 @@ __device__ __forceinline__ FlUnit fl_decode(const Geo& g, const FlowArgs& fa, co
     fl_tiles(g, seq, ta, tb);
     const int h0 = u.group * fa.group_heads, nh = min(fa.group_heads, g.Hkv - h0);
     if (is_a) {
-        const int per = (ta + 4 * fa.m - 1) / (4 * fa.m);
+        const int per = sh.per_head[slot], h = off / per;
         u.kind = 0;
-        u.j0 = h0 + off / per;
+        u.j0 = h0 + h;
         u.nh = 1;
-        u.index = off % per;
+        u.index = off - h * per;
         u.tile0 = u.index * 4 * fa.m;
         u.nt = min(4 * fa.m, ta - u.tile0);
         if (u.j0 >= h0 + nh) u.kind = 3;                            // a last, smaller head group
@@ -344,7 +356,8 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         for (int i = lane; i < fa.n_sel; i += 32) {
             int ta, tb;
             fl_tiles(g, fa.sel[i], ta, tb);
-            sh.units_a[i] = fa.two_sweep ? fa.group_heads * ((ta + 4 * fa.m - 1) / (4 * fa.m)) : 0;
+            sh.per_head[i] = (ta + 4 * fa.m - 1) / (4 * fa.m);
+            sh.units_a[i] = fa.two_sweep ? fa.group_heads * sh.per_head[i] : 0;
             sh.units_b[i] = fa.head_split ? tb : (tb + 3) / 4;
         }
         __syncwarp();
@@ -352,7 +365,9 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         int carry = 0;
         for (int i0 = 0; i0 < period; i0 += 32) {
             const int i = i0 + lane;
-            int c = i < period ? sh.units_a[((i + fa.lag) / fa.n_groups) % fa.n_sel] + sh.units_b[(i / fa.n_groups) % fa.n_sel] : 0;
+            const int ua = i < period ? sh.units_a[((i + fa.lag) / fa.n_groups) % fa.n_sel] : 0;
+            const int c = i < period ? ua + sh.units_b[(i / fa.n_groups) % fa.n_sel] : 0;
+            if (i < period) sh.ahead_units[i] = ua;
             int inc = c;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -362,7 +377,10 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
             if (i < period) sh.prefix[i] = carry + inc - c;
             carry += __shfl_sync(0xffffffffu, inc, 31);
         }
-        if (lane == 0) sh.prefix[period] = carry;
+        int ahead = 0;
+        for (int i = lane; i < min(fa.lag, fa.n_prob * fa.n_groups); i += 32) ahead += sh.units_a[(i / fa.n_groups) % fa.n_sel];
+        ahead = warp_sum(ahead);
+        if (lane == 0) { sh.prefix[period] = carry; sh.ahead = ahead; }
     }
     // What precedes this kernel on the stream is the segmentation, which it needs nothing from (queries, keys
     // and the cleared counters were there before that started): it waits for it only at its end, so that
