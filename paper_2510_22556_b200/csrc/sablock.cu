@@ -547,15 +547,21 @@ sablock_status_t run_flow(const Plan& pl, const sablock_params_t* p, const CUten
     fa.n_prob = g.n_layers * fa.n_sel;
     fa.group_heads = pl.fl_heads; fa.n_groups = pl.fl_groups;
     fa.m = pl.fl_m;
-    // A units run ahead of the B units of the same (problem, head group) by about a unit per SM: enough that the row sums
-    // are there in time (what is late is put aside), little enough that the keys are still in L2
     const int sms = sm_count();
-    const long long ua = tiles * fa.group_heads / (4LL * fa.m * fa.n_sel) + 1;       // on average
-    fa.lag = fa.two_sweep ? (int)fmin(16.0, (double)((sms + ua - 1) / ua)) : 0;
     // four tiles per B unit, or one with the heads spread over the sets where that takes fewer rounds
     units_b *= g.n_layers;
     const long long rounds = (units_b + sms - 1) / sms * fa.group_heads * 4, split = (units_b * 4 + sms - 1) / sms * (fa.group_heads + 1);
     fa.head_split = fa.n_groups == 1 && fa.group_heads >= 4 && split < rounds;
+    // A units run ahead of the B units of the same (problem, head group) by about a unit per SM: enough that the row sums
+    // are there in time, little enough that the keys are still in L2.  A unit of four tiles (20 us) that is early waits where it
+    // is, its products made: a CTA that had put two of them aside was still busy when all others were done.  Units of one
+    // tile take a quarter of that; two may be put aside, and A units run ahead by two per SM.  Two sweeps, 32 / 8 heads of
+    // 128, us a call: 16 layers of 4096 tokens 123 -> 108, 32 of 4211 226 -> 216, 32 of 16 prompts of 4K to 16K 4581 -> 4373; units of
+    // one tile, 32 layers of 1500 tokens 96 -> 89, 8 of nine prompts of up to 2214 176 -> 161.
+    const long long ua = tiles * fa.group_heads / (4LL * fa.m * fa.n_sel) + 1;       // on average
+    const int ahead = fa.head_split ? 2 * sms : sms, most = fa.head_split ? 64 : 16;
+    fa.lag = fa.two_sweep ? (int)fmin((double)most, (double)((ahead + ua - 1) / ua)) : 0;
+    fa.max_aside = fa.head_split ? 2 : 0;
     SAB_TRY(allow_smem<score_flow_tc<W, D>>(fl_smem(D)));
     SAB_TRY(launch(score_flow_tc<W, D>, dim3(sms), kFlThreads, fl_smem(D), stream, 1, tmQ, tmK, g, fa));
     prof_mark(1, stream);

@@ -10,7 +10,7 @@
 // A B unit needs the log-sum-exps of its problem, i.e. A units with smaller numbers: whoever holds those
 // is running, so waiting for them always ends and no CTA has to be resident for another's sake.  The
 // order is A(v + lag), B(v) for v = 0, 1, ...: by the time a B unit is handed out the A units it needs are
-// done or nearly so (a CTA puts a B unit that is early aside and goes on with A units), and as little more
+// done or nearly so (one that is early waits; small ones are put aside while A units go on), and as little more
 // as possible has been read since, so that the keys of a problem of up to about 48 MB are read from L2 the
 // second time.  v counts (problem, group of KV heads); a group is as many heads as have room for their
 // log-sum-exps (1024 window rows), for the usual shapes all of them.  With the row log-sum-exps given there
@@ -69,6 +69,7 @@ struct FlowArgs {
     int group_heads, n_groups;
     int m;                   // A units: tiles per set
     int lag;
+    int max_aside;           // B units that a CTA puts aside: two, or none
     int head_split;          // B units of one tile, the sets share the heads
     float* s_out;
     float* e_out;
@@ -405,7 +406,7 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         uint32_t ks = 0, kpar = 1, qs = 0, qpar = 1;             // next stages and the parities of their last release
         int nu = 0;
         bool ok = true, drained = false;
-        // A B unit whose log-sum-exps are not there yet is put aside (two at most) while A units, which
+        // A B unit whose log-sum-exps are not there yet is put aside (two at most, where units are small) while A units, which
         // wait for nothing, go first.
         FlUnit pend[2];
         int n_pend = 0;
@@ -415,7 +416,7 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         while (ok) {
             FlUnit u;
             bool have = false;
-            if (n_pend > 0 && (drained || n_pend == 2 || ready(pend[0]))) {
+            if (n_pend > 0 && (drained || n_pend == fa.max_aside || ready(pend[0]))) {
                 u = pend[0];
                 pend[0] = pend[1];
                 --n_pend;
@@ -431,7 +432,7 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                     u = fl_decode(g, fa, sh, uniform(t));
                     if (u.kind == 2) { drained = true; continue; }
                     if (u.kind == 3) continue;
-                    if (u.kind == 1 && (n_pend > 0 || !ready(u))) {
+                    if (u.kind == 1 && fa.max_aside > 0 && (n_pend > 0 || !ready(u))) {
                         if (n_pend == 0) pend[0] = u; else pend[1] = u;
                         ++n_pend;
                         continue;
