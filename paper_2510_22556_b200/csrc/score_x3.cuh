@@ -353,19 +353,28 @@ score_x3_sum(const Geo g, const float* __restrict__ x, int ld, float eps, const 
     const int hs = W >= n_warps ? 1 : n_warps / W;     // shares of the heads
     for (int i = threadIdx.x; i < H * W; i += blockDim.x) ls[i] = lse2[(size_t)p * H * W + i];
     __syncthreads();
-    const float* xp = x + (size_t)p * H * W * ld + t0 + lane;
+    // (32-bit positions: 64 MB of logits at most)
+    const float* xp = x + (size_t)p * H * W * ld;
     for (int item = warp; item < W * hs; item += n_warps) {
         const int w = item % W, share = item / W;
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        const size_t step = (size_t)hs * W * ld;
-        const float* row = xp + (size_t)(share * W + w) * ld;
+        const unsigned step = (unsigned)(hs * W * ld), rows = (unsigned)(hs * W);
+        unsigned at = (unsigned)((share * W + w) * ld + t0 + lane);
         const float* lh = ls + share * W + w;
-        for (int n = (H - share + hs - 1) / hs; n > 0; n -= 16, row += 16 * step, lh += 16 * hs * W) {   // heads of the share, sixteen loads in flight
+        int n = (H - share + hs - 1) / hs;           // heads of the share, sixteen loads in flight
+        for (; n >= 16; n -= 16, at += 16 * step, lh += 16 * rows) {
             float v[16];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) v[u] = __ldg(row + min(u, n - 1) * step);
+            for (unsigned u = 0; u < 16; ++u) v[u] = __ldg(xp + (at + u * step));
 #pragma unroll
-            for (int u = 0; u < 16; ++u) acc[u & 3] += u < n ? exp2f(v[u] - lh[min(u, n - 1) * hs * W]) : 0.f;
+            for (unsigned u = 0; u < 16; ++u) acc[u & 3] += exp2f(v[u] - lh[u * rows]);
+        }
+        if (n > 0) {
+            float v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[u] = __ldg(xp + (at + (unsigned)min(u, n - 1) * step));
+#pragma unroll
+            for (int u = 0; u < 16; ++u) acc[u & 3] += u < n ? exp2f(v[u] - lh[(unsigned)min(u, n - 1) * rows]) : 0.f;
         }
         ab[item][lane] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     }
