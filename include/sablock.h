@@ -45,11 +45,13 @@ typedef enum {
 typedef enum { SABLOCK_F32 = 0, SABLOCK_BF16 = 1 } sablock_dtype_t;
 
 /* Which kernel family computes the attention scores.  AUTO picks, for bf16, head_dim 64/128, window
- * 8/16/32 and at most 128 window rows per KV head, the unit-flow tensor-core kernel, except for two sweeps
+ * 8/16/32 and at most 128 window rows per KV head, the unit-flow tensor-core kernel (short prompts: two
+ * kernels of small CTAs in its place), except for two sweeps
  * (row_lse not given) over more than 48 MB of keys per sequence and layer in the shape of the persistent
  * tensor-core kernel (head_dim 128, window 32, four query heads per KV head, at most 7 token tiles of 128
- * per CTA), which takes those; everything else runs on the SIMT kernels (with row_lse these run their
- * second pass only).  FUSED forces the persistent kernel, TENSOR the two-launch tensor-core kernels; both
+ * per CTA), which takes those.  For fp32, head_dim 64/128, window up to 32, at most 128 window rows per KV
+ * head, rows on 16-byte boundaries and at most 64 MB of logits: tensor-core kernels on operands split into three bf16
+ * pieces.  Everything else runs on the SIMT kernels (with row_lse these run their second pass only).  FUSED forces the persistent kernel, TENSOR the two-launch tensor-core kernels; both
  * fail with SABLOCK_ERR_UNSUPPORTED where they cannot run. */
 typedef enum { SABLOCK_SCORE_AUTO = 0, SABLOCK_SCORE_SIMT = 1, SABLOCK_SCORE_TENSOR = 2, SABLOCK_SCORE_FUSED = 3 }
     sablock_score_impl_t;
@@ -147,7 +149,9 @@ sablock_status_t sablock_read_status(const void *ws, sablock_stream_t stream, in
  * loaded, 6 row sums of a phase in shared memory, 7 accumulator complete, 8 log-sum-exps fetched,
  * 9 turn at the exponentials, 11 partial-sum slot free, 12 row sums of all CTAs, 13 merged
  * log-sum-exps, 20 / 21 exchanges inside the epilogue, 22 the other epilogue set's previous step; in the
- * unit flow also 11 row sums taken, 14 / 15 / 17 a unit posted, 16 log-sum-exps taken, 18 / 19 carry of a tile, 21 unit record free), 30 the CTAs of a sequence in the segmentation,
+ * unit flow also 11 row sums taken, 14 / 15 / 17 a unit posted, 16 log-sum-exps taken, 18 / 19 carry of a tile, 21 unit record free; in the kernels for short
+ * prompts 10 products complete, 27 operands loaded; in those for fp32 23 products of a tile complete, 24 stage free, 25 accumulators
+ * free, 26 stage filled), 30 the CTAs of a sequence in the segmentation,
  * 31 the CTAs of one problem in the selection.  Every such wait is limited to about a second of
  * device time; the kernel that gave up returns, the later stages still run on whatever was
  * produced and stay inside their buffers. */

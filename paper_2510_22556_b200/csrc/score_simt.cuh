@@ -1,5 +1,5 @@
-// Stage 2 with plain fp32 FMAs (any head_dim / window the tensor-core kernels do not take,
-// and fp32 inputs).  Two sweeps over K: pass 1 produces the log-sum-exp of every window
+// Stage 2 with plain fp32 FMAs (any head_dim / window the tensor-core kernels do not take, fp32 inputs
+// among them, and fp32 calls of more than 64 MB of logits).  Two sweeps over K: pass 1 produces the log-sum-exp of every window
 // row (h, w) over its causal keys (Eq. 2), pass 2 recomputes the logits, normalises, and
 // reduces over heads and window positions per token (Eqs. 3, 4 and the inner sum of Eq. 6).
 // Logits are kept in log2 units: x2 = (q . k) * log2(e) / sqrt(D).
