@@ -10,7 +10,8 @@
 //
 // What it replaces for these shapes computed the logits twice on multiply-adds, bounded by the 128 bytes per cycle at which
 // shared memory fills registers.  Here a layer's logits (4096 tokens, 32 heads of 128, window 32: 17 MB) stay in L2 between the
-// two kernels, and six products per tile take 1.6 us of an SM.
+// two kernels, and six products per tile take 1.6 us of an SM: 42 + 47 us there, 15 + 7 here, a call 121 -> 48.  Below that the
+// first kernel is latency: a CTA has two tiles there, after 4 us of loading and splitting, and the last to arrive merges.
 #pragma once
 #include "common.cuh"
 #include "score_fused.cuh"
@@ -25,7 +26,7 @@ constexpr int kX3Piece = 128 * 128;                  // one piece of 128 rows x 
 constexpr int kX3MaxW = 32;
 constexpr size_t kX3MaxBytes = 64u << 20;            // logits of a call that this path takes: about half of L2
 constexpr int kX3SumThreads = 1024;                  // half of that for fewer window rows in all than
-constexpr int kX3SumManyRows = 512;                  // (4096 tokens, 1024 rows: 52.8 -> 47.7 us a call; 5000 tokens, 64 rows: 39.3 -> 43.6)
+constexpr int kX3SumManyRows = 512;                  // (512 / 1024 threads: 4096 tokens, 1024 rows 52.8 / 47.7 us a call; 5000, 64 rows 39.3 / 43.6)
 constexpr int kX3SumTokens = 32;                     // tokens of a CTA of the second kernel
 __host__ __device__ constexpr int x3_smem(int D) { return 1024 + (D / 64 + 2) * 3 * kX3Piece; }
 
