@@ -39,7 +39,8 @@ __device__ __forceinline__ void note_giveup(int* status, int code)
 // its post so that the waiting side runs into its limit.  bit 0: CTA 1 of a segmentation cluster never
 // reports its count; bit 1: CTA 0 of every selection cluster never reports its first digit counts; bit
 // 2: CTA 0 of the persistent score kernel never reports its row sums of phase 0, the first unit of the
-// unit flow not its own, the first CTA of score_rows_tc not its products.
+// unit flow not its own, the first CTA of score_rows_tc not its products, that of score_x3_logits not those of its first tile;
+// bit 3: the first CTA of score_heads_tc never reports its products, a warp of that of score_x3_logits not its first keys.
 // Production builds compile none of this.
 #ifdef SABLOCK_TEST_HOOKS
 __device__ int g_test_hooks;

@@ -109,7 +109,7 @@ __device__ __forceinline__ void pr_products(PairShared& sh, const CUtensorMap& t
             if (elect_one()) {
                 fl_issue<D>(sh.tmem_base + (uint32_t)i * 128u, kRows ? q_at : k_lo, kRows ? k_lo : q_at,
                             umma_idesc_bf16(128, kRows ? 128 : RN));
-                if (!(SAB_HOOK(2) && kRows && blockIdx.x + blockIdx.y + blockIdx.z == 0)) tc_commit(smem_u32(&sh.tfull[i]));
+                if (!(SAB_HOOK(kRows ? 2 : 3) && blockIdx.x + blockIdx.y + blockIdx.z == 0)) tc_commit(smem_u32(&sh.tfull[i]));
             }
             __syncwarp();
         }

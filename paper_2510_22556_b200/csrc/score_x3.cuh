@@ -52,6 +52,7 @@ struct X3Shared {
     float2 red[128];
 };
 
+// (All waits are those of whole warps: the lanes of one that gives up all leave, and none of them goes on to tensor memory alone.)
 #define X3_WAIT(code, expr) ((expr) ? true : (note_giveup(a.status, code), false))
 
 // Eight numbers as three pieces of eight bf16 numbers each: x = hi + mid + lo exactly (the differences are exact).
@@ -124,6 +125,7 @@ score_x3_logits(const Geo g, const X3Args a)
         pdl_wait();
         return;
     }
+    [[maybe_unused]] const bool first = chunk + j + p == 0;
     volatile int* abort_flag = &sh.abort_flag;
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -168,7 +170,8 @@ score_x3_logits(const Geo g, const X3Args a)
         bool ok = true;
         auto read_back = [&](int t) {
             const int b = t & 1, t0 = (tile0 + t) * kTcTile + col_half;
-            if (!X3_WAIT(23, mbar_wait(smem_u32(&sh.tfull[b]), (uint32_t)((t >> 1) & 1), abort_flag))) { ok = false; return; }
+            if (!X3_WAIT(23, mbar_wait_warp(smem_u32(&sh.tfull[b]), (uint32_t)((t >> 1) & 1), abort_flag))) { ok = false; return; }
+            __syncwarp();
             tc_fence_after();
             float* dst = a.x + ((size_t)p * g.H * W + (size_t)j * R + row) * a.ld + t0;
             const int lim = Tn + row % W - t0;       // causal (Eq. 2): columns up to here are visible
@@ -234,13 +237,14 @@ score_x3_logits(const Geo g, const X3Args a)
             }
         for (int st = 0; st < n_stage && ok; ++st) {
             const int b = st & 1;
-            if (!X3_WAIT(24, mbar_wait(smem_u32(&sh.empty[b]), (uint32_t)(((st >> 1) & 1) ^ 1), abort_flag))) { ok = false; break; }
+            if (!X3_WAIT(24, mbar_wait_warp(smem_u32(&sh.empty[b]), (uint32_t)(((st >> 1) & 1) ^ 1), abort_flag))) { ok = false; break; }
+            __syncwarp();
             uint8_t* dst = kbuf + b * 3 * kX3Piece;
 #pragma unroll
             for (int i = 0; i < 4; ++i) x3_store(dst, r8 + 32 * i, c8, v[2 * i], v[2 * i + 1]);
             fence_proxy_async();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sh.full[b]));
+            if (lane == 0 && !(SAB_HOOK(3) && first && st == 0 && warp == 0)) mbar_arrive(smem_u32(&sh.full[b]));
             if (st + 1 < n_stage) load(st + 1);
             if ((st + 1) % kHalves == 0 && st >= kHalves) read_back(st / kHalves - 1);
         }
@@ -275,7 +279,7 @@ score_x3_logits(const Geo g, const X3Args a)
                                     step > 0 ? 1u : 0u);
                     }
                     tc_commit(smem_u32(&sh.empty[b]));
-                    if (hf == kHalves - 1) tc_commit(smem_u32(&sh.tfull[tb]));
+                    if (hf == kHalves - 1 && !(SAB_HOOK(2) && first && t == 0)) tc_commit(smem_u32(&sh.tfull[tb]));
                 }
                 __syncwarp();
             }

@@ -17,7 +17,7 @@ from paper_2510_22556_b200.build import build_test_hooks
 pytestmark = pytest.mark.gpu
 
 TIMEOUT = 5          # SABLOCK_ERR_TIMEOUT
-HOOK_SEGMENT, HOOK_TOPB, HOOK_SCORE = 1, 2, 4
+HOOK_SEGMENT, HOOK_TOPB, HOOK_SCORE, HOOK_SCORE2 = 1, 2, 4, 8
 
 
 @pytest.fixture(scope="module")
@@ -131,6 +131,42 @@ def test_unit_flow_gives_up(hooked, H, Hkv, D, W, lens, layers):
     code, raw, where = B.read_status_detail(ws)
     assert code == TIMEOUT and raw & 1
     assert 1 <= _code(where) <= 21
+    for i, L in enumerate(lens):
+        idx = out.out_idx[:, i].cpu().numpy()
+        assert ((idx >= 0) & (idx < L)).all()
+    hooked.sablock_test_set_hooks(0)
+    out = B.compress_layers(*args)
+    torch.cuda.synchronize()
+    assert B.read_status_detail(ws) == (0, 0, 0) and torch.equal(out.out_idx, good)
+
+
+@pytest.mark.parametrize("hook,dtype,H,Hkv,D,W,lens,layers,lse,codes", [
+    (HOOK_SCORE, "f32", 32, 8, 128, 32, [4096], 1, False, [23]),          # products of a tile that are never reported
+    (HOOK_SCORE, "f32", 4, 1, 64, 16, [512, 900], 2, False, [23]),
+    (HOOK_SCORE, "f32", 32, 8, 128, 32, [6000], 1, True, [23]),
+    (HOOK_SCORE2, "f32", 32, 8, 128, 32, [4096], 1, False, [23, 24, 26]),  # keys that are never handed over
+    (HOOK_SCORE2, "f32", 4, 1, 64, 16, [512], 1, False, [23, 24, 26]),
+    (HOOK_SCORE2, "f32", 32, 8, 128, 8, [5000], 3, False, [23, 24, 26]),
+    (HOOK_SCORE, "bf16", 32, 8, 128, 32, [8192], 1, False, [10]),         # short prompts: row sums,
+    (HOOK_SCORE2, "bf16", 32, 8, 128, 32, [8192], 1, False, [10]),        # and sums over the heads
+    (HOOK_SCORE2, "bf16", 4, 1, 64, 16, [900, 700], 1, True, [10])])
+def test_short_prompt_and_fp32_kernels_give_up(hooked, hook, dtype, H, Hkv, D, W, lens, layers, lse, codes):
+    cfg = synth.Config("t", layers, H, Hkv, D, W, tuple(lens), (256,), (1, 2, 4), dtype, 5000, 8, 2.0, 20, (0.4,), 9)
+    b = synth.make_batch(cfg, device="cuda")
+    kw = dict(row_lse=synth.prefill_row_lse(b.q_win, b.k, b.cu_seqlens)) if lse else {}
+    p = B.make_params(H, Hkv, D, W, synth.torch_dtype(dtype), b.bitmap, cfg.vocab, **kw)
+    ws = B.alloc_workspace(p, b.cu_seqlens[-1], max(lens), len(lens), layers)
+    args = (p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, 256, cfg.candidates, ws)
+    out = B.compress_layers(*args)
+    torch.cuda.synchronize()
+    assert B.read_status_detail(ws) == (0, 0, 0)
+    good = out.out_idx.clone()
+    assert hooked.sablock_test_set_hooks(hook) == 0
+    out = B.compress_layers(*args)
+    torch.cuda.synchronize()                                  # every role of every CTA left its loop
+    code, raw, where = B.read_status_detail(ws)
+    assert code == TIMEOUT and raw & 1
+    assert _code(where) in codes
     for i, L in enumerate(lens):
         idx = out.out_idx[:, i].cpu().numpy()
         assert ((idx >= 0) & (idx < L)).all()
