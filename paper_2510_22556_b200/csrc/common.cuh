@@ -13,6 +13,7 @@ namespace sab {
 
 constexpr int kMaxSeqs = SABLOCK_MAX_SEQS;
 constexpr int kMaxCand = SABLOCK_MAX_CANDIDATES;
+constexpr int kSmSharedBytes = 228 * 1024;   // shared memory of an SM, of which every resident CTA takes 1024 bytes beside its own
 
 // Device status word bits.
 constexpr int kStatTimeout = 1;    // a bounded wait ran out

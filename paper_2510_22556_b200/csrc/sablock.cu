@@ -1212,6 +1212,10 @@ int sablock_test_simt_smem(const sablock_params_t* p, int max_L, int n_layers)
     return pl.use_tc ? 0 : pl.simt.smem;
 }
 
+// Dynamic shared memory of a CTA of the kernels for short prompts, and the CTAs of an SM that tensor memory has room for (host only).
+int sablock_test_pair_smem(int head_dim) { return pr_smem(head_dim); }
+int sablock_test_pair_ctas() { return 512 / kPrTmemCols; }
+
 // The problem that a problem of a flow launch waits for before it writes the carry of a tile (host only).
 int sablock_test_carry_tenant(int n_seqs, const int* cu, int window, int n_out, int index, int tile)
 {

@@ -28,7 +28,14 @@ constexpr int kPrMaxHeads = 8;                       // KV heads: CTAs of a clus
 // layer of 8K, 12K, 16K and 18K tokens, four of 8K).  One sweep: 41.7 / 38.4, 42.4 / 44.4, 43.1 / 50.2.
 __host__ __device__ constexpr int pr_max_ctas(bool two_sweep) { return two_sweep ? 3 : 2; }
 constexpr int kPrTmemCols = kPrTiles * 128;
-__host__ __device__ constexpr int pr_smem(int D) { return 1024 + (1 + kPrTiles) * 128 * D * 2; }
+// Shared memory of a CTA: its operands, and never so little that an SM could take three.  Tensor memory has room for two; a third CTA
+// would wait for its columns while its cluster's CTAs on other SMs wait for it, and hold the columns there that a third one waits for.
+__host__ __device__ constexpr int pr_smem(int D)
+{
+    const int operands = 1024 + (1 + kPrTiles) * 128 * D * 2, third = kSmSharedBytes / 3;
+    return operands > third ? operands : third;
+}
+static_assert(2 * kPrTmemCols <= 512, "two CTAs of an SM have their accumulators");
 
 struct PairArgs {
     float c2, eps;

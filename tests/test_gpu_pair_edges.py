@@ -20,3 +20,11 @@ def test_pair_lengths(H, Hkv, D, W, L, lse):
 @pytest.mark.parametrize("lse", [False, True])
 def test_pair_packed_and_its_limit(lens, n_layers, lse):
     _run(32, 8, 128, 32, lens, n_layers, 64, lse)
+
+
+@pytest.mark.parametrize("H,Hkv,W,lens,n_layers", [(32, 8, 32, [7900], 1), (32, 8, 8, [2000], 4), (32, 8, 32, [13000], 1), (16, 4, 16, [4000, 900], 3),
+                                                   (8, 2, 32, [16000], 1)])
+@pytest.mark.parametrize("lse", [False, True])
+def test_pair_with_rows_of_64_fills_the_device(H, Hkv, W, lens, n_layers, lse):
+    """More CTAs than SMs, which the operands alone would let an SM take four of."""
+    _run(H, Hkv, 64, W, lens, n_layers, 64, lse)

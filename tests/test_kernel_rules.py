@@ -128,3 +128,12 @@ def test_a_limit_is_never_lowered_by_another_thread(rules):
     failing = C.CFUNCTYPE(C.c_int, C.c_int)(lambda n: 1)
     assert rules.sablock_test_raise_limit(200, failing) == 1     # a refusal is passed on and not remembered
     assert rules.sablock_test_raise_limit(200, setter) == 0 and now[0] == 200
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_an_sm_takes_no_more_short_prompt_ctas_than_it_has_tensor_memory_for(rules, D):
+    """228 KB of shared memory per SM, 1 KB of it for every resident CTA beside what the CTA asks for: as many CTAs as have their
+    accumulators fit, and not one more, whatever registers the compiler takes."""
+    n, most = rules.sablock_test_pair_smem(D), rules.sablock_test_pair_ctas()
+    static = 5120                                                # barriers, row sums, log-sum-exps, sums of a warp: 4.7 KB
+    assert most * (n + static + 1024) <= 228 * 1024 < (most + 1) * (n + 1024)
