@@ -981,6 +981,7 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
     const long long per_split = (long long)p->n_kv_heads * n_prob;
     dp->cluster = false;
     long long splits;
+    size_t need = 0;
     auto scratch = [&](long long n) { return align_up(sizeof(float) * (size_t)n_prob * p->n_q_heads * n * (p->head_dim + 2)); };
     if (p->dtype == SABLOCK_BF16) {
         // One wave of two CTAs per SM, at least 64 rows (one chunk per warp) each.  Up to eight splits
@@ -992,6 +993,10 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
         const long long by_rows = (n_rows + 63) / 64;
         if (splits > by_rows) splits = by_rows;
         if (splits < 1) splits = 1;
+        // Scratch that is asked for: that of the splits, where they are more than a cluster of the longest cache that always has
+        // one.  (A single split more goes to a cluster too and needs none, but a caller sizes its scratch for the largest batch, and
+        // as the batch shrinks the splits of the others become more: what a batch of nine splits asks for serves them.)
+        need = splits <= kDecMaxCluster || n_rows <= kDecClusterRows ? 256 : scratch(splits);
         if (splits <= kDecClusterSplits || n_rows <= dec_cluster_rows(row_bytes) ||
             (n_rows <= kDecClusterRows && ws_bytes < scratch(splits))) {
             dp->cluster = true;
@@ -1009,8 +1014,8 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
     if (splits > kDecMaxSplits) splits = kDecMaxSplits;
     dp->n_splits = (int)splits;
     dp->rows_per_split = (int)((n_rows + splits - 1) / splits);
-    // the scratch of the clustered form is none; a caller's buffer may not be empty
-    dp->bytes = dp->cluster ? 256 : scratch(splits);
+    // (the scratch of the clustered form is none; a caller's buffer may not be empty)
+    dp->bytes = dp->cluster ? need : scratch(splits);
     return SABLOCK_OK;
 }
 

@@ -169,3 +169,26 @@ def test_workspace_regions(lib):
     ws = torch.zeros(total, dtype=torch.uint8)
     v = B.workspace_view(p, ws, "s_refined", 20000, 8192, 3, 2)
     assert v.shape == (2, 20000) and v.dtype == torch.float32
+
+
+@pytest.mark.parametrize("H,Hkv,D", [(32, 8, 128), (4, 2, 128), (16, 8, 64), (16, 4, 256), (7, 7, 128)])
+@pytest.mark.parametrize("n_rows", [8193, 16384, 131072])
+def test_decode_scratch_of_a_batch_serves_a_smaller_one(lib, H, Hkv, D, n_rows):
+    """What a batch asks for is the partial results of its row splits (two CTAs on each of 148 SMs) where they are more than
+    eight: as sequences finish, batches of 2 / 3 of the size and half of it fit what the whole one asked for."""
+    p = B.make_params(H, Hkv, D, 8, torch.bfloat16)
+    fake = C.c_void_p(256)
+
+    def need(n_prob):
+        return int(lib.sablock_decode_workspace_bytes(C.addressof(p), n_prob, n_rows))
+
+    def call(n_prob, nb):
+        return lib.sablock_decode_attention(C.addressof(p), n_prob, None, fake, fake, n_rows, None, fake, None, fake, nb, None)
+
+    for n_prob in range(1, 40):
+        splits = min(296 // (Hkv * n_prob), -(-n_rows // 64))
+        want = 256 if splits <= 8 else -(-4 * n_prob * H * splits * (D + 2) // 256) * 256
+        assert need(n_prob) == want
+    if Hkv == 8:
+        assert need(4) >= need(3) and need(4) >= need(2)
+    assert call(1, 1 << 30) == 1                                 # (no queries: refused before anything is launched)
