@@ -20,10 +20,23 @@ constexpr int kDecMaxSplits = 512;
 constexpr int kDecMaxD = 256;
 constexpr int kDecMaxG = 4;
 constexpr int kDecClusterRows = 8192;
-// Rows up to which eight splits in a cluster beat as many splits as the device has room for and a second launch, one problem of
-// 8 KV heads (us a layer, cluster / two launches): rows of 256 bytes, 4096 9.7 / 10.5, 6144 12.0 / 12.0, 8192 14.1 / 13.2;
-// rows of 128 bytes, 4096 6.9 / 6.4, 8192 10.5 / 9.0.
-__host__ __device__ constexpr int dec_cluster_rows(int row_bytes) { return row_bytes <= 128 ? 3072 : 6144; }
+// Whether a cache of at most kDecClusterRows rows is better off with as many splits as the device has room for and a second launch
+// than with clusters of eight: long ones are, where the clusters leave most of the device idle, or where there are so many that
+// some CTAs share an SM (wait for one, with rows of 512 bytes) and others have one to themselves.  us for eight layers of 8192 rows
+// launched one after the other, cluster / two launches, by clusters (problems x KV heads):
+//   rows of 256 bytes  1: 109 / 98, 8: 117 / 109, 9: 118 / 108, 10: 119 / 121, 12: 122 / 126, 15: 125 / 138, 16: 151 / 146, 18: 158 / 153,
+//                      20: 159 / 171, 24: 168 / 182, 32: 205 / 225; of 6144 rows 1: 92 / 98, 8: 100 / 101, 12: 103 / 114, 18: 133 / 127
+//   rows of 512 bytes  1: 172 / 97, 3: 174 / 156, 4: 175 / 159, 6: 177 / 177, 8: 180 / 194, 15: 197 / 249, 16: 362 / 262, 24: 370 / 337
+//   rows of 128 bytes  1: 82 / 101, 8: 90 / 98, 12: 93 / 99, 16: 105 / 104, 24: 111 / 118: the second launch costs the host 2.5 us, as
+//                      much as the kernel gains
+constexpr int kDecShortRows = 6144;
+constexpr int kDecLoneClusters = 15;                 // clusters of eight that have an SM for every CTA
+__host__ __device__ constexpr bool dec_two_launches(int row_bytes, int n_rows, long long clusters, int sms)
+{
+    if (row_bytes <= 128 || n_rows <= kDecShortRows) return false;
+    if (clusters * (row_bytes <= 256 ? 16 : 36) <= sms) return true;
+    return clusters > kDecLoneClusters && (row_bytes > 256 || clusters * 8 <= sms);
+}
 constexpr int kDecClusterSplits = 9;                 // four problems, 9 splits: 4096 rows 15.1 / 17.1, 8192 25.0 / 27.4, 16384 47.0 / 48.6
 constexpr int kDecMaxCluster = 8;                    // CTAs that merge through distributed shared memory
 

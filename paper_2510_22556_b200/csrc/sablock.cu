@@ -986,8 +986,8 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
     if (p->dtype == SABLOCK_BF16) {
         // One wave of two CTAs per SM, at least 64 rows (one chunk per warp) each.  Up to eight splits
         // are a cluster that merges on chip.  Beyond that a short cache still goes to clusters of
-        // eight, and so does one that would have a single split more: the rows that a CTA then reads more take less time
-        // than the second launch and the trip through scratch (dec_cluster_rows: where the two cost the same).  And a
+        // eight (dec_two_launches: which do not), and so does one that would have a single split more: the rows that a CTA then
+        // reads more take less time than the second launch and the trip through scratch.  And a
         // cache of at most kDecClusterRows whose caller has brought no scratch for the other form.
         splits = 2LL * sm_count() / per_split;
         const long long by_rows = (n_rows + 63) / 64;
@@ -997,8 +997,8 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
         // one.  (A single split more goes to a cluster too and needs none, but a caller sizes its scratch for the largest batch, and
         // as the batch shrinks the splits of the others become more: what a batch of nine splits asks for serves them.)
         need = splits <= kDecMaxCluster || n_rows <= kDecClusterRows ? 256 : scratch(splits);
-        if (splits <= kDecClusterSplits || n_rows <= dec_cluster_rows(row_bytes) ||
-            (n_rows <= kDecClusterRows && ws_bytes < scratch(splits))) {
+        if (splits <= kDecClusterSplits ||
+            (n_rows <= kDecClusterRows && (!dec_two_launches(row_bytes, n_rows, per_split, sm_count()) || ws_bytes < scratch(splits)))) {
             dp->cluster = true;
             int c = 1;
             while (c < splits && c < kDecMaxCluster) c *= 2;
@@ -1204,6 +1204,14 @@ int sablock_test_host_chunk(const sablock_params_t* p, int n_layers, int n_seqs,
     Plan pl;
     if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, &pl) != SABLOCK_OK) return -1;
     return host_chunk(pl, p, n_layers, n_seqs, cu, max_L, n_out);
+}
+
+// Row splits of a decoding step, negative where they are a cluster (host only).
+int sablock_test_decode_splits(const sablock_params_t* p, int n_prob, int n_rows, size_t ws_bytes)
+{
+    DecodePlan dp;
+    if (decode_plan(p, n_prob, n_rows, ws_bytes, &dp) != SABLOCK_OK) return 0;
+    return dp.cluster ? -dp.n_splits : dp.n_splits;
 }
 
 // Barrier (bit 1) and parity (bit 0) of the n-th exchange of a cluster (host only).

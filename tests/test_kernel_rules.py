@@ -137,3 +137,20 @@ def test_an_sm_takes_no_more_short_prompt_ctas_than_it_has_tensor_memory_for(rul
     n, most = rules.sablock_test_pair_smem(D), rules.sablock_test_pair_ctas()
     static = 5120                                                # barriers, row sums, log-sum-exps, sums of a warp: 4.7 KB
     assert most * (n + static + 1024) <= 228 * 1024 < (most + 1) * (n + 1024)
+
+
+@pytest.mark.parametrize("H,Hkv,D,n_prob,n_rows,two", [
+    (16, 8, 64, 1, 3200, False), (16, 8, 64, 1, 8192, False), (16, 8, 64, 3, 8192, False), (4, 1, 64, 1, 8000, False),     # rows of 128 bytes
+    (32, 8, 128, 1, 6144, False), (32, 8, 128, 1, 6145, True), (32, 8, 128, 2, 8192, True), (32, 8, 128, 3, 6400, False),
+    (32, 8, 128, 3, 8192, False), (4, 1, 128, 9, 8192, True), (4, 1, 128, 10, 8192, False), (4, 1, 128, 15, 8192, False),
+    (4, 1, 128, 16, 8192, True), (4, 1, 128, 18, 8192, True), (4, 1, 128, 19, 8192, False),
+    (8, 2, 256, 2, 6400, True), (8, 2, 256, 3, 6400, False), (16, 8, 256, 1, 8192, False), (16, 8, 256, 2, 6400, True), (8, 2, 256, 12, 7000, True),
+    (32, 8, 128, 1, 8193, True), (16, 8, 64, 1, 8193, True), (32, 8, 128, 4, 16384, False)])
+def test_decode_takes_the_form_that_measured_faster(rules, H, Hkv, D, n_prob, n_rows, two):
+    """A cluster of eight, or as many splits as two CTAs an SM allow and a second launch."""
+    p = B.make_params(H, Hkv, D, 8, torch.bfloat16)
+    rules.sablock_test_decode_splits.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_size_t]
+    n = rules.sablock_test_decode_splits(C.addressof(p), n_prob, n_rows, 1 << 30)
+    assert n == (min(296 // (Hkv * n_prob), -(-n_rows // 64)) if two else -8)
+    if n_rows <= 8192:                                           # and the cluster where there is no scratch for the other form
+        assert rules.sablock_test_decode_splits(C.addressof(p), n_prob, n_rows, 256) == -8
