@@ -354,11 +354,15 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         tmem_relinquish();
     }
     if (warp == 2) {                                             // numbers of units, and their prefix over one period
+        // (Every division here is time in which the CTA has no unit yet: one sweep, which has no A units, does without.)
         for (int i = lane; i < fa.n_sel; i += 32) {
             int ta, tb;
             fl_tiles(g, fa.sel[i], ta, tb);
-            sh.per_head[i] = (ta + 4 * fa.m - 1) / (4 * fa.m);
-            sh.units_a[i] = fa.two_sweep ? fa.group_heads * sh.per_head[i] : 0;
+            if (fa.two_sweep) {
+                const int per = (ta + 4 * fa.m - 1) / (4 * fa.m);
+                sh.per_head[i] = per;
+                sh.units_a[i] = fa.group_heads * per;
+            }
             sh.units_b[i] = fa.head_split ? tb : (tb + 3) / 4;
         }
         __syncwarp();
@@ -366,9 +370,12 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         int carry = 0;
         for (int i0 = 0; i0 < period; i0 += 32) {
             const int i = i0 + lane;
-            const int ua = i < period ? sh.units_a[((i + fa.lag) / fa.n_groups) % fa.n_sel] : 0;
-            const int c = i < period ? ua + sh.units_b[(i / fa.n_groups) % fa.n_sel] : 0;
-            if (i < period) sh.ahead_units[i] = ua;
+            int ua = 0, c = 0;
+            if (i < period) {
+                if (fa.two_sweep) ua = sh.units_a[((i + fa.lag) / fa.n_groups) % fa.n_sel];
+                c = ua + sh.units_b[fa.n_groups == 1 ? i : i / fa.n_groups];
+                sh.ahead_units[i] = ua;
+            }
             int inc = c;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -379,8 +386,10 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
             carry += __shfl_sync(0xffffffffu, inc, 31);
         }
         int ahead = 0;
-        for (int i = lane; i < min(fa.lag, fa.n_prob * fa.n_groups); i += 32) ahead += sh.units_a[(i / fa.n_groups) % fa.n_sel];
-        ahead = warp_sum(ahead);
+        if (fa.two_sweep) {
+            for (int i = lane; i < min(fa.lag, fa.n_prob * fa.n_groups); i += 32) ahead += sh.units_a[(i / fa.n_groups) % fa.n_sel];
+            ahead = warp_sum(ahead);
+        }
         if (lane == 0) { sh.prefix[period] = carry; sh.ahead = ahead; }
     }
     // What precedes this kernel on the stream is the segmentation, which it needs nothing from (queries, keys
