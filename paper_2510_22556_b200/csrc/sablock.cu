@@ -246,8 +246,8 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     // Short prompts: two kernels of few CTAs
     pl->pr_parts = (int)((tiles + kPrTiles - 1) / kPrTiles);
     const bool pair_room = flow_ok && g.Hkv <= kPrMaxHeads && (g.Hkv & (g.Hkv - 1)) == 0;
-    const long long pair_ctas = (long long)pl->pr_parts * g.Hkv * pl->n_prob, pair_max = pr_max_ctas(true) * sm_count();
-    pl->use_pair = pl->use_flow && pair_room && pair_ctas <= pr_max_ctas(p->row_lse == nullptr) * sm_count();
+    const long long pair_ctas = (long long)pl->pr_parts * g.Hkv * pl->n_prob, pair_max = (long long)kPrMaxPerSm * sm_count();
+    pl->use_pair = pl->use_flow && pair_room && pr_takes(pair_ctas, pl->pr_parts, sm_count(), g.Hkv, g.G, p->window, p->row_lse == nullptr);
     pl->use_fused = pl->use_tc && p->score_impl != SABLOCK_SCORE_TENSOR && fused_eligible(p);
     if (pl->use_tc) {
         long long work1 = tiles * g.Hkv * pl->n_prob, work2 = tiles * pl->n_prob;
@@ -1212,6 +1212,15 @@ int sablock_test_decode_splits(const sablock_params_t* p, int n_prob, int n_rows
     DecodePlan dp;
     if (decode_plan(p, n_prob, n_rows, ws_bytes, &dp) != SABLOCK_OK) return 0;
     return dp.cluster ? -dp.n_splits : dp.n_splits;
+}
+
+// The score kernels of a call: 0 multiply-adds, 1 fp32 on tensor cores, 2 the unit flow, 3 the pair for short prompts, 4 the
+// persistent kernel or, where that does not fit, two launches (host only).
+int sablock_test_score_kernels(const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, int max_L, int n_out)
+{
+    Plan pl;
+    if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, &pl) != SABLOCK_OK) return -1;
+    return !pl.use_tc ? (pl.use_x3 ? 1 : 0) : pl.use_pair ? 3 : pl.use_flow ? 2 : 4;
 }
 
 // Barrier (bit 1) and parity (bit 0) of the n-th exchange of a cluster (host only).

@@ -23,10 +23,29 @@ constexpr int kPrEpi0 = 2;                           // first epilogue warp
 constexpr int kPrEpiThreads = kPrTiles * 128;
 constexpr int kPrThreads = kPrEpi0 * 32 + kPrEpiThreads;
 constexpr int kPrMaxHeads = 8;                       // KV heads: CTAs of a cluster
-// CTAs per SM of each kernel up to which the pair takes a call (two are resident).  Two sweeps, 32 / 8 heads of 128, window 32, calls of
-// 1.7, 2.5, 3.5, 3.9 and 6.9 CTAs per SM, unit flow and pair: 53.7 / 44.1, 62.2 / 57.5, 64.3 / 63.3, 66.0 / 71.9, 81.6 / 88.4 us a call (one
-// layer of 8K, 12K, 16K and 18K tokens, four of 8K).  One sweep: 41.7 / 38.4, 42.4 / 44.4, 43.1 / 50.2.
-__host__ __device__ constexpr int pr_max_ctas(bool two_sweep) { return two_sweep ? 3 : 2; }
+// Whether the pair takes a call of so many CTAs a kernel, `parts` of them to a row block, in the place of the unit flow.  Two are
+// resident on an SM, but clusters do not fill every place: from about 7/4 CTAs per SM on a few clusters come in a second wave.  One layer,
+// heads of 128, us a call, unit flow / pair, by query and KV heads and window, at 256, 272, 296 and 440 CTAs:
+//   two sweeps  32/8, 32  52.9/43.6  52.2/49.9  56.6/54.1  61.1/60.0      8/8, 32   47.0/41.7  46.5/46.9  47.6/50.7  52.6/56.1
+//               32/8, 8   46.4/38.9  48.5/45.7  49.4/49.7  51.1/50.1      16/4, 32  50.6/46.0  51.3/46.8  57.3/56.4  65.3/66.2 (400: 63.8/61.3)
+//               8/2, 32   54.5/51.4  54.7/52.5  58.0/55.3  67.6/74.0      16/4, 8   44.3/39.1  48.5/44.1  47.9/49.5  55.8/56.2
+//   one sweep   32/8, 32  40.0/37.0  40.3/40.8  40.3/41.2                 32/8, 8   35.9/34.5  38.7/39.3  38.5/39.4
+//               16/4, 32  38.1/36.6  38.1/39.7  40.5/40.7                 8/2, 32   41.2/39.5  40.8/39.3  40.9/46.1
+// (two sweeps with eight KV heads and four layers 32/8, 32 at 384: 6 % faster, 32/8, 8: 5 %).  Beyond the first wave the pair is still ahead
+// where a CTA has products enough to pay for the exchange of its window's sums: eight KV heads of more than two query heads (16/8, 32 at 440:
+// 54.5/56.0), or four with 128 rows.  One sweep of 8/8, 32 loses a little earlier (rows of 128 bytes, 256: 35.9/37.0, 200: 33.7/32.0).
+// With one KV head there is no cluster that shares a tile's work, and every CTA merges the row sums of the whole layer: 4/1, 32,
+// two sweeps, one layer at 144, 160 and 256 CTAs 51.5/49.3  53.1/55.0  59.0/64.1, four layers at 240 8 % faster, two at 160 the same; one sweep
+// at 96 and 144 2 % faster and 38.5/40.9 (window 8 6 % faster at 160).
+constexpr int kPrMaxPerSm = 3;
+__host__ __device__ constexpr bool pr_takes(long long ctas, int parts, int sms, int Hkv, int G, int W, bool two_sweep)
+{
+    const bool first_wave = 4 * ctas <= 7LL * sms;
+    if (!two_sweep) return Hkv == 1 && W == 32 ? 4 * ctas <= 3LL * sms : Hkv == 8 && G == 1 ? 8 * ctas <= 13LL * sms : first_wave;
+    if (Hkv == 1) return ctas <= sms || (ctas <= 2LL * sms && parts <= 80);
+    if (Hkv == 2) return ctas <= 2LL * sms;
+    return first_wave || (ctas <= (long long)kPrMaxPerSm * sms && (Hkv == 8 ? G > 2 : G * W == 128));
+}
 constexpr int kPrTmemCols = kPrTiles * 128;
 // Shared memory of a CTA: its operands, and never so little that an SM could take three.  Tensor memory has room for two; a third CTA
 // would wait for its columns while its cluster's CTAs on other SMs wait for it, and hold the columns there that a third one waits for.

@@ -154,3 +154,27 @@ def test_decode_takes_the_form_that_measured_faster(rules, H, Hkv, D, n_prob, n_
     assert n == (min(296 // (Hkv * n_prob), -(-n_rows // 64)) if two else -8)
     if n_rows <= 8192:                                           # and the cluster where there is no scratch for the other form
         assert rules.sablock_test_decode_splits(C.addressof(p), n_prob, n_rows, 256) == -8
+
+
+def _kernels(rules, dtype, H, Hkv, D, W, lens, layers, lse=False, impl=B.SCORE_AUTO, n_out=64):
+    p = B.make_params(H, Hkv, D, W, dtype, score_impl=impl, **(dict(row_lse=256) if lse else {}))    # (an address that nothing reads)
+    cu = (C.c_int * (len(lens) + 1))(0)
+    for i, n in enumerate(lens):
+        cu[i + 1] = cu[i] + n
+    return rules.sablock_test_score_kernels(C.c_void_p(C.addressof(p)), layers, len(lens), cu, max(lens), n_out)
+
+
+FLOW, PAIR = 2, 3
+
+
+@pytest.mark.parametrize("H,Hkv,W,L,layers,lse,kernels", [
+    (32, 8, 32, 8192, 1, True, PAIR), (32, 8, 32, 8300, 1, True, FLOW), (32, 8, 8, 9196, 1, True, FLOW),                     # one sweep
+    (32, 8, 32, 2048, 4, True, PAIR), (32, 8, 32, 2305, 4, True, FLOW), (16, 4, 8, 16384, 1, True, PAIR), (16, 4, 8, 17388, 1, True, FLOW),
+    (8, 2, 32, 33000, 1, True, PAIR), (8, 2, 32, 36844, 1, True, FLOW),
+    (4, 1, 32, 25000, 1, True, PAIR), (4, 1, 32, 40940, 1, True, FLOW), (16, 1, 8, 40940, 1, True, PAIR),
+    (32, 8, 32, 14080, 1, False, PAIR), (32, 8, 32, 14081, 1, False, FLOW), (32, 8, 8, 14080, 1, False, PAIR),               # two sweeps
+    (16, 8, 32, 14000, 1, False, FLOW), (8, 8, 32, 7600, 1, True, PAIR), (8, 8, 32, 8192, 1, True, FLOW), (8, 8, 32, 8192, 1, False, PAIR), (8, 8, 32, 9196, 1, False, FLOW), (16, 4, 32, 28000, 1, False, PAIR), (16, 4, 8, 18412, 1, False, FLOW),
+    (16, 4, 8, 16384, 1, False, PAIR), (8, 2, 32, 37800, 1, False, PAIR), (8, 2, 32, 40940, 1, False, FLOW),
+    (4, 1, 32, 36000, 1, False, PAIR), (4, 1, 32, 40940, 1, False, FLOW), (4, 1, 32, 15000, 4, False, PAIR), (4, 1, 32, 30000, 2, False, FLOW)])
+def test_short_prompts_take_the_kernels_that_measured_faster(rules, H, Hkv, W, L, layers, lse, kernels):
+    assert _kernels(rules, torch.bfloat16, H, Hkv, 128, W, [L], layers, lse) == kernels
