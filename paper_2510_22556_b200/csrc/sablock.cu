@@ -553,15 +553,12 @@ sablock_status_t run_flow(const Plan& pl, const sablock_params_t* p, const CUten
     const long long rounds = (units_b + sms - 1) / sms * fa.group_heads * 4, split = (units_b * 4 + sms - 1) / sms * (fa.group_heads + 1);
     fa.head_split = fa.n_groups == 1 && fa.group_heads >= 4 && split < rounds;
     // A units run ahead of the B units of the same (problem, head group) by about a unit per SM: enough that the row sums
-    // are there in time, little enough that the keys are still in L2.  A unit of four tiles (20 us) that is early waits where it
-    // is, its products made: a CTA that had put two of them aside was still busy when all others were done.  Units of one
-    // tile take a quarter of that; two may be put aside, and A units run ahead by two per SM.  Two sweeps, 32 / 8 heads of
-    // 128, us a call: 16 layers of 4096 tokens 123 -> 108, 32 of 4211 226 -> 216, 32 of 16 prompts of 4K to 16K 4581 -> 4373; units of
-    // one tile, 32 layers of 1500 tokens 96 -> 89, 8 of nine prompts of up to 2214 176 -> 161.
+    // are there in time, little enough that the keys are still in L2; by two per SM where B units are one tile and take a quarter
+    // of the time (32 layers of 1500 tokens, two sweeps, 32 / 8 heads of 128: 97.7 -> 90.6 us a call; four of six prompts of up to 6000 140 -> 132).
     const long long ua = tiles * fa.group_heads / (4LL * fa.m * fa.n_sel) + 1;       // on average
     const int ahead = fa.head_split ? 2 * sms : sms, most = fa.head_split ? 64 : 16;
     fa.lag = fa.two_sweep ? (int)fmin((double)most, (double)((ahead + ua - 1) / ua)) : 0;
-    fa.max_aside = fa.head_split ? 2 : 0;
+    fa.max_aside = fl_aside(fa.head_split != 0, fa.group_heads);
     SAB_TRY(allow_smem<score_flow_tc<W, D>>(fl_smem(D)));
     SAB_TRY(launch(score_flow_tc<W, D>, dim3(sms), kFlThreads, fl_smem(D), stream, 1, tmQ, tmK, g, fa));
     prof_mark(1, stream);
@@ -1222,6 +1219,9 @@ int sablock_test_score_kernels(const sablock_params_t* p, int n_layers, int n_se
     if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, &pl) != SABLOCK_OK) return -1;
     return !pl.use_tc ? (pl.use_x3 ? 1 : 0) : pl.use_pair ? 3 : pl.use_flow ? 2 : 4;
 }
+
+// B units that a CTA of the unit flow puts aside (host only).
+int sablock_test_flow_aside(int one_tile, int group_heads) { return fl_aside(one_tile != 0, group_heads); }
 
 // Barrier (bit 1) and parity (bit 0) of the n-th exchange of a cluster (host only).
 int sablock_test_exchange(int n) { return exchange_barrier(n) * 2 + exchange_parity(n); }

@@ -10,7 +10,7 @@
 // A B unit needs the log-sum-exps of its problem, i.e. A units with smaller numbers: whoever holds those
 // is running, so waiting for them always ends and no CTA has to be resident for another's sake.  The
 // order is A(v + lag), B(v) for v = 0, 1, ...: by the time a B unit is handed out the A units it needs are
-// done or nearly so (one that is early waits; small ones are put aside while A units go on), and as little more
+// done or nearly so (one that is early waits; short ones are put aside while A units go on), and as little more
 // as possible has been read since, so that the keys of a problem of up to about 48 MB are read from L2 the
 // second time.  v counts (problem, group of KV heads); a group is as many heads as have room for their
 // log-sum-exps (1024 window rows), for the usual shapes all of them.  With the row log-sum-exps given there
@@ -48,6 +48,14 @@ constexpr int kFlMaxRows = 1024;             // window rows of a head group
 constexpr int kFlMaxSlots = 512;             // (sequence, head group) pairs of a launch
 __host__ __device__ constexpr int fl_kstages(int D) { return D == 128 ? 4 : 8; }
 __host__ __device__ constexpr int fl_smem(int D) { return 1024 + (kFlQStages + fl_kstages(D)) * 128 * D * 2; }
+
+// B units that a CTA puts aside, early ones, while it goes on with A units: two, or none.  A unit of four tiles of many heads (20 us for eight of
+// 128 rows) waits where it is, its products made: a CTA that had put two of them aside was still busy when all others were
+// done.  One of few heads is short, and waiting for it costs more than having it late; so is a unit of one tile.  Two sweeps, us a call, two
+// put aside / none, four query heads of 128 to a KV head, window 32, by KV heads: 16 layers of 9000 tokens 1: 66.3/68.7, 2: 88.8/97.5,
+// 3: 105/109, 4: 105/105, 5: 117/119, 6: 127/130, 7: 144/146, 8: 167/158; 16 of 4096 2: 58.5/59.9, 4: 82.5/82.0, 5: 90.1/80.3, 6: 101/91, 7: 111/97, 8: 121/106;
+// one query head: 9000 2: 76.6/83.8, 3: 87.0/92.3, 4: 89.9/90.8, 5: 102/101, 8: 145/137; 4096 4: 66.9/69.3, 5: 72.2/67.6, 8: 97.4/88.5.
+__host__ __device__ constexpr int fl_aside(bool one_tile, int group_heads) { return one_tile || group_heads < 5 ? 2 : 0; }
 
 struct FlowArgs {
     float c2, eps;
@@ -415,7 +423,7 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         uint32_t ks = 0, kpar = 1, qs = 0, qpar = 1;             // next stages and the parities of their last release
         int nu = 0;
         bool ok = true, drained = false;
-        // A B unit whose log-sum-exps are not there yet is put aside (two at most, where units are small) while A units, which
+        // A B unit whose log-sum-exps are not there yet is put aside (two at most, where units are short) while A units, which
         // wait for nothing, go first.
         FlUnit pend[2];
         int n_pend = 0;

@@ -15,6 +15,7 @@ pytestmark = pytest.mark.gpu
     (32, 8, 64, 16, [2214, 553, 900, 60, 1800, 129, 2000, 640, 1111], 6),
     (32, 8, 128, 32, [12000, 200], 4),
     (4, 2, 64, 32, [30000], 2),                                  # two heads: never one tile a unit
+    (8, 2, 128, 32, [9000, 300], 12), (12, 3, 128, 32, [6000], 16), (4, 4, 128, 32, [9000], 16), (20, 5, 64, 32, [4096], 16),   # few heads: put aside up to four
     (48, 12, 128, 32, [1300, 40, 2600], 5),                      # two head groups
     (32, 8, 128, 32, [19000], 1)])                               # one problem: nothing to run ahead of
 @pytest.mark.parametrize("lse", [False, True])

@@ -178,3 +178,8 @@ FLOW, PAIR = 2, 3
     (4, 1, 32, 36000, 1, False, PAIR), (4, 1, 32, 40940, 1, False, FLOW), (4, 1, 32, 15000, 4, False, PAIR), (4, 1, 32, 30000, 2, False, FLOW)])
 def test_short_prompts_take_the_kernels_that_measured_faster(rules, H, Hkv, W, L, layers, lse, kernels):
     assert _kernels(rules, torch.bfloat16, H, Hkv, 128, W, [L], layers, lse) == kernels
+
+
+@pytest.mark.parametrize("one_tile,group_heads,aside", [(0, 1, 2), (0, 2, 2), (0, 3, 2), (0, 4, 2), (0, 5, 0), (0, 8, 0), (0, 18, 0), (1, 4, 2), (1, 8, 2), (1, 16, 2)])
+def test_units_are_put_aside_where_they_are_short(rules, one_tile, group_heads, aside):
+    assert rules.sablock_test_flow_aside(one_tile, group_heads) == aside
