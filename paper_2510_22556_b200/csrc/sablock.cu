@@ -193,9 +193,10 @@ Strides v_strides(const sablock_params_t* p, long long total_tokens)
 // Bytes of a call's logits.
 size_t x3_logits(const Plan& pl) { return sizeof(float) * (size_t)pl.n_prob * pl.geo.H * pl.geo.window * pl.x3_ld; }
 
-// Builds geometry + workspace layout.  cu == NULL means one sequence of max_L tokens.
+// Builds geometry + workspace layout.  cu == NULL means one sequence of max_L tokens.  `whole`: the plan of a call of which these are some
+// layers, whose choice of kernels they follow.
 sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, long long total_tokens,
-                           int max_L, int n_out, Plan* pl, bool allow_x3 = true)
+                           int max_L, int n_out, Plan* pl, const Plan* whole = nullptr)
 {
     sablock_status_t st = validate_params(p);
     if (st != SABLOCK_OK) return st;
@@ -278,7 +279,9 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
         pl->units = (int)units;
         // fp32 on the tensor cores: one CTA per SM, whole tiles of one KV head each
         pl->x3_ld = (int)(tiles * kTcTile);
-        pl->use_x3 = allow_x3 && x3_eligible(p) && x3_logits(*pl) <= kX3MaxBytes;
+        const long long macs = (long long)n_layers * total_tokens * g.H * g.window * g.D;
+        pl->use_x3 = x3_eligible(p) && x3_logits(*pl) <= kX3MaxBytes &&
+                     (whole ? whole->use_x3 : x3_pays(macs, g.G, p->row_lse == nullptr));
         pl->x3_tpc = (int)((tiles * g.Hkv * pl->n_prob + sm_count() - 1) / sm_count());
         if (pl->x3_tpc > tiles) pl->x3_tpc = (int)tiles;
         pl->x3_chunks = (int)((tiles + pl->x3_tpc - 1) / pl->x3_tpc);
@@ -935,7 +938,7 @@ HostStreams* host_streams()
 bool plan_inside(const Plan& whole, const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, int max_L, int n_out,
                  Plan* pl)
 {
-    if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, pl, whole.use_x3) != SABLOCK_OK || pl->n_regions != whole.n_regions)
+    if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, pl, &whole) != SABLOCK_OK || pl->n_regions != whole.n_regions)
         return false;
     if (pl->use_tc != whole.use_tc || pl->use_x3 != whole.use_x3 || pl->use_flow != whole.use_flow || pl->use_fused != whole.use_fused) return false;
     if (pl->use_tc && (long long)pl->n_prob * pl->geo.H * pl->geo.window < kTcTile) return false;

@@ -28,6 +28,16 @@ constexpr size_t kX3MaxBytes = 64u << 20;            // logits of a call that th
 constexpr int kX3SumThreads = 1024;                  // half of that for fewer window rows in all than
 constexpr int kX3SumManyRows = 512;                  // (512 / 1024 threads: 4096 tokens, 1024 rows 52.8 / 47.7 us a call; 5000, 64 rows 39.3 / 43.6)
 constexpr int kX3SumTokens = 32;                     // tokens of a CTA of the second kernel
+// Whether this path is the faster one.  Two sweeps: always.  With the row log-sum-exps given, one pass of multiply-adds over the keys is all that it replaces,
+// and small calls are done with that before the operands here are split and the logits have gone through scratch.  us a call of one
+// layer, multiply-adds / pieces, by millions of multiply-adds (tokens):
+//   32/8 heads of 128, window 32  39 (300) 35.8/39.5   92 (700) 43.9/40.2     window 16  46 (700) 36.3/38.8   98 (1500) 47.2/42.7
+//                      window 8   49 (1500) 40.4/41.8  98 (3000) 48.9/47.0  164 (5000) 71.2/49.8
+//   8/2 heads of 128, window 16   49 (3000) 41.2/41.6  82 (5000) 50.3/45.3     4/1 of 64, window 32  12 (1500) 32.5/39.1  67 (8192) 46.7/44.5
+// With one query head to a KV head its keys are split for fewer of them, and the line lies higher: 8/8 heads of 128, window 32  49 (1500)
+// 39.6/41.1  98 (3000) 46.8/49.5  164 (5000) 56.4/51.3, window 16  82 (5000) 48.8/49.9  134 (8192) 64.3/53.1.
+constexpr long long kX3MinMacs = 80000000, kX3MinMacsSingle = 100000000;
+__host__ __device__ constexpr bool x3_pays(long long macs, int G, bool two_sweep) { return two_sweep || macs >= (G == 1 ? kX3MinMacsSingle : kX3MinMacs); }
 __host__ __device__ constexpr int x3_smem(int D) { return 1024 + (D / 64 + 2) * 3 * kX3Piece; }
 
 struct X3Args {

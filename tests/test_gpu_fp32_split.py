@@ -58,6 +58,13 @@ def test_scores(H, Hkv, D, W, lens, layers, lse):
         assert err[B.SCORE_AUTO] <= 1.5 * err[B.SCORE_SIMT] + 1e-7
 
 
+@pytest.mark.parametrize("H,Hkv,D,W,lens,layers", [(6, 2, 128, 5, [22000], 1), (5, 1, 64, 25, [11000], 1), (16, 2, 64, 12, [700], 10),
+                                                   (4, 1, 64, 16, [20001], 1), (3, 3, 128, 1, [26049], 10), (8, 8, 128, 4, [8100, 30], 4)])
+def test_given_normalisers_of_calls_large_enough(H, Hkv, D, W, lens, layers):
+    """(smaller ones are left to the multiply-adds)"""
+    test_scores(H, Hkv, D, W, lens, layers, True)
+
+
 @pytest.mark.parametrize("offset", [0, 1])
 def test_strided_keys(offset):
     """Keys inside a larger buffer, with gaps between heads, tokens and layers; one element further on their rows are not on

@@ -183,3 +183,16 @@ def test_short_prompts_take_the_kernels_that_measured_faster(rules, H, Hkv, W, L
 @pytest.mark.parametrize("one_tile,group_heads,aside", [(0, 1, 2), (0, 2, 2), (0, 3, 2), (0, 4, 2), (0, 5, 0), (0, 8, 0), (0, 18, 0), (1, 4, 2), (1, 8, 2), (1, 16, 2)])
 def test_units_are_put_aside_where_they_are_short(rules, one_tile, group_heads, aside):
     assert rules.sablock_test_flow_aside(one_tile, group_heads) == aside
+
+
+SIMT, X3 = 0, 1
+
+
+@pytest.mark.parametrize("H,Hkv,D,W,L,layers,lse,kernels", [
+    (32, 8, 128, 32, 300, 1, True, SIMT), (32, 8, 128, 32, 700, 1, True, X3), (32, 8, 128, 16, 700, 1, True, SIMT), (32, 8, 128, 16, 1500, 1, True, X3),
+    (32, 8, 128, 8, 1500, 1, True, SIMT), (32, 8, 128, 8, 1500, 3, True, X3), (4, 1, 64, 16, 512, 1, True, SIMT), (8, 8, 128, 32, 3000, 1, True, SIMT),
+    (8, 8, 128, 32, 5000, 1, True, X3), (4, 1, 64, 16, 512, 1, False, X3), (32, 8, 128, 32, 300, 1, False, X3), (1, 1, 64, 1, 200, 1, False, X3),
+    (32, 8, 128, 32, 16384, 1, False, X3), (32, 8, 128, 32, 16385, 1, False, SIMT), (32, 8, 128, 32, 4096, 4, False, X3),     # 64 MB of logits
+    (32, 8, 128, 32, 4096, 5, False, SIMT)])
+def test_fp32_scores_take_the_kernels_that_measured_faster(rules, H, Hkv, D, W, L, layers, lse, kernels):
+    assert _kernels(rules, torch.float32, H, Hkv, D, W, [L], layers, lse) == kernels
