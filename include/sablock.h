@@ -123,7 +123,9 @@ size_t sablock_params_sizeof(void);   /* sizeof(sablock_params_t) as the library
 /* Bytes of device scratch needed for a call over n_layers x n_seqs problems whose
  * sequences have at most max_L tokens and total_tokens tokens in all.  Single-problem
  * entry points use n_layers = n_seqs = 1, total_tokens = max_L = L.  Returns 0 on
- * invalid arguments. */
+ * invalid arguments.  (fp32 calls that keep their logits, see sablock_score_impl_t, need up to 64 MB for them; with what the
+ * same call needs under SABLOCK_SCORE_SIMT they run too, on those kernels.  The bytes do not grow with every one of the sizes: a
+ * buffer that several calls share has the largest of their sizes.) */
 size_t sablock_workspace_bytes(const sablock_params_t *p, long long total_tokens, int max_L,
                                int n_seqs, int n_layers);
 

@@ -312,10 +312,7 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
                                      : (size_t)pl->n_prob * pl->units * pl->n_chunks * pl->simt.gb * g.window;
     const size_t pair_n = pair_room ? (size_t)(pair_ctas < pair_max ? pair_ctas : pair_max) * g.G * g.window : 0;
     const size_t flow_n = flow_ok ? (size_t)pl->n_prob * g.Hkv * (pl->fl_parts + (pl->fl_parts + kFlMerge - 1) / kFlMerge) * g.G * g.window : 0;
-    // (Scratch that only calls up to some size use is kept in larger ones' plans too: a workspace that is sized for the longest
-    // prompt serves the shorter ones.)
-    const bool x3_room = !pl->use_tc && x3_eligible(p);
-    const size_t x3_n = x3_room ? ((size_t)sm_count() + (size_t)pl->n_prob * g.Hkv) * g.G * g.window : 0;
+    const size_t x3_n = pl->use_x3 ? ((size_t)sm_count() + (size_t)pl->n_prob * g.Hkv) * g.G * g.window : 0;
     size_t most = part_n > flow_n ? part_n : flow_n;
     if (x3_n > most) most = x3_n;
     if (pair_n > most) most = pair_n;
@@ -326,10 +323,24 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     take(&Plan::o_keep, sizeof(unsigned) * (size_t)pl->n_prob * pl->keep_words);
     take(&Plan::o_phi, sizeof(double) * ntok);
     take(&Plan::o_fpart, pl->use_fused ? sizeof(float2) * (size_t)kFuMaxCtas * kFuPartSlots * 128 : 0);
-    const size_t x3_bytes = x3_room ? x3_logits(*pl) : 0;                  // (rows start on 32-byte boundaries wherever the workspace does)
-    take(&Plan::o_x3, x3_room ? (x3_bytes < kX3MaxBytes ? x3_bytes : kX3MaxBytes) + 32 : 0);
+    take(&Plan::o_x3, pl->use_x3 ? x3_logits(*pl) + 32 : 0);               // (rows start on 32-byte boundaries wherever the workspace does)
     pl->total = o;
     return SABLOCK_OK;
+}
+
+// The plan of a call with ws_bytes of workspace.  The logits of the fp32 kernels are most of theirs, up to 64 MB: a workspace
+// without room for them (sized for a larger call, which does not use them, or for one with the row log-sum-exps given) is still good for the
+// multiply-adds.
+sablock_status_t plan_call(const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, long long total_tokens, int max_L, int n_out,
+                           const void* ws, size_t ws_bytes, Plan* pl)
+{
+    sablock_status_t st = make_plan(p, n_layers, n_seqs, cu, total_tokens, max_L, n_out, pl);
+    if (st == SABLOCK_OK && pl->use_x3 && ws_bytes < pl->total) {
+        const Plan without = {};
+        st = make_plan(p, n_layers, n_seqs, cu, total_tokens, max_L, n_out, pl, &without);
+    }
+    if (st != SABLOCK_OK) return st;
+    return !ws || ws_bytes < pl->total ? SABLOCK_ERR_WORKSPACE_TOO_SMALL : SABLOCK_OK;
 }
 
 template <typename T> T* at(void* ws, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(ws) + off); }
@@ -1216,10 +1227,10 @@ int sablock_test_decode_splits(const sablock_params_t* p, int n_prob, int n_rows
 
 // The score kernels of a call: 0 multiply-adds, 1 fp32 on tensor cores, 2 the unit flow, 3 the pair for short prompts, 4 the
 // persistent kernel or, where that does not fit, two launches (host only).
-int sablock_test_score_kernels(const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, int max_L, int n_out)
+int sablock_test_score_kernels(const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, int max_L, int n_out, size_t ws_bytes)
 {
     Plan pl;
-    if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, &pl) != SABLOCK_OK) return -1;
+    if (plan_call(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, p, ws_bytes, &pl) != SABLOCK_OK) return -1;
     return !pl.use_tc ? (pl.use_x3 ? 1 : 0) : pl.use_pair ? 3 : pl.use_flow ? 2 : 4;
 }
 
@@ -1261,8 +1272,7 @@ sablock_status_t sablock_segment(const sablock_params_t* p, const int* token_ids
     t_launches = 0;
     if (!p || L <= p->window) return SABLOCK_ERR_INVALID_ARG;
     Plan pl;
-    SAB_TRY(make_plan(p, 1, 1, nullptr, L, L, p->window + 1, &pl));
-    if (!ws || ws_bytes < pl.total) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
+    SAB_TRY(plan_call(p, 1, 1, nullptr, L, L, p->window + 1, ws, ws_bytes, &pl));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     return run_segment(pl, p, token_ids, seg_id, seg_start, n_seg, ws, st);
 }
@@ -1297,8 +1307,7 @@ sablock_status_t sablock_score(const sablock_params_t* p, const void* q_win, con
     Plan pl;
     // no budget here: "output rows" = the window alone, so that no sequence with a compressible
     // token (L > W) counts as one that is returned unchanged
-    SAB_TRY(make_plan(p, 1, 1, nullptr, L, L, p->window, &pl));
-    if (!ws || ws_bytes < pl.total) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
+    SAB_TRY(plan_call(p, 1, 1, nullptr, L, L, p->window, ws, ws_bytes, &pl));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     SAB_TRY(zero_control(pl, ws, st));
     float* e_buf = e ? e : at<float>(ws, pl.o_e);
@@ -1318,8 +1327,7 @@ sablock_status_t sablock_select(const sablock_params_t* p, const float* s_refine
     Cands cands;
     SAB_TRY(check_candidates(block_candidates, n_candidates, &cands));
     Plan pl;
-    SAB_TRY(make_plan(p, 1, 1, nullptr, L, L, rows_out(p, budget), &pl));
-    if (!ws || ws_bytes < pl.total) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
+    SAB_TRY(plan_call(p, 1, 1, nullptr, L, L, rows_out(p, budget), ws, ws_bytes, &pl));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // the retained count is written to workspace (n_seg slot is free here)
     return run_select(pl, p, nullptr, nullptr, const_cast<float*>(s_refined), seg_start, n_seg, cands, out_idx,
@@ -1361,8 +1369,7 @@ sablock_status_t sablock_compress_layers(const sablock_params_t* p, int n_layers
     Cands cands;
     SAB_TRY(check_candidates(block_candidates, n_candidates, &cands));
     Plan pl;
-    SAB_TRY(make_plan(p, n_layers, n_seqs, cu_seqlens, cu_seqlens[n_seqs], max_L, rows_out(p, budget), &pl));
-    if (!ws || ws_bytes < pl.total) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
+    SAB_TRY(plan_call(p, n_layers, n_seqs, cu_seqlens, cu_seqlens[n_seqs], max_L, rows_out(p, budget), ws, ws_bytes, &pl));
     return run_pass(pl, p, cands, q_win, k, v, token_ids, out_k, out_v, out_idx, out_n_keep, ws, static_cast<cudaStream_t>(stream));
 }
 
@@ -1450,8 +1457,7 @@ sablock_status_t sablock_compress_layers_host(const sablock_params_t* p, int n_l
     Cands cands;
     SAB_TRY(check_candidates(block_candidates, n_candidates, &cands));
     Plan pl;
-    SAB_TRY(make_plan(p, n_layers, n_seqs, cu_seqlens, cu_seqlens[n_seqs], max_L, rows_out(p, budget), &pl));
-    if (!ws || ws_bytes < pl.total) return SABLOCK_ERR_WORKSPACE_TOO_SMALL;
+    SAB_TRY(plan_call(p, n_layers, n_seqs, cu_seqlens, cu_seqlens[n_seqs], max_L, rows_out(p, budget), ws, ws_bytes, &pl));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const size_t es = elem_size(p);
     const size_t total = (size_t)cu_seqlens[n_seqs];

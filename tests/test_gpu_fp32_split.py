@@ -107,3 +107,27 @@ def test_a_key_that_is_no_number(value):
     p = B.make_params(H, Hkv, D, W, torch.float32, b.bitmap, cfg.vocab)
     s, _, status = _scores(p, b, [L], 1, 64)
     assert bool(torch.isnan(s[0, :L - W]).all()) and status == 6
+
+
+@pytest.mark.parametrize("lse", [False, True])
+def test_a_workspace_without_room_for_logits(lse):
+    """One sized for the multiply-adds, between two guards: the call takes those, and what they compute."""
+    H, Hkv, D, W, L = 32, 8, 128, 32, 3000
+    cfg, b = _batch(H, Hkv, D, W, [L], 1, 64)
+    kw = dict(row_lse=synth.prefill_row_lse(b.q_win, b.k, b.cu_seqlens)) if lse else {}
+    plain = B.make_params(H, Hkv, D, W, torch.float32, b.bitmap, cfg.vocab, score_impl=B.SCORE_SIMT, **kw)
+    p = B.make_params(H, Hkv, D, W, torch.float32, b.bitmap, cfg.vocab, **kw)
+    n = B.workspace_bytes(plain, L, L)
+    assert n < B.workspace_bytes(p, L, L)
+    buf = torch.full((n + 512,), 0x5a, dtype=torch.uint8, device="cuda")
+    res = []
+    for q, ws in ((plain, torch.empty(n, dtype=torch.uint8, device="cuda")), (p, buf[256: 256 + n])):
+        out = B.compress_layers(q, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, 64, cfg.candidates, ws)
+        torch.cuda.synchronize()
+        assert B.read_status(ws) == 0
+        res.append([B.workspace_view(q, ws, x, L, L)[0, :L - W].clone() for x in ("s", "e", "s_refined")] + [out.out_idx, out.out_k])
+    assert all(torch.equal(x, y) for x, y in zip(*res))
+    assert bool((buf[:256] == 0x5a).all()) and bool((buf[256 + n:] == 0x5a).all())
+    with pytest.raises(B.SablockError) as err:
+        B.compress_layers(p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, 64, cfg.candidates, buf[256: 255 + n])
+    assert err.value.code == 3

@@ -156,12 +156,12 @@ def test_decode_takes_the_form_that_measured_faster(rules, H, Hkv, D, n_prob, n_
         assert rules.sablock_test_decode_splits(C.addressof(p), n_prob, n_rows, 256) == -8
 
 
-def _kernels(rules, dtype, H, Hkv, D, W, lens, layers, lse=False, impl=B.SCORE_AUTO, n_out=64):
+def _kernels(rules, dtype, H, Hkv, D, W, lens, layers, lse=False, impl=B.SCORE_AUTO, n_out=64, ws_bytes=1 << 40):
     p = B.make_params(H, Hkv, D, W, dtype, score_impl=impl, **(dict(row_lse=256) if lse else {}))    # (an address that nothing reads)
     cu = (C.c_int * (len(lens) + 1))(0)
     for i, n in enumerate(lens):
         cu[i + 1] = cu[i] + n
-    return rules.sablock_test_score_kernels(C.c_void_p(C.addressof(p)), layers, len(lens), cu, max(lens), n_out)
+    return rules.sablock_test_score_kernels(C.c_void_p(C.addressof(p)), layers, len(lens), cu, max(lens), n_out, C.c_size_t(ws_bytes))
 
 
 FLOW, PAIR = 2, 3
@@ -196,3 +196,28 @@ SIMT, X3 = 0, 1
     (32, 8, 128, 32, 4096, 5, False, SIMT)])
 def test_fp32_scores_take_the_kernels_that_measured_faster(rules, H, Hkv, D, W, L, layers, lse, kernels):
     assert _kernels(rules, torch.float32, H, Hkv, D, W, [L], layers, lse) == kernels
+
+
+def _scratch(rules, dtype, H, Hkv, D, W, L, layers, impl=B.SCORE_AUTO):
+    p = B.make_params(H, Hkv, D, W, dtype, score_impl=impl)
+    rules.sablock_workspace_bytes.restype = C.c_size_t
+    return rules.sablock_workspace_bytes(C.c_void_p(C.addressof(p)), C.c_longlong(L), L, 1, layers)
+
+
+@pytest.mark.parametrize("H,Hkv,D,W", [(32, 8, 128, 32), (4, 1, 64, 16), (8, 8, 64, 8)])
+def test_scratch_for_logits_is_that_of_calls_which_have_them(rules, H, Hkv, D, W):
+    """A call that is too large for kept logits needs what it needs on the multiply-adds, and its workspace, or one sized for
+    those, is good for smaller calls too: they then take the multiply-adds themselves."""
+    f32 = torch.float32
+    for L, layers in ((131072, 1), (4096, 32), (16384, 40)):
+        if _kernels(rules, f32, H, Hkv, D, W, [L], layers) == SIMT:
+            assert _scratch(rules, f32, H, Hkv, D, W, L, layers) == _scratch(rules, f32, H, Hkv, D, W, L, layers, B.SCORE_SIMT)
+    for L in (200, 259, 312, 1000, 4096):
+        full, plain = (_scratch(rules, f32, H, Hkv, D, W, L, 1, impl) for impl in (B.SCORE_AUTO, B.SCORE_SIMT))
+        logits = H * W * -(-L // 128) * 128 * 4
+        assert plain < full and logits <= full - plain + 512 * 1024          # (the partial row sums are smaller or larger by some)
+        assert _kernels(rules, f32, H, Hkv, D, W, [L], 1, ws_bytes=full) == X3
+        assert _kernels(rules, f32, H, Hkv, D, W, [L], 1, ws_bytes=full - 1) == SIMT
+        assert _kernels(rules, f32, H, Hkv, D, W, [L], 1, ws_bytes=plain) == SIMT
+        assert _kernels(rules, f32, H, Hkv, D, W, [L], 1, ws_bytes=plain - 1) == -1
+    assert _kernels(rules, f32, H, Hkv, D, W, [259], 1, ws_bytes=_scratch(rules, f32, H, Hkv, D, W, 312, 1)) >= 0
