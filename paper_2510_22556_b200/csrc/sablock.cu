@@ -248,7 +248,8 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     pl->pr_parts = (int)((tiles + kPrTiles - 1) / kPrTiles);
     const bool pair_room = flow_ok && g.Hkv <= kPrMaxHeads && (g.Hkv & (g.Hkv - 1)) == 0;
     const long long pair_ctas = (long long)pl->pr_parts * g.Hkv * pl->n_prob, pair_max = (long long)kPrMaxPerSm * sm_count();
-    pl->use_pair = pl->use_flow && pair_room && pr_takes(pair_ctas, pl->pr_parts, sm_count(), g.Hkv, g.G, p->window, p->row_lse == nullptr);
+    pl->use_pair = pl->use_flow && pair_room && (!whole || whole->use_pair) &&
+                   pr_takes(pair_ctas, pl->pr_parts, sm_count(), g.Hkv, g.G, p->window, p->row_lse == nullptr);
     pl->use_fused = pl->use_tc && p->score_impl != SABLOCK_SCORE_TENSOR && fused_eligible(p);
     if (pl->use_tc) {
         long long work1 = tiles * g.Hkv * pl->n_prob, work2 = tiles * pl->n_prob;
@@ -944,14 +945,16 @@ HostStreams* host_streams()
 }
 
 // The plan of n_layers of a larger call's layers inside that call's workspace; false if a region would not
-// hold what it needs, or if so few layers would go to other kernels than the whole call (the tensor maps need 128
-// rows of queries).
+// hold what it needs, or if so few layers cannot go to the kernels of the whole call (the tensor maps need 128
+// rows of queries).  What the pass over host buffers selects is what the pass over device buffers does.
 bool plan_inside(const Plan& whole, const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, int max_L, int n_out,
                  Plan* pl)
 {
     if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, pl, &whole) != SABLOCK_OK || pl->n_regions != whole.n_regions)
         return false;
-    if (pl->use_tc != whole.use_tc || pl->use_x3 != whole.use_x3 || pl->use_flow != whole.use_flow || pl->use_fused != whole.use_fused) return false;
+    if (pl->use_tc != whole.use_tc || pl->use_x3 != whole.use_x3 || pl->use_flow != whole.use_flow || pl->use_pair != whole.use_pair ||
+        pl->use_fused != whole.use_fused)
+        return false;
     if (pl->use_tc && (long long)pl->n_prob * pl->geo.H * pl->geo.window < kTcTile) return false;
     for (int i = 0; i < pl->n_regions; ++i) {
         if (pl->regions[i].bytes > whole.regions[i].bytes) return false;
@@ -1217,6 +1220,8 @@ int sablock_test_host_chunk(const sablock_params_t* p, int n_layers, int n_seqs,
     return host_chunk(pl, p, n_layers, n_seqs, cu, max_L, n_out);
 }
 
+static int score_kernels(const Plan& pl) { return !pl.use_tc ? (pl.use_x3 ? 1 : 0) : pl.use_pair ? 3 : pl.use_flow ? 2 : 4; }
+
 // Row splits of a decoding step, negative where they are a cluster (host only).
 int sablock_test_decode_splits(const sablock_params_t* p, int n_prob, int n_rows, size_t ws_bytes)
 {
@@ -1231,7 +1236,15 @@ int sablock_test_score_kernels(const sablock_params_t* p, int n_layers, int n_se
 {
     Plan pl;
     if (plan_call(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, p, ws_bytes, &pl) != SABLOCK_OK) return -1;
-    return !pl.use_tc ? (pl.use_x3 ? 1 : 0) : pl.use_pair ? 3 : pl.use_flow ? 2 : 4;
+    return score_kernels(pl);
+}
+
+// The same of `layers` of the call's layers, as a host-buffer pass takes them.
+int sablock_test_chunk_kernels(const sablock_params_t* p, int n_layers, int n_seqs, const int* cu, int max_L, int n_out, int layers)
+{
+    Plan pl, part;
+    if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, &pl) != SABLOCK_OK) return -1;
+    return plan_inside(pl, p, layers, n_seqs, cu, max_L, n_out, &part) ? score_kernels(part) : -1;
 }
 
 // B units that a CTA of the unit flow puts aside (host only).

@@ -221,3 +221,22 @@ def test_scratch_for_logits_is_that_of_calls_which_have_them(rules, H, Hkv, D, W
         assert _kernels(rules, f32, H, Hkv, D, W, [L], 1, ws_bytes=plain) == SIMT
         assert _kernels(rules, f32, H, Hkv, D, W, [L], 1, ws_bytes=plain - 1) == -1
     assert _kernels(rules, f32, H, Hkv, D, W, [259], 1, ws_bytes=_scratch(rules, f32, H, Hkv, D, W, 312, 1)) >= 0
+
+
+@pytest.mark.parametrize("dtype,H,Hkv,D,W,lens,layers,lse", [
+    (torch.bfloat16, 32, 8, 128, 32, [8192], 4, False), (torch.bfloat16, 32, 8, 128, 32, [8192], 4, True), (torch.bfloat16, 32, 8, 128, 8, [2500], 9, False),
+    (torch.bfloat16, 4, 1, 64, 16, [30000], 9, False), (torch.bfloat16, 32, 8, 128, 32, [2048], 4, False), (torch.bfloat16, 32, 8, 128, 32, [3000, 100], 20, True),
+    (torch.float32, 32, 8, 128, 32, [4096], 5, False), (torch.float32, 32, 8, 128, 32, [4096], 4, False), (torch.float32, 32, 8, 128, 16, [700], 4, True)])
+def test_layers_of_a_host_pass_take_the_kernels_of_the_whole_call(rules, dtype, H, Hkv, D, W, lens, layers, lse):
+    """A few layers alone would take other kernels than all of them.  Inside the whole call they take its own, or are no chunk of it (-1:
+    they would not fit its workspace)."""
+    p = B.make_params(H, Hkv, D, W, dtype, **(dict(row_lse=256) if lse else {}))
+    cu = (C.c_int * (len(lens) + 1))(0)
+    for i, n in enumerate(lens):
+        cu[i + 1] = cu[i] + n
+    whole = _kernels(rules, dtype, H, Hkv, D, W, lens, layers, lse)
+    at = C.c_void_p(C.addressof(p))
+    for some in range(1, layers):
+        assert rules.sablock_test_chunk_kernels(at, layers, len(lens), cu, max(lens), 64, some) in (whole, -1)
+    per = rules.sablock_test_host_chunk(at, layers, len(lens), cu, max(lens), 64)
+    assert rules.sablock_test_chunk_kernels(at, layers, len(lens), cu, max(lens), 64, per) == whole
