@@ -352,8 +352,7 @@ score_x3_logits(const Geo g, const X3Args a)
 // there are fewer positions than warps): the head-summed attention of Eq. 3 is a sum down the rows of logits, 128
 // bytes per warp and row.  Then a warp per token, a lane per window position (Eqs. 4, 6).
 __global__ void __launch_bounds__(kX3SumThreads, 1)
-score_x3_sum(const Geo g, const float* __restrict__ x, int ld, float eps, const float* __restrict__ lse2, float* __restrict__ s_out,
-             float* __restrict__ e_out)
+score_x3_sum(const Geo g, const float* x, int ld, float eps, const float* lse2, float* s_out, float* e_out)
 {
     constexpr int kMaxWarps = kX3SumThreads / 32;
     const int n_warps = blockDim.x >> 5;
@@ -366,9 +365,10 @@ score_x3_sum(const Geo g, const float* __restrict__ x, int ld, float eps, const 
     if (geo_identity(g, seq) || t0 >= T) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int hs = W >= n_warps ? 1 : n_warps / W;     // shares of the heads
-    for (int i = threadIdx.x; i < H * W; i += blockDim.x) ls[i] = lse2[(size_t)p * H * W + i];
+    for (int i = threadIdx.x; i < H * W; i += blockDim.x) ls[i] = __ldcg(lse2 + (size_t)p * H * W + i);
     __syncthreads();
-    // (32-bit positions: 64 MB of logits at most)
+    // (32-bit positions: 64 MB of logits at most.  Loads from L2: this kernel may have started before the logits were written, so they
+    // are no constants of its lifetime, which the read-only path wants.)
     const float* xp = x + (size_t)p * H * W * ld;
     for (int item = warp; item < W * hs; item += n_warps) {
         const int w = item % W, share = item / W;
@@ -380,14 +380,14 @@ score_x3_sum(const Geo g, const float* __restrict__ x, int ld, float eps, const 
         for (; n >= 16; n -= 16, at += 16 * step, lh += 16 * rows) {
             float v[16];
 #pragma unroll
-            for (unsigned u = 0; u < 16; ++u) v[u] = __ldg(xp + (at + u * step));
+            for (unsigned u = 0; u < 16; ++u) v[u] = __ldcg(xp + (at + u * step));
 #pragma unroll
             for (unsigned u = 0; u < 16; ++u) acc[u & 3] += exp2f(v[u] - lh[u * rows]);
         }
         if (n > 0) {
             float v[16];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) v[u] = __ldg(xp + (at + (unsigned)min(u, n - 1) * step));
+            for (int u = 0; u < 16; ++u) v[u] = __ldcg(xp + (at + (unsigned)min(u, n - 1) * step));
 #pragma unroll
             for (int u = 0; u < 16; ++u) acc[u & 3] += u < n ? exp2f(v[u] - lh[(unsigned)min(u, n - 1) * rows]) : 0.f;
         }
