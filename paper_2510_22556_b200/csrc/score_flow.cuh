@@ -121,12 +121,6 @@ __device__ __forceinline__ bool elect_one()
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
     return p != 0;
 }
-// mbar_wait by a whole warp; the result is uniform.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag)
-{
-    if (__any_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
-}
 __device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 #define FL_WAIT(code, expr) ((expr) ? true : (note_giveup(fa.status, code), false))
@@ -540,18 +534,19 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
     } else if (warp == 2) {
         // ------------------------------------------------------------------ log-sum-exps of B units
         int nb = 0;
+        bool ok = true;                                          // (waits and votes as in the epilogue below)
         for (int nu = 0;; ++nu) {
             const int slot = nu % kFlUnits;
-            if (!FL_WAIT(15, mbar_wait(smem_u32(&sh.ufull[slot]), (nu / kFlUnits) & 1, abort_flag))) break;
+            ok = FL_WAIT(15, mbar_wait(smem_u32(&sh.ufull[slot]), (nu / kFlUnits) & 1, abort_flag)) && ok;
             const int kind = sh.unit[slot].kind, prob = sh.unit[slot].prob, j0 = sh.unit[slot].j0, nh = sh.unit[slot].nh,
                       group = sh.unit[slot].group;
-            __syncwarp();
+            if (!__all_sync(0xffffffffu, ok)) break;
             if (lane == 0) mbar_arrive(smem_u32(&sh.uempty[slot]));
             if (kind == 2) break;
             if (kind == 0) continue;
             const int b = nb & 1;
-            if (!FL_WAIT(16, mbar_wait(smem_u32(&sh.lempty[b]), ((nb >> 1) & 1) ^ 1, abort_flag))) break;
-            if (fa.two_sweep && !FL_WAIT(13, wait_counter(fa.done + prob * fa.n_groups + group, nh, abort_flag, fa.status))) break;
+            ok = FL_WAIT(16, mbar_wait(smem_u32(&sh.lempty[b]), ((nb >> 1) & 1) ^ 1, abort_flag)) && ok;
+            if (fa.two_sweep) ok = FL_WAIT(13, wait_counter(fa.done + prob * fa.n_groups + group, nh, abort_flag, fa.status)) && ok;
             const size_t at = (size_t)prob * g.H * W + (size_t)j0 * R;
             float* dst = sh.lse[b];
 #pragma unroll 8
@@ -567,17 +562,18 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         // row block to arrive merges the partials, in order.  Reference exponents are integers, so
         // rescaling is exact.
         int na = 0;
+        bool ok = true;
         for (int nu = 0;; ++nu) {
             const int slot = nu % kFlUnits;
-            if (!FL_WAIT(14, mbar_wait(smem_u32(&sh.ufull[slot]), (nu / kFlUnits) & 1, abort_flag))) break;
+            ok = FL_WAIT(14, mbar_wait(smem_u32(&sh.ufull[slot]), (nu / kFlUnits) & 1, abort_flag)) && ok;
             const int kind = sh.unit[slot].kind, prob = sh.unit[slot].prob, j = sh.unit[slot].j0, index = sh.unit[slot].index,
                       group = sh.unit[slot].group;
-            __syncwarp();
+            if (!__all_sync(0xffffffffu, ok)) break;
             if (lane == 0) mbar_arrive(smem_u32(&sh.uempty[slot]));
             if (kind == 2) break;
             if (kind == 1) continue;
             const int b = na & 3;
-            if (!FL_WAIT(6, mbar_wait(smem_u32(&sh.afull[b]), (na >> 2) & 1, abort_flag))) break;
+            ok = FL_WAIT(6, mbar_wait(smem_u32(&sh.afull[b]), (na >> 2) & 1, abort_flag)) && ok;
             ++na;
             const int pj = prob * g.Hkv + j;
             float2* part = fa.part + (size_t)pj * (fa.max_part_units + fa.max_grp) * R;
@@ -625,22 +621,25 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         const uint32_t acc_addr = lane_addr + (uint32_t)set * 128u;
         const float c2 = fa.c2;
         uint32_t n_mine = 0, na = 0, nb = 0, n_hs = 0;
+        // The waits inside a unit are those of lanes, and a lane that gives up goes on with whatever is there: lanes that left alone would be
+        // missing where a warp reads tensor memory.  All leave together, at the next unit's record (a vote a unit; one a
+        // tile cost 1 %: 16 layers of 4096 tokens 104.5 -> 105.6 us).
+        bool ok = true;
         // waits for this set's next product; the accumulator is given back with release()
-        auto product = [&]() -> bool {
-            const bool ok = FL_WAIT(7, mbar_wait(smem_u32(&sh.tfull[set]), n_mine & 1u, abort_flag));
+        auto product = [&]() {
+            ok = FL_WAIT(7, mbar_wait(smem_u32(&sh.tfull[set]), n_mine & 1u, abort_flag)) && ok;
             ++n_mine;
+            __syncwarp();
             tc_fence_after();
-            return ok;
         };
         auto release = [&]() {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sh.tempty[set]));
         };
-        bool ok = true;
-        for (int nu = 0; ok; ++nu) {
+        for (int nu = 0;; ++nu) {
             const int slot = nu % kFlUnits;
-            if (!FL_WAIT(17, mbar_wait(smem_u32(&sh.ufull[slot]), (nu / kFlUnits) & 1, abort_flag))) break;
+            if (!__all_sync(0xffffffffu, FL_WAIT(17, mbar_wait(smem_u32(&sh.ufull[slot]), (nu / kFlUnits) & 1, abort_flag)) && ok)) break;
             const FlUnit& u = sh.unit[slot];
             const int kind = u.kind, nt = u.nt;
             if (kind == 2) break;
@@ -651,7 +650,7 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                 RowSum rs;
                 rs.reset();
                 for (int i = set; i < nt; i += 4) {
-                    if (!product()) { ok = false; break; }
+                    product();
                     if (q4 >= fl_shift(R, set) && (q4 - fl_shift(R, set)) * 32 < R) {
                         const int tok0 = (tile0 + i) * kTcTile;
                         const bool mask = tok0 + kTcTile - 1 > Tn;
@@ -674,9 +673,8 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                         release();
                     }
                 }
-                if (!ok) break;
                 const int ab = na & 3;
-                if (!FL_WAIT(11, mbar_wait(smem_u32(&sh.aempty[ab]), ((na >> 2) & 1u) ^ 1u, abort_flag))) break;
+                ok = FL_WAIT(11, mbar_wait(smem_u32(&sh.aempty[ab]), ((na >> 2) & 1u) ^ 1u, abort_flag)) && ok;
                 ++na;
                 if (r0 >= 0 && r0 < R) sh.sums[ab][set][r0] = make_float2(rs.m, rs.l);       // (a set without tiles: zero)
                 __syncwarp();
@@ -688,7 +686,7 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                 ++nb;
                 const bool split = fa.head_split != 0;
                 const int tile = u.tile0 + (split ? 0 : set);
-                if (!FL_WAIT(8, mbar_wait(smem_u32(&sh.lfull[lb]), lpar, abort_flag))) break;
+                ok = FL_WAIT(8, mbar_wait(smem_u32(&sh.lfull[lb]), lpar, abort_flag)) && ok;
                 if (split || set < nt) {
                     float acc[W];
 #pragma unroll
@@ -696,14 +694,14 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                     float* carry = fa.carry + ((size_t)(u.index % kFlCarryRing) * fa.max_tiles + tile) * W * 128 + row;
                     int* bdone = fa.bdone + (size_t)prob * fa.max_tiles + tile;
                     if (u.group > 0) {                           // what the earlier head groups of this tile have summed
-                        if (lane == 0) ok = FL_WAIT(18, wait_counter(bdone, 4 * u.group, abort_flag, fa.status));
-                        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-                        if (!ok) break;
+                        bool there = true;
+                        if (lane == 0) there = FL_WAIT(18, wait_counter(bdone, 4 * u.group, abort_flag, fa.status));
+                        if (!__shfl_sync(0xffffffffu, there ? 1 : 0, 0)) break;
 #pragma unroll
                         for (int i = 0; i < W; ++i) acc[i] = __ldcg(carry + i * 128);
                     }
                     for (int h = split ? set : 0; h < nh; h += split ? 4 : 1) {
-                        if (!product()) { ok = false; break; }
+                        product();
                         const float* nl = &sh.lse[lb][h * R];
 #pragma unroll 1
                         for (int c = 0; c * 32 < R; ++c) {
@@ -720,7 +718,6 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                             }
                         }
                     }
-                    if (!ok) break;
                     if (split) {
                         // the sets' sums of a token meet in tensor memory: a set leaves its sums where its last
                         // logits were, set 0 adds them in order and then gives back all four accumulators
@@ -733,7 +730,8 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&sh.hs[q4]));
                         if (set == 0) {
-                            if (!FL_WAIT(20, mbar_wait(smem_u32(&sh.hs[q4]), n_hs & 1u, abort_flag))) break;
+                            ok = FL_WAIT(20, mbar_wait(smem_u32(&sh.hs[q4]), n_hs & 1u, abort_flag)) && ok;
+                            __syncwarp();
                             tc_fence_after();
 #pragma unroll
                             for (int x = 1; x < 4; ++x)
@@ -755,11 +753,11 @@ score_flow_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                     } else if (u.group < fa.n_groups - 1) {
                         if (u.group == 0) {                      // the slot's previous tenant is through
                             const int prev = lane == 0 ? fl_carry_tenant(g, fa, u.index, tile) : -1;
+                            bool there = true;
                             if (prev >= 0)
-                                ok = FL_WAIT(19, wait_counter(fa.bdone + (size_t)prev * fa.max_tiles + tile, 4 * fa.n_groups,
-                                                              abort_flag, fa.status));
-                            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-                            if (!ok) break;
+                                there = FL_WAIT(19, wait_counter(fa.bdone + (size_t)prev * fa.max_tiles + tile, 4 * fa.n_groups,
+                                                                 abort_flag, fa.status));
+                            if (!__shfl_sync(0xffffffffu, there ? 1 : 0, 0)) break;
                         }
 #pragma unroll
                         for (int i = 0; i < W; ++i) __stcg(carry + i * 128, acc[i]);

@@ -162,7 +162,7 @@ score_p1_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         float m2 = -INFINITY, l = 0.f;
         for (int it = 0; it < ntl; ++it) {
             const int acc = it & 1, aph = (it >> 1) & 1;
-            if (!mbar_wait(smem_u32(&sh.tfull[acc]), aph, abort_flag)) break;
+            if (!mbar_wait_warp(smem_u32(&sh.tfull[acc]), aph, abort_flag)) break;
             tc_fence_after();
             const int tok0 = (tile0 + it) * kTcTile;
             const bool need_mask = tok0 + kTcTile - 1 > Tn;
@@ -310,7 +310,7 @@ score_p2_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             for (int j = 0; j < Hkv; ++j) {
                 const int it = tl * Hkv + j;
                 const int acc = it & 1, aph = (it >> 1) & 1;
-                if (!mbar_wait(smem_u32(&sh.tfull[acc]), aph, abort_flag)) { ok = false; break; }
+                if (!mbar_wait_warp(smem_u32(&sh.tfull[acc]), aph, abort_flag)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t taddr = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)acc * 128u;
                 const float* lj = lse_s + j * R;
