@@ -26,6 +26,11 @@ using namespace sab;
 namespace {
 
 thread_local int t_launches = 0;
+#ifdef SABLOCK_TEST_HOOKS
+int g_test_no_pair = 0;            // test builds: short prompts take the unit flow
+#else
+constexpr int g_test_no_pair = 0;
+#endif
 
 // ---- optional per-stage event timing ---------------------------------------------------
 constexpr int kProfStages = 9;
@@ -248,7 +253,7 @@ sablock_status_t make_plan(const sablock_params_t* p, int n_layers, int n_seqs, 
     pl->pr_parts = (int)((tiles + kPrTiles - 1) / kPrTiles);
     const bool pair_room = flow_ok && g.Hkv <= kPrMaxHeads && (g.Hkv & (g.Hkv - 1)) == 0;
     const long long pair_ctas = (long long)pl->pr_parts * g.Hkv * pl->n_prob, pair_max = (long long)kPrMaxPerSm * sm_count();
-    pl->use_pair = pl->use_flow && pair_room && (!whole || whole->use_pair) &&
+    pl->use_pair = pl->use_flow && pair_room && (!whole || whole->use_pair) && !g_test_no_pair &&
                    pr_takes(pair_ctas, pl->pr_parts, sm_count(), g.Hkv, g.G, p->window, p->row_lse == nullptr);
     pl->use_fused = pl->use_tc && p->score_impl != SABLOCK_SCORE_TENSOR && fused_eligible(p);
     if (pl->use_tc) {
@@ -563,10 +568,7 @@ sablock_status_t run_flow(const Plan& pl, const sablock_params_t* p, const CUten
     fa.group_heads = pl.fl_heads; fa.n_groups = pl.fl_groups;
     fa.m = pl.fl_m;
     const int sms = sm_count();
-    // four tiles per B unit, or one with the heads spread over the sets where that takes fewer rounds
-    units_b *= g.n_layers;
-    const long long rounds = (units_b + sms - 1) / sms * fa.group_heads * 4, split = (units_b * 4 + sms - 1) / sms * (fa.group_heads + 1);
-    fa.head_split = fa.n_groups == 1 && fa.group_heads >= 4 && split < rounds;
+    fa.head_split = fl_one_tile(units_b * g.n_layers, sms, fa.n_groups, fa.group_heads);
     // A units run ahead of the B units of the same (problem, head group) by about a unit per SM: enough that the row sums
     // are there in time, little enough that the keys are still in L2; by two per SM where B units are one tile and take a quarter
     // of the time (32 layers of 1500 tokens, two sweeps, 32 / 8 heads of 128: 97.7 -> 90.6 us a call; four of six prompts of up to 6000 140 -> 132).
@@ -1245,6 +1247,16 @@ int sablock_test_chunk_kernels(const sablock_params_t* p, int n_layers, int n_se
     Plan pl, part;
     if (make_plan(p, n_layers, n_seqs, cu, cu[n_seqs], max_L, n_out, &pl) != SABLOCK_OK) return -1;
     return plan_inside(pl, p, layers, n_seqs, cu, max_L, n_out, &part) ? score_kernels(part) : -1;
+}
+
+// Whether short prompts take the unit flow (host only).
+void sablock_test_no_pair(int on) { g_test_no_pair = on; }
+
+// Whether the unit flow takes a call of equal sequences in units of one tile (host only).
+int sablock_test_flow_one_tile(int n_kv_heads, int window_rows, int n_layers, int tiles)
+{
+    const int most = kFlMaxRows / window_rows, groups = (n_kv_heads + most - 1) / most;
+    return fl_one_tile((long long)n_layers * ((tiles + 3) / 4), sm_count(), groups, (n_kv_heads + groups - 1) / groups);
 }
 
 // B units that a CTA of the unit flow puts aside (host only).

@@ -57,6 +57,13 @@ __host__ __device__ constexpr int fl_smem(int D) { return 1024 + (kFlQStages + f
 // one query head: 9000 2: 76.6/83.8, 3: 87.0/92.3, 4: 89.9/90.8, 5: 102/101, 8: 145/137; 4096 4: 66.9/69.3, 5: 72.2/67.6, 8: 97.4/88.5.
 __host__ __device__ constexpr int fl_aside(bool one_tile, int group_heads) { return one_tile || group_heads < 5 ? 2 : 0; }
 
+// Whether B units are one tile, with the heads spread over the sets, instead of four: where that takes fewer rounds.
+__host__ __device__ constexpr bool fl_one_tile(long long units_b, int sms, int n_groups, int group_heads)
+{
+    return n_groups == 1 && group_heads >= 4 &&
+           (units_b * 4 + sms - 1) / sms * (group_heads + 1) < (units_b + sms - 1) / sms * group_heads * 4;
+}
+
 struct FlowArgs {
     float c2, eps;
     float2* part;            // [problem * Hkv + j][max_part_units + max_grp][R] row statistics (m, l) of the A units and of groups

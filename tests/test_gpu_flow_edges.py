@@ -1,8 +1,9 @@
 """The unit-flow score kernel at the edges of its schedule: lengths around a token tile and a unit, every
 number of window rows per KV head, long sequences of few window rows, several head groups (more than 1024 window rows:
 their sums pass through scratch that has fewer slots than there are problems) in one and two sweeps, packed
-sequences of very different length among them ones that are returned unchanged.  Reference: the
-scores and entropies in float64 on the stored values.
+sequences of very different length among them ones that are returned unchanged.  Short prompts with one, two, four or eight KV heads take
+the pair of kernels of score_pair.cuh in the product, and the same cases are run on the unit flow with a test build that leaves them to
+it.  Reference: the scores and entropies in float64 on the stored values.
 
 Tolerance: a logit is an fp32 sum of D <= 128 exact products, partial sums below 64 in log2 units, so its
 rounding error is about sqrt(128) * 2^-24 * 64 = 4e-5, times ln 2 the relative error of a weight: 3e-5; the
@@ -15,8 +16,35 @@ import torch
 
 import synth
 from paper_2510_22556_b200 import binding as B
+from paper_2510_22556_b200.build import build_test_hooks
 
 pytestmark = pytest.mark.gpu
+
+
+FLOW, PAIR = 2, 3
+
+
+@pytest.fixture(scope="module")
+def hooked():
+    return B._load(build_test_hooks())
+
+
+@pytest.fixture
+def on_the_flow(hooked):
+    """The test build for the duration of a test, with every call that could take the pair on the unit flow."""
+    saved, B._lib = B._lib, hooked
+    hooked.sablock_test_no_pair(1)
+    yield hooked
+    hooked.sablock_test_no_pair(0)
+    B._lib = saved
+
+
+def _kernels(lib, H, Hkv, D, W, lens, n_layers, lse=False):
+    p = B.make_params(H, Hkv, D, W, torch.bfloat16, **(dict(row_lse=256) if lse else {}))
+    cu = (B.C.c_int * (len(lens) + 1))(0)
+    for i, n in enumerate(lens):
+        cu[i + 1] = cu[i] + n
+    return lib.sablock_test_score_kernels(B.C.c_void_p(B.C.addressof(p)), n_layers, len(lens), cu, max(lens), 64, B.C.c_size_t(1 << 40))
 
 
 def _reference(q, k, W):
@@ -68,10 +96,25 @@ def test_lengths(L, lse):
     _run(32, 8, 128, 32, [L], 1, 64, lse)
 
 
+@pytest.mark.parametrize("L", [129, 160, 161, 255, 511, 512, 513, 545, 2047, 2049, 8193])
+@pytest.mark.parametrize("lse", [False, True])
+def test_lengths_on_the_flow(on_the_flow, L, lse):
+    assert _kernels(on_the_flow, 32, 8, 128, 32, [L], 1, lse) == FLOW
+    _run(32, 8, 128, 32, [L], 1, 64, lse)
+
+
 @pytest.mark.parametrize("H,Hkv,W,D", [(8, 8, 8, 128), (4, 2, 8, 64), (6, 2, 8, 128), (10, 2, 8, 64), (16, 2, 16, 128), (6, 2, 32, 128),
                                        (32, 2, 8, 128), (3, 3, 32, 64), (8, 2, 32, 64), (14, 2, 16, 64)])
 @pytest.mark.parametrize("lse", [False, True])
 def test_window_rows(H, Hkv, W, D, lse):
+    _run(H, Hkv, D, W, [1500], 3, 64, lse)
+
+
+@pytest.mark.parametrize("H,Hkv,W,D", [(8, 8, 8, 128), (6, 2, 8, 64), (10, 2, 8, 64), (16, 2, 16, 128), (6, 2, 32, 128),
+                                       (32, 2, 8, 128), (8, 2, 32, 64), (14, 2, 16, 64), (7, 1, 16, 128), (4, 4, 32, 64)])
+@pytest.mark.parametrize("lse", [False, True])
+def test_window_rows_on_the_flow(on_the_flow, H, Hkv, W, D, lse):
+    assert _kernels(on_the_flow, H, Hkv, D, W, [1500], 3, lse) == FLOW
     _run(H, Hkv, D, W, [1500], 3, 64, lse)
 
 
@@ -126,3 +169,11 @@ def test_a_key_that_is_no_number(H, Hkv, D, W, value, L):
     s = B.workspace_view(p, ws, "s", L, L)[0, :L - W]
     assert bool(torch.isnan(rs).all()) and bool(torch.isnan(s).all())
     assert B.read_status(ws) == 6
+
+
+@pytest.mark.parametrize("H,Hkv,D,W", [(32, 8, 128, 32), (16, 4, 64, 8), (8, 2, 128, 16), (48, 12, 64, 8)])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("L", [700, 5000, 9000])
+def test_a_key_that_is_no_number_on_the_flow(on_the_flow, H, Hkv, D, W, value, L):
+    assert _kernels(on_the_flow, H, Hkv, D, W, [L], 1) == FLOW
+    test_a_key_that_is_no_number(H, Hkv, D, W, value, L)

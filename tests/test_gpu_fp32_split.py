@@ -131,3 +131,51 @@ def test_a_workspace_without_room_for_logits(lse):
     with pytest.raises(B.SablockError) as err:
         B.compress_layers(p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, 64, cfg.candidates, buf[256: 255 + n])
     assert err.value.code == 3
+
+
+@pytest.mark.parametrize("H,Hkv,D,W,lens,layers", [(32, 8, 128, 32, [4096], 1), (4, 1, 64, 16, [512], 1), (8, 2, 128, 8, [16000], 1), (32, 8, 128, 16, [900, 2100], 3)])
+def test_the_same_from_run_to_run(H, Hkv, D, W, lens, layers):
+    """Whichever CTA of a row block comes last merges the partial sums, in one order."""
+    cfg, b = _batch(H, Hkv, D, W, lens, layers, 64)
+    p = B.make_params(H, Hkv, D, W, torch.float32, b.bitmap, cfg.vocab)
+    first = None
+    for _ in range(20):
+        s, e, status = _scores(p, b, lens, layers, 64)
+        assert status == 0
+        res = [torch.cat([x[l, b.cu_seqlens[i]: b.cu_seqlens[i + 1] - W] for l in range(layers) for i in range(len(lens))]) for x in (s, e)]
+        if first is None:
+            first = [x.clone() for x in res]
+        assert torch.equal(first[0], res[0]) and torch.equal(first[1], res[1])
+
+
+@pytest.mark.parametrize("L", [16384, 16385])
+def test_the_largest_call_that_keeps_its_logits(L):
+    """64 MB of them, and a token more."""
+    H, Hkv, D, W = 32, 8, 128, 32
+    cfg, b = _batch(H, Hkv, D, W, [L], 1, 64)
+    p = B.make_params(H, Hkv, D, W, torch.float32, b.bitmap, cfg.vocab)
+    assert (B.workspace_bytes(p, L, L) > 64 << 20) == (L == 16384)
+    s, e, status = _scores(p, b, [L], 1, 64)
+    rs, re = _reference(b.q_win[0, 0], b.k[0], W)
+    assert status == 0
+    assert float(((s[0, :L - W].double() - rs) / rs).abs().max()) <= (4e-5 if L == 16384 else 2e-4)
+    assert float((e[0, :L - W].double() - re).abs().max()) <= (1e-4 if L == 16384 else 4e-4)
+
+
+@pytest.mark.parametrize("H,Hkv,D,W,L", [(32, 8, 128, 32, 256), (32, 8, 128, 32, 1025), (32, 8, 128, 32, 4096), (32, 8, 128, 32, 8192), (4, 1, 64, 16, 512),
+                                         (8, 8, 64, 8, 5000), (32, 8, 128, 8, 8192)])
+def test_no_further_from_64_bits_than_multiply_adds(H, Hkv, D, W, L):
+    """What the file says of its sums: their error is no larger than that of a chain of fp32 multiply-adds, in its root mean square (a twentieth for
+    the sample) nor, though tensor memory loses what it drops in one direction, in its mean."""
+    cfg, b = _batch(H, Hkv, D, W, [L], 1, 64)
+    rs, _ = _reference(b.q_win[0, 0], b.k[0], W)
+    rms, mean = {}, {}
+    for impl in (B.SCORE_AUTO, B.SCORE_SIMT):
+        p = B.make_params(H, Hkv, D, W, torch.float32, b.bitmap, cfg.vocab, score_impl=impl)
+        s, _, status = _scores(p, b, [L], 1, 64)
+        assert status == 0
+        d = (s[0, :L - W].double() - rs) / rs
+        rms[impl], mean[impl] = float(d.pow(2).mean().sqrt()), float(d.mean())
+    print(f"{H}/{Hkv} {D} W{W} L{L}: rms {rms[B.SCORE_AUTO]:.3g} / {rms[B.SCORE_SIMT]:.3g}, mean {mean[B.SCORE_AUTO]:+.3g} / {mean[B.SCORE_SIMT]:+.3g}")
+    assert rms[B.SCORE_AUTO] <= 1.05 * rms[B.SCORE_SIMT]
+    assert abs(mean[B.SCORE_AUTO]) <= rms[B.SCORE_SIMT]

@@ -109,11 +109,11 @@ def test_score_kernel_handover_gives_up(hooked):
     assert B.read_status_detail(ws) == (0, 0, 0) and torch.equal(out.out_idx, good)
 
 
-@pytest.mark.parametrize("H,Hkv,D,W,lens,layers", [(32, 8, 128, 32, [8192], 1),              # few tiles: the sets share the heads
+@pytest.mark.parametrize("H,Hkv,D,W,lens,layers", [(32, 8, 128, 32, [8192], 1),              # (the pair of kernels for short prompts)
                                                    (32, 8, 128, 32, [3000, 700, 5000], 6),   # four tiles a unit
                                                    (64, 16, 64, 32, [900, 2500], 3)])        # head groups waiting for one another
 def test_unit_flow_gives_up(hooked, H, Hkv, D, W, lens, layers):
-    """The kernel that the default choice takes: the row sums of one unit are missing, so one problem's log-sum-exps never
+    """The kernels that the default choice takes: the row sums of one unit are missing, so one problem's log-sum-exps never
     come, and whoever waits for them runs out."""
     cfg = synth.Config("t", layers, H, Hkv, D, W, tuple(lens), (256,), (1, 2, 4), "bf16", 5000, 8, 2.0, 20, (0.4,), 9)
     b = synth.make_batch(cfg, device="cuda")
@@ -174,3 +174,10 @@ def test_short_prompt_and_fp32_kernels_give_up(hooked, hook, dtype, H, Hkv, D, W
     out = B.compress_layers(*args)
     torch.cuda.synchronize()
     assert B.read_status_detail(ws) == (0, 0, 0) and torch.equal(out.out_idx, good)
+
+
+@pytest.mark.parametrize("H,Hkv,D,W,lens,layers", [(32, 8, 128, 32, [1500], 16), (32, 8, 64, 8, [2000, 700], 12), (16, 4, 128, 32, [20000], 1)])
+def test_unit_flow_with_units_of_one_tile_gives_up(hooked, H, Hkv, D, W, lens, layers):
+    """Few tiles: the sets share the heads."""
+    assert hooked.sablock_test_flow_one_tile(Hkv, H // Hkv * W, layers * len(lens), -(-max(lens) // 128))
+    test_unit_flow_gives_up(hooked, H, Hkv, D, W, lens, layers)

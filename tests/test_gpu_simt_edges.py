@@ -96,3 +96,35 @@ def test_an_infinite_key_under_given_normalisers(H, Hkv, layers, L):
     s = B.workspace_view(p, ws, "s", L, L, 1, layers)[:, :L - W]
     assert bool((s[:, t] == float("inf")).all())
     assert int(torch.isfinite(s).sum()) == s.numel() - layers
+
+
+@pytest.mark.parametrize("H,Hkv,D,W,L", [
+    (4, 1, 64, 16, 129), (4, 1, 64, 16, 512), (32, 8, 128, 32, 700), (32, 8, 128, 32, 4097), (8, 8, 64, 8, 2500), (3, 3, 128, 1, 200),
+    (16, 8, 64, 7, 6001), (5, 1, 64, 12, 3000), (6, 2, 128, 25, 900), (7, 1, 64, 16, 400)])
+@pytest.mark.parametrize("layers", [1, 5])
+@pytest.mark.parametrize("lse", [False, True])
+def test_fp32_scores_of_shapes_that_the_tensor_cores_could_take(H, Hkv, D, W, L, layers, lse):
+    """(larger calls of these shapes come here by themselves)"""
+    cfg = synth.Config("t", layers, H, Hkv, D, W, (L,), (W + 20,), (1, 2, 4), "f32", 5000, 8, 2.0, 20, (), 3)
+    b = synth.make_batch(cfg, device="cuda")
+    kw = dict(row_lse=synth.prefill_row_lse(b.q_win, b.k, b.cu_seqlens)) if lse else {}
+    p = B.make_params(H, Hkv, D, W, torch.float32, b.bitmap, cfg.vocab, score_impl=B.SCORE_SIMT, **kw)
+    ws = B.alloc_workspace(p, L, L, 1, layers)
+    B.compress_layers(p, b.q_win, b.k, b.v, b.token_ids, b.cu_seqlens, W + 20, cfg.candidates, ws)
+    torch.cuda.synchronize()
+    assert B.read_status(ws) == 0
+    s = B.workspace_view(p, ws, "s", L, L, 1, layers)
+    e = B.workspace_view(p, ws, "e", L, L, 1, layers)
+    for l in range(layers):
+        rs, re = _reference(b.q_win[l, 0], b.k[l], W)
+        assert float(((s[l, :L - W].double() - rs).abs() / rs).max()) <= 2e-4
+        assert float((e[l, :L - W].double() - re).abs().max()) <= 4e-4
+
+
+@pytest.mark.parametrize("H,Hkv", [(5, 1), (6, 2), (7, 1), (8, 2)])
+@pytest.mark.parametrize("layers,L", [(1, 300), (8, 6000)])
+def test_an_infinite_key_under_given_normalisers_on_multiply_adds(monkeypatch, H, Hkv, layers, L):
+    """The same where the call is told to take the multiply-adds: the variant of their second pass with absent heads."""
+    plain = B.make_params
+    monkeypatch.setattr(B, "make_params", lambda *a, **kw: plain(*a, score_impl=B.SCORE_SIMT, **kw))
+    test_an_infinite_key_under_given_normalisers(H, Hkv, layers, L)
