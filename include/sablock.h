@@ -45,14 +45,15 @@ typedef enum {
 typedef enum { SABLOCK_F32 = 0, SABLOCK_BF16 = 1 } sablock_dtype_t;
 
 /* Which kernel family computes the attention scores.  AUTO picks, for bf16, head_dim 64/128, window
- * 8/16/32 and at most 128 window rows per KV head, the unit-flow tensor-core kernel (short prompts: two
- * kernels of small CTAs in its place), except for two sweeps
+ * 8/16/32 and at most 128 window rows per KV head, the unit-flow tensor-core kernel (short prompts with one, two, four or
+ * eight KV heads: two kernels of small CTAs in its place), except for two sweeps
  * (row_lse not given) over more than 48 MB of keys per sequence and layer in the shape of the persistent
  * tensor-core kernel (head_dim 128, window 32, four query heads per KV head, at most 7 token tiles of 128
  * per CTA), which takes those.  For fp32, head_dim 64/128, window up to 32, at most 128 window rows per KV
- * head, rows on 16-byte boundaries and at most 64 MB of logits: tensor-core kernels on operands split into three bf16
- * pieces.  Everything else runs on the SIMT kernels (with row_lse these run their second pass only).  FUSED forces the persistent kernel, TENSOR the two-launch tensor-core kernels; both
- * fail with SABLOCK_ERR_UNSUPPORTED where they cannot run. */
+ * head, rows on 16-byte boundaries and at most 64 MB of logits in all layers together: tensor-core kernels on operands split into
+ * three bf16 pieces (with row_lse from 80 to 100 million multiply-adds on; in a workspace with room for the logits).
+ * Everything else runs on the SIMT kernels (with row_lse these run their second pass only).  FUSED forces the
+ * persistent kernel, TENSOR the two-launch tensor-core kernels; both fail with SABLOCK_ERR_UNSUPPORTED where they cannot run. */
 typedef enum { SABLOCK_SCORE_AUTO = 0, SABLOCK_SCORE_SIMT = 1, SABLOCK_SCORE_TENSOR = 2, SABLOCK_SCORE_FUSED = 3 }
     sablock_score_impl_t;
 
@@ -286,8 +287,9 @@ sablock_status_t sablock_decode_attention(const sablock_params_t *p, int n_prob,
  * milliseconds of each stage interval; it returns the number of intervals (0 if the slot
  * was never used).  sablock_profile_stage_name(i) names interval i.  The stages are:
  * segment, score_pass1, score_merge, score_pass2, refine, topb, search, index, compact.  Where one kernel is several
- * stages the first of them has its time and the others are zero: score_pass1 for the tensor kernels in one launch,
- * score_pass2 for the single sweep of the others, search for everything from the refinement to the index list.
+ * stages the first of them has its time and the others are zero: score_pass1 for the unit flow and the persistent kernel,
+ * score_pass2 for the single sweep of the kernels for short prompts, in two launches and on multiply-adds (fp32 on split operands: the
+ * logits are score_pass1, the sums score_pass2, in either mode), search for everything from the refinement to the index list.
  * sablock_compress_layers_host takes all layers at once while timing is enabled (one slot, like the device call; its
  * copies then do not overlap with its kernels). */
 #define SABLOCK_PROFILE_MAX_SLOTS 512

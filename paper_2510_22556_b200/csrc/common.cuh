@@ -73,12 +73,20 @@ __device__ __forceinline__ bool geo_identity(const Geo& g, int seq) { return geo
 __device__ __forceinline__ float ld_as_float(const float* p) { return *p; }
 __device__ __forceinline__ float ld_as_float(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 
-// Programmatic dependent launch.  Every kernel of the library is launched with the attribute that
-// lets it start while its predecessor on the stream still runs, and opens with pdl_wait(), which
-// returns once the predecessor has completed and its writes are visible: nothing but set-up that
-// touches no global memory comes before it.  pdl_launch() lets the successor's CTAs be scheduled as
-// soon as there is room for them; they then wait in their own pdl_wait().  What this hides is launch
-// latency (about 2 us from kernel to kernel becomes about 1), which short calls are made of.
+// Programmatic dependent launch.  Every kernel of the library but the cooperative one is launched with the attribute that
+// lets it start while its predecessor on the stream still runs.  pdl_launch() lets the successor's CTAs be scheduled as
+// soon as all CTAs of this kernel have called it (or ended) and there is room; pdl_wait() returns once the predecessor has completed and
+// its writes are visible.  What this hides is launch latency (about 2 us from kernel to kernel becomes about 1), which short calls are made of.
+// What holds:
+//  - Every kernel calls pdl_wait() in every CTA before it ends, so that a kernel's completion means that of all before it on the stream.
+//  - A kernel that calls pdl_wait() before pdl_launch() fences what came before it off from its successor: nothing that precedes it on the stream
+//    still runs when the successor starts.  The segmentation, clear_kernel and lse_import_kernel do.
+//  - All others open with pdl_wait(), before any access to global memory, except the four that come right behind such a fence and need nothing from
+//    it but what it wrote before its pdl_launch() (the cleared counters): score_flow_tc, score_rows_tc, score_heads_tc with given log-sum-exps
+//    and score_x3_logits read queries and keys, and write scores, logits and partial sums, before they wait.  (score_heads_tc behind
+//    score_rows_tc waits before it reads the row sums and writes.)  A kernel put between the fence and one of them has to be a fence itself.
+//  - A kernel whose successor takes tensor memory too (score_rows_tc) calls pdl_launch() only once it has its own: the successor's CTAs take theirs
+//    and then wait for it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

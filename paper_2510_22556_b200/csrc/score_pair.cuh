@@ -11,7 +11,7 @@
 // ticket, load, product, exponentials, then three trips through global memory to merge the row sums (two levels, each store,
 // fence, counter, load) and a fourth to wait for the result, and all heads of a tile on one SM: 27 us for 8192
 // tokens, of which 4.3 are exponentials.  Here every trip but one is gone, nothing waits for a CTA that is still to come, and the
-// exponentials of a tile are spread over eight SMs: 8 us and 11 us, a call 52.4 -> 43.1 (2681 tokens of window 16 44.3 -> 36.6).
+// exponentials of a tile are spread over eight SMs: 8 us and 11 us, a call 52-54 -> 43-45, from one GPU to another (2681 tokens of window 16 44.3 -> 36.6).
 #pragma once
 #include "common.cuh"
 #include "score_flow.cuh"
