@@ -55,6 +55,7 @@ __host__ __device__ constexpr int fl_smem(int D) { return 1024 + (kFlQStages + f
 // put aside / none, four query heads of 128 to a KV head, window 32, by KV heads: 16 layers of 9000 tokens 1: 66.3/68.7, 2: 88.8/97.5,
 // 3: 105/109, 4: 105/105, 5: 117/119, 6: 127/130, 7: 144/146, 8: 167/158; 16 of 4096 2: 58.5/59.9, 4: 82.5/82.0, 5: 90.1/80.3, 6: 101/91, 7: 111/97, 8: 121/106;
 // one query head: 9000 2: 76.6/83.8, 3: 87.0/92.3, 4: 89.9/90.8, 5: 102/101, 8: 145/137; 4096 4: 66.9/69.3, 5: 72.2/67.6, 8: 97.4/88.5.
+// (Not at every size, for the last units of a launch fall as they fall: eight heads, window 16, 2 layers of 30000 tokens 103/92, 8 of 43930 297/309, 8 of 60000 388/379.)
 __host__ __device__ constexpr int fl_aside(bool one_tile, int group_heads) { return one_tile || group_heads < 5 ? 2 : 0; }
 
 // Whether B units are one tile, with the heads spread over the sets, instead of four: where that takes fewer rounds.
