@@ -995,6 +995,7 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
     if ((G != 1 && G != 2 && G != 4) || p->head_dim > kDecMaxD || (row_bytes != 128 && row_bytes != 256 && row_bytes != 512))
         return SABLOCK_ERR_UNSUPPORTED;
     const long long per_split = (long long)p->n_kv_heads * n_prob;
+    const int sms = sm_count();
     dp->cluster = false;
     long long splits;
     size_t need = 0;
@@ -1005,7 +1006,7 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
         // eight (dec_two_launches: which do not), and so does one that would have a single split more: the rows that a CTA then
         // reads more take less time than the second launch and the trip through scratch.  And a
         // cache of at most kDecClusterRows whose caller has brought no scratch for the other form.
-        splits = 2LL * sm_count() / per_split;
+        splits = 2LL * sms / per_split;
         const long long by_rows = (n_rows + 63) / 64;
         if (splits > by_rows) splits = by_rows;
         if (splits < 1) splits = 1;
@@ -1014,7 +1015,7 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
         // as the batch shrinks the splits of the others become more: what a batch of nine splits asks for serves them.)
         need = splits <= kDecMaxCluster || n_rows <= kDecClusterRows ? 256 : scratch(splits);
         if (splits <= kDecClusterSplits ||
-            (n_rows <= kDecClusterRows && (!dec_two_launches(row_bytes, n_rows, per_split, sm_count()) || ws_bytes < scratch(splits)))) {
+            (n_rows <= kDecClusterRows && (!dec_two_launches(row_bytes, n_rows, per_split, sms) || ws_bytes < scratch(splits)))) {
             dp->cluster = true;
             int c = 1;
             while (c < splits && c < kDecMaxCluster) c *= 2;
@@ -1024,7 +1025,7 @@ sablock_status_t decode_plan(const sablock_params_t* p, int n_prob, int n_rows, 
         // Row splits: at least 256 rows each, and no more CTAs than two waves of the device (two CTAs
         // per SM are resident): the merge that follows reads one partial result per split.
         splits = (n_rows + kDecThreads - 1) / kDecThreads;
-        const long long cap = 4LL * sm_count() / per_split;
+        const long long cap = 4LL * sms / per_split;
         if (splits > cap) splits = cap < 1 ? 1 : cap;
     }
     if (splits > kDecMaxSplits) splits = kDecMaxSplits;
